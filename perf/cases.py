@@ -13,7 +13,10 @@ Kinds of case:
   gated     one layer with the convolutional local attention gate, forward and backward.
   features  the positional features of one layer from their generator's weights, and the weights' gradients.
 """
+import math
+
 import torch
+import torch.nn.functional as F
 
 from paper_2603_06738_b200 import binding
 
@@ -110,7 +113,7 @@ def _generator(case, source):
     return [source.f32(rows, dh, sigma=rows ** -0.5), source.f32(dh, sigma=0.1), source.f32(dh, r, sigma=dh ** -0.5), source.f32(dh, r, sigma=dh ** -0.5)]
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
     source = _Source(seed)
     if case["kind"] == "features":
         n = case["window"] ** 2
@@ -130,16 +133,22 @@ def prepare(case, seed):
     if case["kind"] == "infer":
         return state
     state["dout"] = source.bf16(*image)
-    shape = (B, H, W, heads, d, r, case["window"])
-    if case.get("headwise"):
-        need = binding.rib_window_attn_bwd_headwise_workspace(n * r, *shape)
-    else:
-        need = binding.rib_window_attn_bwd_workspace(*shape)
-    state["workspace"] = torch.empty(need, dtype=torch.uint8, device="cuda")
     if case["kind"] == "gated":
         D = heads * d
         state["x"] = source.bf16(B, H, W, D)
         state["conv"] = [source.f32(D, 3, 3, sigma=1 / 3), source.f32(D, sigma=0.1), source.f32(D, D, sigma=D ** -0.5), source.f32(D, sigma=0.1)]
+    return state
+
+
+def prepare(case, seed):
+    state = _inputs(case, seed)
+    if case["kind"] in ("train", "gated"):
+        shape = tuple(case[k] for k in ("B", "H", "W", "heads", "d", "r", "window"))
+        if case.get("headwise"):
+            need = binding.rib_window_attn_bwd_headwise_workspace(case["window"] ** 2 * case["r"], *shape)
+        else:
+            need = binding.rib_window_attn_bwd_workspace(*shape)
+        state["workspace"] = torch.empty(need, dtype=torch.uint8, device="cuda")
     return state
 
 
@@ -174,6 +183,105 @@ def run(state):
         return out, lse, binding.rib_window_attn_bwd_headwise(*args, out, lse, dout, window, shift, workspace=workspace)
     out, lse = binding.rib_window_attn_fwd(*args, window, shift)
     return out, lse, binding.rib_window_attn_bwd(*args, out, lse, dout, window, shift, workspace=workspace)
+
+
+def _to_windows(t, window, shift):
+    """[B, H, W, ...] laid over the extended map, rolled by the shift and cut: [B * windows, window^2, ...]."""
+    B, H, W = t.shape[:3]
+    Hp, Wp = -(-H // window) * window, -(-W // window) * window
+    t = F.pad(t, [0, 0] * (t.dim() - 3) + [0, Wp - W, 0, Hp - H]).roll((-shift, -shift), (1, 2))
+    t = t.reshape(B, Hp // window, window, Wp // window, window, -1).transpose(2, 3)
+    return t.reshape(B * (Hp // window) * (Wp // window), window * window, -1)
+
+
+def _from_windows(t, shape, window, shift):
+    """The inverse of _to_windows for a map of shape (B, H, W)."""
+    B, H, W = shape
+    ny, nx = -(-H // window), -(-W // window)
+    t = t.reshape(B, ny, nx, window, window, -1).transpose(2, 3).reshape(B, ny * window, nx * window, -1)
+    return t.roll((shift, shift), (1, 2))[:, :H, :W]
+
+
+def _attention(q, k, v, pq, pk, dout, window, shift, masked):
+    """out, lse (and, given dout, dq, dk, dv, dpq, dpk) in float64, one group of windows of one head at a time."""
+    B, H, W, heads, d = q.shape
+    r = pq.shape[-1]
+    images = [_to_windows(t, window, shift).unflatten(-1, (heads, d)) for t in (q, k, v) + ((dout,) if dout is not None else ())]
+    # a label per position: different labels do not attend to each other, label 0 is no token
+    label = torch.zeros((1, -(-H // window) * window, -(-W // window) * window), device=q.device)
+    label[:, :H, :W] = 1
+    if masked and shift:
+        rows, cols = (torch.arange(side, device=q.device) < shift for side in (H, W))
+        label = label + rows[None, :, None] + 2 * cols[None, None, :]
+    label = _to_windows(label[..., None], window, shift)[..., 0].repeat(B, 1)
+    pq, pk = (t.double().expand(heads, -1, -1) if t.dim() == 2 else t.double() for t in (pq, pk))
+    results = [torch.zeros(images[0].shape, dtype=torch.float64, device=q.device) for _ in range(1 if dout is None else 4)]
+    lse = torch.zeros(images[0].shape[:-1], dtype=torch.float64, device=q.device)
+    dpq, dpk = torch.zeros_like(pq, memory_format=torch.contiguous_format), torch.zeros_like(pk, memory_format=torch.contiguous_format)
+    group = max(1, (1 << 27) // window ** 4)
+    for h in range(heads):
+        for start in range(0, label.shape[0], group):
+            part = slice(start, start + group)
+            qw, kw, vw = (t[part, :, h].double() for t in images[:3])
+            logits = qw @ kw.mT / math.sqrt(d) + pq[h] @ pk[h].T / math.sqrt(r)
+            logits = logits.masked_fill_(label[part, :, None] != label[part, None, :], -math.inf)
+            lse[part, :, h] = logits.logsumexp(-1)
+            p = torch.exp(logits.sub_(lse[part, :, h, None]))
+            results[0][part, :, h] = p @ vw
+            if dout is None:
+                continue
+            gw = images[3][part, :, h].double()
+            results[3][part, :, h] = p.mT @ gw
+            ds = p * (gw @ vw.mT - (gw * results[0][part, :, h]).sum(-1, keepdim=True))
+            results[1][part, :, h] = ds @ kw / math.sqrt(d)
+            results[2][part, :, h] = ds.mT @ qw / math.sqrt(d)
+            total = (ds * (label[part] > 0)[:, :, None]).sum(0)
+            dpq[h] += total @ pk[h] / math.sqrt(r)
+            dpk[h] += total.T @ pq[h] / math.sqrt(r)
+    results = [_from_windows(t.flatten(-2), (B, H, W), window, shift).unflatten(-1, (heads, d)) for t in results]
+    lse = _from_windows(lse, (B, H, W), window, shift).permute(0, 3, 1, 2)
+    return results[0], lse, results[1:], dpq, dpk
+
+
+def _gate(x, w_dw, b_dw, w_pw, b_pw):
+    D = x.shape[-1]
+    y = F.conv2d(x.permute(0, 3, 1, 2), w_dw[:, None], b_dw, padding=1, groups=D).permute(0, 2, 3, 1)
+    return torch.sigmoid(y @ w_pw.T + b_pw)
+
+
+def exact(case, seed):
+    """What `run` returns, from the definitions in float64."""
+    state = _inputs(case, seed)
+    kind = case["kind"]
+    if kind == "features":
+        w_h, b_h, w_pq, w_pk = weights = [t.double().requires_grad_() for t in state["weights"]]
+        axis = torch.linspace(-1, 1, case["window"], dtype=torch.float64, device="cuda")
+        x = torch.stack(torch.meshgrid(axis, axis, indexing="ij"), -1).reshape(-1, 2)
+        rows = torch.cat([x] + [f(2.0 ** l * x) for l in range(case["L"]) for f in (torch.sin, torch.cos)], 1)
+        hidden = torch.relu(rows @ w_h + b_h)
+        pq, pk = hidden @ w_pq, hidden @ w_pk
+        grads = torch.autograd.grad([pq, pk], weights, [state["dpq"].double(), state["dpk"].double()])
+        return pq.detach(), pk.detach(), grads
+    if kind == "block":
+        layers = [_attention(*(state[k][l] for k in ("q", "k", "v", "pq", "pk", "dout")), w, 0, False) for l, w in enumerate(state["windows"])]
+        tables = [(dpq.sum(0), dpk.sum(0)) for _, _, _, dpq, dpk in layers]
+        return [l[0] for l in layers], tuple([l[2][i] for l in layers] for i in range(3)) + tuple([t[i] for t in tables] for i in range(2))
+    dout = state.get("dout")
+    if kind == "gated":
+        x, *conv = leaves = [t.double().requires_grad_() for t in [state["x"], *state["conv"]]]
+        gate = _gate(x, *conv)
+        dout = dout.double() * gate.detach().reshape(dout.shape)
+    out, lse, grads, dpq, dpk = _attention(*(state[k] for k in ("q", "k", "v", "pq", "pk")), dout, case["window"], case["shift"],
+                                           case.get("masked", False))
+    if kind == "infer":
+        return out
+    if not case.get("headwise"):
+        dpq, dpk = dpq.sum(0), dpk.sum(0)
+    grads = (*grads, dpq, dpk)
+    if kind == "gated":
+        dgate = (state["dout"].double() * out).reshape(gate.shape)
+        return out * gate.detach().reshape(out.shape), grads, torch.autograd.grad(gate, leaves, dgate)
+    return out, lse, grads
 
 
 def _attending(side, window, shift, masked):
