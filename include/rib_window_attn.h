@@ -131,7 +131,8 @@ size_t rib_window_attn_bwd_headwise_workspace(long long pos_head_stride, int B, 
  * and lse have the real sizes H and W: nothing is padded in memory.  With H and W multiples of the window this is
  * rib_window_attn_fwd_headwise; other arguments, layouts and error codes as there.  H and W multiples of 8 (and
  * the shape conditions above) take the tcgen05 kernel, where a patch of the extension costs a zero-filled TMA box;
- * any other H, W take the any-shape kernel.
+ * any other H, W (windows a multiple of 16, shift a multiple of 8, d and r as above, r up to 32) take a tcgen05 kernel of their
+ * own that keeps probabilities, sums and scaled features at fp32 precision; what is left takes the any-shape kernel.
  */
 int rib_window_attn_fwd_padded(const void* q, const void* k, const void* v, const void* pq, const void* pk,
                                long long pos_head_stride,

@@ -349,13 +349,14 @@ int fwd_impl(const void* q, const void* k, const void* v, const void* pq, const 
     if (int rc = device_status_ptr(&p.status)) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int forced = g_forced_path.load();
-    bool fast = forced != RIB_PATH_GENERIC && rib::sm100_fwd_supported(p);
+    const bool frame = rib::sm100_frame_supported(p);
+    bool fast = forced != RIB_PATH_GENERIC && (frame || rib::sm100_fwd_supported(p));
     p.exact_softmax = forced == RIB_PATH_SM100_EXACT;
     int launches = 1;
     cudaError_t e;
     if (fast) {
-        e = rib::sm100_fwd(p, st);
-    } else if (forced != RIB_PATH_GENERIC && rib::sm100_repack_supported(p)) {
+        e = frame ? rib::sm100_fwd_frame(p, st) : rib::sm100_fwd(p, st);
+    } else if (forced != RIB_PATH_GENERIC && rib::sm100_repack_fwd_supported(p)) {
         // rows TMA cannot address (d = 30, r = 18, ...): the tensor-core kernels on zero-padded copies
         e = rib::sm100_fwd_repacked(p, st, &launches);
         fast = e == cudaSuccess;
@@ -390,7 +391,7 @@ size_t rib_window_attn_bwd_headwise_workspace(long long pos_head_stride, int B, 
     size_t need = rowdot_bytes(B, H, W, heads);
     rib::Problem p{};
     fill_shape(p, B, H, W, heads, d, r, window, 0);
-    if (rib::sm100_bwd_supported(p) || rib::sm100_repack_supported(p)) {   // whatever the shift: one size per shape
+    if (rib::sm100_bwd_supported(p) || rib::sm100_repack_bwd_supported(p)) {   // whatever the shift: one size per shape
         const size_t fast = rib::sm100_bwd_workspace_bytes(p.pairs, p.n, pos_head_stride ? heads : 1, rib::repacked_width(r));
         if (fast > need) need = fast;
     }
@@ -428,7 +429,7 @@ size_t rib_window_attn_bwd_padded_workspace(long long pos_head_stride, int B, in
     size_t need = rowdot_bytes(B, H, W, heads);
     rib::Problem p{};
     fill_shape(p, B, H, W, heads, d, r, window, 0);
-    if (rib::sm100_bwd_supported(p) || rib::sm100_repack_supported(p)) {        // sized by the windows of the extended map
+    if (rib::sm100_bwd_supported(p) || rib::sm100_repack_bwd_supported(p)) {        // sized by the windows of the extended map
         const size_t fast = rib::sm100_bwd_workspace_bytes(p.pairs, p.n, pos_head_stride ? heads : 1, rib::repacked_width(r));
         if (fast > need) need = fast;
     }
@@ -481,7 +482,7 @@ static int bwd_impl(const void* q, const void* k, const void* v, const void* pq,
     cudaError_t e;
     if (fast) {
         e = rib::sm100_bwd(p, st);
-    } else if (allowed && rib::sm100_repack_supported(p)) {
+    } else if (allowed && rib::sm100_repack_bwd_supported(p)) {
         e = rib::sm100_bwd_repacked(p, st, &launches);
         fast = e == cudaSuccess;
         if (e == cudaErrorMemoryAllocation) {

@@ -65,13 +65,18 @@ cudaError_t rowdot_prepass(const Problem& p, cudaStream_t stream);
 
 bool sm100_fwd_supported(const Problem& p);
 cudaError_t sm100_fwd(const Problem& p, cudaStream_t stream);
+// Frames with a side that is no multiple of 8, at the precision of the any-shape kernel (rib_fwd_frame_sm100.cu).
+bool sm100_frame_supported(const Problem& p);
+cudaError_t sm100_fwd_frame(const Problem& p, cudaStream_t stream);
 bool sm100_bwd_supported(const Problem& p);
 size_t sm100_bwd_workspace_bytes(long long pairs, int n, int tables, int r);
 cudaError_t sm100_bwd(const Problem& p, cudaStream_t stream);   // launches 3 kernels
 // Even head widths and ranks up to 32 whose rows TMA cannot address (60-byte rows of d = 30, 36-byte rows of r = 18):
 // the tensors are copied into zero-padded scratch (stream-ordered allocation), the tcgen05 kernels run on the copies,
 // and the results are copied back.  `launches` receives the number of kernels enqueued.
-bool sm100_repack_supported(const Problem& p);
+// The forward pass takes frames of any size, the backward pass sides that are multiples of 8.
+bool sm100_repack_fwd_supported(const Problem& p);
+bool sm100_repack_bwd_supported(const Problem& p);
 int repacked_width(int w);                    // the next multiple of 8
 cudaError_t sm100_fwd_repacked(const Problem& p, cudaStream_t stream, int* launches);
 cudaError_t sm100_bwd_repacked(const Problem& p, cudaStream_t stream, int* launches);

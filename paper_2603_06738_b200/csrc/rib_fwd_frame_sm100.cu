@@ -1,0 +1,456 @@
+// Forward RIB window attention for B200 (sm_100a) on frames whose sides are not multiples of 8: tcgen05 MMAs, TMEM, TMA.
+//
+// These shapes are defined by the fp32 any-shape kernels (rib_generic.cu), which keep the probabilities, their sums and the
+// scaled positional features in fp32.  This kernel keeps that precision on the bf16 tensor cores by splitting what is not
+// a bf16 number to begin with into bf16 terms whose sum carries it:
+//     P            = hi + lo           two terms, 16 significant bits: the PV contraction runs twice, into one accumulator;
+//     Pq sqrt(d/r) = hi + mid + lo     three terms, all 24 bits: one K16 step (two at R = 32) of the score chain per term
+//                                      (one term where d / r is a power of 4 and the product is a bf16 number);
+// q, k, v and Pk are bf16 as given and enter exactly, sums are fp32, every exponential is ex2.approx (2 ulp), the row sum
+// adds the unrounded fp32 probabilities.
+//
+// What bounds it: the exponentials (16 per cycle and SM: 1024 cycles per tile of 128 x 128 scores) and, next to them, 21
+// MMAs per tile (about 950 cycles).  Measured (180 x 320 tokens, 32 x 32 windows, 6 heads of 32 channels, rank 16, with the
+// launch): 176 us = 308 TFLOP/s of the layer's own flops, about 2000 cycles per tile and SM; the any-shape kernel 13 460 us.
+// Error of `out` against float64 as that kernel's (1.7e-3, the rounding to bf16).
+//
+// Work item = one (batch, window, head) pair x two query tiles of 128 tokens (two 8x8-token patches each).  Only patches that
+// hold tokens are walked (LiveWindows in rib_sm100_common.cuh); a patch that straddles the border of the frame is filled up
+// with zeros by TMA, its keys beyond the frame get the score -inf and its queries beyond it are not stored.
+//
+// Tensor memory: three score buffers of 128 columns and 2 x 2 output accumulators (query tile, key half) of 32.  Unit u =
+// 2 * block + query tile uses buffer u mod 3.  A softmax thread holds one row's 64 scores of its key half in registers and
+// writes P over them (hi 32 columns, lo 32 columns), so a buffer is handed back to the one issuing thread with P in it; that
+// thread issues PV(u) and behind it S(u + 3) into the same columns, in which order the tensor pipe executes them.  The scores
+// of one tile's next block are thus under way while the other tile's exponentials run.
+//
+// Roles (640 threads): warp 0 TMA producer, which also stages the scaled query RIB rows; warp 1 issues all MMAs; warp 2 owns
+// the TMEM allocation; warps 4-11 softmax / epilogue of query tile 0 (4-7 first key half, 8-11 second half), 12-19 of tile 1.
+// Every wait is bounded.
+#include "rib_sm100_common.cuh"
+
+namespace rib {
+namespace {
+
+using namespace sm100;
+
+constexpr int kThreads = 640;
+constexpr int kTerms = 3;                 // bf16 terms of a scaled query RIB row
+constexpr int kBuffers = 3;               // score / P buffers in tensor memory
+
+// shared-memory map (offsets from a 1024-byte aligned base); RIB rows of 16 elements (32 bytes, SWIZZLE_32B) or 32 (SWIZZLE_64B)
+template <int R>
+struct Frame {
+    static constexpr int kStages = R == 16 ? 4 : 3;                              // K / V ring: what fits
+    static constexpr uint32_t kPos = kTile * R * 2, kPatchP = kPos / 2;
+    static constexpr uint32_t kOffQc = 0;                                        // [2 items][2 tiles] query content
+    static constexpr uint32_t kOffQp = kOffQc + 4 * kContentBytes;               // [2 items][2 tiles][kTerms] query RIB rows
+    static constexpr uint32_t kOffKc = kOffQp + 4 * kTerms * kPos;               // [kStages] key content, key RIB rows, values
+    static constexpr uint32_t kOffKp = kOffKc + kStages * kContentBytes;
+    static constexpr uint32_t kOffV = kOffKp + kStages * kPos;
+    static constexpr uint32_t kOffBar = kOffV + kStages * kContentBytes;
+    // barriers: query buffers, ring stages, score buffers, completed PV per tile, merge per tile and quarter of the rows, drain
+    enum Bar { kQFull = 0, kQEmpty = 2, kQPos = 4, kFull = 6, kEmpty = kFull + kStages, kSFull = kEmpty + kStages, kPReady = kSFull + kBuffers,
+               kPVDone = kPReady + kBuffers, kMerge = kPVDone + 2, kDrain = kMerge + 8, kNumBars };
+    static constexpr uint32_t kOffMisc = kOffBar + kNumBars * 8;                 // tmem base, abort flags
+    static constexpr uint32_t kOffMerge = (kOffMisc + 16 + 15) & ~15u;           // [2 item parities][2 tiles][2 halves][128 rows] (max, sum)
+    static constexpr uint32_t kSmemBytes = kOffMerge + 8 * kTile * 8 + 1024;     // + slack for manual alignment
+    static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
+};
+
+constexpr uint32_t kColO = kBuffers * kTile, kTmemCols = 512;                    // O: [2 tiles][2 key halves][32]
+static_assert(kColO + 4 * kD <= kTmemCols, "tensor memory has 512 columns");
+
+constexpr uint32_t kIdescS = idesc_bf16_f32(kTile, kTile, false);
+constexpr uint32_t kIdescPV = idesc_bf16_f32(kTile, kD, true);
+
+struct FrameParams {
+    const __nv_bfloat16* pq;
+    __nv_bfloat16* out;
+    float* lse;
+    int* status;
+    int H, W, heads, d, r;
+    WindowGeom geom;           // sides of the extended map, window, shift
+    int terms;                 // terms of the scaled query RIB rows in use: 1 or kTerms
+    float scale_log2;          // log2(e) / sqrt(d)
+    float inv_sqrt_d;
+    float pos_scale;           // sqrt(d / r): folds 1/sqrt(r) into the content scale
+    long long pos_head_stride;
+    int pos_per_head;
+    LiveWindows live;
+};
+
+template <int R>
+__global__ void __launch_bounds__(kThreads, 1)
+rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                           const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ FrameParams p)
+{
+    using L = Frame<R>;
+    constexpr int kStages = L::kStages;
+    constexpr uint32_t kPos = L::kPos;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
+    auto bar = [&](int i) { return base + L::kOffBar + 8u * i; };
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + L::kOffMisc);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + L::kOffMisc + 4);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int items = p.live.offset[9];
+
+    if (threadIdx.x == 0) {
+        abort_flag[0] = 0; abort_flag[1] = 0;   // [1] stays 0: used by the drain waits
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar(L::kQFull + i), 1); mbar_init(bar(L::kQEmpty + i), 1); mbar_init(bar(L::kQPos + i), 1); mbar_init(bar(L::kPVDone + i), 1);
+            for (int q4 = 0; q4 < 4; ++q4) mbar_init(bar(L::kMerge + 4 * i + q4), 2);
+        }
+        for (int i = 0; i < kBuffers; ++i) { mbar_init(bar(L::kSFull + i), 1); mbar_init(bar(L::kPReady + i), 8); }
+        for (int s = 0; s < kStages; ++s) { mbar_init(bar(L::kFull + s), 1); mbar_init(bar(L::kEmpty + s), 1); }
+        mbar_init(bar(L::kDrain), 1);
+        fence_barrier_init();
+        prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v); prefetch_tensormap(&tm_pk);
+    }
+    if (warp == 2) {
+        tmem_alloc(base + L::kOffMisc, kTmemCols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    bool ok = true;
+    if (warp == 0) {
+        // ===================== TMA producer (lane 0) and the query RIB rows Pq * sqrt(d/r) of the same item, in terms (whole warp)
+        uint32_t io = 0, blk = 0;
+        for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++io) {
+            const LiveItem c = decode_live_item(p.live, item);
+            const uint32_t buf = io & 1;
+            if (io >= 2 && !mbar_wait_warp(bar(L::kQEmpty + buf), ((io >> 1) - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+            if (lane == 0) {
+                mbar_arrive_expect_tx(bar(L::kQFull + buf), 2 * kContentBytes);
+                for (int q4 = 0; q4 < 4; ++q4) {
+                    int py, px, Y0, X0;
+                    live_patch_origin(p.live, p.geom, c, min(4 * c.tp + q4, c.patches - 1), py, px, Y0, X0);
+                    tma_load_5d(base + L::kOffQc + 2 * buf * kContentBytes + q4 * kPatchContent, &tm_q, bar(L::kQFull + buf), 0, c.h, X0, Y0, c.b);
+                }
+            }
+            for (int k = 0; k < 8; ++k) {
+                const int r256 = lane + 32 * k, qt = r256 >> 7, row = r256 & 127;
+                int py, px, Y0, X0;
+                live_patch_origin(p.live, p.geom, c, min(4 * c.tp + (r256 >> 6), c.patches - 1), py, px, Y0, X0);
+                const int token = (py + ((row >> 3) & 7)) * p.geom.M + px + (row & 7);      // row of the table
+                const uint4* src = reinterpret_cast<const uint4*>(p.pq + (size_t)c.h * p.pos_head_stride + (size_t)token * p.r);
+                uint8_t* dst = base_ptr + L::kOffQp + (2 * buf + qt) * kTerms * kPos + row * (2 * R);
+                const int sw = R == 16 ? (row >> 2) & 1 : (row >> 1) & 3;                   // SWIZZLE_32B / SWIZZLE_64B
+#pragma unroll
+                for (int ck = 0; ck < R / 8; ++ck) {                                        // 16-byte chunks of the row
+                    const uint4 v = 8 * ck < p.r ? __ldg(src + ck) : make_uint4(0u, 0u, 0u, 0u);
+                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                    uint32_t t[kTerms][4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        float lo = __uint_as_float(w[e] << 16) * p.pos_scale, hi = __uint_as_float(w[e] & 0xffff0000u) * p.pos_scale;
+#pragma unroll
+                        for (int term = 0; term < kTerms; ++term) {
+                            t[term][e] = pack_bf16x2(lo, hi);
+                            lo -= __uint_as_float(t[term][e] << 16);
+                            hi -= __uint_as_float(t[term][e] & 0xffff0000u);
+                        }
+                    }
+#pragma unroll
+                    for (int term = 0; term < kTerms; ++term)
+                        if (term < p.terms) *reinterpret_cast<uint4*>(dst + term * kPos + ((ck ^ sw) << 4)) = make_uint4(t[term][0], t[term][1], t[term][2], t[term][3]);
+                }
+            }
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(bar(L::kQPos + buf));
+                const int nblk = (c.patches + 1) >> 1;
+                for (int j = 0; j < nblk; ++j, ++blk) {
+                    const uint32_t st = blk % kStages, use = blk / kStages;
+                    if (use > 0 && !mbar_wait(bar(L::kEmpty + st), (use - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                    mbar_arrive_expect_tx(bar(L::kFull + st), 2 * kContentBytes + kPos);
+                    for (int sub = 0; sub < 2; ++sub) {
+                        int py, px, Y0, X0;
+                        live_patch_origin(p.live, p.geom, c, min(2 * j + sub, c.patches - 1), py, px, Y0, X0);
+                        tma_load_5d(base + L::kOffKc + st * kContentBytes + sub * kPatchContent, &tm_k, bar(L::kFull + st), 0, c.h, X0, Y0, c.b);
+                        tma_load_4d(base + L::kOffKp + st * kPos + sub * L::kPatchP, &tm_pk, bar(L::kFull + st), 0, px, py, c.h * p.pos_per_head);
+                        tma_load_5d(base + L::kOffV + st * kContentBytes + sub * kPatchContent, &tm_v, bar(L::kFull + st), 0, c.h, X0, Y0, c.b);
+                    }
+                }
+            } else {
+                blk += (uint32_t)((c.patches + 1) >> 1);
+            }
+            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            if (!ok && lane == 0) ++io;                      // this item's query tiles are armed as well
+        }
+        if (!ok && lane == 0) {
+            // Gave up: let the copies already in flight land before the CTA may exit.
+            for (uint32_t b2 = io > 2u ? io - 2 : 0; b2 < io; ++b2)
+                mbar_wait(bar(L::kQFull + (b2 & 1)), (b2 >> 1) & 1, abort_flag + 1, p.status);
+            for (uint32_t b2 = blk > (uint32_t)kStages ? blk - kStages : 0; b2 < blk; ++b2)
+                mbar_wait(bar(L::kFull + b2 % kStages), (b2 / kStages) & 1, abort_flag + 1, p.status);
+        }
+    } else if (warp == 1) {
+        // ===================== issuer: S(0), S(1), S(2), then PV(u), S(u + 3) for u = 0, 1, ...; the whole warp walks and waits
+        constexpr uint64_t kDesc64 = smem_desc_const(16, 512, kSwizzle64B), kDesc32 = smem_desc_const(16, 256, kSwizzle32B);
+        constexpr uint64_t kDescP = R == 16 ? kDesc32 : kDesc64;
+        // two cursors over the same sequence of blocks: scores run three units ahead of PV
+        struct Cursor { int item; int nblk, j; uint32_t io, blk, u; } s{}, v{};
+        auto enter = [&](Cursor& c) { if (c.item < items) c.nblk = (decode_live_item(p.live, c.item).patches + 1) >> 1; };
+        auto advance = [&](Cursor& c) {
+            if (++c.u & 1) return;                           // the block's second query tile is next
+            ++c.blk;
+            if (++c.j < c.nblk) return;
+            c.j = 0; c.item += gridDim.x; ++c.io;
+            enter(c);
+        };
+        s.item = v.item = blockIdx.x;
+        enter(s); enter(v);
+        auto issue_scores = [&]() {
+            if (s.item >= items) return true;
+            const uint32_t buf = s.io & 1, st = s.blk % kStages, qt = s.u & 1, sb = s.u % kBuffers;
+            if (qt == 0) {
+                if (s.j == 0 && (!mbar_wait_warp(bar(L::kQFull + buf), (s.io >> 1) & 1, abort_flag, p.status) ||
+                                 !mbar_wait_warp(bar(L::kQPos + buf), (s.io >> 1) & 1, abort_flag, p.status))) return false;
+                if (!mbar_wait_warp(bar(L::kFull + st), (s.blk / kStages) & 1, abort_flag, p.status)) return false;
+            }
+            if (elect_one()) {
+                const uint64_t kc = smem_desc_at(kDesc64, base + L::kOffKc + st * kContentBytes), kp = smem_desc_at(kDescP, base + L::kOffKp + st * kPos);
+                const uint64_t qc = smem_desc_at(kDesc64, base + L::kOffQc + (2 * buf + qt) * kContentBytes);
+                const uint64_t qp = smem_desc_at(kDescP, base + L::kOffQp + (2 * buf + qt) * kTerms * kPos);
+                const uint32_t d_s = tmem + sb * kTile;
+                mma_ss(d_s, qc, kc, kIdescS, 0u);
+                mma_ss(d_s, qc + 2, kc + 2, kIdescS, 1u);          // + 32 bytes: second K16 step of the content rows
+                for (int term = 0; term < p.terms; ++term) {
+                    mma_ss(d_s, qp + term * (kPos >> 4), kp, kIdescS, 1u);
+                    if (R == 32) mma_ss(d_s, qp + term * (kPos >> 4) + 2, kp + 2, kIdescS, 1u);
+                }
+                mma_commit(bar(L::kSFull + sb));
+                if (qt == 1 && s.j == s.nblk - 1) mma_commit(bar(L::kQEmpty + buf));
+            }
+            __syncwarp();
+            advance(s);
+            return true;
+        };
+        for (int i = 0; i < kBuffers && ok; ++i) ok = issue_scores();
+        while (ok && v.item < items) {
+            const uint32_t st = v.blk % kStages, qt = v.u & 1, sb = v.u % kBuffers;
+            // P of the unit is there.  (The first block of an item overwrites O: the softmax warps have read it before they
+            // arrive here for that block.)
+            if (!mbar_wait_warp(bar(L::kPReady + sb), (v.u / kBuffers) & 1, abort_flag, p.status)) { ok = false; break; }
+            tc_fence_after();
+            if (elect_one()) {
+                const uint64_t vd = smem_desc_at(kDesc64, base + L::kOffV + st * kContentBytes);
+                const uint32_t a_p = tmem + sb * kTile, d_o = tmem + kColO + qt * 2 * kD;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {                   // keys 16 kk ..: key half kk / 4 has its own accumulator
+                    const uint32_t a = a_p + (kk >> 2) * 64 + 8 * (kk & 3), d = d_o + (kk >> 2) * kD;
+                    mma_ts(d, a, vd + 64 * kk, kIdescPV, (v.j == 0 && (kk & 3) == 0) ? 0u : 1u);
+                    mma_ts(d, a + 32, vd + 64 * kk, kIdescPV, 1u);
+                }
+                mma_commit(bar(L::kPVDone + qt));
+                if (qt == 1) mma_commit(bar(L::kEmpty + st));
+            }
+            __syncwarp();
+            advance(v);
+            ok = issue_scores();
+        }
+        // everything issued by this warp's leader must have finished before TMEM is released
+        if (elect_one()) mma_commit(bar(L::kDrain));
+        __syncwarp();
+        mbar_wait(bar(L::kDrain), 0, abort_flag + 1, p.status);
+    } else if (warp >= 4) {
+        // ================ softmax + epilogue: two threads per query row, one per half of the keys
+        const int qt = (warp - 4) >> 3;
+        const int half = ((warp - 4) >> 2) & 1;
+        const int quarter = warp & 3;
+        const int row = quarter * 32 + lane;                 // row of the tile == TMEM lane
+        const uint32_t t_half = tmem + ((uint32_t)(quarter * 32) << 16) + half * 64;                // + buffer: own scores, own P
+        const uint32_t t_o = tmem + ((uint32_t)(quarter * 32) << 16) + kColO + qt * 2 * kD;         // both halves' accumulators
+        // [half][row]; two sets, so that a warp that is an item ahead of its partner does not overwrite what that one still reads
+        float2* const merge_sets = reinterpret_cast<float2*>(base_ptr + L::kOffMerge) + qt * 2 * kTile;
+        const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
+        const float rescale_threshold = 8.0f / p.scale_log2; // raw-logit units: probabilities stay <= 2^8 relative to the reference
+        uint32_t blk = 0, nmerge = 0, sb = qt, use = 0;      // sb, use: (2 blk + qt) mod and div kBuffers
+        for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++nmerge) {
+            const LiveItem c = decode_live_item(p.live, item);
+            const int nblk = (c.patches + 1) >> 1;
+            // does the window reach beyond the frame?  (only then can a patch hold fewer than 64 tokens)
+            const bool edge = c.wy * p.geom.M + p.geom.s + p.geom.M > p.H || c.wx * p.geom.M + p.geom.s + p.geom.M > p.W;
+            float m_used = -INFINITY, l = 0.f;
+            for (int j = 0; j < nblk; ++j, ++blk) {
+                // warp-uniform outcome: the TMEM accesses below are warp-collective
+                if (!mbar_wait_warp(bar(L::kSFull + sb), use & 1, abort_flag, p.status)) { ok = false; break; }
+                tc_fence_after();
+                uint32_t s[2][32];
+                tmem_ld32(t_half + sb * kTile, s[0]);
+                tmem_ld32(t_half + sb * kTile + 32, s[1]);
+                tmem_wait_ld();
+                if (edge) {
+                    // this thread's 64 keys are one 8x8 patch: tokens beyond the frame (or all of a missing last patch) get -inf
+                    int py, px, Y0, X0, rows = 0, cols = 0;
+                    if (2 * j + half < c.patches) {
+                        live_patch_origin(p.live, p.geom, c, 2 * j + half, py, px, Y0, X0);
+                        rows = p.H - Y0; cols = p.W - X0;
+                    }
+                    if (rows < 8 || cols < 8) {              // warp-uniform
+#pragma unroll
+                        for (int e = 0; e < 64; ++e)
+                            if ((e >> 3) >= rows || (e & 7) >= cols) s[e >> 5][e & 31] = 0xff800000u;
+                    }
+                }
+                float mx0 = -INFINITY, mx1 = -INFINITY;
+#pragma unroll
+                for (int e = 0; e < 32; e += 2) {
+                    mx0 = max3(mx0, __uint_as_float(s[0][e]), __uint_as_float(s[0][e + 1]));
+                    mx1 = max3(mx1, __uint_as_float(s[1][e]), __uint_as_float(s[1][e + 1]));
+                }
+                const float mx = fmaxf(mx0, mx1);
+                if (j == 0) {
+                    m_used = mx;
+                } else {
+                    // Move the reference (and rescale O, l) only when the maximum grew by more than the threshold; the result
+                    // is exact after the final normalisation because l carries the same reference.
+                    const bool need = mx > m_used + rescale_threshold;
+                    if (__any_sync(0xffffffffu, need)) {
+                        if (!mbar_wait_warp(bar(L::kPVDone + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                        tc_fence_after();
+                        const float factor = need ? ex2_approx((m_used - mx) * p.scale_log2) : 1.f;
+                        if (need) { l *= factor; m_used = mx; }
+                        for (int g = 0; g < 4; ++g) {
+                            uint32_t o[8];
+                            tmem_ld8(t_o + half * kD + 8 * g, o);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * factor);
+                            tmem_st8(t_o + half * kD + 8 * g, o);
+                        }
+                    }
+                }
+                // a half that has seen no token yet has no reference: its scores are all -inf, its probabilities 0
+                const float neg = m_used == -INFINITY ? 0.f : -m_used * p.scale_log2;
+                const float2 neg2 = make_float2(neg, neg);
+                float2 sum_a = make_float2(0.f, 0.f), sum_b = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int ch = 0; ch < 2; ++ch) {
+                    uint32_t hi[16], lo[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[ch][2 * i]), __uint_as_float(s[ch][2 * i + 1])), scale2, neg2);
+                        const float2 e = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+                        if (i & 1) sum_b = __fadd2_rn(sum_b, e); else sum_a = __fadd2_rn(sum_a, e);
+                        hi[i] = pack_bf16x2(e.x, e.y);
+                        const float2 rest = __fadd2_rn(e, make_float2(-__uint_as_float(hi[i] << 16), -__uint_as_float(hi[i] & 0xffff0000u)));
+                        lo[i] = pack_bf16x2(rest.x, rest.y);
+                    }
+                    tmem_st16(t_half + sb * kTile + 16 * ch, hi);
+                    tmem_st16(t_half + sb * kTile + 32 + 16 * ch, lo);
+                }
+                l += (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(L::kPReady + sb));
+                sb += 2;
+                if (sb >= kBuffers) { sb -= kBuffers; ++use; }
+            }
+            if (!ok) break;
+            // ---- merge the two key halves and write this thread's 16 output columns
+            float2* const merge = merge_sets + (nmerge & 1) * 4 * kTile;
+            merge[half * kTile + row] = make_float2(m_used, l);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(L::kMerge + 4 * qt + quarter));
+            // The partner's (m, l) must be there and the item's last PV must have completed.
+            if (!mbar_wait_warp(bar(L::kMerge + 4 * qt + quarter), nmerge & 1, abort_flag, p.status) ||
+                !mbar_wait_warp(bar(L::kPVDone + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+            tc_fence_after();
+            uint32_t oa[16], ob[16];
+            tmem_ld16(t_o + half * 16, oa);
+            tmem_ld16(t_o + kD + half * 16, ob);
+            tmem_wait_ld();
+            tc_fence_before();
+            const float2 other = merge[(half ^ 1) * kTile + row];
+            const float m_a = half ? other.x : m_used, l_a = half ? other.y : l;
+            const float m_b = half ? m_used : other.x, l_b = half ? l : other.y;
+            const float m = fmaxf(m_a, m_b);
+            const float f_a = ex2_approx((m_a - m) * p.scale_log2), f_b = ex2_approx((m_b - m) * p.scale_log2);
+            const float l_all = l_a * f_a + l_b * f_b;
+            const float w_a = f_a / l_all, w_b = f_b / l_all;
+            const int k = 4 * c.tp + 2 * qt + (row >> 6);
+            int py, px, Y0, X0;
+            live_patch_origin(p.live, p.geom, c, min(k, c.patches - 1), py, px, Y0, X0);
+            const int Y = Y0 + ((row >> 3) & 7), X = X0 + (row & 7);
+            if (k < c.patches && Y < p.H && X < p.W) {       // (else: no token, nothing to store)
+                const size_t tok = (((size_t)c.b * p.H + Y) * p.W + X) * p.heads + c.h;
+                uint4* dst = reinterpret_cast<uint4*>(p.out + tok * p.d + half * 16);
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    if (half * 16 + 8 * g >= p.d) break;     // a head narrower than 32 channels: the rest of the row is padding
+                    uint32_t w[4];
+#pragma unroll
+                    for (int k2 = 0; k2 < 4; ++k2) {
+                        const int e = 8 * g + 2 * k2;
+                        w[k2] = pack_bf16x2(__uint_as_float(oa[e]) * w_a + __uint_as_float(ob[e]) * w_b,
+                                            __uint_as_float(oa[e + 1]) * w_a + __uint_as_float(ob[e + 1]) * w_b);
+                    }
+                    dst[g] = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+                if (p.lse && half == 0) p.lse[(((size_t)c.b * p.heads + c.h) * p.H + Y) * p.W + X] = m * p.inv_sqrt_d + logf(l_all);
+            }
+            __syncwarp();
+        }
+    }
+    // ================================================================================ common tail
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 2) {
+        tc_fence_after();
+        tmem_dealloc(tmem, kTmemCols);
+    }
+}
+
+}  // namespace
+
+template <int R>
+cudaError_t launch_fwd_frame(const Problem& p, cudaStream_t stream)
+{
+    if (!encode_fn()) return cudaErrorNotSupported;
+    FrameParams fp{};
+    if (!make_live_windows(p, &fp.live)) return cudaErrorInvalidValue;
+    CUtensorMap tm_q, tm_k, tm_v, tm_pk;
+    if (!encode_image_map(&tm_q, p.q, p) || !encode_image_map(&tm_k, p.k, p) || !encode_image_map(&tm_v, p.v, p) ||
+        !encode_pos_map(&tm_pk, p.pk, p, pos_tables(p), p.pos_head_stride))
+        return cudaErrorInvalidValue;
+    static KernelSetup setup;       // one per instantiation of this launcher, i.e. per kernel
+    int sm_count = 0;
+    if (cudaError_t e = setup.prepare(rib_fwd_frame_sm100_kernel<R>, Frame<R>::kSmemBytes, &sm_count)) return e;
+    fp.pq = p.pq; fp.out = p.out_w; fp.lse = p.lse_w; fp.status = p.status;
+    fp.H = p.H; fp.W = p.W; fp.heads = p.heads; fp.d = p.d; fp.r = p.r;
+    fp.geom = WindowGeom{p.Hp, p.Wp, p.M, p.s};
+    const float d = scale_width_d(p), r = scale_width_r(p);
+    fp.scale_log2 = 1.4426950408889634f / sqrtf(d);
+    fp.inv_sqrt_d = 1.f / sqrtf(d);
+    fp.pos_scale = sqrtf(d / r);
+    fp.terms = d == r || d == 4.f * r || 4.f * d == r ? 1 : kTerms;      // sqrt(d / r) a power of two: the product is a bf16 number
+    fp.pos_head_stride = p.pos_head_stride;
+    fp.pos_per_head = p.pos_head_stride ? 1 : 0;
+    const int items = fp.live.offset[9], grid = items < sm_count ? items : sm_count;
+    { ProfileScope scope(RIB_KERNEL_FWD_MAIN, stream); rib_fwd_frame_sm100_kernel<R><<<grid, kThreads, Frame<R>::kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_pk, fp); }
+    return cudaGetLastError();
+}
+
+bool sm100_frame_supported(const Problem& p)
+{
+    return p.d % 8 == 0 && p.d >= 8 && p.d <= kD && p.r % 8 == 0 && p.r >= 8 && p.r <= 32 && p.M % 16 == 0 && p.M <= 256 && p.s % 8 == 0 &&
+           (p.H % 8 || p.W % 8) && !p.masked && !p.gate && !p.packed8;
+}
+
+cudaError_t sm100_fwd_frame(const Problem& p, cudaStream_t stream)
+{
+    return padded_rank(p.r) == 32 ? launch_fwd_frame<32>(p, stream) : launch_fwd_frame<16>(p, stream);
+}
+
+}  // namespace rib

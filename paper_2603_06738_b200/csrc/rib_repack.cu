@@ -233,14 +233,23 @@ cudaError_t pack_qk(const Problem& p, const __nv_bfloat16* q, __nv_bfloat16* q2,
 
 int repacked_width(int w) { return (w + 7) & ~7; }
 
-bool sm100_repack_supported(const Problem& p)
+static bool repack_supported(const Problem& p)
 {
     if (p.d < 2 || p.d > 32 || p.r < 2 || (p.d & 1) || (p.r & 1) || p.d_true || p.r_true) return false;
     if (p.r > 32 && p.r - 32 > repacked_width(p.d) - p.d) return false;      // no room for the columns above 32
     if (p.d % 8 == 0 && p.r % 8 == 0) return false;          // these run on the kernels as they are
     if ((long long)p.B * p.H * p.W * p.heads * 16 > 0x7fffffffLL && p.r > 32) return false;   // 32-bit indices of the tail kernels
+    return true;
+}
+
+bool sm100_repack_bwd_supported(const Problem& p) { return repack_supported(p) && sm100_bwd_supported(padded_shape(p)); }
+
+bool sm100_repack_fwd_supported(const Problem& p)
+{
+    if (!repack_supported(p)) return false;
     const Problem pp = padded_shape(p);
-    return sm100_fwd_supported(pp) && sm100_bwd_supported(pp);
+    // (frames keep the precision of the any-shape kernel, which the rank tail in bf16 channels would not)
+    return sm100_fwd_supported(pp) || (sm100_frame_supported(pp) && !rank_tail(p));
 }
 
 cudaError_t sm100_fwd_repacked(const Problem& p, cudaStream_t stream, int* launches)
@@ -267,7 +276,7 @@ cudaError_t sm100_fwd_repacked(const Problem& p, cudaStream_t stream, int* launc
     if (!e) e = copy_tables<uint32_t>(p.pk, p.pos_head_stride, p.r, pk2, tstride, pp.r, tables, p.n, stream, launches);
     if (!e) {
         pp.q = q2; pp.k = k2; pp.v = v2; pp.pq = pq2; pp.pk = pk2; pp.out_w = o2;
-        e = sm100_fwd(pp, stream);
+        e = sm100_frame_supported(pp) ? sm100_fwd_frame(pp, stream) : sm100_fwd(pp, stream);
         ++*launches;
     }
     if (!e) e = resize_rows(o2, pp.d, p.out_w, p.d, rows, stream, launches);

@@ -78,6 +78,104 @@ __host__ __device__ __forceinline__ void window_order_token(const WindowGeom& g,
     X = X0 + tx;
 }
 
+// ------------------------------------------------------------------------- windows of a map that they do not divide
+// Windows are laid over the map extended to Hp x Wp; positions beyond H x W are no tokens.  Attention does not depend on
+// the order of a window's tokens, so a kernel may walk only the patches that hold some: along each axis a window has a list
+// of such patch rows (columns), which is one or two runs, and patch k of the window is (row k / cols, column k % cols) of
+// the two lists.  Along an axis every window but the last one or two is full (the positions beyond the map are fewer than
+// a window, and the shift is smaller than one), which gives at most three kinds of window per axis and nine in the map;
+// the work items (two query tiles = four patches each) are numbered kind by kind, full windows first, so that the items
+// dealt out last are the short ones.
+struct AxisKind { int count, start0, len0, start1, first; FastDiv by_count, by_windows; };      // patches; first window and number of windows of the kind
+struct LiveWindows {
+    AxisKind y[3], x[3];
+    int offset[10];                  // first item of kind 3 * ky + kx; offset[9]: all items
+    FastDiv items_per_window[9];
+    FastDiv by_heads;
+};
+struct LiveItem { int b, h, wy, wx, tp, ky, kx, patches; };
+
+__host__ __device__ __forceinline__ LiveItem decode_live_item(const LiveWindows& g, int item)
+{
+    LiveItem c;
+    int kind = 0;
+#pragma unroll
+    for (int k = 1; k < 9; ++k) kind += item >= g.offset[k] ? 1 : 0;
+    c.ky = kind / 3; c.kx = kind - 3 * c.ky;
+    int rest = item - g.offset[kind], i;
+    g.items_per_window[kind].divmod(rest, rest, c.tp);
+    g.by_heads.divmod(rest, rest, c.h);
+    g.x[c.kx].by_windows.divmod(rest, rest, i);
+    c.wx = g.x[c.kx].first + i;
+    g.y[c.ky].by_windows.divmod(rest, c.b, i);
+    c.wy = g.y[c.ky].first + i;
+    c.patches = g.y[c.ky].count * g.x[c.kx].count;
+    return c;
+}
+// Patch k of the item's window: top-left token in window coordinates and in shifted, wrapped coordinates of the extended map.
+__host__ __device__ __forceinline__ void live_patch_origin(const LiveWindows& g, const WindowGeom& w, const LiveItem& c, int k, int& py, int& px,
+                                                           int& Y0, int& X0)
+{
+    const AxisKind &ay = g.y[c.ky], &ax = g.x[c.kx];
+    int r, l;
+    ax.by_count.divmod(k, r, l);
+    py = (r < ay.len0 ? ay.start0 + r : ay.start1 + r - ay.len0) << 3;
+    px = (l < ax.len0 ? ax.start0 + l : ax.start1 + l - ax.len0) << 3;
+    Y0 = c.wy * w.M + py + w.s; if (Y0 >= w.H) Y0 -= w.H;
+    X0 = c.wx * w.M + px + w.s; if (X0 >= w.W) X0 -= w.W;
+}
+
+// The kinds of window along an axis of `size` positions; returns their number, 0 if the axis is not of the form above.
+inline int axis_kinds(int size, int M, int s, AxisKind (&kinds)[3], int (&windows)[3])
+{
+    const int n = (size + M - 1) / M, extended = n * M, per_row = M / 8;
+    int used = 0;
+    for (int w = 0; w < n; ++w) {
+        AxisKind k{};
+        int runs = 0, last = -2;
+        for (int l = 0; l < per_row; ++l) {
+            if ((w * M + 8 * l + s) % extended >= size) continue;
+            if (last != l - 1) {
+                if (runs == 0) k.start0 = l; else k.start1 = l;
+                ++runs;
+            }
+            if (runs == 1) ++k.len0;
+            last = l;
+            ++k.count;
+        }
+        if (k.count == 0 || runs > 2) return 0;
+        k.first = w;
+        const bool full = k.count == per_row;
+        if (full && used == 1 && kinds[0].count == per_row) { ++windows[0]; continue; }
+        if (used == 3 || (full && used > 0)) return 0;
+        kinds[used] = k;
+        windows[used++] = 1;
+    }
+    for (int i = 0; i < used; ++i) { kinds[i].by_count = make_fast_div(kinds[i].count); kinds[i].by_windows = make_fast_div(windows[i]); }
+    return used;
+}
+
+inline bool make_live_windows(const Problem& p, LiveWindows* g)
+{
+    int ny_windows[3] = {0, 0, 0}, nx_windows[3] = {0, 0, 0};
+    *g = LiveWindows{};
+    const int ny = axis_kinds(p.H, p.M, p.s, g->y, ny_windows), nx = axis_kinds(p.W, p.M, p.s, g->x, nx_windows);
+    if (!ny || !nx) return false;
+    long long at = 0;
+    for (int k = 0; k < 9; ++k) {
+        g->offset[k] = (int)at;
+        const int ky = k / 3, kx = k % 3;
+        if (ky >= ny || kx >= nx) { g->items_per_window[k] = make_fast_div(1); continue; }
+        const int per_window = (g->y[ky].count * g->x[kx].count + 3) / 4;
+        g->items_per_window[k] = make_fast_div(per_window);
+        at += (long long)p.B * p.heads * ny_windows[ky] * nx_windows[kx] * per_window;
+        if (at > 0x7fffffffLL) return false;
+    }
+    g->offset[9] = (int)at;
+    g->by_heads = make_fast_div(p.heads);
+    return true;
+}
+
 // ---------------------------------------------------------------------------------- host side
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
