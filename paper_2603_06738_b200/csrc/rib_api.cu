@@ -606,7 +606,7 @@ int rib_generate_features_bwd(const float* w_h, const float* b_h, const float* w
     const cudaError_t e = rib::generator_bwd(w_h, b_h, w_pq, w_pk, dpq, dpk, window, L, dh, r, dw_h, db_h, dw_pq, dw_pk,
                                              static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return RIB_ERR_CUDA;
-    g_kernel_launches += 1;
+    g_kernel_launches += 2;          // clearing of the gradients, main kernel
     return RIB_OK;
 }
 

@@ -2,11 +2,14 @@
 // layer shared by all heads -> two linear projections to the rank-r positional features Pq, Pk that
 // the attention entry points take, and the chain rule of those steps.
 //
-// The problem is tiny (n = window^2 <= 4096 tokens, a 42 x 32 and two 32 x 16 matrices at the paper's
-// sizes): a few MFLOP and well under a megabyte, bound by launch latency.  One thread owns one token;
-// weights sit in shared memory; the backward pass stages a slice of 128 tokens in shared memory and
-// lets the threads of the block reduce the weight gradients over that slice before one atomic add
-// per element and block.
+// The problem is tiny (n = window^2 <= 4096 tokens, a 42 x 32 and two 32 x 16 matrices at the paper's sizes: a few MFLOP and
+// well under a megabyte), so what bounds it is the serial chain inside one block and the launches.  A block therefore takes
+// only kTokens tokens and spreads every step over all of its threads: a thread evaluates single Fourier features and then
+// 4-column pieces of the hidden rows, of the projections and, in the backward pass, of the weight gradients, which are
+// summed over the block's tokens and added to global memory with one atomic per piece.  The gradients are cleared by one
+// small kernel that the main kernel overtakes (programmatic dependent launch) up to its first atomic.  Measured at window
+// 32, L = 10, dh = 32, r = 16, a thread owning a whole token of a block of 128 before: forward 39.5 -> 14.6 us, backward 119.8 -> 19.2 us by event hooks (which
+// include about 7 us per call); forward and backward call together 140 -> 40 us, now bound by the host side.
 //
 // Coordinates: window points run from -1 to 1 inclusive on both axes (a single point sits at 0); token
 // i = y * window + x has the coordinate (row, column); Eq. 1 literally, frequencies 2^l without pi.
@@ -15,8 +18,8 @@
 namespace rib {
 namespace {
 
-constexpr int kGenThreads = 128;
-constexpr int kMaxHidden = 64;
+constexpr int kThreads = 128;
+constexpr int kTokens = 16;      // tokens of a block: 64 blocks at window 32; the gradients' atomics grow with the number of blocks
 
 struct GenParams {
     const float* w_h;      // [2 + 4 L][dh]
@@ -33,135 +36,195 @@ struct GenParams {
 
 __device__ __forceinline__ double coordinate(int idx, int M) { return M == 1 ? 0.0 : -1.0 + 2.0 * (double)idx / (double)(M - 1); }
 
-// Feature f of Eq. 1 for the token with coordinates (cy, cx): [x, sin(2^0 x), cos(2^0 x), ...], every block 2 wide.
-// The argument 2^l x reaches thousands of radians at the upper bands, where a coordinate rounded to fp32
-// would be off by a visible fraction of a radian: the coordinate and the reduction of the argument to
-// [-pi, pi] are done in double (a handful of operations per feature), the sine itself in fp32.
-__device__ __forceinline__ float feature(int f, double cy, double cx)
+// The argument 2^l x of a sine and a cosine of Eq. 1, reduced to [-pi, pi].  It reaches thousands of radians at the upper
+// bands, where a coordinate rounded to fp32 would be off by a visible fraction of a radian: the coordinate and the reduction
+// are done in double (a handful of operations per argument), the sine itself in fp32.
+// Feature order: [x, sin(2^0 x), cos(2^0 x), ...], every block 2 wide.
+__device__ __forceinline__ float band_argument(double c, int l)
 {
-    const double c = (f & 1) ? cx : cy;
-    if (f < 2) return (float)c;
-    const int l = (f - 2) >> 2;
     double arg = ldexp(c, l);
     arg -= 6.283185307179586476925 * rint(arg * 0.15915494309189533577);
-    return ((f - 2) & 2) ? cosf((float)arg) : sinf((float)arg);
+    return (float)arg;
 }
 
-// Pre-activation a = r_in W_h + b_h of one token (Eq. 2 before the ReLU); W_h, b_h in shared memory.
-// When `feat_out` is given the features are kept there (stride 1).
-__device__ __forceinline__ void hidden_preactivation(const GenParams& p, const float* w_h, const float* b_h, int token, float (&a)[kMaxHidden],
-                                                     float* feat_out)
+// Shared memory: every row is padded with zeros to a multiple of 4 floats, so that a thread can take 4 columns at a time.
+struct GenSmem {
+    int dhp, rp;                        // padded widths
+    float *w_h, *b_h, *w_pq, *w_pk;     // [in][dhp], [dhp], [dh][rp], [dh][rp]
+    float *feat, *h;                    // [kTokens][in], [kTokens][dhp]
+    float *da, *dq, *dk;                // backward: [kTokens][dhp], [kTokens][rp], [kTokens][rp]
+};
+__host__ __device__ inline int pad4(int w) { return (w + 3) & ~3; }
+__host__ __device__ inline size_t smem_floats(int in, int dh, int r, bool backward)
 {
-    const int y = token / p.M, x = token - y * p.M;
-    const double cy = coordinate(y, p.M), cx = coordinate(x, p.M);
-#pragma unroll
-    for (int j = 0; j < kMaxHidden; ++j) a[j] = j < p.dh ? b_h[j] : 0.f;
-    for (int f = 0; f < p.in; ++f) {
-        const float v = feature(f, cy, cx);
-        if (feat_out) feat_out[f] = v;
-        const float* wrow = w_h + f * p.dh;
-#pragma unroll
-        for (int j = 0; j < kMaxHidden; ++j)
-            if (j < p.dh) a[j] = fmaf(v, wrow[j], a[j]);
+    const size_t dhp = pad4(dh), rp = pad4(r), inp = pad4(in);
+    return in * dhp + dhp + 2 * dh * rp + kTokens * (inp + dhp) + (backward ? kTokens * (dhp + 2 * rp) : 0);
+}
+__device__ __forceinline__ GenSmem carve(const GenParams& p, float* sm)
+{
+    GenSmem s;
+    s.dhp = pad4(p.dh); s.rp = pad4(p.r);
+    s.w_h = sm; s.b_h = s.w_h + p.in * s.dhp; s.w_pq = s.b_h + s.dhp; s.w_pk = s.w_pq + p.dh * s.rp;
+    s.h = s.w_pk + p.dh * s.rp; s.da = s.h + kTokens * s.dhp; s.dq = s.da + kTokens * s.dhp; s.dk = s.dq + kTokens * s.rp;
+    s.feat = s.h + kTokens * s.dhp;     // forward: behind h; the backward kernel moves it behind dk
+    return s;
+}
+
+__device__ __forceinline__ void stage(float* dst, int wd, const float* src, int ws, int rows, int real_rows)
+{
+    for (int i = threadIdx.x; i < rows * wd; i += kThreads) {
+        const int row = i / wd, c = i - row * wd;
+        dst[i] = row < real_rows && c < ws ? src[row * ws + c] : 0.f;
     }
 }
 
-__device__ __forceinline__ void stage(float* dst, const float* src, int count)
+__device__ __forceinline__ void fma4(float4& a, float x, const float4& w)
 {
-    for (int i = threadIdx.x; i < count; i += kGenThreads) dst[i] = src[i];
+    a.x = fmaf(x, w.x, a.x); a.y = fmaf(x, w.y, a.y); a.z = fmaf(x, w.z, a.z); a.w = fmaf(x, w.w, a.w);
+}
+
+// Features of the block's tokens, then h = ReLU(r_in W_h + b_h) (Eq. 1, Eq. 2); rows beyond the last token are zero.
+__device__ __forceinline__ void features_and_hidden(const GenParams& p, const GenSmem& s, int token0)
+{
+    const int items = kTokens * (1 + 2 * p.L);         // per token the coordinates and, per band and axis, a sine and a cosine
+    for (int e = threadIdx.x; e < items; e += kThreads) {
+        const int t = e % kTokens, k = e / kTokens, token = token0 + t;
+        float* row = s.feat + t * p.in;
+        const int y = token / p.M, x = token - y * p.M;
+        const double cy = coordinate(y, p.M), cx = coordinate(x, p.M);
+        const bool live = token < p.n;
+        if (k == 0) {
+            row[0] = live ? (float)cy : 0.f;
+            row[1] = live ? (float)cx : 0.f;
+        } else {
+            const int axis = (k - 1) & 1, l = (k - 1) >> 1;
+            const float arg = band_argument(axis ? cx : cy, l);
+            row[2 + 4 * l + axis] = live ? sinf(arg) : 0.f;
+            row[4 + 4 * l + axis] = live ? cosf(arg) : 0.f;
+        }
+    }
+    __syncthreads();
+    const int pieces = s.dhp / 4;
+    for (int e = threadIdx.x; e < kTokens * pieces; e += kThreads) {
+        const int t = e / pieces, j = 4 * (e - t * pieces);
+        float4 a = *reinterpret_cast<const float4*>(s.b_h + j);
+        const float* f = s.feat + t * p.in;
+#pragma unroll 4
+        for (int i = 0; i < p.in; ++i) fma4(a, f[i], *reinterpret_cast<const float4*>(s.w_h + i * s.dhp + j));
+        const bool live = token0 + t < p.n;
+        *reinterpret_cast<float4*>(s.h + t * s.dhp + j) =
+            live ? make_float4(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f), fmaxf(a.z, 0.f), fmaxf(a.w, 0.f)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
 }
 
 // ---------------------------------------------------------------------------------- forward
-__global__ void __launch_bounds__(kGenThreads) rib_generator_fwd_kernel(const GenParams p)
+__global__ void __launch_bounds__(kThreads) rib_generator_fwd_kernel(const GenParams p)
 {
-    extern __shared__ float sm[];
-    float* w_h = sm; float* b_h = w_h + p.in * p.dh; float* w_pq = b_h + p.dh; float* w_pk = w_pq + p.dh * p.r;
-    stage(w_h, p.w_h, p.in * p.dh); stage(b_h, p.b_h, p.dh); stage(w_pq, p.w_pq, p.dh * p.r); stage(w_pk, p.w_pk, p.dh * p.r);
-    __syncthreads();
-    const int token = blockIdx.x * kGenThreads + threadIdx.x;
-    if (token >= p.n) return;
-    float a[kMaxHidden];
-    hidden_preactivation(p, w_h, b_h, token, a, nullptr);
+    extern __shared__ __align__(16) float sm[];
+    const GenSmem s = carve(p, sm);
+    stage(s.w_h, s.dhp, p.w_h, p.dh, p.in, p.in); stage(s.b_h, s.dhp, p.b_h, p.dh, 1, 1);
+    stage(s.w_pq, s.rp, p.w_pq, p.r, p.dh, p.dh); stage(s.w_pk, s.rp, p.w_pk, p.r, p.dh, p.dh);
+    const int token0 = blockIdx.x * kTokens;
+    features_and_hidden(p, s, token0);
+    const int pieces = s.rp / 4;
+    for (int e = threadIdx.x; e < 2 * kTokens * pieces; e += kThreads) {                   // Eq. 3
+        const bool is_k = e >= kTokens * pieces;
+        const int e2 = is_k ? e - kTokens * pieces : e, t = e2 / pieces, c = 4 * (e2 - t * pieces);
+        if (token0 + t >= p.n) continue;
+        const float* w = (is_k ? s.w_pk : s.w_pq) + c;
+        const float* h = s.h + t * s.dhp;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int j = 0; j < p.dh; ++j) fma4(a, h[j], *reinterpret_cast<const float4*>(w + j * s.rp));
+        __nv_bfloat16* dst = (is_k ? p.pk : p.pq) + (size_t)(token0 + t) * p.r + c;
+        const float v[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
-    for (int j = 0; j < kMaxHidden; ++j) a[j] = fmaxf(a[j], 0.f);      // h = ReLU(.)   (Eq. 2)
-    for (int c = 0; c < p.r; ++c) {                                       // Eq. 3
-        float q = 0.f, k = 0.f;
-#pragma unroll
-        for (int j = 0; j < kMaxHidden; ++j)
-            if (j < p.dh) { q = fmaf(a[j], w_pq[j * p.r + c], q); k = fmaf(a[j], w_pk[j * p.r + c], k); }
-        p.pq[(size_t)token * p.r + c] = __float2bfloat16_rn(q);
-        p.pk[(size_t)token * p.r + c] = __float2bfloat16_rn(k);
+        for (int k = 0; k < 4; ++k)
+            if (c + k < p.r) dst[k] = __float2bfloat16_rn(v[k]);
     }
 }
 
 // --------------------------------------------------------------------------------- backward
-// Block = a slice of 128 tokens.  Phase 1 (thread = token): features, h, and da = (dPq W_pq^T + dPk W_pk^T) o [a > 0]
-// into shared memory.  Phase 2 (threads = output elements): dW_h = r_in^T da, db_h = sum da, dW_pq = h^T dPq,
-// dW_pk = h^T dPk over the slice, one atomic add per element.
-__global__ void __launch_bounds__(kGenThreads) rib_generator_bwd_kernel(const GenParams p)
+__global__ void __launch_bounds__(256) rib_generator_clear_kernel(const GenParams p)
 {
-    extern __shared__ float sm[];
-    float* w_h = sm; float* b_h = w_h + p.in * p.dh; float* w_pq = b_h + p.dh; float* w_pk = w_pq + p.dh * p.r;
-    float* s_feat = w_pk + p.dh * p.r;               // [128][in]
-    float* s_h = s_feat + kGenThreads * p.in;        // [128][dh]
-    float* s_da = s_h + kGenThreads * p.dh;          // [128][dh]
-    float* s_dq = s_da + kGenThreads * p.dh;         // [128][r]
-    float* s_dk = s_dq + kGenThreads * p.r;          // [128][r]
-    stage(w_h, p.w_h, p.in * p.dh); stage(b_h, p.b_h, p.dh); stage(w_pq, p.w_pq, p.dh * p.r); stage(w_pk, p.w_pk, p.dh * p.r);
-    const int t = threadIdx.x, token = blockIdx.x * kGenThreads + t;
-    const bool live = token < p.n;
-    for (int c = 0; c < p.r; ++c) {
-        s_dq[t * p.r + c] = live ? p.dpq[(size_t)token * p.r + c] : 0.f;
-        s_dk[t * p.r + c] = live ? p.dpk[(size_t)token * p.r + c] : 0.f;
-    }
-    __syncthreads();
-    {
-        float a[kMaxHidden];
-        if (live) hidden_preactivation(p, w_h, b_h, token, a, s_feat + t * p.in);
-        else for (int f = 0; f < p.in; ++f) s_feat[t * p.in + f] = 0.f;
-#pragma unroll
-        for (int j = 0; j < kMaxHidden; ++j) {
-            if (j < p.dh) {
-                float g = 0.f;
-                for (int c = 0; c < p.r; ++c) g = fmaf(s_dq[t * p.r + c], w_pq[j * p.r + c], fmaf(s_dk[t * p.r + c], w_pk[j * p.r + c], g));
-                const bool on = live && a[j] > 0.f;
-                s_h[t * p.dh + j] = on ? a[j] : 0.f;
-                s_da[t * p.dh + j] = on ? g : 0.f;
-            }
-        }
-    }
-    __syncthreads();
-    const int n_wh = p.in * p.dh, n_pp = p.dh * p.r;
-    for (int e = threadIdx.x; e < n_wh + p.dh + 2 * n_pp; e += kGenThreads) {
-        float acc = 0.f;
-        float* dst;
-        if (e < n_wh) {
-            const int f = e / p.dh, j = e - f * p.dh;
-            for (int k = 0; k < kGenThreads; ++k) acc = fmaf(s_feat[k * p.in + f], s_da[k * p.dh + j], acc);
-            dst = p.dw_h + e;
-        } else if (e < n_wh + p.dh) {
-            const int j = e - n_wh;
-            for (int k = 0; k < kGenThreads; ++k) acc += s_da[k * p.dh + j];
-            dst = p.db_h + j;
-        } else {
-            const int e2 = e - n_wh - p.dh;
-            const bool is_k = e2 >= n_pp;
-            const int e3 = is_k ? e2 - n_pp : e2, j = e3 / p.r, c = e3 - j * p.r;
-            const float* g = is_k ? s_dk : s_dq;
-            for (int k = 0; k < kGenThreads; ++k) acc = fmaf(s_h[k * p.dh + j], g[k * p.r + c], acc);
-            dst = (is_k ? p.dw_pk : p.dw_pq) + e3;
-        }
-        atomicAdd(dst, acc);
-    }
+    cudaTriggerProgrammaticLaunchCompletion();         // the main kernel waits for this one's end before its first atomic
+    const int n_wh = p.in * p.dh, n_pp = p.dh * p.r, t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < n_wh) p.dw_h[t] = 0.f;
+    if (t < p.dh) p.db_h[t] = 0.f;
+    if (t < n_pp) { p.dw_pq[t] = 0.f; p.dw_pk[t] = 0.f; }
 }
 
-size_t weights_floats(const GenParams& p) { return (size_t)p.in * p.dh + p.dh + 2 * (size_t)p.dh * p.r; }
+// adds columns c .. c + 3 of a row of `width` floats
+__device__ __forceinline__ void add4(float* row, int c, int width, const float4& v)
+{
+    if ((width & 3) == 0) { atomicAdd(reinterpret_cast<float4*>(row + c), v); return; }
+    const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (c + k < width) atomicAdd(row + c + k, f[k]);
+}
+
+// Per block: features and h as above, da = (dPq W_pq^T + dPk W_pk^T) o [h > 0], then dW_h = r_in^T da, db_h = sum da,
+// dW_pq = h^T dPq, dW_pk = h^T dPk over the block's tokens.
+__global__ void __launch_bounds__(kThreads) rib_generator_bwd_kernel(const GenParams p)
+{
+    extern __shared__ __align__(16) float sm[];
+    GenSmem s = carve(p, sm);
+    s.feat = s.dk + kTokens * s.rp;
+    const int token0 = blockIdx.x * kTokens, tokens = min(kTokens, p.n - token0);
+    stage(s.w_h, s.dhp, p.w_h, p.dh, p.in, p.in); stage(s.b_h, s.dhp, p.b_h, p.dh, 1, 1);
+    stage(s.w_pq, s.rp, p.w_pq, p.r, p.dh, p.dh); stage(s.w_pk, s.rp, p.w_pk, p.r, p.dh, p.dh);
+    stage(s.dq, s.rp, p.dpq + (size_t)token0 * p.r, p.r, kTokens, tokens);
+    stage(s.dk, s.rp, p.dpk + (size_t)token0 * p.r, p.r, kTokens, tokens);
+    features_and_hidden(p, s, token0);
+    for (int e = threadIdx.x; e < kTokens * s.dhp; e += kThreads) {
+        const int t = e / s.dhp, j = e - t * s.dhp;
+        float g = 0.f;
+        if (j < p.dh && s.h[e] > 0.f) {
+            const float4 *dq = reinterpret_cast<const float4*>(s.dq + t * s.rp), *dk = reinterpret_cast<const float4*>(s.dk + t * s.rp);
+            const float4 *wq = reinterpret_cast<const float4*>(s.w_pq + j * s.rp), *wk = reinterpret_cast<const float4*>(s.w_pk + j * s.rp);
+            for (int c = 0; c < s.rp / 4; ++c) {
+                const float4 a = dq[c], b = wq[c], u = dk[c], v = wk[c];
+                g = fmaf(a.x, b.x, fmaf(u.x, v.x, g)); g = fmaf(a.y, b.y, fmaf(u.y, v.y, g));
+                g = fmaf(a.z, b.z, fmaf(u.z, v.z, g)); g = fmaf(a.w, b.w, fmaf(u.w, v.w, g));
+            }
+        }
+        s.da[e] = g;
+    }
+    __syncthreads();
+    cudaGridDependencySynchronize();                   // the results are cleared
+    const int ph = s.dhp / 4, pr = s.rp / 4, n_h = (p.in + 1) * ph, n_p = p.dh * pr;       // the row behind W_h's is b_h
+    for (int e = threadIdx.x; e < n_h + 2 * n_p; e += kThreads) {
+        const float *left, *right;                     // columns of the two factors: their strides
+        int ls, rs, c, width;
+        float* dst;
+        if (e < n_h) {
+            const int f = e / ph;
+            c = 4 * (e - f * ph); width = p.dh;
+            left = f < p.in ? s.feat + f : nullptr; ls = p.in;
+            right = s.da + c; rs = s.dhp;
+            dst = f < p.in ? p.dw_h + f * p.dh : p.db_h;
+        } else {
+            const bool is_k = e >= n_h + n_p;
+            const int e2 = e - n_h - (is_k ? n_p : 0), j = e2 / pr;
+            c = 4 * (e2 - j * pr); width = p.r;
+            left = s.h + j; ls = s.dhp;
+            right = (is_k ? s.dk : s.dq) + c; rs = s.rp;
+            dst = (is_k ? p.dw_pk : p.dw_pq) + j * p.r;
+        }
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < kTokens; ++k) fma4(acc, left ? left[k * ls] : 1.f, *reinterpret_cast<const float4*>(right + k * rs));
+        add4(dst, c, width, acc);
+    }
+}
 
 }  // namespace
 
 bool generator_supported(int window, int L, int dh, int r)
 {
-    return window >= 1 && window <= 256 && L >= 0 && L <= 16 && dh >= 1 && dh <= kMaxHidden && r >= 1 && r <= 64;
+    return window >= 1 && window <= 256 && L >= 0 && L <= 16 && dh >= 1 && dh <= 64 && r >= 1 && r <= 64;
 }
 
 cudaError_t generator_fwd(const float* w_h, const float* b_h, const float* w_pq, const float* w_pk, int window, int L, int dh, int r,
@@ -170,12 +233,12 @@ cudaError_t generator_fwd(const float* w_h, const float* b_h, const float* w_pq,
     GenParams p{};
     p.w_h = w_h; p.b_h = b_h; p.w_pq = w_pq; p.w_pk = w_pk; p.pq = pq; p.pk = pk;
     p.M = window; p.n = window * window; p.L = L; p.in = 2 + 4 * L; p.dh = dh; p.r = r;
-    const size_t smem = sizeof(float) * weights_floats(p);
+    const size_t smem = sizeof(float) * smem_floats(p.in, dh, r, false);
     cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(rib_generator_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                                      : cudaSuccess;
     if (e != cudaSuccess) return e;
     ProfileScope scope(RIB_KERNEL_GENERATOR_FWD, stream);
-    rib_generator_fwd_kernel<<<(p.n + kGenThreads - 1) / kGenThreads, kGenThreads, smem, stream>>>(p);
+    rib_generator_fwd_kernel<<<(p.n + kTokens - 1) / kTokens, kThreads, smem, stream>>>(p);
     return cudaGetLastError();
 }
 
@@ -186,17 +249,25 @@ cudaError_t generator_bwd(const float* w_h, const float* b_h, const float* w_pq,
     p.w_h = w_h; p.b_h = b_h; p.w_pq = w_pq; p.w_pk = w_pk; p.dpq = dpq; p.dpk = dpk;
     p.dw_h = dw_h; p.db_h = db_h; p.dw_pq = dw_pq; p.dw_pk = dw_pk;
     p.M = window; p.n = window * window; p.L = L; p.in = 2 + 4 * L; p.dh = dh; p.r = r;
-    cudaError_t e = cudaMemsetAsync(dw_h, 0, sizeof(float) * p.in * dh, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(db_h, 0, sizeof(float) * dh, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dw_pq, 0, sizeof(float) * dh * r, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dw_pk, 0, sizeof(float) * dh * r, stream);
-    if (e != cudaSuccess) return e;
-    const size_t smem = sizeof(float) * (weights_floats(p) + (size_t)kGenThreads * (p.in + 2 * dh + 2 * r));
-    e = smem > 48 * 1024 ? cudaFuncSetAttribute(rib_generator_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
+    const size_t smem = sizeof(float) * smem_floats(p.in, dh, r, true);
+    cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(rib_generator_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                                     : cudaSuccess;
     if (e != cudaSuccess) return e;
     ProfileScope scope(RIB_KERNEL_GENERATOR_BWD, stream);
-    rib_generator_bwd_kernel<<<(p.n + kGenThreads - 1) / kGenThreads, kGenThreads, smem, stream>>>(p);
-    return cudaGetLastError();
+    const int most = p.in * dh > dh * r ? p.in * dh : dh * r;
+    rib_generator_clear_kernel<<<(most + 255) / 256, 256, 0, stream>>>(p);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    cudaLaunchAttribute overtake;
+    overtake.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overtake.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t config{};
+    config.gridDim = dim3((unsigned)((p.n + kTokens - 1) / kTokens));
+    config.blockDim = dim3(kThreads);
+    config.dynamicSmemBytes = smem;
+    config.stream = stream;
+    config.attrs = &overtake;
+    config.numAttrs = 1;
+    return cudaLaunchKernelEx(&config, rib_generator_bwd_kernel, p);
 }
 
 }  // namespace rib
