@@ -478,7 +478,7 @@ static int bwd_impl(const void* q, const void* k, const void* v, const void* pq,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const bool allowed = g_forced_path.load() != RIB_PATH_GENERIC;
     bool fast = allowed && rib::sm100_bwd_supported(p);
-    int launches = 3;          // prepare, main, finish : rowdot, dq, dk/dv
+    int launches = fast ? rib::sm100_bwd_launches(p) : 3;          // any-shape kernels: rowdot, dq, dk/dv
     cudaError_t e;
     if (fast) {
         e = rib::sm100_bwd(p, st);

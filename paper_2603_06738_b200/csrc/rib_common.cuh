@@ -41,9 +41,6 @@ struct Problem {
     bool masked;                      // shifted windows: the wrapped parts of a border window do not attend to each other
     int d_true, r_true;               // tcgen05 kernels on zero-padded copies (rib_repack.cu): the widths the scales 1/sqrt(d),
                                       // 1/sqrt(r) are taken from; 0 = d, r themselves
-    bool packed8;                     // tcgen05 kernels only: M, n, nWy, nWx, pairs describe 16 x 16 windows that each stand for
-                                      // 2 x 2 windows of 8 x 8 tokens (a token attends to the 8 x 8 patch it lies in; the tables
-                                      // pq, pk, dpq, dpk have 64 rows)
 };
 
 // Pq/Pk tables: one shared by the heads, or one per head (Sec. 3.1, after Eq. 3: head-wise projections of the shared h).
@@ -70,7 +67,12 @@ bool sm100_frame_supported(const Problem& p);
 cudaError_t sm100_fwd_frame(const Problem& p, cudaStream_t stream);
 bool sm100_bwd_supported(const Problem& p);
 size_t sm100_bwd_workspace_bytes(long long pairs, int n, int tables, int r);
-cudaError_t sm100_bwd(const Problem& p, cudaStream_t stream);   // launches 3 kernels
+cudaError_t sm100_bwd(const Problem& p, cudaStream_t stream);
+int sm100_bwd_launches(const Problem& p);     // kernels it enqueues
+// Windows of 8 x 8 tokens (rib_window8_sm100.cu); the backward launches 2 kernels.
+bool sm100_window8(const Problem& p);
+cudaError_t sm100_window8_fwd(const Problem& p, cudaStream_t stream);
+cudaError_t sm100_window8_bwd(const Problem& p, cudaStream_t stream);
 // Even head widths and ranks up to 32 whose rows TMA cannot address (60-byte rows of d = 30, 36-byte rows of r = 18):
 // the tensors are copied into zero-padded scratch (stream-ordered allocation), the tcgen05 kernels run on the copies,
 // and the results are copied back.  `launches` receives the number of kernels enqueued.

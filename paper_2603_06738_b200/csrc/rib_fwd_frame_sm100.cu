@@ -445,7 +445,7 @@ cudaError_t launch_fwd_frame(const Problem& p, cudaStream_t stream)
 bool sm100_frame_supported(const Problem& p)
 {
     return p.d % 8 == 0 && p.d >= 8 && p.d <= kD && p.r % 8 == 0 && p.r >= 8 && p.r <= 32 && p.M % 16 == 0 && p.M <= 256 && p.s % 8 == 0 &&
-           (p.H % 8 || p.W % 8) && !p.masked && !p.gate && !p.packed8;
+           (p.H % 8 || p.W % 8) && !p.masked && !p.gate;
 }
 
 cudaError_t sm100_fwd_frame(const Problem& p, cudaStream_t stream)

@@ -311,7 +311,7 @@ cudaError_t sm100_bwd_repacked(const Problem& p, cudaStream_t stream, int* launc
         pp.dq = image(5); pp.dk = image(6); pp.dv = image(7);
         pp.pq = pq2; pp.pk = pk2; pp.dpq = dpq2; pp.dpk = dpk2;
         e = sm100_bwd(pp, stream);
-        *launches += 3;
+        *launches += sm100_bwd_launches(pp);
     }
     __nv_bfloat16* outs[3] = {p.dq, p.dk, p.dv};
     for (int i = 0; i < 3 && !e; ++i) e = resize_rows(image(5 + i), pp.d, outs[i], p.d, rows, stream, launches);
