@@ -363,8 +363,10 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             merge[half * kTile + row] = make_float2(m_used, l);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(L::kMerge + 4 * qt + quarter));
-            // The partner's (m, l) must be there and the item's last PV must have completed.
+            // The partner's (m, l) must be there and the item's last PV must have completed.  (A parity wait cannot tell "two
+            // phases ahead" from "not yet", and nothing above has waited for the PV before the last one: it is waited for first.)
             if (!mbar_wait_warp(bar(L::kMerge + 4 * qt + quarter), nmerge & 1, abort_flag, p.status) ||
+                !(blk < 2 || mbar_wait_warp(bar(L::kPVDone + qt), (blk - 2) & 1, abort_flag, p.status)) ||
                 !mbar_wait_warp(bar(L::kPVDone + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
             uint32_t oa[16], ob[16];
