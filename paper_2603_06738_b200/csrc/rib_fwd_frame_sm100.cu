@@ -350,6 +350,9 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     tmem_st16(t_half + sb * kTile + 32 + 16 * ch, lo);
                 }
                 l += (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
+                // The epilogue waits for this block's PV.  A parity wait cannot tell "two phases ahead" from "not yet", so the
+                // phase before it is seen here, while P of this block is still held back and its own phase cannot complete.
+                if (j == nblk - 1 && blk > 0 && !mbar_wait_warp(bar(L::kPVDone + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
@@ -363,10 +366,8 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             merge[half * kTile + row] = make_float2(m_used, l);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(L::kMerge + 4 * qt + quarter));
-            // The partner's (m, l) must be there and the item's last PV must have completed.  (A parity wait cannot tell "two
-            // phases ahead" from "not yet", and nothing above has waited for the PV before the last one: it is waited for first.)
+            // The partner's (m, l) must be there and the item's last PV must have completed.
             if (!mbar_wait_warp(bar(L::kMerge + 4 * qt + quarter), nmerge & 1, abort_flag, p.status) ||
-                !(blk < 2 || mbar_wait_warp(bar(L::kPVDone + qt), (blk - 2) & 1, abort_flag, p.status)) ||
                 !mbar_wait_warp(bar(L::kPVDone + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
             uint32_t oa[16], ob[16];
