@@ -832,11 +832,12 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-int sm100_bwd_launches(const Problem& p) { return sm100_window8(p) ? 2 : 3; }      // clear, main; prepare, main, finish
+int sm100_bwd_launches(const Problem& p) { return sm100_window8(p) ? 2 : 3; }      // clear, main; else two clears, main or prepare, main, finish
 
 cudaError_t sm100_bwd(const Problem& p, cudaStream_t stream)
 {
     if (sm100_window8(p)) return sm100_window8_bwd(p, stream);
+    if (sm100_window16(p)) return sm100_window16_bwd(p, stream);
     const bool wide = padded_rank(p.r) == 32;      // accumulators with 32 RIB columns (ranks 24 and 32), else 16 (ranks 8 and 16)
     if (p.Hp != p.H || p.Wp != p.W || p.masked) return wide ? launch_bwd<32, true>(p, stream) : launch_bwd<16, true>(p, stream);
     return wide ? launch_bwd<32, false>(p, stream) : launch_bwd<16, false>(p, stream);

@@ -73,6 +73,11 @@ int sm100_bwd_launches(const Problem& p);     // kernels it enqueues
 bool sm100_window8(const Problem& p);
 cudaError_t sm100_window8_fwd(const Problem& p, cudaStream_t stream);
 cudaError_t sm100_window8_bwd(const Problem& p, cudaStream_t stream);
+// Windows of 16 x 16 tokens (rib_window16_sm100.cu); the backward launches 3 kernels.
+bool sm100_window16(const Problem& p);
+bool sm100_window16_prefers(const Problem& p);        // ... the forward kernel
+cudaError_t sm100_window16_fwd(const Problem& p, cudaStream_t stream);
+cudaError_t sm100_window16_bwd(const Problem& p, cudaStream_t stream);
 // Even head widths and ranks up to 32 whose rows TMA cannot address (60-byte rows of d = 30, 36-byte rows of r = 18):
 // the tensors are copied into zero-padded scratch (stream-ordered allocation), the tcgen05 kernels run on the copies,
 // and the results are copied back.  `launches` receives the number of kernels enqueued.

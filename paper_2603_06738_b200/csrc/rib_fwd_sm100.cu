@@ -963,6 +963,7 @@ cudaError_t launch_fwd(const Problem& p, cudaStream_t stream)
 cudaError_t sm100_fwd(const Problem& p, cudaStream_t stream)
 {
     if (sm100_window8(p)) return sm100_window8_fwd(p, stream);
+    if (sm100_window16_prefers(p)) return sm100_window16_fwd(p, stream);
     const bool wide = padded_rank(p.r) == 32;      // RIB rows of 32 elements (ranks 24 and 32), else of 16 (ranks 8 and 16)
     if (p.Hp != p.H || p.Wp != p.W || p.masked) return wide ? launch_fwd<32, true, false>(p, stream) : launch_fwd<16, true, false>(p, stream);
     if (p.gate) return wide ? launch_fwd<32, false, true>(p, stream) : launch_fwd<16, false, true>(p, stream);

@@ -16,33 +16,16 @@
 //
 // A score tile is computed 128 x 128 although only its two diagonal 64 x 64 blocks are meant (an M128 N128 MMA costs what
 // two M64 N64 would); rows read their own block, and the other block of P (dS) is zero wherever it is contracted.
-#include "rib_sm100_common.cuh"
+#include "rib_small_window.cuh"
 
 namespace rib {
 namespace {
 
 using namespace sm100;
 
-struct Win8Params {
-    const __nv_bfloat16* pq;
-    const __nv_bfloat16* pk;
-    const float* lse_in;       // backward
-    float* lse;                // forward, may be null
-    float* dpq;
-    float* dpk;
-    int* status;
-    int H, W, heads, r;
-    int tiles, groups;         // tiles of one head; CTAs of one head
-    FastDiv by_heads, by_nx, by_ny;      // heads, W / 16, H / 8
-    float scale_log2;          // log2(e) / sqrt(d)
-    float inv_sqrt_d, inv_sqrt_r;
-    float pos_scale;           // sqrt(d / r)
-    long long pos_head_stride;
-};
-
 struct Win8Tile { int b, Y0, X0; };      // first token of the left window
 
-__device__ __forceinline__ Win8Tile decode_tile(const Win8Params& p, int tile)
+__device__ __forceinline__ Win8Tile decode_tile(const SmallWindowParams& p, int tile)
 {
     Win8Tile t;
     int y, x;
@@ -50,38 +33,6 @@ __device__ __forceinline__ Win8Tile decode_tile(const Win8Params& p, int tile)
     p.by_ny.divmod(tile, t.b, y);
     t.Y0 = 8 * y; t.X0 = 16 * x;
     return t;
-}
-
-// The RIB rows of a head as 64-byte rows (32 elements, zeros from column r on; SWIZZLE_64B like a content tile), the 64 rows
-// of the table twice; thread t < 128 writes row t of both tiles.  Query rows are scaled by sqrt(d / r) and rounded to bf16.
-__device__ __forceinline__ void stage_rib_rows(const Win8Params& p, int head, uint8_t* q_tile, uint8_t* k_tile, int row)
-{
-    const size_t at = (size_t)head * p.pos_head_stride + (size_t)(row & 63) * p.r;
-    const uint4 *q = reinterpret_cast<const uint4*>(p.pq + at), *k = reinterpret_cast<const uint4*>(p.pk + at);
-    const int sw = (row >> 1) & 3;
-#pragma unroll
-    for (int ck = 0; ck < 4; ++ck) {
-        const uint4 zero = make_uint4(0u, 0u, 0u, 0u), a = 8 * ck < p.r ? __ldg(q + ck) : zero, b = 8 * ck < p.r ? __ldg(k + ck) : zero;
-        uint32_t w[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            w[e] = pack_bf16x2(__uint_as_float(w[e] << 16) * p.pos_scale, __uint_as_float(w[e] & 0xffff0000u) * p.pos_scale);
-        *reinterpret_cast<uint4*>(q_tile + row * 64 + ((ck ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-        *reinterpret_cast<uint4*>(k_tile + row * 64 + ((ck ^ sw) << 4)) = b;
-    }
-}
-
-// 32 fp32 columns of a row (times f) as a bf16 row of a 64-byte-row tile
-__device__ __forceinline__ void write_row(uint8_t* tile, int row, const uint32_t (&a)[32], float f)
-{
-    const int sw = (row >> 1) & 3;
-#pragma unroll
-    for (int ck = 0; ck < 4; ++ck)
-        *reinterpret_cast<uint4*>(tile + row * 64 + ((ck ^ sw) << 4)) =
-            make_uint4(pack_bf16x2(__uint_as_float(a[8 * ck]) * f, __uint_as_float(a[8 * ck + 1]) * f),
-                       pack_bf16x2(__uint_as_float(a[8 * ck + 2]) * f, __uint_as_float(a[8 * ck + 3]) * f),
-                       pack_bf16x2(__uint_as_float(a[8 * ck + 4]) * f, __uint_as_float(a[8 * ck + 5]) * f),
-                       pack_bf16x2(__uint_as_float(a[8 * ck + 6]) * f, __uint_as_float(a[8 * ck + 7]) * f));
 }
 
 constexpr uint64_t kDesc64 = smem_desc_const(16, 512, kSwizzle64B);
@@ -107,7 +58,7 @@ static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 template <int R>
 __global__ void __launch_bounds__(kThreads, 1)
 rib_window8_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                       const __grid_constant__ CUtensorMap tm_out, const __grid_constant__ Win8Params p)
+                       const __grid_constant__ CUtensorMap tm_out, const __grid_constant__ SmallWindowParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -135,7 +86,8 @@ rib_window8_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         tmem_relinquish();
     }
     if (warp >= 4 && warp < 8) {
-        stage_rib_rows(p, head, base_ptr + kOffRib, base_ptr + kOffRib + kContentBytes, (int)threadIdx.x - 128);
+        const int row = (int)threadIdx.x - 128;             // the 64 rows of the tables twice
+        stage_rib_row(p, head, row & 63, base_ptr + kOffRib, base_ptr + kOffRib + kContentBytes, row);
         fence_proxy_async();
     }
     tc_fence_before();
@@ -325,7 +277,7 @@ template <int R>
 __global__ void __launch_bounds__(kThreads, 1)
 rib_window8_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                        const __grid_constant__ CUtensorMap tm_do, const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ CUtensorMap tm_dq,
-                       const __grid_constant__ CUtensorMap tm_dk, const __grid_constant__ CUtensorMap tm_dv, const __grid_constant__ Win8Params p)
+                       const __grid_constant__ CUtensorMap tm_dk, const __grid_constant__ CUtensorMap tm_dv, const __grid_constant__ SmallWindowParams p)
 {
     constexpr uint32_t kIdescGrad = idesc_bf16_f32_ab(kTile, kD + R, false, true);       // dQ~: A in TMEM
     constexpr uint32_t kIdescGradT = idesc_bf16_f32_ab(kTile, kD + R, true, true);       // dK~: A MN-major
@@ -356,7 +308,7 @@ rib_window8_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
     if (warp >= 4 && warp < 8) {
         const int t = (int)threadIdx.x - 128;
-        stage_rib_rows(p, head, base_ptr + kOffRib, base_ptr + kOffRib + kContentBytes, t);
+        stage_rib_row(p, head, t & 63, base_ptr + kOffRib, base_ptr + kOffRib + kContentBytes, t);
         *reinterpret_cast<uint4*>(base_ptr + kOffZeroLo + 16 * t) = make_uint4(0u, 0u, 0u, 0u);
         *reinterpret_cast<uint4*>(base_ptr + kOffZeroHi + 16 * t) = make_uint4(0u, 0u, 0u, 0u);
         fence_proxy_async();
@@ -585,11 +537,8 @@ rib_window8_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 #pragma unroll
                 for (int q4 = 0; q4 < 4; ++q4) {
                     if (16 * part + 4 * q4 >= p.r) break;                      // ranks are multiples of 8
-                    const float fq = p.inv_sqrt_r, fk = p.inv_sqrt_d;          // (the query rows carried sqrt(d / r))
-                    atomicAdd(reinterpret_cast<float4*>(gq + 16 * part + 4 * q4),
-                              make_float4(__uint_as_float(a[4 * q4]) * fq, __uint_as_float(a[4 * q4 + 1]) * fq, __uint_as_float(a[4 * q4 + 2]) * fq, __uint_as_float(a[4 * q4 + 3]) * fq));
-                    atomicAdd(reinterpret_cast<float4*>(gk + 16 * part + 4 * q4),
-                              make_float4(__uint_as_float(b[4 * q4]) * fk, __uint_as_float(b[4 * q4 + 1]) * fk, __uint_as_float(b[4 * q4 + 2]) * fk, __uint_as_float(b[4 * q4 + 3]) * fk));
+                    add_columns(gq + 16 * part + 4 * q4, a + 4 * q4, p.inv_sqrt_r);
+                    add_columns(gk + 16 * part + 4 * q4, b + 4 * q4, p.inv_sqrt_d);      // (the query rows carried sqrt(d / r))
                 }
             }
         }
@@ -616,24 +565,6 @@ __global__ void __launch_bounds__(256) rib_window8_clear_kernel(float* dpq, floa
 }
 }  // namespace bwd8
 
-// One CTA per SM, a whole number per head; with more heads than SMs a CTA per head.
-void fill_win8(const Problem& p, int sm_count, Win8Params* w, int* grid)
-{
-    w->pq = p.pq; w->pk = p.pk; w->status = p.status;
-    w->H = p.H; w->W = p.W; w->heads = p.heads; w->r = p.r;
-    w->tiles = p.B * (p.H / 8) * (p.W / 16);
-    w->groups = sm_count / p.heads > 1 ? sm_count / p.heads : 1;
-    if (w->groups > w->tiles) w->groups = w->tiles;
-    *grid = w->groups * p.heads;
-    w->by_heads = make_fast_div(p.heads); w->by_nx = make_fast_div(p.W / 16); w->by_ny = make_fast_div(p.H / 8);
-    const float d = scale_width_d(p), r = scale_width_r(p);
-    w->scale_log2 = 1.4426950408889634f / sqrtf(d);
-    w->inv_sqrt_d = 1.f / sqrtf(d);
-    w->inv_sqrt_r = 1.f / sqrtf(r);
-    w->pos_scale = sqrtf(d / r);
-    w->pos_head_stride = p.pos_head_stride;
-}
-
 template <int R>
 cudaError_t launch_win8_fwd(const Problem& p, cudaStream_t stream)
 {
@@ -642,10 +573,10 @@ cudaError_t launch_win8_fwd(const Problem& p, cudaStream_t stream)
     if (!encode_image_map(&tm_q, p.q, p) || !encode_image_map(&tm_k, p.k, p) || !encode_image_map(&tm_v, p.v, p) || !encode_image_map(&tm_out, p.out_w, p))
         return cudaErrorInvalidValue;
     static KernelSetup setup;       // one per instantiation of this launcher, i.e. per kernel
-    int sm_count = 0, grid = 0;
+    int sm_count = 0;
     if (cudaError_t e = setup.prepare(fwd8::rib_window8_fwd_kernel<R>, fwd8::kSmemBytes, &sm_count)) return e;
-    Win8Params w{};
-    fill_win8(p, sm_count, &w, &grid);
+    SmallWindowParams w{};
+    const int grid = fill_small_window(p, sm_count, p.H / 8, p.W / 16, &w);
     w.lse = p.lse_w;
     ProfileScope scope(RIB_KERNEL_FWD_MAIN, stream);
     fwd8::rib_window8_fwd_kernel<R><<<grid, fwd8::kThreads, fwd8::kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_out, w);
@@ -661,27 +592,17 @@ cudaError_t launch_win8_bwd(const Problem& p, cudaStream_t stream)
         !encode_image_map(&tm_o, p.out, p) || !encode_image_map(&tm_dq, p.dq, p) || !encode_image_map(&tm_dk, p.dk, p) || !encode_image_map(&tm_dv, p.dv, p))
         return cudaErrorInvalidValue;
     static KernelSetup setup;
-    int sm_count = 0, grid = 0;
+    int sm_count = 0;
     if (cudaError_t e = setup.prepare(bwd8::rib_window8_bwd_kernel<R>, bwd8::kSmemBytes, &sm_count)) return e;
-    Win8Params w{};
-    fill_win8(p, sm_count, &w, &grid);
+    SmallWindowParams w{};
+    const int grid = fill_small_window(p, sm_count, p.H / 8, p.W / 16, &w);
     w.lse_in = p.lse_in; w.dpq = p.dpq; w.dpk = p.dpk;
     const int tables = pos_tables(p), per_table = 64 * p.r;
     bwd8::rib_window8_clear_kernel<<<(tables * per_table + 255) / 256 < 64 ? (tables * per_table + 255) / 256 : 64, 256, 0, stream>>>(
         p.dpq, p.dpk, tables, per_table, p.pos_head_stride);
     if (cudaError_t e = cudaGetLastError()) return e;
-    cudaLaunchAttribute overtake;
-    overtake.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    overtake.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t config{};
-    config.gridDim = dim3((unsigned)grid);
-    config.blockDim = dim3(bwd8::kThreads);
-    config.dynamicSmemBytes = bwd8::kSmemBytes;
-    config.stream = stream;
-    config.attrs = &overtake;
-    config.numAttrs = 1;
     ProfileScope scope(RIB_KERNEL_BWD_MAIN, stream);
-    return cudaLaunchKernelEx(&config, bwd8::rib_window8_bwd_kernel<R>, tm_q, tm_k, tm_v, tm_do, tm_o, tm_dq, tm_dk, tm_dv, w);
+    return launch_overtaking(bwd8::rib_window8_bwd_kernel<R>, grid, bwd8::kThreads, bwd8::kSmemBytes, stream, tm_q, tm_k, tm_v, tm_do, tm_o, tm_dq, tm_dk, tm_dv, w);
 }
 
 }  // namespace
