@@ -39,11 +39,9 @@
 //   integer pipes instead of the MUFU.
 //   Exact form (second pass): classic online softmax per key half
 //   with a running maximum, lazy rescaling of O, separate accumulators and a log-sum-exp merge.
-//   On maps with partial windows (kPartial) key patches in the extension of the map contribute probability 0 in
-//   both forms, the fast form takes its reference from the first block that holds real keys, and items whose query
-//   patches all lie in the extension are skipped by every role alike.
-//   Shifted windows with a mask run on the kPartial instantiation too: for a query patch the patches of the other part
-//   of its border window count as patches of the extension.
+//   On maps with partial windows (kPartial) only patches that hold tokens are walked (LiveWindows in rib_sm100_common.cuh), and
+//   with a mask the parts of a border window are windows of their own; an odd number of patches leaves the second half
+//   of the last block without keys: zero rows of K and V, left out of the row sum by a second tile of ones.
 //
 // Tiles are two 8x8-token patches (see rib_sm100_common.cuh), fetched by one TMA box each.
 //
@@ -68,10 +66,6 @@ using namespace sm100;
 constexpr int kStages = 4;            // K/V ring depth
 constexpr int kThreads = 640;
 constexpr int kMaxRedo = 64;          // items a CTA can note for the exact pass (more: all of its items are redone)
-constexpr int kMaxListed = 1023;      // kPartial: items of a CTA whose masks are worked out once and kept in shared memory
-
-// kPartial with skipping: an item of the CTA that holds tokens, with what every role needs to walk it
-struct ItemRec { int item; uint32_t row_dead, col_dead, range; };       // range = first | last << 16 key block with tokens
 constexpr uint32_t kPolyMask = RIB_FWD_POLY_MASK;
 
 // kSFull .. kOFree: one per query tile; kDrain: one per issuing warp; kMerge: 4 * tile + quarter of the rows
@@ -90,14 +84,13 @@ struct Layout {
     static constexpr uint32_t kOffKp = kOffKc + kStages * kContentBytes;         // [kStages] key RIB rows
     static constexpr uint32_t kOffV = kOffKp + kStages * kPosBytes;              // [kStages] values
     static constexpr uint32_t kOffOnes = kOffV + kStages * kContentBytes;        // [128 keys][32] column 0 = 1: second atom of V
-    static constexpr uint32_t kOffBar = kOffOnes + kContentBytes;
+    static constexpr uint32_t kOffHalfOnes = kOffOnes + kContentBytes;           // the same with 0 in keys 64 .. 127 (kPartial)
+    static constexpr uint32_t kOffBar = kOffHalfOnes + kContentBytes;
     static constexpr uint32_t kOffMisc = kOffBar + kNumBars * 8;                 // tmem base, abort flags, redo count
     static constexpr uint32_t kOffRedo = kOffMisc + 16;                          // [kMaxRedo] item ordinals of the exact pass
     static constexpr uint32_t kOffMerge = kOffRedo + kMaxRedo * 4;               // [2 tiles][2 halves][128 rows] (max, sum)
-    static constexpr uint32_t kOffItems = kOffMerge + 4 * kTile * 8;             // [1 + kMaxListed] ItemRec; entry 0 holds the count
-    static constexpr uint32_t kSmemBytes = kOffItems + 1024;                           // + slack for manual alignment
-    static constexpr uint32_t kSmemBytesPartial = kOffItems + (1 + kMaxListed) * 16 + 1024;   // kPartial instantiations: with the item list
-    static_assert(kSmemBytesPartial <= 232448, "shared memory of one CTA");
+    static constexpr uint32_t kSmemBytes = kOffMerge + 4 * kTile * 8 + 1024;     // + slack for manual alignment
+    static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
     static_assert(kOffV % 1024 == 0 && kOffOnes % 1024 == 0, "swizzle atoms need aligned tiles");
 };
 
@@ -127,14 +120,14 @@ struct FwdParams {
     long long pos_head_stride; // elements between the heads' Pq tables (0: one table for all heads)
     int pos_per_head;          // 1 when Pq/Pk are head-wise: table index = head
     int exact_only;            // 1: skip the fast form (every item takes the exact softmax)
-    int skip_dead;             // kPartial: 1 = items and key blocks without tokens are skipped, 0 = walked with probability 0
-    int masked;                // kPartial: shifted windows with a mask -- a query sees the keys of its own part of a border window only
     FastDiv div_tp, div_heads, div_nwx, div_nwy, div_per_row;   // tiles_per_item_pair, heads, nWx, nWy, M / 8
 };
+template <bool kPartial> struct Params : FwdParams {};
+template <> struct Params<true> : FwdParams { LiveWindows live; };
 
 struct ItemCoord { int b, wy, wx, h, tp; };
 
-__device__ __forceinline__ ItemCoord decode_item(const FwdParams& p, int item)
+__device__ __forceinline__ ItemCoord decode_item(const Params<false>& p, int item)
 {
     ItemCoord c;
     p.div_tp.divmod(item, item, c.tp);
@@ -143,12 +136,20 @@ __device__ __forceinline__ ItemCoord decode_item(const FwdParams& p, int item)
     p.div_nwy.divmod(item, c.b, c.wy);
     return c;
 }
-
-__device__ __forceinline__ void patch_origin(const FwdParams& p, const ItemCoord& c, int sp, int& py, int& px,
-                                             int& Y0, int& X0)
+__device__ __forceinline__ void patch_origin(const Params<false>& p, const ItemCoord& c, int sp, int& py, int& px, int& Y0, int& X0)
 {
     sm100::patch_origin(WindowGeom{p.Hp, p.Wp, p.M, p.s}, p.div_per_row, c.wy, c.wx, sp, py, px, Y0, X0);
 }
+__device__ __forceinline__ int patches_of(const Params<false>& p, const ItemCoord&) { return p.n / 64; }
+
+// kPartial: `sp` counts the patches of the window that hold tokens; beyond the last one lies nothing (TMA fills in zeros)
+__device__ __forceinline__ LiveItem decode_item(const Params<true>& p, int item) { return decode_live_item(p.live, item); }
+__device__ __forceinline__ void patch_origin(const Params<true>& p, const LiveItem& c, int sp, int& py, int& px, int& Y0, int& X0)
+{
+    live_patch_origin(p.live, WindowGeom{p.Hp, p.Wp, p.M, p.s}, c, min(sp, c.patches - 1), py, px, Y0, X0);
+    if (sp >= c.patches) X0 = p.Wp;
+}
+__device__ __forceinline__ int patches_of(const Params<true>&, const LiveItem& c) { return c.patches; }
 
 // 2^x for a pair of arguments on the FMA and integer pipes, for the fast softmax form.  x = n + f with
 // n = round(x), |f| <= 1/2.  The cubic (relative error 7.5e-5) is evaluated with coefficients scaled by
@@ -171,18 +172,17 @@ __device__ __forceinline__ float2 ex2_poly2_ranged(float2 x)
     return make_float2(__uint_as_float(__float_as_uint(q.x) + (vx << 23)), __uint_as_float(__float_as_uint(q.y) + (vy << 23)));
 }
 
-// kPartial: H or W is not a multiple of the window (but of 8).  Windows are laid over the map extended to Hp x Wp;
-// an 8x8 patch of the extension holds no tokens: TMA fills it with zeros, the softmax warps give its keys the
-// probability 0, and nothing is stored for its queries.
+// kPartial: windows of several kinds (LiveWindows): H or W is not a multiple of the window (but of 8), or a mask between the
+// wrapped parts of shifted windows.
 // kGated: the output is multiplied by the CLA gate (Eq. 9) before it is stored.
 template <int R, bool kPartial, bool kGated>
 __global__ void __launch_bounds__(kThreads, 1)
 rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_pk,
-                     const FwdParams p)
+                     const __grid_constant__ Params<kPartial> p)
 {
     using L = Layout<R>;
-    constexpr uint32_t kOffQc = L::kOffQc, kOffQp = L::kOffQp, kOffKc = L::kOffKc, kOffKp = L::kOffKp, kOffV = L::kOffV, kOffOnes = L::kOffOnes,
+    constexpr uint32_t kOffQc = L::kOffQc, kOffQp = L::kOffQp, kOffKc = L::kOffKc, kOffKp = L::kOffKp, kOffV = L::kOffV, kOffOnes = L::kOffOnes, kOffHalfOnes = L::kOffHalfOnes,
                        kOffBar = L::kOffBar, kOffMisc = L::kOffMisc, kOffRedo = L::kOffRedo, kOffMerge = L::kOffMerge, kPosBytes = L::kPosBytes,
                        kPatchPos = L::kPatchPos;
     extern __shared__ uint8_t smem_raw[];
@@ -226,61 +226,17 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         const int sw = (row >> 1) & 3;
 #pragma unroll
         for (int ck = 0; ck < 4; ++ck) dst[ck] = make_uint4(ck == sw ? 0x00003F80u : 0u, 0u, 0u, 0u);
+        if (kPartial) {
+            dst = reinterpret_cast<uint4*>(base_ptr + kOffHalfOnes + row * 64);
+#pragma unroll
+            for (int ck = 0; ck < 4; ++ck) dst[ck] = make_uint4(ck == sw && row < 64 ? 0x00003F80u : 0u, 0u, 0u, 0u);
+        }
         fence_proxy_async();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-
-    // kPartial: one warp works out, once, which of this CTA's items hold tokens and their dead-patch masks; every role then
-    // walks that list instead of testing every item itself (the tests were the cost of skipping: a few hundred cycles per
-    // role and item).
-    ItemRec* const item_list = reinterpret_cast<ItemRec*>(base_ptr + L::kOffItems) + 1;
-    int* const list_count = reinterpret_cast<int*>(base_ptr + L::kOffItems);
-    const bool listed = kPartial && !p.masked && my_items <= kMaxListed;     // the same for every thread of the CTA
-    if (listed) {
-        if (warp == 4) {
-            const int per_row = p.M >> 3;
-            const uint32_t in_window = per_row == 32 ? 0xffffffffu : (1u << per_row) - 1u;
-            int kept = 0;
-            for (int i0 = 0; i0 < my_items; i0 += 32) {
-                const int i = i0 + lane;
-                bool live = false;
-                ItemRec rec{};
-                if (i < my_items) {
-                    rec.item = (int)blockIdx.x + i * (int)gridDim.x;
-                    const ItemCoord c = decode_item(p, rec.item);
-                    for (int l = 0; l < per_row; ++l) {
-                        int y = c.wy * p.M + 8 * l + p.s; if (y >= p.Hp) y -= p.Hp;
-                        int x = c.wx * p.M + 8 * l + p.s; if (x >= p.Wp) x -= p.Wp;
-                        rec.row_dead |= (uint32_t)(y >= p.H) << l;
-                        rec.col_dead |= (uint32_t)(x >= p.W) << l;
-                    }
-                    for (int sp = 0; sp < 4; ++sp) {
-                        int pr, pc;
-                        p.div_per_row.divmod(4 * c.tp + sp, pr, pc);
-                        live = live || (((rec.row_dead >> pr) | (rec.col_dead >> pc)) & 1u) == 0u;
-                    }
-                    const uint32_t rows = ~rec.row_dead & in_window;
-                    const uint32_t pairs = ~(rec.col_dead & (rec.col_dead >> 1)) & 0x55555555u & in_window;
-                    const int jf = (__ffs(rows) - 1) * (per_row >> 1) + ((__ffs(pairs) - 1) >> 1);
-                    const int jl = (31 - __clz(rows)) * (per_row >> 1) + ((31 - __clz(pairs)) >> 1);
-                    rec.range = (uint32_t)jf | ((uint32_t)jl << 16);
-                    if (!p.skip_dead) {                  // small windows: everything is walked, the list only saves the roles the masks
-                        live = true;
-                        rec.range = (uint32_t)(nblk - 1) << 16;
-                    }
-                }
-                const uint32_t votes = __ballot_sync(0xffffffffu, live);
-                if (live) item_list[kept + __popc(votes & ((1u << lane) - 1u))] = rec;
-                kept += __popc(votes);
-            }
-            if (lane == 0) *list_count = kept;
-        }
-        __syncthreads();
-    }
-    const int live_items = listed ? *list_count : my_items;
 
     // Role state that carries over from the first pass to the exact pass: block and item counters give the barrier phases.
     uint32_t blk = 0, io = 0, nmerge = 0;
@@ -292,89 +248,15 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         // pass 0: every item of this CTA; pass 1: the items noted by the fast form (all of them when the notes overflowed)
         const int noted = pass == 0 ? 0 : *redo_count;
         const bool all_items = pass == 0 || noted > kMaxRedo;
-        const int count = all_items ? (kPartial ? live_items : my_items) : noted;
-        auto ordinal = [&](int i) { return all_items ? i : (int)redo_list[i]; };      // place in the CTA's sequence of items
-        auto item_at = [&](int i) {
-            if (kPartial && listed) return item_list[ordinal(i)].item;
-            return (int)blockIdx.x + (all_items ? i : redo_list[i]) * (int)gridDim.x;
-        };
-        // kPartial: an item whose four query patches all lie in the extension of the map has nothing to compute; every role
-        // skips it by the same test, so the item and block counters that give the barrier phases stay in step.  The tests cost
-        // every role some hundred cycles per item, which pays from windows of 32 x 32 tokens on (skip_dead); in smaller
-        // windows an item is a block or two long and everything is walked.
-        auto item_live = [&](int item) {
-            if (!kPartial || !p.skip_dead || listed) return true;         // (a listed item is walked)
-            const ItemCoord c = decode_item(p, item);
-            bool live = false;
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp) {
-                int py, px, Y0, X0;
-                patch_origin(p, c, 4 * c.tp + sp, py, px, Y0, X0);
-                live = live || (Y0 < p.H && X0 < p.W);
-            }
-            return live;
-        };
-        // kPartial: which patch rows / patch columns of the item's window lie in the extension of the map, one bit each
-        // (lane l votes for row and column l; a window has at most 32 of either).  Warp-collective.
-        auto dead_masks = [&](const ItemCoord& c, uint32_t& row_dead, uint32_t& col_dead) {
-            int y = c.wy * p.M + 8 * lane + p.s; if (y >= p.Hp) y -= p.Hp;
-            int x = c.wx * p.M + 8 * lane + p.s; if (x >= p.Wp) x -= p.Wp;
-            row_dead = __ballot_sync(0xffffffffu, y >= p.H);
-            col_dead = __ballot_sync(0xffffffffu, x >= p.W);
-        };
-        // Masked shifted windows (p.masked, a use of the kPartial instantiation on a map the window divides): in the last window
-        // row (column) the patch rows (columns) from (M - s) / 8 on hold the wrapped part of the map.  For the query patch
-        // q_patch the patch rows and columns of the OTHER part count as dead, which hands the mask to the code that gives the
-        // keys beyond a map probability 0.  (The shift is a multiple of 8: a patch lies in one part.)
-        auto mask_masks = [&](const ItemCoord& c, int q_patch, uint32_t& row_dead, uint32_t& col_dead) {
-            const int per_row = p.M >> 3, thr = (p.M - p.s) >> 3;
-            const uint32_t in_window = per_row == 32 ? 0xffffffffu : (1u << per_row) - 1u;
-            const uint32_t wrapped = in_window & ~(thr >= 32 ? 0xffffffffu : (1u << thr) - 1u);
-            const uint32_t rows_w = c.wy == p.nWy - 1 ? wrapped : 0u, cols_w = c.wx == p.nWx - 1 ? wrapped : 0u;
-            int pr, pc;
-            p.div_per_row.divmod(q_patch, pr, pc);
-            row_dead = ((rows_w >> pr) & 1u) ? in_window & ~rows_w : rows_w;
-            col_dead = ((cols_w >> pc) & 1u) ? in_window & ~cols_w : cols_w;
-        };
-        auto patch_dead = [&](int sp, uint32_t row_dead, uint32_t col_dead) {
-            int pr, pc;
-            p.div_per_row.divmod(sp, pr, pc);
-            return (((row_dead >> pr) | (col_dead >> pc)) & 1u) != 0u;
-        };
-        // kPartial: a key block is two neighbouring patches of one patch row (a window row holds an even number of patches); it
-        // holds no token when its row is dead or both of its columns are.  Every role walks the blocks jf .. jl of an item
-        // (its first and last block with tokens; a live item has some: its own query patches) and skips the dead ones in
-        // between by the same test, so the block counters that give the barrier phases stay in step.
-        auto block_dead = [&](int j, uint32_t row_dead, uint32_t col_dead) {
-            int pr, pc;
-            p.div_per_row.divmod(2 * j, pr, pc);
-            return (((row_dead >> pr) | ((col_dead & (col_dead >> 1)) >> pc)) & 1u) != 0u;
-        };
-        auto live_range = [&](uint32_t row_dead, uint32_t col_dead, int& jf, int& jl) {
-            const int per_row = p.M >> 3;
-            const uint32_t in_window = per_row == 32 ? 0xffffffffu : (1u << per_row) - 1u;
-            const uint32_t rows = ~row_dead & in_window;
-            const uint32_t pairs = ~(col_dead & (col_dead >> 1)) & 0x55555555u & in_window;     // bit 2c: columns 2c, 2c + 1
-            jf = (__ffs(rows) - 1) * (per_row >> 1) + ((__ffs(pairs) - 1) >> 1);
-            jl = (31 - __clz(rows)) * (per_row >> 1) + ((31 - __clz(pairs)) >> 1);
-        };
-        // the masks and the block range of item i of this pass: from the list, or worked out here (warp-collective)
-        auto item_masks = [&](int i, const ItemCoord& c, uint32_t& row_dead, uint32_t& col_dead, int& jf, int& jl) {
-            if (listed) {
-                const ItemRec rec = item_list[ordinal(i)];
-                row_dead = rec.row_dead; col_dead = rec.col_dead;
-                jf = (int)(rec.range & 0xffffu); jl = (int)(rec.range >> 16);
-            } else {
-                dead_masks(c, row_dead, col_dead);
-                if (p.skip_dead) live_range(row_dead, col_dead, jf, jl);
-            }
-        };
+        const int count = all_items ? my_items : noted;
+        auto item_at = [&](int i) { return (int)blockIdx.x + (all_items ? i : redo_list[i]) * (int)gridDim.x; };
+        // key blocks of item i of this pass
+        auto blocks_at = [&](int i) { return kPartial ? (patches_of(p, decode_item(p, item_at(i))) + 1) >> 1 : nblk; };
 
         if (warp == 0) {
             // ===================== TMA producer (lane 0) and query RIB rows bf16(Pq * sqrt(d/r)) of the same item (whole warp)
             for (int i = 0; i < count && ok; ++i, ++io) {
-                if (!item_live(item_at(i))) { --io; continue; }
-                const ItemCoord c = decode_item(p, item_at(i));
+                const auto c = decode_item(p, item_at(i));
                 const uint32_t buf = io & 1;
                 if (io >= 2 && !mbar_wait_warp(bar(kQEmpty + buf), ((io >> 1) - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                 if (lane == 0) {
@@ -413,13 +295,10 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 }
                 fence_proxy_async();
                 __syncwarp();
-                uint32_t row_dead = 0u, col_dead = 0u;
-                int jf = 0, jl = nblk - 1;
-                if (kPartial) item_masks(i, c, row_dead, col_dead, jf, jl);
+                const int nb = kPartial ? (patches_of(p, c) + 1) >> 1 : nblk;
                 if (lane == 0) {
                     mbar_arrive(bar(kQPos + buf));
-                    for (int j = jf; j <= jl; ++j, ++blk) {
-                        if (kPartial && p.skip_dead && (row_dead | col_dead) != 0u && block_dead(j, row_dead, col_dead)) { --blk; continue; }
+                    for (int j = 0; j < nb; ++j, ++blk) {
                         const uint32_t st = blk % kStages, use = blk / kStages;
                         if (use > 0 && !mbar_wait(bar(kKEmpty + st), (use - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                         mbar_arrive_expect_tx(bar(kKFull + st), kContentBytes + kPosBytes);
@@ -458,15 +337,11 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             // and waits; one elected lane issues (this keeps descriptors in uniform registers).
             constexpr uint64_t kDesc64 = smem_desc_const(16, 512, kSwizzle64B), kDesc32 = smem_desc_const(16, 256, kSwizzle32B);
             for (int i = 0; i < count && ok; ++i, ++io) {
-                if (!item_live(item_at(i))) { --io; continue; }
                 const uint32_t buf = io & 1;
                 if (!mbar_wait_warp(bar(kQFull + buf), (io >> 1) & 1, abort_flag, p.status) ||
                     !mbar_wait_warp(bar(kQPos + buf), (io >> 1) & 1, abort_flag, p.status)) { ok = false; break; }
-                uint32_t row_dead = 0u, col_dead = 0u;
-                int jf = 0, jl = nblk - 1;
-                if (kPartial && (p.skip_dead || listed)) item_masks(i, listed ? ItemCoord{} : decode_item(p, item_at(i)), row_dead, col_dead, jf, jl);
-                for (int j = jf; j <= jl && ok; ++j, ++blk) {
-                    if (kPartial && p.skip_dead && (row_dead | col_dead) != 0u && block_dead(j, row_dead, col_dead)) { --blk; continue; }
+                const int nb = blocks_at(i);
+                for (int j = 0; j < nb && ok; ++j, ++blk) {
                     const uint32_t st = blk % kStages;
                     if (!mbar_wait_warp(bar(kKFull + st), (blk / kStages) & 1, abort_flag, p.status)) { ok = false; break; }
                     const uint64_t kc = smem_desc_at(kDesc64, base + kOffKc + st * kContentBytes);
@@ -487,7 +362,7 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                             mma_commit(bar(kSFull + qt));
                             if (qt == 1) {
                                 mma_commit(bar(kKEmpty + st));
-                                if (j == jl) mma_commit(bar(kQEmpty + buf));
+                                if (j == nb - 1) mma_commit(bar(kQEmpty + buf));
                             }
                         }
                         __syncwarp();
@@ -502,32 +377,31 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             const uint32_t d_o = tmem + kColO + qt * 2 * kD;              // exact form: one accumulator per key half
             const uint32_t d_o1 = tmem + kColO + qt * kFastOCols;         // fast form: one accumulator
             for (int i = 0; i < count && ok; ++i, ++io) {
-                if (!item_live(item_at(i))) { --io; continue; }
-                uint32_t row_dead = 0u, col_dead = 0u;
-                int jf = 0, jl = nblk - 1;
-                if (kPartial && (p.skip_dead || listed)) item_masks(i, listed ? ItemCoord{} : decode_item(p, item_at(i)), row_dead, col_dead, jf, jl);
-                for (int j = jf; j <= jl; ++j, ++blk) {
-                    if (kPartial && p.skip_dead && (row_dead | col_dead) != 0u && block_dead(j, row_dead, col_dead)) { --blk; continue; }
+                const int patches = kPartial ? patches_of(p, decode_item(p, item_at(i))) : 0, nb = kPartial ? (patches + 1) >> 1 : nblk;
+                const bool odd = kPartial && (patches & 1);
+                for (int j = 0; j < nb; ++j, ++blk) {
                     const uint32_t st = blk % kStages;
                     // warp-uniform outcomes, so that the warp stays converged.  The first block of an item overwrites the
                     // accumulator: the epilogue of the item before must have read it.
                     if (!mbar_wait_warp(bar(kVFull + st), (blk / kStages) & 1, abort_flag, p.status) ||
-                        !(j > jf || io == 0 || mbar_wait_warp(bar(kOFree + qt), (io - 1) & 1, abort_flag, p.status)) ||
+                        !(j > 0 || io == 0 || mbar_wait_warp(bar(kOFree + qt), (io - 1) & 1, abort_flag, p.status)) ||
                         !mbar_wait_warp(bar(kPReady + qt), blk & 1, abort_flag, p.status)) { ok = false; break; }
                     tc_fence_after();
                     if (elect_one()) {
                         const uint32_t v_addr = base + kOffV + st * kContentBytes;
                         if (fast) {
                             // [V | ones] as one MN-major operand of 48 columns, the second 32-column atom `lbo` bytes behind the first
-                            const uint64_t v = smem_desc(v_addr, kOffOnes - (kOffV + st * kContentBytes), 512, kSwizzle64B);
+                            // (kPartial: half a block without tokens has zero rows of V and of the second atom)
+                            const uint32_t ones = kPartial && j == nb - 1 && odd ? kOffHalfOnes : kOffOnes;
+                            const uint64_t v = smem_desc(v_addr, ones - (kOffV + st * kContentBytes), 512, kSwizzle64B);
 #pragma unroll
                             for (int kk = 0; kk < 8; ++kk)
-                                mma_ts(d_o1, a_p + 8 * kk, v + 64 * kk, kIdescPV1, (j == jf && kk == 0) ? 0u : 1u);
+                                mma_ts(d_o1, a_p + 8 * kk, v + 64 * kk, kIdescPV1, (j == 0 && kk == 0) ? 0u : 1u);
                         } else {
                             const uint64_t v = smem_desc_at(kDesc64, v_addr);
 #pragma unroll
                             for (int kk = 0; kk < 8; ++kk)     // keys 16 kk ..: key half kk / 4 has its own accumulator
-                                mma_ts(d_o + (kk >> 2) * kD, a_p + 8 * kk, v + 64 * kk, kIdescPV, (j == jf && (kk & 3) == 0) ? 0u : 1u);
+                                mma_ts(d_o + (kk >> 2) * kD, a_p + 8 * kk, v + 64 * kk, kIdescPV, (j == 0 && (kk & 3) == 0) ? 0u : 1u);
                         }
                         mma_commit(bar(kPFree + qt));
                         mma_commit(bar(kVEmpty + st));
@@ -567,12 +441,12 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 float* pend_lse = nullptr;
                 float pend_ref = 0.f;
                 int pend_ordinal = -1;                      // -1: nothing pending
-                // Full windows: the wait for the next block's scores is asked between the stores of P and their completion,
+                // The wait for the next block's scores is asked between the stores of P and their completion,
                 // in straight-line code (with a branch around the question the gain is gone: 3 % of the kernel).  After the
                 // last block of the pass no scores follow; there the question names the phase just used, which is complete,
                 // so that no warp sits out the time limit of a wait that nothing answers.
                 bool s_polled = false, s_ready = false;
-                const uint32_t last_blk = blk + (uint32_t)count * (uint32_t)nblk - 1u;
+                const uint32_t last_blk = kPartial ? 0u : blk + (uint32_t)count * (uint32_t)nblk - 1u;
                 // O and l of the pending item are complete (the caller has waited for its last PV): normalise, store, note overflow
                 auto epilogue = [&]() {
                     uint32_t o[16], lsum[1];
@@ -584,9 +458,7 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     if (lane == 0) mbar_arrive(bar(kOFree + qt));
                     const float l_all = __uint_as_float(lsum[0]);
                     // a score left the range the fixed reference covers: the exact form redoes the item
-                    // (kPartial: or the row sum is so small that the weights of keys beyond the map could show in it)
-                    const float l_min = kPartial ? 8.6736174e-19f : 0.f;                                   // 2^-60
-                    const bool bad = pend_out != nullptr && !(l_all > l_min && l_all < 1.2676506e30f);     // 2^100
+                    const bool bad = pend_out != nullptr && !(l_all > 0.f && l_all < 1.2676506e30f);     // 2^100
                     if (__any_sync(0xffffffffu, bad) && lane == 0) {
                         const int slot = atomicAdd(redo_count, 1);
                         if (slot < kMaxRedo) redo_list[slot] = pend_ordinal;
@@ -615,32 +487,26 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     pend_ordinal = -1;
                 };
                 for (int i = 0; i < count && ok; ++i, ++io) {
-                    const int item = item_at(i);
-                    if (!item_live(item)) { --io; continue; }
-                    const ItemCoord c = decode_item(p, item);
+                    const auto c = decode_item(p, item_at(i));
                     // where this thread's half row of the item goes
                     int py, px, Y0, X0;
                     patch_origin(p, c, 2 * (2 * c.tp + qt) + (row >> 6), py, px, Y0, X0);
                     const int Y = Y0 + ((row >> 3) & 7), X = X0 + (row & 7);   // the patch does not straddle the border
-                    const bool no_query = kPartial && (Y0 >= p.H || X0 >= p.W);   // a patch of the extension: no tokens, nothing to store
+                    const bool no_query = kPartial && 2 * (2 * c.tp + qt) + (row >> 6) >= patches_of(p, c);   // half a tile without tokens: nothing to store
                     const size_t tok = (((size_t)c.b * p.H + Y) * p.W + X) * p.heads + c.h;
                     __nv_bfloat16* const out_row = no_query ? nullptr : p.out + tok * p.d + half * 16;
                     const __nv_bfloat16* const gate_row = kGated ? p.gate + tok * p.d + half * 16 : nullptr;
                     float* const lse_row = (p.lse && half == 0 && !no_query) ? p.lse + (((size_t)c.b * p.heads + c.h) * p.H + Y) * p.W + X : nullptr;
                     float m_ref = 0.f;
                     float2 neg2 = make_float2(0.f, 0.f);
-                    uint32_t row_dead = 0u, col_dead = 0u;
-                    int jf = 0, jl = nblk - 1;
-                    if (kPartial) item_masks(i, c, row_dead, col_dead, jf, jl);
-                    if (kPartial && p.masked) mask_masks(c, 2 * (2 * c.tp + qt) + (row >> 6), row_dead, col_dead);
-                    for (int j = jf; j <= jl; ++j, ++blk) {
-                        if (kPartial && p.skip_dead && (row_dead | col_dead) != 0u && block_dead(j, row_dead, col_dead)) { --blk; continue; }
+                    const int patches = patches_of(p, c), nb = kPartial ? (patches + 1) >> 1 : nblk;
+                    for (int j = 0; j < nb; ++j, ++blk) {
                         // warp-uniform outcome: the TMEM loads below are warp-collective
                         if (!(s_polled && __all_sync(0xffffffffu, s_ready)) && !mbar_wait_warp(bar(kSFull + qt), blk & 1, abort_flag, p.status)) { ok = false; break; }
                         s_polled = false;
                         tc_fence_after();
                         uint32_t sa[32], sb[32];
-                        if (j == jf) {
+                        if (j == 0) {
                             // the row's reference: the maximum over keys 0-31 of the window, the same for both key halves
                             tmem_ld32(tmem + lane_base + kColS + qt * kTile, sa);
                             tmem_wait_ld();
@@ -662,32 +528,21 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         __syncwarp();
                         if (lane == 0) mbar_arrive(bar(kSFree + qt));   // the next block's scores may overwrite the accumulator
                         uint32_t pa[16], pb[16];
-                        float2 sc2 = scale2, ng2 = neg2;
-                        if (kPartial && (row_dead | col_dead) != 0u && patch_dead(2 * j + half, row_dead, col_dead)) {
-                            // This thread's 64 keys are one 8x8 patch; in the extension of the map it holds no tokens.  The block
-                            // runs through the same instructions with scale 0 and offset -119: each such key gets the weight
-                            // 2^-119 (the smallest both exponential paths deliver), its zero-filled value row adds nothing to
-                            // O, and the at most 2^16 such keys add less than 2^-103 to a row sum that the epilogue accepts
-                            // only from 2^-60 upwards.  The reference above may come from such keys: any finite score serves.
-                            sc2 = make_float2(0.f, 0.f);
-                            ng2 = make_float2(-119.f, -119.f);
-                        }
-                        // P of the tile is free once the previous block's PV has completed (long ago, as a rule).  Full windows ask
-                        // before the exponentials, so that the answer is there when they are done.
-                        const bool p_free = blk == 0 || (!kPartial && mbar_try_wait(b_free, (blk - 1) & 1));
-                        exp_chunk1(sa, sc2, ng2, pa);
-                        exp_chunk1(sb, sc2, ng2, pb);
+                        // P of the tile is free once the previous block's PV has completed (long ago, as a rule).  It is asked before the
+                        // exponentials, so that the answer is there when they are done.
+                        const bool p_free = blk == 0 || mbar_try_wait(b_free, (blk - 1) & 1);
+                        exp_chunk1(sa, scale2, neg2, pa);
+                        exp_chunk1(sb, scale2, neg2, pb);
                         if (blk > 0) {
                             if (!__all_sync(0xffffffffu, p_free) && !mbar_wait_warp(b_free, (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                             tc_fence_after();
                         }
-                        if (j == jf && pend_ordinal >= 0) epilogue();     // that PV was the last one of the item before
+                        if (j == 0 && pend_ordinal >= 0) epilogue();     // that PV was the last one of the item before
                         tmem_st16(t_p, pa);
                         tmem_st16(t_p + 16, pb);
-                        if (!kPartial) {
-                            s_ready = mbar_try_wait(bar(kSFull + qt), (blk + (blk != last_blk ? 1u : 0u)) & 1);
-                            s_polled = true;
-                        }
+                        const bool more = kPartial ? i != count - 1 || j != nb - 1 : blk != last_blk;
+                        s_ready = mbar_try_wait(bar(kSFull + qt), (blk + (more ? 1u : 0u)) & 1);
+                        s_polled = true;
                         tmem_wait_st();
                         tc_fence_before();
                         __syncwarp();
@@ -719,24 +574,17 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     return (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
                 };
                 for (int i = 0; i < count && ok; ++i, ++io, ++nmerge) {
-                    const int item = item_at(i);
-                    if (!item_live(item)) { --io; --nmerge; continue; }
-                    const ItemCoord c = decode_item(p, item);
+                    const auto c = decode_item(p, item_at(i));
                     float m_used = -INFINITY, l = 0.f;
-                    bool have_ref = false;            // kPartial: a block with real keys has set the reference
-                    uint32_t row_dead = 0u, col_dead = 0u;
-                    int jf = 0, jl = nblk - 1;
-                    if (kPartial) item_masks(i, c, row_dead, col_dead, jf, jl);
-                    if (kPartial && p.masked) mask_masks(c, 2 * (2 * c.tp + qt) + (row >> 6), row_dead, col_dead);
-                    for (int j = jf; j <= jl; ++j, ++blk) {
-                        if (kPartial && p.skip_dead && (row_dead | col_dead) != 0u && block_dead(j, row_dead, col_dead)) { --blk; continue; }
+                    const int patches = patches_of(p, c), nb = kPartial ? (patches + 1) >> 1 : nblk;
+                    for (int j = 0; j < nb; ++j, ++blk) {
                         // warp-uniform outcome: the TMEM loads below are warp-collective
                         if (!mbar_wait_warp(bar(kSFull + qt), blk & 1, abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
                         bool p_free = blk == 0;       // P (and O) of this half are free once the previous block's PV has completed
                         if (kPartial) {
-                            // this thread's 64 keys are one 8x8 patch: beyond the image it holds no tokens
-                            if (patch_dead(2 * j + half, row_dead, col_dead)) {
+                            // half a block without tokens (the last one of an odd number of patches)
+                            if (half != 0 && 2 * j + 1 >= patches) {
                                 tc_fence_before();
                                 __syncwarp();
                                 if (lane == 0) mbar_arrive(bar(kSFree + qt));
@@ -756,8 +604,7 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                                 continue;
                             }
                         }
-                        const bool first_ref = kPartial ? !have_ref : j == jf;
-                        have_ref = true;
+                        const bool first_ref = j == 0;
 #pragma unroll
                         for (int ch = 0; ch < 2; ++ch) {
                             uint32_t s[32];
@@ -785,7 +632,7 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                                     }
                                     const float factor = need ? ex2_approx((m_used - mx) * p.scale_log2) : 1.f;
                                     if (need) { l *= factor; m_used = mx; }
-                                    if (j > jf) {
+                                    if (j > 0) {
                                         uint32_t o[32];
                                         tmem_ld32(t_o + half * kD, o);
                                         tmem_wait_ld();
@@ -851,7 +698,7 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     int py, px, Y0, X0;
                     patch_origin(p, c, 2 * (2 * c.tp + qt) + (row >> 6), py, px, Y0, X0);
                     const int Y = Y0 + ((row >> 3) & 7), X = X0 + (row & 7);   // the patch does not straddle the border
-                    if (kPartial && (Y0 >= p.H || X0 >= p.W)) continue;        // a patch of the extension: no tokens, nothing to store
+                    if (kPartial && 2 * (2 * c.tp + qt) + (row >> 6) >= patches) continue;     // half a tile without tokens: nothing to store
                     const size_t tok = (((size_t)c.b * p.H + Y) * p.W + X) * p.heads + c.h;
                     uint4* dst = reinterpret_cast<uint4*>(p.out + tok * p.d + half * 16);
                     const uint4* gsrc = reinterpret_cast<const uint4*>(p.gate + tok * p.d + half * 16);
@@ -932,11 +779,11 @@ cudaError_t launch_fwd(const Problem& p, cudaStream_t stream)
     if (!encode_image_map(&tm_q, p.q, p) || !encode_image_map(&tm_k, p.k, p) || !encode_image_map(&tm_v, p.v, p) ||
         !encode_pos_map(&tm_pk, p.pk, p, pos_tables(p), p.pos_head_stride))
         return cudaErrorInvalidValue;
-    constexpr uint32_t kSmemBytes = kPartial ? Layout<R>::kSmemBytesPartial : Layout<R>::kSmemBytes;
+    constexpr uint32_t kSmemBytes = Layout<R>::kSmemBytes;
     static KernelSetup setup;       // one per instantiation of this launcher, i.e. per kernel
     int sm_count = 0;
     if (cudaError_t e = setup.prepare(rib_fwd_sm100_kernel<R, kPartial, kGated>, kSmemBytes, &sm_count)) return e;
-    FwdParams fp{};
+    Params<kPartial> fp{};
     fp.pq = p.pq; fp.gate = p.gate; fp.out = p.out_w; fp.lse = p.lse_w; fp.status = p.status;
     fp.H = p.H; fp.W = p.W; fp.heads = p.heads; fp.M = p.M; fp.s = p.s; fp.n = p.n; fp.nWy = p.nWy; fp.nWx = p.nWx;
     fp.d = p.d; fp.r = p.r;
@@ -949,12 +796,12 @@ cudaError_t launch_fwd(const Problem& p, cudaStream_t stream)
     fp.pos_head_stride = p.pos_head_stride;
     fp.pos_per_head = p.pos_head_stride ? 1 : 0;
     fp.exact_only = p.exact_softmax ? 1 : 0;
-    fp.masked = p.masked ? 1 : 0;
-    // (a mask differs from query patch to query patch; in windows below 32 x 32 an item is a block or two long and the tests of
-    // the blocks cost more than the skipped ones save: measured +6 % at 16 x 16 even with the per-CTA list of live items)
-    fp.skip_dead = kPartial && !p.masked && p.n / kTile >= 8 ? 1 : 0;
     fp.div_tp = make_fast_div(fp.tiles_per_item_pair); fp.div_heads = make_fast_div(p.heads);
     fp.div_nwx = make_fast_div(p.nWx); fp.div_nwy = make_fast_div(p.nWy); fp.div_per_row = make_fast_div(p.M >> 3);
+    if constexpr (kPartial) {
+        if (!make_live_windows(p, &fp.live)) return cudaErrorInvalidValue;
+        fp.items = fp.live.offset[9];
+    }
     const int grid = fp.items < sm_count ? fp.items : sm_count;
     { ProfileScope scope(RIB_KERNEL_FWD_MAIN, stream); rib_fwd_sm100_kernel<R, kPartial, kGated><<<grid, kThreads, kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_pk, fp); }
     return cudaGetLastError();

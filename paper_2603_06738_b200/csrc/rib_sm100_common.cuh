@@ -125,6 +125,21 @@ __host__ __device__ __forceinline__ void live_patch_origin(const LiveWindows& g,
     X0 = c.wx * w.M + px + w.s; if (X0 >= w.W) X0 -= w.W;
 }
 
+// With a mask between the wrapped parts of shifted windows the parts of the last window are windows of their own: two kinds,
+// the patch rows (columns) before position M - s and those from it on.
+inline int masked_axis_kinds(int size, int M, int s, AxisKind (&kinds)[3], int (&windows)[3])
+{
+    const int n = size / M, per_row = M / 8, cut = (M - s) / 8;
+    int used = 0;
+    auto add = [&](int first, int count, int start, int len) {
+        kinds[used] = AxisKind{len, start, len, 0, first, make_fast_div(len), make_fast_div(count)};
+        windows[used++] = count;
+    };
+    if (n - (s ? 1 : 0) > 0) add(0, n - (s ? 1 : 0), 0, per_row);
+    if (s) { add(n - 1, 1, 0, cut); add(n - 1, 1, cut, per_row - cut); }
+    return used;
+}
+
 // The kinds of window along an axis of `size` positions; returns their number, 0 if the axis is not of the form above.
 inline int axis_kinds(int size, int M, int s, AxisKind (&kinds)[3], int (&windows)[3])
 {
@@ -159,7 +174,8 @@ inline bool make_live_windows(const Problem& p, LiveWindows* g)
 {
     int ny_windows[3] = {0, 0, 0}, nx_windows[3] = {0, 0, 0};
     *g = LiveWindows{};
-    const int ny = axis_kinds(p.H, p.M, p.s, g->y, ny_windows), nx = axis_kinds(p.W, p.M, p.s, g->x, nx_windows);
+    const int ny = p.masked ? masked_axis_kinds(p.H, p.M, p.s, g->y, ny_windows) : axis_kinds(p.H, p.M, p.s, g->y, ny_windows);
+    const int nx = p.masked ? masked_axis_kinds(p.W, p.M, p.s, g->x, nx_windows) : axis_kinds(p.W, p.M, p.s, g->x, nx_windows);
     if (!ny || !nx) return false;
     long long at = 0;
     for (int k = 0; k < 9; ++k) {
