@@ -21,8 +21,9 @@
 // Tensor memory: three score buffers of 128 columns and 2 x 2 output accumulators (query tile, key half) of 32.  Unit u =
 // 2 * block + query tile uses buffer u mod 3.  A softmax thread holds one row's 64 scores of its key half in registers and
 // writes P over them (hi 32 columns, lo 32 columns), so a buffer is handed back to the one issuing thread with P in it; that
-// thread issues PV(u) and behind it S(u + 3) into the same columns, in which order the tensor pipe executes them.  The scores
-// of one tile's next block are thus under way while the other tile's exponentials run.
+// thread issues PV(u), waits for its completion (nothing orders an MMA that overwrites columns behind one of another shape and
+// accumulator that reads them as its A operand) and issues S(u + 3) into the same columns.  The scores of one tile's next block
+// are thus under way while the other tile's exponentials run.
 //
 // Roles (640 threads): warp 0 TMA producer, which also stages the scaled query RIB rows; warp 1 issues all MMAs; warp 2 owns
 // the TMEM allocation; warps 4-11 softmax / epilogue of query tile 0 (4-7 first key half, 8-11 second half), 12-19 of tile 1.
@@ -194,7 +195,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 mbar_wait(bar(L::kFull + b2 % kStages), (b2 / kStages) & 1, abort_flag + 1, p.status);
         }
     } else if (warp == 1) {
-        // ===================== issuer: S(0), S(1), S(2), then PV(u), S(u + 3) for u = 0, 1, ...; the whole warp walks and waits
+        // ===================== issuer: S(0), S(1), S(2), then PV(u), its completion, S(u + 3) for u = 0, 1, ...; the whole warp walks and waits
         constexpr uint64_t kDesc64 = smem_desc_const(16, 512, kSwizzle64B), kDesc32 = smem_desc_const(16, 256, kSwizzle32B);
         constexpr uint64_t kDescP = R == 16 ? kDesc32 : kDesc64;
         // two cursors over the same sequence of blocks: scores run three units ahead of PV
@@ -255,6 +256,9 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 if (qt == 1) mma_commit(bar(L::kEmpty + st));
             }
             __syncwarp();
+            // S(u + 3) overwrites the columns that PV(u) reads P from: it is not issued before PV(u) has completed
+            if (!mbar_wait_warp(bar(L::kPVDone + qt), v.blk & 1, abort_flag, p.status)) { ok = false; break; }
+            tc_fence_after();
             advance(v);
             ok = issue_scores();
         }

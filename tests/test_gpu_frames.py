@@ -76,3 +76,25 @@ def test_a_frame_beside_others_reads_and_writes_nothing_beyond_itself():
     compare("out", out[1:2], ref_out)
     compare("lse", lse[1:2], ref_lse)
     assert np.isnan(out[0]).all() and np.isnan(out[2]).all()
+
+
+# several items per CTA (148 SMs at most): query buffers, accumulators, score buffers and barrier phases cross from item to item
+MANY = [
+    Workload("f_125x203_w16", 2, 125, 203, 6, 32, 16, 16, 0, seed=215),                # 1248 items of one or two blocks
+    Workload("f_77x107_w32_r32", 4, 77, 107, 6, 32, 32, 32, 0, seed=216),              # items of 1 to 8 blocks, odd patch counts, rank 32
+    Workload("f_83x61_w32_s8", 6, 83, 61, 6, 32, 16, 32, 8, seed=217),
+]
+
+
+@pytest.mark.parametrize("wl", MANY, ids=lambda w: w.name)
+def test_frames_with_many_items_per_cta(wl):
+    cpu = synthetic.make_inputs(wl, with_dout=False)
+    gpu = {k: v.cuda() for k, v in cpu.items()}
+    ref_out, ref_lse = pad.fwd(*(to_f64(cpu[k]) for k in ("q", "k", "v", "pq", "pk")), wl.window, wl.shift)
+    out, lse, used = run(wl, gpu, binding.RIB_PATH_NONE)
+    assert used == binding.RIB_PATH_SM100
+    compare("out", out, ref_out)
+    assert np.linalg.norm(lse - ref_lse) <= 2e-6 * np.linalg.norm(ref_lse)
+    for _ in range(3):                                   # no sum's order depends on timing
+        again, lse_again, _ = run(wl, gpu, binding.RIB_PATH_NONE)
+        assert np.array_equal(out, again) and np.array_equal(lse, lse_again)
