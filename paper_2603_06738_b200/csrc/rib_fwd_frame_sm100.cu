@@ -74,12 +74,21 @@ struct FrameParams {
     WindowGeom geom;           // sides of the extended map, window, shift
     int terms;                 // terms of the scaled query RIB rows in use: 1 or kTerms
     float scale_log2;          // log2(e) / sqrt(d)
-    float inv_sqrt_d;
     float pos_scale;           // sqrt(d / r): folds 1/sqrt(r) into the content scale
     long long pos_head_stride;
     int pos_per_head;
     LiveWindows live;
 };
+
+// ln(2^-n l), rounded once: the logarithm of l's mantissa is small, the rest is added up in double (once per row).  With logf(l)
+// and a product in fp32, and the scores' steps the other way round, lse was 1.36 times as far from float64 as the any-shape
+// kernel's (180 x 320 tokens, 32 x 32 windows: 4.1e-8 against 3.0e-8); now 2.4e-8.
+__device__ __forceinline__ float log_sum(float n, float l)
+{
+    if (!(l > 0.f && l < INFINITY)) return -n + logf(l);             // no finite logit, or one that is no number
+    const int k = ((int)__float_as_uint(l) - 0x3f3504f3) >> 23;      // l = 2^k f, f in [sqrt(1/2), sqrt(2))
+    return (float)(((double)k - (double)n) * 0.69314718055994531 + (double)logf(__uint_as_float(__float_as_uint(l) - ((uint32_t)k << 23))));
+}
 
 template <int R>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -223,12 +232,13 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 const uint64_t qc = smem_desc_at(kDesc64, base + L::kOffQc + (2 * buf + qt) * kContentBytes);
                 const uint64_t qp = smem_desc_at(kDescP, base + L::kOffQp + (2 * buf + qt) * kTerms * kPos);
                 const uint32_t d_s = tmem + sb * kTile;
-                mma_ss(d_s, qc, kc, kIdescS, 0u);
-                mma_ss(d_s, qc + 2, kc + 2, kIdescS, 1u);          // + 32 bytes: second K16 step of the content rows
-                for (int term = 0; term < p.terms; ++term) {
-                    mma_ss(d_s, qp + term * (kPos >> 4), kp, kIdescS, 1u);
+                // smallest terms first: a step drops what lies below the last place of the sum so far
+                for (int term = p.terms - 1; term >= 0; --term) {
+                    mma_ss(d_s, qp + term * (kPos >> 4), kp, kIdescS, term == p.terms - 1 ? 0u : 1u);
                     if (R == 32) mma_ss(d_s, qp + term * (kPos >> 4) + 2, kp + 2, kIdescS, 1u);
                 }
+                mma_ss(d_s, qc, kc, kIdescS, 1u);
+                mma_ss(d_s, qc + 2, kc + 2, kIdescS, 1u);          // + 32 bytes: second K16 step of the content rows
                 mma_commit(bar(L::kSFull + sb));
                 if (qt == 1 && s.j == s.nblk - 1) mma_commit(bar(L::kQEmpty + buf));
             }
@@ -322,7 +332,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     if (__any_sync(0xffffffffu, need)) {
                         if (!mbar_wait_warp(bar(L::kPVDone + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
-                        const float factor = need ? ex2_approx((m_used - mx) * p.scale_log2) : 1.f;
+                        const float factor = need ? ex2_approx(__fmul_rn(m_used, p.scale_log2) - __fmul_rn(mx, p.scale_log2)) : 1.f;
                         if (need) { l *= factor; m_used = mx; }
                         for (int g = 0; g < 4; ++g) {
                             uint32_t o[8];
@@ -335,7 +345,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     }
                 }
                 // a half that has seen no token yet has no reference: its scores are all -inf, its probabilities 0
-                const float neg = m_used == -INFINITY ? 0.f : -m_used * p.scale_log2;
+                const float neg = m_used == -INFINITY ? 0.f : __fmul_rn(-m_used, p.scale_log2);
                 const float2 neg2 = make_float2(neg, neg);
                 float2 sum_a = make_float2(0.f, 0.f), sum_b = make_float2(0.f, 0.f);
 #pragma unroll
@@ -382,8 +392,10 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             const float2 other = merge[(half ^ 1) * kTile + row];
             const float m_a = half ? other.x : m_used, l_a = half ? other.y : l;
             const float m_b = half ? m_used : other.x, l_b = half ? l : other.y;
-            const float m = fmaxf(m_a, m_b);
-            const float f_a = ex2_approx((m_a - m) * p.scale_log2), f_b = ex2_approx((m_b - m) * p.scale_log2);
+            // the offsets as the exponentials took them, so that their rounding cancels
+            const float n_a = __fmul_rn(-m_a, p.scale_log2), n_b = __fmul_rn(-m_b, p.scale_log2), n = fminf(n_a, n_b);
+            // (a half without a finite logit, offset inf, adds nothing)
+            const float f_a = n_a == INFINITY ? 0.f : ex2_approx(n - n_a), f_b = n_b == INFINITY ? 0.f : ex2_approx(n - n_b);
             const float l_all = l_a * f_a + l_b * f_b;
             const float w_a = f_a / l_all, w_b = f_b / l_all;
             const int k = 4 * c.tp + 2 * qt + (row >> 6);
@@ -405,7 +417,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     }
                     dst[g] = make_uint4(w[0], w[1], w[2], w[3]);
                 }
-                if (p.lse && half == 0) p.lse[(((size_t)c.b * p.heads + c.h) * p.H + Y) * p.W + X] = m * p.inv_sqrt_d + logf(l_all);
+                if (p.lse && half == 0) p.lse[(((size_t)c.b * p.heads + c.h) * p.H + Y) * p.W + X] = log_sum(n, l_all);
             }
             __syncwarp();
         }
@@ -438,8 +450,7 @@ cudaError_t launch_fwd_frame(const Problem& p, cudaStream_t stream)
     fp.H = p.H; fp.W = p.W; fp.heads = p.heads; fp.d = p.d; fp.r = p.r;
     fp.geom = WindowGeom{p.Hp, p.Wp, p.M, p.s};
     const float d = scale_width_d(p), r = scale_width_r(p);
-    fp.scale_log2 = 1.4426950408889634f / sqrtf(d);
-    fp.inv_sqrt_d = 1.f / sqrtf(d);
+    fp.scale_log2 = (float)(1.4426950408889634 / sqrt((double)d));
     fp.pos_scale = sqrtf(d / r);
     fp.terms = d == r || d == 4.f * r || 4.f * d == r ? 1 : kTerms;      // sqrt(d / r) a power of two: the product is a bf16 number
     fp.pos_head_stride = p.pos_head_stride;

@@ -98,3 +98,13 @@ def test_frames_with_many_items_per_cta(wl):
     for _ in range(3):                                   # no sum's order depends on timing
         again, lse_again, _ = run(wl, gpu, binding.RIB_PATH_NONE)
         assert np.array_equal(out, again) and np.array_equal(lse, lse_again)
+
+
+@pytest.mark.parametrize("wl", [CASES[6], CASES[8], MANY[0], MANY[2]], ids=lambda w: w.name)
+def test_lse_of_frames_is_no_further_off_than_from_the_any_shape_kernel(wl):
+    cpu = synthetic.make_inputs(wl, with_dout=False)
+    gpu = {k: v.cuda() for k, v in cpu.items()}
+    _, ref = pad.fwd(*(to_f64(cpu[k]) for k in ("q", "k", "v", "pq", "pk")), wl.window, wl.shift)
+    off = [np.linalg.norm(run(wl, gpu, path)[1] - ref) / np.linalg.norm(ref) for path in (binding.RIB_PATH_NONE, binding.RIB_PATH_GENERIC)]
+    print(f"lse: relative error {off[0]:.3e}, any-shape kernel {off[1]:.3e}")
+    assert off[0] <= off[1], off
