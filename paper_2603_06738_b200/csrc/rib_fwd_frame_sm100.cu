@@ -7,7 +7,8 @@
 //     Pq sqrt(d/r) = hi + mid + lo     three terms, all 24 bits: one K16 step (two at R = 32) of the score chain per term
 //                                      (one term where d / r is a power of 4 and the product is a bf16 number);
 // q, k, v and Pk are bf16 as given and enter exactly, sums are fp32, every exponential is ex2.approx (2 ulp), the row sum
-// adds the unrounded fp32 probabilities.
+// adds the unrounded fp32 probabilities.  Infinities: the terms of a number times an infinity may cancel to NaN where the number
+// itself times it would not, so a row that comes out as NaN is computed once more from the plain numbers (plain_row).
 //
 // What bounds it: the exponentials (16 per cycle and SM: 1024 cycles per tile of 128 x 128 scores) and, next to them, 21
 // MMAs per tile (about 950 cycles).  Measured (180 x 320 tokens, 32 x 32 windows, 6 heads of 32 channels, rank 16, with the
@@ -66,6 +67,7 @@ constexpr uint32_t kIdescS = idesc_bf16_f32(kTile, kTile, false);
 constexpr uint32_t kIdescPV = idesc_bf16_f32(kTile, kD, true);
 
 struct FrameParams {
+    const __nv_bfloat16 *q, *k, *v, *pk;       // read by plain_row only
     const __nv_bfloat16* pq;
     __nv_bfloat16* out;
     float* lse;
@@ -74,6 +76,7 @@ struct FrameParams {
     WindowGeom geom;           // sides of the extended map, window, shift
     int terms;                 // terms of the scaled query RIB rows in use: 1 or kTerms
     float scale_log2;          // log2(e) / sqrt(d)
+    float inv_sqrt_d, inv_sqrt_r;
     float pos_scale;           // sqrt(d / r): folds 1/sqrt(r) into the content scale
     long long pos_head_stride;
     int pos_per_head;
@@ -88,6 +91,67 @@ __device__ __forceinline__ float log_sum(float n, float l)
     if (!(l > 0.f && l < INFINITY)) return -n + logf(l);             // no finite logit, or one that is no number
     const int k = ((int)__float_as_uint(l) - 0x3f3504f3) >> 23;      // l = 2^k f, f in [sqrt(1/2), sqrt(2))
     return (float)(((double)k - (double)n) * 0.69314718055994531 + (double)logf(__uint_as_float(__float_as_uint(l) - ((uint32_t)k << 23))));
+}
+
+// s plus the products of two rows of bf16 (16-byte aligned, widths are multiples of 8), the first scaled, in fp32
+__device__ __forceinline__ float add_products(float s, const __nv_bfloat16* a, float scale, const __nv_bfloat16* b, int width)
+{
+    for (int e = 0; e < width; e += 8) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4*>(a + e)), y = __ldg(reinterpret_cast<const uint4*>(b + e));
+        const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            s = fmaf(__uint_as_float(xs[w] << 16) * scale, __uint_as_float(ys[w] << 16), s);
+            s = fmaf(__uint_as_float(xs[w] & 0xffff0000u) * scale, __uint_as_float(ys[w] & 0xffff0000u), s);
+        }
+    }
+    return s;
+}
+
+// The output row (16 channels) and lse of one query, as rib_generic.cu defines them: fp32, one number per factor.  Called for
+// rows with a NaN only, by one thread per half.
+__device__ __noinline__ void plain_row(const FrameParams* pp, int item, int row256, int half)
+{
+    const FrameParams& p = *pp;
+    const LiveItem c = decode_live_item(p.live, item);
+    auto place = [&](int patch, int in, int& table_row, size_t& token) {      // false: no token
+        int py, px, Y0, X0;
+        live_patch_origin(p.live, p.geom, c, patch, py, px, Y0, X0);
+        const int Y = Y0 + (in >> 3), X = X0 + (in & 7);
+        table_row = (py + (in >> 3)) * p.geom.M + px + (in & 7);
+        token = (((size_t)c.b * p.H + Y) * p.W + X) * p.heads + c.h;
+        return Y < p.H && X < p.W;
+    };
+    int i;
+    size_t query;
+    place(4 * c.tp + (row256 >> 6), row256 & 63, i, query);
+    const __nv_bfloat16 *pq = p.pq + (size_t)c.h * p.pos_head_stride + (size_t)i * p.r, *pk = p.pk + (size_t)c.h * p.pos_head_stride;
+    auto logit = [&](int j, size_t key) {
+        return add_products(add_products(0.f, p.q + query * p.d, p.inv_sqrt_d, p.k + key * p.d, p.d), pq, p.inv_sqrt_r, pk + (size_t)j * p.r, p.r);
+    };
+    float m = -INFINITY, l = 0.f, o[16];
+    for (int key = 0; key < 64 * c.patches; ++key) {
+        int j;
+        size_t token;
+        if (place(key >> 6, key & 63, j, token)) m = fmaxf(m, logit(j, token));
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) o[e] = 0.f;
+    for (int key = 0; key < 64 * c.patches && m > -INFINITY; ++key) {
+        int j;
+        size_t token;
+        if (!place(key >> 6, key & 63, j, token)) continue;
+        const float w = expf(logit(j, token) - m);
+        l += w;
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+            if (half * 16 + e < p.d) o[e] = fmaf(w, __bfloat162float(p.v[token * p.d + half * 16 + e]), o[e]);
+    }
+    const float inv = 1.f / l;
+#pragma unroll
+    for (int e = 0; e < 16; ++e)
+        if (half * 16 + e < p.d) p.out[query * p.d + half * 16 + e] = __float2bfloat16_rn(o[e] * inv);
+    if (p.lse && half == 0) p.lse[((size_t)c.b * p.heads + c.h) * p.H * p.W + (query / p.heads - (size_t)c.b * p.H * p.W)] = m + logf(l);
 }
 
 template <int R>
@@ -185,6 +249,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     for (int sub = 0; sub < 2; ++sub) {
                         int py, px, Y0, X0;
                         live_patch_origin(p.live, p.geom, c, min(2 * j + sub, c.patches - 1), py, px, Y0, X0);
+                        if (2 * j + sub >= c.patches) X0 = p.geom.W;         // no such patch: beyond the map, zeros
                         tma_load_5d(base + L::kOffKc + st * kContentBytes + sub * kPatchContent, &tm_k, bar(L::kFull + st), 0, c.h, X0, Y0, c.b);
                         tma_load_4d(base + L::kOffKp + st * kPos + sub * L::kPatchP, &tm_pk, bar(L::kFull + st), 0, px, py, c.h * p.pos_per_head);
                         tma_load_5d(base + L::kOffV + st * kContentBytes + sub * kPatchContent, &tm_v, bar(L::kFull + st), 0, c.h, X0, Y0, c.b);
@@ -405,6 +470,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             if (k < c.patches && Y < p.H && X < p.W) {       // (else: no token, nothing to store)
                 const size_t tok = (((size_t)c.b * p.H + Y) * p.W + X) * p.heads + c.h;
                 uint4* dst = reinterpret_cast<uint4*>(p.out + tok * p.d + half * 16);
+                float sum = 0.f;                             // NaN if a value is NaN
 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
                     if (half * 16 + 8 * g >= p.d) break;     // a head narrower than 32 channels: the rest of the row is padding
@@ -412,12 +478,14 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
 #pragma unroll
                     for (int k2 = 0; k2 < 4; ++k2) {
                         const int e = 8 * g + 2 * k2;
-                        w[k2] = pack_bf16x2(__uint_as_float(oa[e]) * w_a + __uint_as_float(ob[e]) * w_b,
-                                            __uint_as_float(oa[e + 1]) * w_a + __uint_as_float(ob[e + 1]) * w_b);
+                        const float x = __uint_as_float(oa[e]) * w_a + __uint_as_float(ob[e]) * w_b, y = __uint_as_float(oa[e + 1]) * w_a + __uint_as_float(ob[e + 1]) * w_b;
+                        sum += x + y;
+                        w[k2] = pack_bf16x2(x, y);
                     }
                     dst[g] = make_uint4(w[0], w[1], w[2], w[3]);
                 }
                 if (p.lse && half == 0) p.lse[(((size_t)c.b * p.heads + c.h) * p.H + Y) * p.W + X] = log_sum(n, l_all);
+                if (isnan(sum)) plain_row(&p, item, 128 * qt + row, half);
             }
             __syncwarp();
         }
@@ -446,10 +514,12 @@ cudaError_t launch_fwd_frame(const Problem& p, cudaStream_t stream)
     static KernelSetup setup;       // one per instantiation of this launcher, i.e. per kernel
     int sm_count = 0;
     if (cudaError_t e = setup.prepare(rib_fwd_frame_sm100_kernel<R>, Frame<R>::kSmemBytes, &sm_count)) return e;
+    const float d = scale_width_d(p), r = scale_width_r(p);
+    fp.q = p.q; fp.k = p.k; fp.v = p.v; fp.pk = p.pk;
+    fp.inv_sqrt_d = 1.f / sqrtf(d); fp.inv_sqrt_r = 1.f / sqrtf(r);
     fp.pq = p.pq; fp.out = p.out_w; fp.lse = p.lse_w; fp.status = p.status;
     fp.H = p.H; fp.W = p.W; fp.heads = p.heads; fp.d = p.d; fp.r = p.r;
     fp.geom = WindowGeom{p.Hp, p.Wp, p.M, p.s};
-    const float d = scale_width_d(p), r = scale_width_r(p);
     fp.scale_log2 = (float)(1.4426950408889634 / sqrt((double)d));
     fp.pos_scale = sqrtf(d / r);
     fp.terms = d == r || d == 4.f * r || 4.f * d == r ? 1 : kTerms;      // sqrt(d / r) a power of two: the product is a bf16 number

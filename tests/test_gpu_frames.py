@@ -100,6 +100,34 @@ def test_frames_with_many_items_per_cta(wl):
         assert np.array_equal(out, again) and np.array_equal(lse, lse_again)
 
 
+@pytest.mark.parametrize("what", ["v", "k", "pk", "pq", "pq_all"])
+@pytest.mark.parametrize("shape", [(20, 28, 32, 16, 16), (45, 27, 32, 32, 32), (20, 28, 30, 18, 16)], ids=lambda s: "x".join(map(str, s)))
+def test_infinities_come_out_as_from_the_any_shape_kernel(shape, what):
+    """One infinite (or -inf) entry: NaN, inf and -inf at the same places as from the fp32 kernel, finite values beside them."""
+    H, W, d, r, window = shape
+    wl = Workload("f_inf", 2, H, W, 2, d, r, window, 0, seed=218)
+    cpu = synthetic.make_inputs(wl, with_dout=False)
+    inf = float("inf")
+    if what in ("v", "k"):
+        for y, x, c, value in ((0, 1, 3, inf), (H - 1, W - 1, 5, -inf)):      # the last patch as well: it may fill half a key block
+            cpu[what][1, y, x, 1, c] = value
+    elif what == "pk":
+        cpu["pk"][window + 1, 2], cpu["pk"][3, 4] = inf, -inf
+    else:
+        cpu["pq"][window + 2, 3] = -inf
+        if what == "pq_all":                                                  # every logit of that row is -inf
+            cpu["pk"][:, 3] = cpu["pk"][:, 3].abs() + 0.5
+    gpu = {k: v.cuda() for k, v in cpu.items()}
+    out, lse, used = run(wl, gpu, binding.RIB_PATH_NONE)
+    wide_out, wide_lse, _ = run(wl, gpu, binding.RIB_PATH_GENERIC)
+    assert used == binding.RIB_PATH_SM100 and not (np.isfinite(wide_out).all() and np.isfinite(wide_lse).all())
+    for got, want in ((out, wide_out), (lse, wide_lse)):
+        assert np.array_equal(np.isnan(got), np.isnan(want))
+        assert np.array_equal(np.isposinf(got), np.isposinf(want)) and np.array_equal(np.isneginf(got), np.isneginf(want))
+        fine = np.isfinite(want)                 # the roundings to bf16 that the order of an fp32 sum decides: one step of values up to 2
+        compare("finite values", got[fine], want[fine], max_abs=2.0 ** -7, rel_l2=3e-4)
+
+
 @pytest.mark.parametrize("wl", [CASES[6], CASES[8], MANY[0], MANY[2]], ids=lambda w: w.name)
 def test_lse_of_frames_is_no_further_off_than_from_the_any_shape_kernel(wl):
     cpu = synthetic.make_inputs(wl, with_dout=False)
