@@ -358,10 +358,12 @@ const char* rib_status_string(int status);
 
 /*
  * Debugging knobs, per process.  rib_set_path(RIB_PATH_GENERIC) forces the any-shape kernels,
- * rib_set_path(RIB_PATH_SM100_EXACT) keeps automatic selection but makes the tcgen05 forward kernel
- * take its exact softmax form (running maximum, rescaling) for every item instead of only for the
+ * rib_set_path(RIB_PATH_SM100_EXACT) keeps automatic selection but makes the tcgen05 forward kernels
+ * take the exact softmax form (a maximum of the row's own, every exponential on the special-function unit, fp32 sum of
+ * the unrounded exponentials in lse) for every item instead of only for the
  * items whose scores leave the range of the fast form (Sec. 3.1: the steps after Eq. 6 are those of
- * standard attention; both forms compute the same SoftMax), rib_set_path(RIB_PATH_NONE) restores
+ * standard attention; both forms compute the same SoftMax); windows of 8 x 8 tokens and frames with a side that is no
+ * multiple of 8 have that form only.  rib_set_path(RIB_PATH_NONE) restores
  * automatic selection; returns the previous setting (other values: nothing changes).
  * rib_last_path() tells which family the last successful fwd/bwd call of this thread launched.
  */

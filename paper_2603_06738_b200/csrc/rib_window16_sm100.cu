@@ -727,7 +727,9 @@ bool sm100_window16(const Problem& p) { return p.M == 16 && p.s % 8 == 0 && p.H 
 // Forward: on windows that are all whole and alike the general kernel is the faster one (10 x 64 x 64 tokens, 6 heads, rank 16:
 // 37 against 43 us with the launch); with a mask or windows beyond the map it is the slower one (4 x 96 x 96 tokens, 12 heads
 // of 16 channels, rank 24, masked: 83 against 63 us).
-bool sm100_window16_prefers(const Problem& p) { return sm100_window16(p) && (p.masked || p.Hp != p.H || p.Wp != p.W); }
+// This kernel has the fast form of the softmax only (one exponential in four on the FMA pipe, lse from rounded probabilities):
+// calls that ask for the exact form take the general kernel.
+bool sm100_window16_prefers(const Problem& p) { return sm100_window16(p) && !p.exact_softmax && (p.masked || p.Hp != p.H || p.Wp != p.W); }
 cudaError_t sm100_window16_fwd(const Problem& p, cudaStream_t stream)
 {
     return padded_rank(p.r) == 32 ? launch_win16_fwd<32>(p, stream) : launch_win16_fwd<16>(p, stream);

@@ -54,3 +54,28 @@ def test_windows_of_16(wl, spread):
 @pytest.mark.parametrize("wl", [w for w in CASES if w.H % 16 == 0 and w.W % 16 == 0], ids=lambda w: w.name)
 def test_masked_windows_of_16(wl):
     check(wl, 1.0, rib_masked_oracle, binding.rib_window_attn_fwd_masked, binding.rib_window_attn_bwd_masked)
+
+
+@pytest.mark.parametrize("wl", [
+    Workload("w16_exact_masked", 1, 48, 32, 3, 32, 32, 16, 8, seed=510),
+    Workload("w16_exact_masked_headwise", 2, 32, 32, 2, 8, 32, 16, 8, seed=511, headwise=True),
+    Workload("w16_exact_partial", 1, 24, 72, 6, 32, 32, 16, 8, seed=512),
+], ids=lambda w: w.name)
+def test_the_exact_form_is_taken_where_it_is_asked_for(wl):
+    """rib_set_path(RIB_PATH_SM100_EXACT): lse from fp32 sums of unrounded exponentials, also for masks and windows beyond the map."""
+    cpu = synthetic.make_inputs(wl, with_dout=False)
+    args = [cpu[k].cuda() for k in ("q", "k", "v", "pq", "pk")]
+    masked = wl.H % 16 == 0 and wl.W % 16 == 0
+    fwd, oracle = (binding.rib_window_attn_fwd_masked, rib_masked_oracle) if masked else (binding.rib_window_attn_fwd_padded, rib_padded_oracle)
+    binding.rib_set_path(binding.RIB_PATH_SM100_EXACT)
+    try:
+        out, lse = fwd(*args, wl.window, wl.shift)
+        assert binding.rib_last_path() == binding.RIB_PATH_SM100
+    finally:
+        binding.rib_set_path(binding.RIB_PATH_NONE)
+    torch.cuda.synchronize()
+    ref_out, ref_lse = oracle.fwd(*(to_f64(cpu[k]) for k in ("q", "k", "v", "pq", "pk")), wl.window, wl.shift)
+    compare("out", to_f64(out), ref_out)
+    # sqrt(d / r) is a power of two here, so the scaled query rows are exact: what is left are fp32 logits and sums (2^-24 each);
+    # probabilities rounded to bf16 (2^-9 each over up to 256 keys) would leave some 1e-5 of lse
+    compare("lse", to_f64(lse), ref_lse, rel_l2=2e-6)
