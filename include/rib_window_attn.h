@@ -383,8 +383,8 @@ void rib_tensor_map_cache_counts(long long* hits, long long* misses);
 
 /*
  * Per-kernel device timing, for benchmarks (not part of the method).  Between rib_profile_begin and
- * rib_profile_end every kernel launch of this library is bracketed by two CUDA events on the launch
- * stream, up to `max_launches` launches (later ones are not recorded).  rib_profile_end waits for
+ * rib_profile_end every kernel launch of the attention, generator and gate calls but the copies of zero-padded rows is bracketed
+ * by two CUDA events on the launch stream (a kernel that would overtake the one before it then does not), up to `max_launches` launches (later ones are not recorded).  rib_profile_end waits for
  * the recorded events, writes for launch i its kernel id (RIB_KERNEL_*) to kernel_ids[i] and its
  * device time in milliseconds to ms[i] (at most `capacity` entries), releases the events and
  * returns the number of entries written, or a negative RIB_ERR_* code.  Both calls create or
@@ -394,7 +394,9 @@ void rib_tensor_map_cache_counts(long long* hits, long long* misses);
 enum { RIB_KERNEL_FWD_MAIN = 1, RIB_KERNEL_BWD_PREPARE = 2, RIB_KERNEL_BWD_MAIN = 3, RIB_KERNEL_BWD_FINISH = 4,
        RIB_KERNEL_RESERVED = 5, RIB_KERNEL_ANY_FWD = 6, RIB_KERNEL_ANY_ROWDOT = 7, RIB_KERNEL_ANY_BWD_DQ = 8,
        RIB_KERNEL_ANY_BWD_DKV = 9, RIB_KERNEL_GENERATOR_FWD = 10, RIB_KERNEL_GENERATOR_BWD = 11,
-    RIB_KERNEL_CLA_GATE = 12, RIB_KERNEL_CLA_BWD_PW = 13, RIB_KERNEL_CLA_BWD_DW = 14, RIB_KERNEL_CLA_PRODUCT = 15, RIB_KERNEL_CLA_BWD_TC = 16 };
+    RIB_KERNEL_CLA_GATE = 12, RIB_KERNEL_CLA_BWD_PW = 13, RIB_KERNEL_CLA_BWD_DW = 14, RIB_KERNEL_CLA_PRODUCT = 15, RIB_KERNEL_CLA_BWD_TC = 16,
+    RIB_KERNEL_FWD_FRAME = 17, RIB_KERNEL_WINDOW8_FWD = 18, RIB_KERNEL_WINDOW8_CLEAR = 19, RIB_KERNEL_WINDOW8_BWD = 20,
+    RIB_KERNEL_WINDOW16_FWD = 21, RIB_KERNEL_WINDOW16_CLEAR = 22, RIB_KERNEL_WINDOW16_BWD = 23, RIB_KERNEL_GENERATOR_CLEAR = 24 };
 int rib_profile_begin(int max_launches);
 int rib_profile_end(int* kernel_ids, float* ms, int capacity);
 

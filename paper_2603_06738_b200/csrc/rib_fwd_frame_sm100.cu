@@ -526,7 +526,7 @@ cudaError_t launch_fwd_frame(const Problem& p, cudaStream_t stream)
     fp.pos_head_stride = p.pos_head_stride;
     fp.pos_per_head = p.pos_head_stride ? 1 : 0;
     const int items = fp.live.offset[9], grid = items < sm_count ? items : sm_count;
-    { ProfileScope scope(RIB_KERNEL_FWD_MAIN, stream); rib_fwd_frame_sm100_kernel<R><<<grid, kThreads, Frame<R>::kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_pk, fp); }
+    { ProfileScope scope(RIB_KERNEL_FWD_FRAME, stream); rib_fwd_frame_sm100_kernel<R><<<grid, kThreads, Frame<R>::kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_pk, fp); }
     return cudaGetLastError();
 }
 

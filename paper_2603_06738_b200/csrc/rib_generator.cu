@@ -253,10 +253,10 @@ cudaError_t generator_bwd(const float* w_h, const float* b_h, const float* w_pq,
     cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(rib_generator_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                                      : cudaSuccess;
     if (e != cudaSuccess) return e;
-    ProfileScope scope(RIB_KERNEL_GENERATOR_BWD, stream);
     const int most = p.in * dh > dh * r ? p.in * dh : dh * r;
-    rib_generator_clear_kernel<<<(most + 255) / 256, 256, 0, stream>>>(p);
+    { ProfileScope scope(RIB_KERNEL_GENERATOR_CLEAR, stream); rib_generator_clear_kernel<<<(most + 255) / 256, 256, 0, stream>>>(p); }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    ProfileScope scope(RIB_KERNEL_GENERATOR_BWD, stream);
     cudaLaunchAttribute overtake;
     overtake.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     overtake.val.programmaticStreamSerializationAllowed = 1;

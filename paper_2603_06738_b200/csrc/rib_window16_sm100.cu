@@ -693,7 +693,7 @@ cudaError_t launch_win16_fwd(const Problem& p, cudaStream_t stream)
     SmallWindowParams w{};
     const int grid = fill_small_window(p, sm_count, p.nWy, p.nWx, &w);
     w.lse = p.lse_w;
-    ProfileScope scope(RIB_KERNEL_FWD_MAIN, stream);
+    ProfileScope scope(RIB_KERNEL_WINDOW16_FWD, stream);
     fwd16::rib_window16_fwd_kernel<R><<<grid, fwd16::kThreads, fwd16::kSmemBytes, stream>>>(tm_q, tm_k, tm_v, p.out_w, w);
     return cudaGetLastError();
 }
@@ -713,10 +713,16 @@ cudaError_t launch_win16_bwd(const Problem& p, cudaStream_t stream)
     const int grid = fill_small_window(p, sm_count, p.nWy, p.nWx, &w);
     w.out = p.out; w.dout = p.dout; w.lse_in = p.lse_in; w.dpq = p.dpq; w.dpk = p.dpk;
     const int tables = pos_tables(p), per_table = 256 * p.r, blocks = (tables * per_table + 255) / 256 < 64 ? (tables * per_table + 255) / 256 : 64;
-    bwd16::rib_window16_clear_kernel<<<blocks, 256, 0, stream>>>(p.dpq, tables, per_table, p.pos_head_stride);
+    {
+        ProfileScope scope(RIB_KERNEL_WINDOW16_CLEAR, stream);
+        bwd16::rib_window16_clear_kernel<<<blocks, 256, 0, stream>>>(p.dpq, tables, per_table, p.pos_head_stride);
+    }
     if (cudaError_t e = cudaGetLastError()) return e;
-    if (cudaError_t e = launch_overtaking(bwd16::rib_window16_clear_kernel, blocks, 256, 0, stream, p.dpk, tables, per_table, p.pos_head_stride)) return e;
-    ProfileScope scope(RIB_KERNEL_BWD_MAIN, stream);
+    {
+        ProfileScope scope(RIB_KERNEL_WINDOW16_CLEAR, stream);
+        if (cudaError_t e = launch_overtaking(bwd16::rib_window16_clear_kernel, blocks, 256, 0, stream, p.dpk, tables, per_table, p.pos_head_stride)) return e;
+    }
+    ProfileScope scope(RIB_KERNEL_WINDOW16_BWD, stream);
     return launch_overtaking(bwd16::rib_window16_bwd_kernel<R>, grid, bwd16::kThreads, bwd16::kSmemBytes, stream, tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, p.dv, w);
 }
 

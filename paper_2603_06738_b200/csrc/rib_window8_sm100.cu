@@ -578,7 +578,7 @@ cudaError_t launch_win8_fwd(const Problem& p, cudaStream_t stream)
     SmallWindowParams w{};
     const int grid = fill_small_window(p, sm_count, p.H / 8, p.W / 16, &w);
     w.lse = p.lse_w;
-    ProfileScope scope(RIB_KERNEL_FWD_MAIN, stream);
+    ProfileScope scope(RIB_KERNEL_WINDOW8_FWD, stream);
     fwd8::rib_window8_fwd_kernel<R><<<grid, fwd8::kThreads, fwd8::kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_out, w);
     return cudaGetLastError();
 }
@@ -598,10 +598,13 @@ cudaError_t launch_win8_bwd(const Problem& p, cudaStream_t stream)
     const int grid = fill_small_window(p, sm_count, p.H / 8, p.W / 16, &w);
     w.lse_in = p.lse_in; w.dpq = p.dpq; w.dpk = p.dpk;
     const int tables = pos_tables(p), per_table = 64 * p.r;
-    bwd8::rib_window8_clear_kernel<<<(tables * per_table + 255) / 256 < 64 ? (tables * per_table + 255) / 256 : 64, 256, 0, stream>>>(
-        p.dpq, p.dpk, tables, per_table, p.pos_head_stride);
+    const int blocks = (tables * per_table + 255) / 256 < 64 ? (tables * per_table + 255) / 256 : 64;
+    {
+        ProfileScope scope(RIB_KERNEL_WINDOW8_CLEAR, stream);
+        bwd8::rib_window8_clear_kernel<<<blocks, 256, 0, stream>>>(p.dpq, p.dpk, tables, per_table, p.pos_head_stride);
+    }
     if (cudaError_t e = cudaGetLastError()) return e;
-    ProfileScope scope(RIB_KERNEL_BWD_MAIN, stream);
+    ProfileScope scope(RIB_KERNEL_WINDOW8_BWD, stream);
     return launch_overtaking(bwd8::rib_window8_bwd_kernel<R>, grid, bwd8::kThreads, bwd8::kSmemBytes, stream, tm_q, tm_k, tm_v, tm_do, tm_o, tm_dq, tm_dk, tm_dv, w);
 }
 
