@@ -132,7 +132,10 @@ size_t rib_window_attn_bwd_headwise_workspace(long long pos_head_stride, int B, 
  * rib_window_attn_fwd_headwise; other arguments, layouts and error codes as there.  H and W multiples of 8 (and
  * the shape conditions above) take the tcgen05 kernel, where a patch of the extension costs a zero-filled TMA box;
  * any other H, W (windows a multiple of 16, shift a multiple of 8, d and r as above, r up to 32) take a tcgen05 kernel of their
- * own that keeps probabilities, sums and scaled features at fp32 precision; what is left takes the any-shape kernel.
+ * own: scaled features enter its products with 24 significant bits, probabilities with 16 (the any-shape kernel: 24), sums are
+ * fp32; the error of out against float64 is the rounding to bf16 with either (1.7e-3, equal to 4 parts in a million), that of lse
+ * is below the any-shape kernel's; NaN and infinite inputs give what the any-shape kernel gives, a row that comes out as NaN being
+ * computed once more without tensor cores.  What is left takes the any-shape kernel.
  */
 int rib_window_attn_fwd_padded(const void* q, const void* k, const void* v, const void* pq, const void* pk,
                                long long pos_head_stride,
@@ -313,7 +316,7 @@ int rib_window_attn_bwd_noalloc(const void* q, const void* k, const void* v, con
  * Backward: given dpq, dpk (fp32 [n][r], e.g. from rib_window_attn_bwd) it overwrites
  *   dw_h [2 + 4 L][dh], db_h [dh], dw_pq, dw_pk [dh][r] (fp32) with the gradients of
  *   sum(Pq o dpq) + sum(Pk o dpk); the bf16 rounding of pq / pk is treated as the identity.
- *   The results are zero-filled on `stream` and accumulated with atomic adds over slices of 128 tokens.
+ *   The results are zero-filled on `stream` and accumulated with atomic adds over slices of 16 tokens.
  * Limits: 1 <= window <= 256, 0 <= L <= 16, 1 <= dh <= 64, 1 <= r <= 64; otherwise RIB_ERR_UNSUPPORTED
  * (RIB_ERR_SHAPE for non-positive sizes).  Pointers 16-byte aligned.  Both calls only enqueue work.
  */
