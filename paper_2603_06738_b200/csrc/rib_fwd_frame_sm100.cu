@@ -259,7 +259,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 blk += (uint32_t)((c.patches + 1) >> 1);
             }
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok && lane == 0) ++io;                      // this item's query tiles are armed as well
+            // (giving up here: the loop counts this item, whose query tiles are armed)
         }
         if (!ok && lane == 0) {
             // Gave up: let the copies already in flight land before the CTA may exit.
