@@ -730,12 +730,20 @@ cudaError_t launch_win16_bwd(const Problem& p, cudaStream_t stream)
 
 // (sides that are no multiples of 8 have kernels of their own)
 bool sm100_window16(const Problem& p) { return p.M == 16 && p.s % 8 == 0 && p.H % 8 == 0 && p.W % 8 == 0 && !p.gate; }
-// Forward: on windows that are all whole and alike the general kernel is the faster one (10 x 64 x 64 tokens, 6 heads, rank 16:
-// 37 against 43 us with the launch); with a mask or windows beyond the map it is the slower one (4 x 96 x 96 tokens, 12 heads
-// of 16 channels, rank 24, masked: 83 against 63 us).
+// Forward, this kernel against the general one, us with the launch (6 heads of 32 channels unless stated; 12 x 16: 12 heads of 16):
+//   whole windows          rank 16: 10 x 64 x 64 tokens 40 / 35, 256 x 256 60 / 50; rank 32: 41 / 40, 62 / 59; 12 x 16, rank 24: 65 / 63, 98 / 96;
+//   with a mask            rank 16: 10 x 64 x 64 40 / 47, 16 x 96 x 96 122 / 135, 256 x 256 60 / 59; rank 32: 41 / 58, 62 / 73; 12 x 16, rank 24: 63 / 106;
+//   beyond the map         rank 16: 48 x 40 10.4 / 12.3, 120 x 200 28.8 / 28.8, 200 x 328 64 / 59, 360 x 632 189 / 175; rank 32: 120 x 200 30 / 33,
+//                          360 x 632 193 / 217; 12 x 16, rank 24: 315 / 393.
+// So whole windows stay with the general kernel, masks come here, and windows beyond the map come here with RIB rows of 32 elements or
+// while there is little work (120 x 200 tokens are four windows per SM).
 // This kernel has the fast form of the softmax only (one exponential in four on the FMA pipe, lse from rounded probabilities):
 // calls that ask for the exact form take the general kernel.
-bool sm100_window16_prefers(const Problem& p) { return sm100_window16(p) && !p.exact_softmax && (p.masked || p.Hp != p.H || p.Wp != p.W); }
+bool sm100_window16_prefers(const Problem& p)
+{
+    if (!sm100_window16(p) || p.exact_softmax) return false;
+    return p.masked || ((p.Hp != p.H || p.Wp != p.W) && (padded_rank(p.r) == 32 || p.pairs <= 4 * 148));
+}
 cudaError_t sm100_window16_fwd(const Problem& p, cudaStream_t stream)
 {
     return padded_rank(p.r) == 32 ? launch_win16_fwd<32>(p, stream) : launch_win16_fwd<16>(p, stream);

@@ -46,3 +46,24 @@ def test_the_generator_backward_is_two_launches():
     grads = [torch.randn(256, 16, device="cuda") for _ in range(2)]
     _, names = bracketed(lambda: binding.rib_generate_features_bwd(*ws, *grads, 16))
     assert names == ["rib_generator_clear_kernel", "rib_generator_bwd_kernel"]
+
+
+@pytest.mark.parametrize("H,W,r,masked,kernel", [
+    (128, 128, 16, False, "rib_fwd_sm100_kernel"),                  # whole windows
+    (128, 128, 16, True, "rib_window16_fwd_kernel"),
+    (120, 136, 16, False, "rib_window16_fwd_kernel"),               # 8 x 9 windows, 8 heads: 576 pairs
+    (120, 152, 16, False, "rib_fwd_sm100_kernel"),                  # 8 x 10: 640
+    (120, 152, 32, False, "rib_window16_fwd_kernel"),
+])
+def test_the_forward_kernel_of_windows_of_16(H, W, r, masked, kernel):
+    cpu = synthetic.make_inputs(Workload("rule", 1, H, W, 8, 32, r, 16, 8, seed=702), with_dout=False)
+    args = [cpu[k].cuda() for k in ("q", "k", "v", "pq", "pk")]
+    fwd = binding.rib_window_attn_fwd_masked if masked else binding.rib_window_attn_fwd_padded
+    (out, lse), names = bracketed(lambda: fwd(*args, 16, 8))
+    assert names == [kernel]
+    binding.rib_set_path(binding.RIB_PATH_SM100_EXACT)              # the other kernel agrees: two bf16 roundings of values up to 4
+    try:
+        other, other_lse = fwd(*args, 16, 8)
+    finally:
+        binding.rib_set_path(binding.RIB_PATH_NONE)
+    assert (out.float() - other.float()).abs().max() <= 2.0 ** -6 and (lse - other_lse).abs().max() <= 2e-3
