@@ -131,6 +131,23 @@ struct ProfileScope {
     ~ProfileScope() { profile_mark(id, 1, stream); }
 };
 
+// Launch of a kernel that may start while the kernel before it on the stream still runs (it waits for that one's end by itself).
+template <typename Kernel, typename... Args>
+inline cudaError_t launch_overtaking(Kernel kernel, int grid, int threads, size_t smem, cudaStream_t stream, const Args&... args)
+{
+    cudaLaunchAttribute overtake;
+    overtake.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overtake.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t config{};
+    config.gridDim = dim3((unsigned)grid);
+    config.blockDim = dim3((unsigned)threads);
+    config.dynamicSmemBytes = smem;
+    config.stream = stream;
+    config.attrs = &overtake;
+    config.numAttrs = 1;
+    return cudaLaunchKernelEx(&config, kernel, args...);
+}
+
 // Window partition with cyclic shift: token i = y*M + x of window (wy, wx) -> image pixel.
 __host__ __device__ inline void token_pixel(int H, int W, int M, int s, int wy, int wx, int i,
                                             int& Y, int& X)

@@ -257,17 +257,7 @@ cudaError_t generator_bwd(const float* w_h, const float* b_h, const float* w_pq,
     { ProfileScope scope(RIB_KERNEL_GENERATOR_CLEAR, stream); rib_generator_clear_kernel<<<(most + 255) / 256, 256, 0, stream>>>(p); }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     ProfileScope scope(RIB_KERNEL_GENERATOR_BWD, stream);
-    cudaLaunchAttribute overtake;
-    overtake.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    overtake.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t config{};
-    config.gridDim = dim3((unsigned)((p.n + kTokens - 1) / kTokens));
-    config.blockDim = dim3(kThreads);
-    config.dynamicSmemBytes = smem;
-    config.stream = stream;
-    config.attrs = &overtake;
-    config.numAttrs = 1;
-    return cudaLaunchKernelEx(&config, rib_generator_bwd_kernel, p);
+    return launch_overtaking(rib_generator_bwd_kernel, (p.n + kTokens - 1) / kTokens, kThreads, smem, stream, p);
 }
 
 }  // namespace rib

@@ -85,22 +85,5 @@ __device__ __forceinline__ void add_columns(float* dst, const uint32_t* a, float
     atomicAdd(reinterpret_cast<float4*>(dst), make_float4(__uint_as_float(a[0]) * f, __uint_as_float(a[1]) * f, __uint_as_float(a[2]) * f, __uint_as_float(a[3]) * f));
 }
 
-// Launch of a kernel that may start while the kernel before it on the stream still runs (it waits for that one's end by itself).
-template <typename Kernel, typename... Args>
-inline cudaError_t launch_overtaking(Kernel kernel, int grid, int threads, size_t smem, cudaStream_t stream, const Args&... args)
-{
-    cudaLaunchAttribute overtake;
-    overtake.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    overtake.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t config{};
-    config.gridDim = dim3((unsigned)grid);
-    config.blockDim = dim3((unsigned)threads);
-    config.dynamicSmemBytes = smem;
-    config.stream = stream;
-    config.attrs = &overtake;
-    config.numAttrs = 1;
-    return cudaLaunchKernelEx(&config, kernel, args...);
-}
-
 }  // namespace sm100
 }  // namespace rib
