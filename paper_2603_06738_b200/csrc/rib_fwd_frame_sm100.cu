@@ -1,8 +1,8 @@
 // Forward RIB window attention for B200 (sm_100a) on frames whose sides are not multiples of 8: tcgen05 MMAs, TMEM, TMA.
 //
 // These shapes are defined by the fp32 any-shape kernels (rib_generic.cu), which keep the probabilities, their sums and the
-// scaled positional features in fp32.  This kernel keeps that precision on the bf16 tensor cores by splitting what is not
-// a bf16 number to begin with into bf16 terms whose sum carries it:
+// scaled positional features in fp32.  This kernel stays close to that on the bf16 tensor cores by splitting what is not
+// a bf16 number to begin with into bf16 terms:
 //     P            = hi + lo           two terms, 16 significant bits: the PV contraction runs twice, into one accumulator;
 //     Pq sqrt(d/r) = hi + mid + lo     three terms, all 24 bits: one K16 step (two at R = 32) of the score chain per term
 //                                      (one term where d / r is a power of 4 and the product is a bf16 number);
@@ -12,8 +12,8 @@
 //
 // What bounds it: the exponentials (16 per cycle and SM: 1024 cycles per tile of 128 x 128 scores) and, next to them, 21
 // MMAs per tile (about 950 cycles).  Measured (180 x 320 tokens, 32 x 32 windows, 6 heads of 32 channels, rank 16, with the
-// launch): 176 us = 308 TFLOP/s of the layer's own flops, about 2000 cycles per tile and SM; the any-shape kernel 13 460 us.
-// Error of `out` against float64 as that kernel's (1.7e-3, the rounding to bf16).
+// launch): 178 us = 305 TFLOP/s of the layer's own flops, about 2000 cycles per tile and SM; the any-shape kernel 13 460 us.
+// Error of `out` against float64 as that kernel's (1.7e-3, the rounding to bf16; 4 parts in a million more at most), of lse below it.
 //
 // Work item = one (batch, window, head) pair x two query tiles of 128 tokens (two 8x8-token patches each).  Only patches that
 // hold tokens are walked (LiveWindows in rib_sm100_common.cuh); a patch that straddles the border of the frame is filled up

@@ -7,8 +7,8 @@
 // outside the chip.  What bounds it: the serial program of the softmax (arithmetic) warps.  A unit of the forward (128 rows x 256
 // keys) takes about 3900 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) about 3200: 1050 of loads
 // and exponentials, 1600 of stores of P and dS and their fences, with 1470 cycles of MMAs beside it.  Measured (4 x 96 x 96 tokens,
-// 12 heads of 16 channels, rank 24, shift 8, masked, by event hooks): forward 83 -> 62 us, backward 31 + 142 + 48 -> 103 us, both
-// calls 288 -> 156 us; backward on 10 x 64 x 64 tokens, 6 heads of 32 channels, rank 16: 21 + 64 + 25 -> 73 us.
+// 12 heads of 16 channels, rank 24, shift 8, masked, by event hooks): forward 82 -> 60 us, backward 30 + 140 + 46 -> 12 (two
+// clearings) + 104 us, both calls 288 -> 156 us; backward on 10 x 64 x 64 tokens, 6 heads of 32 channels, rank 16: 20 + 66 + 23 -> 12 + 71 us.
 //
 // Windows may be shifted (multiples of 8), masked, or reach beyond the map (sides multiples of 8): a window is four 8x8-token
 // patches (one TMA box each), and a query patch attends to a key patch or not.

@@ -4,9 +4,9 @@
 // 64 * (2 d + r) products, so a tile of 128 tokens has 1420 cycles at the measured copy bandwidth and needs 512 of the exp
 // pipe and about 550 of the tensor pipe; the backward has 2840 cycles per tile and needs 512 and about 1400.  Hence: every
 // input is read once and every output written once, nothing goes through accumulators in global memory, and several tiles are
-// under way per SM.  Measured (16 x 96 x 96 tokens, 6 heads of 32 channels, rank 16, kernel with launch, by event hooks):
-// forward 52 us, backward 87 us (each with about 7 us of launch) for 226 and 456 MB; the two calls together 141 us.  (Before: 128
-// us, 57 + 322 + 80 us and 560 us; these windows ran four at a time as 16 x 16 windows of the general kernels with three quarters of
+// under way per SM.  Measured (16 x 96 x 96 tokens, 6 heads of 32 channels, rank 16, by event hooks, which include some us per
+// launch): forward 45 us, backward 6 (clearing) + 83 us for 226 and 456 MB; the two calls together 141 us.  (Before: 125
+// us, 56 + 311 + 80 us and 582 us; these windows ran four at a time as 16 x 16 windows of the general kernels with three quarters of
 // every score tile discarded; the backward added dq in global memory and needed a preparation and a finishing kernel.)
 //
 // Tile = two horizontally adjacent windows of one head, 64 rows each (one 8x8-token patch, one TMA box).  A CTA keeps to one
