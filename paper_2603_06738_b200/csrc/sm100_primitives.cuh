@@ -227,25 +227,19 @@ __device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t (&r)[1])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[0]) : "r"(taddr) : "memory");
 }
-// 16 lanes x 32 fp32 columns.  Thread t of the warp receives rows t / 4 and t / 4 + 8 of the 16 lanes that start at
+// 16 lanes x 16 fp32 columns.  Thread t of the warp receives rows t / 4 and t / 4 + 8 of the 16 lanes that start at
 // the lane of `taddr`, and of each group g of 8 columns the two columns 8 g + 2 (t % 4), + 1:
 // r[4 g + 0], r[4 g + 1] = row t / 4, r[4 g + 2], r[4 g + 3] = row t / 4 + 8.  (Layout checked on the device.)
-__device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, uint32_t (&r)[16])
+__device__ __forceinline__ void tmem_ld_16x256b_x2(uint32_t taddr, uint32_t (&r)[8])
 {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
 }
-// 16 lanes x 16 columns of 32 bits.  Thread t writes, for each group g of 4 columns, column 4 g + t % 4 of rows t / 4
+// 16 lanes x 8 columns of 32 bits.  Thread t writes, for each group g of 4 columns, column 4 g + t % 4 of rows t / 4
 // (r[2 g]) and t / 4 + 8 (r[2 g + 1]): with two bf16 per column this is the packed image of the load above.
-__device__ __forceinline__ void tmem_st_16x128b_x4(uint32_t taddr, const uint32_t (&r)[8])
+__device__ __forceinline__ void tmem_st_16x128b_x2(uint32_t taddr, const uint32_t (&r)[4])
 {
-    asm volatile(
-        "tcgen05.st.sync.aligned.16x128b.x4.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
-        ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(taddr) : "memory");
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x2.b32 [%4], {%0, %1, %2, %3};" ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32])
 {
@@ -269,6 +263,12 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
           "r"(taddr) : "memory");
 }
 
+// Four 8 x 8 blocks of 16-bit elements to shared memory: lane 8 m + i gives the address of row i of block m (16 bytes), register m
+// of thread t holds elements 2 (t % 4), + 1 of row t / 4 of block m -- the layout of the 16-lane fragments above.
+__device__ __forceinline__ void stmatrix_x4(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
 {
     asm volatile(
@@ -327,10 +327,17 @@ __device__ __forceinline__ void mma_commit(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// Fire-and-forget fp32 add to global memory (relaxed, device scope).
-__device__ __forceinline__ void red_add_f32(float* addr, float v)
+// Fire-and-forget add of four fp32 columns to global memory (16-byte aligned; relaxed, device scope).
+__device__ __forceinline__ void red_add_f32x4(float* addr, const uint32_t* v)
 {
-    asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(addr), "f"(v) : "memory");
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};"
+                 ::"l"(addr), "f"(__uint_as_float(v[0])), "f"(__uint_as_float(v[1])), "f"(__uint_as_float(v[2])), "f"(__uint_as_float(v[3])) : "memory");
+}
+__device__ __forceinline__ float lds_f32(uint32_t addr)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+    return v;
 }
 
 __device__ __forceinline__ float ex2_approx(float x)
