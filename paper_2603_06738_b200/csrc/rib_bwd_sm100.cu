@@ -87,7 +87,6 @@ template <int R> struct Cols {
 constexpr uint32_t kHalfCols = kTile / 2;
 constexpr uint32_t kTmemCols = 512;
 
-constexpr uint32_t kIdescSS = idesc_bf16_f32(kTile, kTile / 2, false);        // S^T, dP^T of a half-tile: both operands K-major
 constexpr uint32_t kIdescT32 = idesc_bf16_f32(kTile, kD, true);               // A in TMEM, B MN-major, N = 32
 // dK~ (A in TMEM or K-major in shared memory, B MN-major) and dQ~ (A and B MN-major), N = kD + R
 template <int R> struct Idesc {
@@ -139,6 +138,8 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 {
     constexpr int kDk = kD + R;
     constexpr uint32_t kColDS = Cols<R>::kColDS, kColDV = Cols<R>::kColDV, kColDK = Cols<R>::kColDK, kColDQ = Cols<R>::kColDQ;
+    constexpr uint32_t kSUnits = R == 32 ? 2 : 1;         // half-tiles whose S^T, dP^T are issued together
+    constexpr uint32_t kIdescSS = idesc_bf16_f32(kTile, kSUnits * kTile / 2, false);    // both operands K-major
     constexpr uint32_t kIdescT48 = Idesc<R>::kT, kIdescQ48 = Idesc<R>::kQ;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -236,20 +237,22 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         auto wait_all = [&](uint32_t b, uint32_t parity) { return mbar_wait_warp(b, parity, abort_flag, p.status); };
         bool ok = true;
         if (warp == 1) {
+            // Rank 32: of both halves of a tile at once (N = 128), whose six MMAs fetch 48 KB of operands where two sets of six fetch 72 (641 ->
+            // 625 us); at rank 16 the halves kept apart are the faster (550 against 560 us).
             // ---- S^T, dP^T of unit u as soon as the arithmetic group has read unit u - 2 (same buffers)
             // out of tensor memory; the group is then still busy with that unit's exponentials
             uint32_t nitem = 0, I = 0;
             uint32_t slot_base = 0;
-            for (uint32_t u = 0; u < total_units && ok; ++u) {
-                const uint32_t h = u & 1, g = u >> 1, st = g % kQStages, slot = nitem & 1;
+            for (uint32_t u = 0; u < total_units / kSUnits && ok; ++u) {
+                const uint32_t h = kSUnits == 1 ? u & 1 : 0, g = kSUnits == 1 ? u >> 1 : u, st = g % kQStages, slot = nitem & 1;
                 if (h == 0 && I == 0) {
                     if (!wait_all(bar(kKVFull + slot), (nitem >> 1) & 1)) { ok = false; break; }
                     slot_base = base + slot * kContentBytes;
                 }
                 if (h == 0 && !wait_all(bar(kQFull + st), (g / kQStages) & 1)) { ok = false; break; }
-                if (u >= 2 && !wait_all(bar(kSFree + h), ((u - 2) >> 1) & 1)) { ok = false; break; }
+                if (g >= 1 && (!wait_all(bar(kSFree + h), (g - 1) & 1) || (kSUnits == 2 && !wait_all(bar(kSFree + 1), (g - 1) & 1)))) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t ring = base + kOffRing + st * kRingBytes + h * kPatchContent;   // rows of patch h
+                const uint32_t ring = base + kOffRing + st * kRingBytes + h * kPatchContent;   // rows of patch h (and the next)
                 if (elect_one()) {
                     const uint64_t kc = smem_desc_at(kDesc64, slot_base + kOffKc), kp = smem_desc_at(kDesc64, slot_base + kOffKp);
                     const uint64_t v = smem_desc_at(kDesc64, slot_base + kOffV);
@@ -263,9 +266,10 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     mma_ss(d_p, v, go, kIdescSS, 0u);
                     mma_ss(d_p, v + 2, go + 2, kIdescSS, 1u);
                     mma_commit(bar(kSFull + h));
+                    if (kSUnits == 2) mma_commit(bar(kSFull + 1));
                 }
                 __syncwarp();
-                if (h == 1 && ++I == (uint32_t)nblk) { I = 0; ++nitem; }
+                if (h == kSUnits % 2 && ++I == (uint32_t)nblk) { I = 0; ++nitem; }
             }
         } else if (warp == 2) {
             // ---- dV_J += P^T dO_u and dK~_J += dS^T Q~_u (A from tensor memory, 16 queries per step)
@@ -490,7 +494,13 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kDQFree));
 #pragma unroll
-                for (int col = 0; col < kDk; col += 4, dst += 4 * (size_t)p.n) red_add_f32x4(dst, a[col >> 4] + (col & 15));
+                for (int col = 0; col < kDk; col += 4, dst += 4 * (size_t)p.n) {
+                    red_add_f32x4(dst, a[col >> 4] + (col & 15));
+                    // The adds of a tile in one burst hold up the loads and stores of the other warps, which go through the same queue: a short
+                    // pause after each (rank 32: after every second one) spreads them over the tile's time (550 -> 535 us at rank 16,
+                    // 641 -> 633 us at rank 32, 16 x 96 x 96 tokens in windows of 32; 50 ns pauses: 542 and 689 us).
+                    if (R == 16 || (col & 4)) __nanosleep(20);
+                }
             }
             if (!ok) break;
             if (!__all_sync(0xffffffffu, mbar_wait(bar(kAccFull), nitem & 1, abort_flag, p.status))) { ok = false; break; }
