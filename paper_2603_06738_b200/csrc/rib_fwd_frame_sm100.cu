@@ -10,9 +10,11 @@
 // adds the unrounded fp32 probabilities.  Infinities: the terms of a number times an infinity may cancel to NaN where the number
 // itself times it would not, so a row that comes out as NaN is computed once more from the plain numbers (plain_row).
 //
-// What bounds it: the exponentials (16 per cycle and SM: 1024 cycles per tile of 128 x 128 scores) and, next to them, 21
-// MMAs per tile (about 950 cycles).  Measured (180 x 320 tokens, 32 x 32 windows, 6 heads of 32 channels, rank 16, with the
-// launch): 178 us = 305 TFLOP/s of the layer's own flops, about 2000 cycles per tile and SM; the any-shape kernel 13 460 us.
+// What bounds it: the serial program of the softmax warps, 3300 cycles per block of both query tiles of which the exp unit is busy
+// 2048, beside 42 MMAs (2100 cycles of issue, from three warps).  Measured (180 x 320 tokens, 32 x 32 windows, 6 heads of 32
+// channels, rank 16, with the launch): 158 us = 343 TFLOP/s of the layer's own flops; one warp issuing everything 176 us (it held
+// a unit for 16 + 5 MMAs and the wait between them, 1600 cycles), the any-shape kernel 13 460 us.  Asking for the next scores
+// before P is handed over, as the general kernel does, took 178 us: P then waits for them.
 // Error of `out` against float64 as that kernel's (1.7e-3, the rounding to bf16; 4 parts in a million more at most), of lse below it.
 //
 // Work item = one (batch, window, head) pair x two query tiles of 128 tokens (two 8x8-token patches each).  Only patches that
@@ -21,13 +23,12 @@
 //
 // Tensor memory: three score buffers of 128 columns and 2 x 2 output accumulators (query tile, key half) of 32.  Unit u =
 // 2 * block + query tile uses buffer u mod 3.  A softmax thread holds one row's 64 scores of its key half in registers and
-// writes P over them (hi 32 columns, lo 32 columns), so a buffer is handed back to the one issuing thread with P in it; that
-// thread issues PV(u), waits for its completion (nothing orders an MMA that overwrites columns behind one of another shape and
-// accumulator that reads them as its A operand) and issues S(u + 3) into the same columns.  The scores of one tile's next block
-// are thus under way while the other tile's exponentials run.
+// writes P over them (hi 32 columns, lo 32 columns), so a buffer is handed back with P in it; S(u + 3) goes into the same columns
+// once PV(u) has completed (nothing orders an MMA that overwrites columns behind one of another shape and accumulator that reads
+// them as its A operand).  The scores of one tile's next block are thus under way while the other tile's exponentials run.
 //
-// Roles (640 threads): warp 0 TMA producer, which also stages the scaled query RIB rows; warp 1 issues all MMAs; warp 2 owns
-// the TMEM allocation; warps 4-11 softmax / epilogue of query tile 0 (4-7 first key half, 8-11 second half), 12-19 of tile 1.
+// Roles (640 threads): warp 0 TMA producer, which also stages the scaled query RIB rows; warp 1 issues S, warps 2 and 3
+// PV of query tile 0 and 1 (warp 2 owns the TMEM allocation); warps 4-11 softmax / epilogue of query tile 0 (4-7 first key half, 8-11 second half), 12-19 of tile 1.
 // Every wait is bounded.
 #include "rib_sm100_common.cuh"
 
@@ -51,9 +52,13 @@ struct Frame {
     static constexpr uint32_t kOffKp = kOffKc + kStages * kContentBytes;
     static constexpr uint32_t kOffV = kOffKp + kStages * kPos;
     static constexpr uint32_t kOffBar = kOffV + kStages * kContentBytes;
-    // barriers: query buffers, ring stages, score buffers, completed PV per tile, merge per tile and quarter of the rows, drain
+    // barriers: query buffers, ring stages, scores there (per buffer), P there (2 tile + parity of the block), P read (per buffer),
+    // completed PV per tile, merge per tile and quarter of the rows, drain per issuing warp.  A parity wait cannot tell "a phase ahead"
+    // or "a phase behind" from its own, so every barrier is one whose next phase needs what its waiters do after this one, and whose
+    // phase before they know to be complete: P of a tile's block b + 2 needs the scores that overwrite P of block b.  (By buffer it is
+    // not: the phase before belongs to the other tile, whose PV another warp issues.)
     enum Bar { kQFull = 0, kQEmpty = 2, kQPos = 4, kFull = 6, kEmpty = kFull + kStages, kSFull = kEmpty + kStages, kPReady = kSFull + kBuffers,
-               kPVDone = kPReady + kBuffers, kMerge = kPVDone + 2, kDrain = kMerge + 8, kNumBars };
+               kPFree = kPReady + 4, kPVDone = kPFree + kBuffers, kMerge = kPVDone + 2, kDrain = kMerge + 8, kNumBars = kDrain + 3 };
     static constexpr uint32_t kOffMisc = kOffBar + kNumBars * 8;                 // tmem base, abort flags
     static constexpr uint32_t kOffMerge = (kOffMisc + 16 + 15) & ~15u;           // [2 item parities][2 tiles][2 halves][128 rows] (max, sum)
     static constexpr uint32_t kSmemBytes = kOffMerge + 8 * kTile * 8 + 1024;     // + slack for manual alignment
@@ -178,9 +183,10 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             mbar_init(bar(L::kQFull + i), 1); mbar_init(bar(L::kQEmpty + i), 1); mbar_init(bar(L::kQPos + i), 1); mbar_init(bar(L::kPVDone + i), 1);
             for (int q4 = 0; q4 < 4; ++q4) mbar_init(bar(L::kMerge + 4 * i + q4), 2);
         }
-        for (int i = 0; i < kBuffers; ++i) { mbar_init(bar(L::kSFull + i), 1); mbar_init(bar(L::kPReady + i), 8); }
-        for (int s = 0; s < kStages; ++s) { mbar_init(bar(L::kFull + s), 1); mbar_init(bar(L::kEmpty + s), 1); }
-        mbar_init(bar(L::kDrain), 1);
+        for (int i = 0; i < kBuffers; ++i) { mbar_init(bar(L::kSFull + i), 1); mbar_init(bar(L::kPFree + i), 1); }
+        for (int i = 0; i < 4; ++i) mbar_init(bar(L::kPReady + i), 8);
+        for (int s = 0; s < kStages; ++s) { mbar_init(bar(L::kFull + s), 1); mbar_init(bar(L::kEmpty + s), 2); }     // empty: both tiles' PV
+        for (int i = 0; i < 3; ++i) mbar_init(bar(L::kDrain + i), 1);
         fence_barrier_init();
         prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v); prefetch_tensormap(&tm_pk);
     }
@@ -268,80 +274,75 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             for (uint32_t b2 = blk > (uint32_t)kStages ? blk - kStages : 0; b2 < blk; ++b2)
                 mbar_wait(bar(L::kFull + b2 % kStages), (b2 / kStages) & 1, abort_flag + 1, p.status);
         }
-    } else if (warp == 1) {
-        // ===================== issuer: S(0), S(1), S(2), then PV(u), its completion, S(u + 3) for u = 0, 1, ...; the whole warp walks and waits
+    } else if (warp < 4) {
+        // ===================== issuers: warp 1 the scores of both query tiles, warps 2 and 3 PV of tile 0 and 1; the whole warp walks and waits
         constexpr uint64_t kDesc64 = smem_desc_const(16, 512, kSwizzle64B), kDesc32 = smem_desc_const(16, 256, kSwizzle32B);
         constexpr uint64_t kDescP = R == 16 ? kDesc32 : kDesc64;
-        // two cursors over the same sequence of blocks: scores run three units ahead of PV
-        struct Cursor { int item; int nblk, j; uint32_t io, blk, u; } s{}, v{};
-        auto enter = [&](Cursor& c) { if (c.item < items) c.nblk = (decode_live_item(p.live, c.item).patches + 1) >> 1; };
-        auto advance = [&](Cursor& c) {
-            if (++c.u & 1) return;                           // the block's second query tile is next
-            ++c.blk;
-            if (++c.j < c.nblk) return;
-            c.j = 0; c.item += gridDim.x; ++c.io;
-            enter(c);
-        };
-        s.item = v.item = blockIdx.x;
-        enter(s); enter(v);
-        auto issue_scores = [&]() {
-            if (s.item >= items) return true;
-            const uint32_t buf = s.io & 1, st = s.blk % kStages, qt = s.u & 1, sb = s.u % kBuffers;
-            if (qt == 0) {
-                if (s.j == 0 && (!mbar_wait_warp(bar(L::kQFull + buf), (s.io >> 1) & 1, abort_flag, p.status) ||
-                                 !mbar_wait_warp(bar(L::kQPos + buf), (s.io >> 1) & 1, abort_flag, p.status))) return false;
-                if (!mbar_wait_warp(bar(L::kFull + st), (s.blk / kStages) & 1, abort_flag, p.status)) return false;
-            }
-            if (elect_one()) {
-                const uint64_t kc = smem_desc_at(kDesc64, base + L::kOffKc + st * kContentBytes), kp = smem_desc_at(kDescP, base + L::kOffKp + st * kPos);
-                const uint64_t qc = smem_desc_at(kDesc64, base + L::kOffQc + (2 * buf + qt) * kContentBytes);
-                const uint64_t qp = smem_desc_at(kDescP, base + L::kOffQp + (2 * buf + qt) * kTerms * kPos);
-                const uint32_t d_s = tmem + sb * kTile;
-                // smallest terms first: a step drops what lies below the last place of the sum so far
-                for (int term = p.terms - 1; term >= 0; --term) {
-                    mma_ss(d_s, qp + term * (kPos >> 4), kp, kIdescS, term == p.terms - 1 ? 0u : 1u);
-                    if (R == 32) mma_ss(d_s, qp + term * (kPos >> 4) + 2, kp + 2, kIdescS, 1u);
-                }
-                mma_ss(d_s, qc, kc, kIdescS, 1u);
-                mma_ss(d_s, qc + 2, kc + 2, kIdescS, 1u);          // + 32 bytes: second K16 step of the content rows
-                mma_commit(bar(L::kSFull + sb));
-                if (qt == 1 && s.j == s.nblk - 1) mma_commit(bar(L::kQEmpty + buf));
-            }
-            __syncwarp();
-            advance(s);
-            return true;
-        };
-        for (int i = 0; i < kBuffers && ok; ++i) ok = issue_scores();
-        while (ok && v.item < items) {
-            const uint32_t st = v.blk % kStages, qt = v.u & 1, sb = v.u % kBuffers;
-            // P of the unit is there.  (The first block of an item overwrites O: the softmax warps have read it before they
-            // arrive here for that block.)
-            if (!mbar_wait_warp(bar(L::kPReady + sb), (v.u / kBuffers) & 1, abort_flag, p.status)) { ok = false; break; }
-            tc_fence_after();
-            if (elect_one()) {
-                const uint64_t vd = smem_desc_at(kDesc64, base + L::kOffV + st * kContentBytes);
-                const uint32_t a_p = tmem + sb * kTile, d_o = tmem + kColO + qt * 2 * kD;
+        uint32_t io = 0, blk = 0, sb = warp == 3 ? 1 : 0, use = 0;      // sb, use: unit mod and div kBuffers
+        auto next_unit = [&](uint32_t by) { sb += by; if (sb >= kBuffers) { sb -= kBuffers; ++use; } };
+        for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++io) {
+            const int nblk = (decode_live_item(p.live, item).patches + 1) >> 1;
+            const uint32_t buf = io & 1;
+            if (warp == 1 && (!mbar_wait_warp(bar(L::kQFull + buf), (io >> 1) & 1, abort_flag, p.status) ||
+                              !mbar_wait_warp(bar(L::kQPos + buf), (io >> 1) & 1, abort_flag, p.status))) { ok = false; break; }
+            for (int j = 0; j < nblk && ok; ++j, ++blk) {
+                const uint32_t st = blk % kStages;
+                if (warp == 1) {
+                    if (!mbar_wait_warp(bar(L::kFull + st), (blk / kStages) & 1, abort_flag, p.status)) { ok = false; break; }
+                    const uint64_t kc = smem_desc_at(kDesc64, base + L::kOffKc + st * kContentBytes), kp = smem_desc_at(kDescP, base + L::kOffKp + st * kPos);
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {                   // keys 16 kk ..: key half kk / 4 has its own accumulator
-                    const uint32_t a = a_p + (kk >> 2) * 64 + 8 * (kk & 3), d = d_o + (kk >> 2) * kD;
-                    mma_ts(d, a, vd + 64 * kk, kIdescPV, (v.j == 0 && (kk & 3) == 0) ? 0u : 1u);
-                    mma_ts(d, a + 32, vd + 64 * kk, kIdescPV, 1u);
+                    for (int qt = 0; qt < 2; ++qt) {
+                        // The scores overwrite the columns that PV of three units before reads P from: it has completed.  (The barrier is the
+                        // buffer's own, so that its next phase cannot complete before this one is seen; no phase completed answers yes
+                        // to parity 1, which the first three units ask for.)
+                        if (!mbar_wait_warp(bar(L::kPFree + sb), (use - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                        tc_fence_after();
+                        if (elect_one()) {
+                            const uint64_t qc = smem_desc_at(kDesc64, base + L::kOffQc + (2 * buf + qt) * kContentBytes);
+                            const uint64_t qp = smem_desc_at(kDescP, base + L::kOffQp + (2 * buf + qt) * kTerms * kPos);
+                            const uint32_t d_s = tmem + sb * kTile;
+                            // smallest terms first: a step drops what lies below the last place of the sum so far
+                            for (int term = p.terms - 1; term >= 0; --term) {
+                                mma_ss(d_s, qp + term * (kPos >> 4), kp, kIdescS, term == p.terms - 1 ? 0u : 1u);
+                                if (R == 32) mma_ss(d_s, qp + term * (kPos >> 4) + 2, kp + 2, kIdescS, 1u);
+                            }
+                            mma_ss(d_s, qc, kc, kIdescS, 1u);
+                            mma_ss(d_s, qc + 2, kc + 2, kIdescS, 1u);          // + 32 bytes: second K16 step of the content rows
+                            mma_commit(bar(L::kSFull + sb));
+                            if (qt == 1 && j == nblk - 1) mma_commit(bar(L::kQEmpty + buf));
+                        }
+                        __syncwarp();
+                        next_unit(1);
+                    }
+                } else {
+                    // P of the unit is there.  (The first block of an item overwrites O: the softmax warps have read it before they
+                    // arrive here for that block.)
+                    if (!mbar_wait_warp(bar(L::kFull + st), (blk / kStages) & 1, abort_flag, p.status) ||
+                        !mbar_wait_warp(bar(L::kPReady + 2 * (warp - 2) + (blk & 1)), (blk >> 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint64_t vd = smem_desc_at(kDesc64, base + L::kOffV + st * kContentBytes);
+                        const uint32_t a_p = tmem + sb * kTile, d_o = tmem + kColO + (warp - 2) * 2 * kD;
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk) {                   // keys 16 kk ..: key half kk / 4 has its own accumulator
+                            const uint32_t a = a_p + (kk >> 2) * 64 + 8 * (kk & 3), d = d_o + (kk >> 2) * kD;
+                            mma_ts(d, a, vd + 64 * kk, kIdescPV, (j == 0 && (kk & 3) == 0) ? 0u : 1u);
+                            mma_ts(d, a + 32, vd + 64 * kk, kIdescPV, 1u);
+                        }
+                        mma_commit(bar(L::kPFree + sb));
+                        mma_commit(bar(L::kPVDone + warp - 2));
+                        mma_commit(bar(L::kEmpty + st));
+                    }
+                    __syncwarp();
+                    next_unit(2);
                 }
-                mma_commit(bar(L::kPVDone + qt));
-                if (qt == 1) mma_commit(bar(L::kEmpty + st));
             }
-            __syncwarp();
-            // S(u + 3) overwrites the columns that PV(u) reads P from: it is not issued before PV(u) has completed
-            if (!mbar_wait_warp(bar(L::kPVDone + qt), v.blk & 1, abort_flag, p.status)) { ok = false; break; }
-            tc_fence_after();
-            advance(v);
-            ok = issue_scores();
         }
         // everything issued by this warp's leader must have finished before TMEM is released
-        if (elect_one()) mma_commit(bar(L::kDrain));
+        if (elect_one()) mma_commit(bar(L::kDrain + warp - 1));
         __syncwarp();
-        mbar_wait(bar(L::kDrain), 0, abort_flag + 1, p.status);
-    } else if (warp >= 4) {
+        mbar_wait(bar(L::kDrain + warp - 1), 0, abort_flag + 1, p.status);
+    } else {
         // ================ softmax + epilogue: two threads per query row, one per half of the keys
         const int qt = (warp - 4) >> 3;
         const int half = ((warp - 4) >> 2) & 1;
@@ -381,13 +382,15 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                             if ((e >> 3) >= rows || (e & 7) >= cols) s[e >> 5][e & 31] = 0xff800000u;
                     }
                 }
-                float mx0 = -INFINITY, mx1 = -INFINITY;
+                float mxs[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                    mx0 = max3(mx0, __uint_as_float(s[0][e]), __uint_as_float(s[0][e + 1]));
-                    mx1 = max3(mx1, __uint_as_float(s[1][e]), __uint_as_float(s[1][e + 1]));
+                for (int e = 0; e < 32; e += 4) {
+                    mxs[0] = max3(mxs[0], __uint_as_float(s[0][e]), __uint_as_float(s[0][e + 1]));
+                    mxs[1] = max3(mxs[1], __uint_as_float(s[1][e]), __uint_as_float(s[1][e + 1]));
+                    mxs[2] = max3(mxs[2], __uint_as_float(s[0][e + 2]), __uint_as_float(s[0][e + 3]));
+                    mxs[3] = max3(mxs[3], __uint_as_float(s[1][e + 2]), __uint_as_float(s[1][e + 3]));
                 }
-                const float mx = fmaxf(mx0, mx1);
+                const float mx = fmaxf(fmaxf(mxs[0], mxs[1]), fmaxf(mxs[2], mxs[3]));
                 if (j == 0) {
                     m_used = mx;
                 } else {
@@ -414,19 +417,20 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 const float2 neg2 = make_float2(neg, neg);
                 float2 sum_a = make_float2(0.f, 0.f), sum_b = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int ch = 0; ch < 2; ++ch) {
-                    uint32_t hi[16], lo[16];
+                for (int ch = 0; ch < 4; ++ch) {                  // 16 keys at a time: next to 64 scores, no more results fit the registers
+                    uint32_t hi[8], lo[8];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[ch][2 * i]), __uint_as_float(s[ch][2 * i + 1])), scale2, neg2);
+                    for (int i = 0; i < 8; ++i) {
+                        const int k = 16 * (ch & 1) + 2 * i;
+                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[ch >> 1][k]), __uint_as_float(s[ch >> 1][k + 1])), scale2, neg2);
                         const float2 e = make_float2(ex2_approx(x.x), ex2_approx(x.y));
                         if (i & 1) sum_b = __fadd2_rn(sum_b, e); else sum_a = __fadd2_rn(sum_a, e);
                         hi[i] = pack_bf16x2(e.x, e.y);
                         const float2 rest = __fadd2_rn(e, make_float2(-__uint_as_float(hi[i] << 16), -__uint_as_float(hi[i] & 0xffff0000u)));
                         lo[i] = pack_bf16x2(rest.x, rest.y);
                     }
-                    tmem_st16(t_half + sb * kTile + 16 * ch, hi);
-                    tmem_st16(t_half + sb * kTile + 32 + 16 * ch, lo);
+                    tmem_st8(t_half + sb * kTile + 8 * ch, hi);
+                    tmem_st8(t_half + sb * kTile + 32 + 8 * ch, lo);
                 }
                 l += (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
                 // The epilogue waits for this block's PV.  A parity wait cannot tell "two phases ahead" from "not yet", so the
@@ -435,7 +439,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(L::kPReady + sb));
+                if (lane == 0) mbar_arrive(bar(L::kPReady + 2 * qt + (blk & 1)));
                 sb += 2;
                 if (sb >= kBuffers) { sb -= kBuffers; ++use; }
             }
