@@ -567,6 +567,7 @@ struct AuxParams {
     float* dpk;
     int H, W, heads, M, s, n, nWy, nWx, pairs;
     int d, r;                    // head width and rank of the caller's tensors (the accumulators are 32 + R columns wide)
+    int narrow;                  // kNarrow: width of the rows of out and dq (even, less than d)
     int Hp, Wp;                  // sides of the extended map (equal to H, W when they are multiples of the window)
     int tables;                  // Pq/Pk tables: 1 (shared by the heads) or heads
     long long pos_head_stride;   // elements between the tables in pq, dpq, dpk (pq_scaled is packed: n * 16 apart)
@@ -590,7 +591,8 @@ __device__ __forceinline__ bool decode_pair_token(const AuxParams& p, int pair, 
 // One thread per (pair, token in window order): D = dO . O and lse in the layout the main kernel
 // streams; the dQ~ accumulators are cleared with 16-byte stores, (d + r) / 4 per thread, as one flat array;
 // the first threads also stage bf16(Pq sqrt(d/r)) and clear dPq, dPk.
-template <int R>
+// kNarrow: the rows of out are p.narrow < d elements wide and aligned to 4 bytes only.
+template <int R, bool kNarrow>
 __global__ void __launch_bounds__(256) rib_bwd_prepare_kernel(const AuxParams p)
 {
     constexpr int kDk = kD + R;
@@ -625,14 +627,25 @@ __global__ void __launch_bounds__(256) rib_bwd_prepare_kernel(const AuxParams p)
         return;
     }
     const uint4* a = reinterpret_cast<const uint4*>(p.dout + tok * p.d);
-    const uint4* b = reinterpret_cast<const uint4*>(p.out + tok * p.d);
+    const uint4* b = reinterpret_cast<const uint4*>(p.out + tok * (kNarrow ? p.narrow : p.d));
     float acc = 0.f;
 #pragma unroll
     for (int q4 = 0; q4 < 4; ++q4) {
         // (predicated, not a break: the loads of all four pieces are in flight together)
         const bool on = 8 * q4 < p.d;
         const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-        const uint4 x = on ? __ldg(a + q4) : zero, y = on ? __ldg(b + q4) : zero;
+        const uint4 x = on ? __ldg(a + q4) : zero;
+        uint4 y = zero;
+        if (kNarrow) {
+            const uint32_t* w = reinterpret_cast<const uint32_t*>(b) + 4 * q4;
+            const int left = p.narrow - 8 * q4;
+            if (left > 0) y.x = __ldg(w);
+            if (left > 2) y.y = __ldg(w + 1);
+            if (left > 4) y.z = __ldg(w + 2);
+            if (left > 6) y.w = __ldg(w + 3);
+        } else if (on) {
+            y = __ldg(b + q4);
+        }
         const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -656,7 +669,7 @@ __global__ void __launch_bounds__(256) rib_bwd_prepare_kernel(const AuxParams p)
 // piece of dQ~[:, :d] / sqrt(d) into bf16, and it keeps running sums of its RIB columns of dQ~ (-> dPq, times
 // 1/sqrt(r)) and of dK~ (-> dPk); the group's sums go to the zeroed results with one vector atomic each (these
 // adds all land on the same n x r addresses: a group is long enough that their number does not set the time).
-template <int R>
+template <int R, bool kNarrow>       // kNarrow: the rows of dq are p.narrow < d elements wide
 __global__ void __launch_bounds__(128, 8) rib_bwd_finish_kernel(const AuxParams p, int pairs_per_group)
 {
     constexpr int kDk = kD + R;
@@ -690,8 +703,17 @@ __global__ void __launch_bounds__(128, 8) rib_bwd_finish_kernel(const AuxParams 
         const float4 gq = src[(size_t)((kD + col0) / 4) * p.n], gk = srk[(size_t)(col0 / 4) * p.n];
         if (piece) {
             const float f = p.inv_sqrt_d;
-            reinterpret_cast<uint4*>(p.dq + tok * p.d)[cg] =
-                make_uint4(pack_bf16x2(f0.x * f, f0.y * f), pack_bf16x2(f0.z * f, f0.w * f), pack_bf16x2(f1.x * f, f1.y * f), pack_bf16x2(f1.z * f, f1.w * f));
+            const uint4 v = make_uint4(pack_bf16x2(f0.x * f, f0.y * f), pack_bf16x2(f0.z * f, f0.w * f), pack_bf16x2(f1.x * f, f1.y * f), pack_bf16x2(f1.z * f, f1.w * f));
+            if (kNarrow) {
+                uint32_t* w = reinterpret_cast<uint32_t*>(p.dq + tok * p.narrow) + 4 * cg;
+                const int left = p.narrow - 8 * cg;
+                if (left > 0) w[0] = v.x;
+                if (left > 2) w[1] = v.y;
+                if (left > 4) w[2] = v.z;
+                if (left > 6) w[3] = v.w;
+            } else {
+                reinterpret_cast<uint4*>(p.dq + tok * p.d)[cg] = v;
+            }
         }
         sq[0] += gq.x; sq[1] += gq.y; sq[2] += gq.z; sq[3] += gq.w;
         sk[0] += gk.x; sk[1] += gk.y; sk[2] += gk.z; sk[3] += gk.w;
@@ -758,7 +780,7 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     ap.H = p.H; ap.W = p.W; ap.heads = p.heads; ap.M = p.M; ap.s = p.s; ap.n = p.n; ap.nWy = p.nWy; ap.nWx = p.nWx;
     ap.Hp = p.Hp; ap.Wp = p.Wp;
     ap.pairs = p.pairs;
-    ap.d = p.d; ap.r = p.r;
+    ap.d = p.d; ap.r = p.r; ap.narrow = p.narrow;
     ap.tables = tables;
     ap.pos_head_stride = p.pos_head_stride;
     ap.pos_scale = sqrtf(scale_width_d(p) / scale_width_r(p));
@@ -766,7 +788,7 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     ap.inv_sqrt_r = 1.f / sqrtf(scale_width_r(p));
     const size_t tokens = (size_t)p.pairs * p.n;
     const unsigned aux_blocks = (unsigned)((tokens + 255) / 256);
-    { ProfileScope scope(RIB_KERNEL_BWD_PREPARE, stream); rib_bwd_prepare_kernel<R><<<aux_blocks, 256, 0, stream>>>(ap); }
+    { ProfileScope scope(RIB_KERNEL_BWD_PREPARE, stream); (p.narrow ? rib_bwd_prepare_kernel<R, true> : rib_bwd_prepare_kernel<R, false>)<<<aux_blocks, 256, 0, stream>>>(ap); }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
 
@@ -794,9 +816,11 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     const int per_group = in_line >= 1024 ? 8 : in_line >= 16 ? 4 : 1;
     const unsigned groups = (tables == 1 ? 1u : (unsigned)p.heads) * (unsigned)((in_line + per_group - 1) / per_group);
     dim3 grid_fin((unsigned)(p.n / 32), groups, (unsigned)(R / 16));
-    { ProfileScope scope(RIB_KERNEL_BWD_FINISH, stream); rib_bwd_finish_kernel<R><<<grid_fin, 128, 0, stream>>>(ap, per_group); }
+    { ProfileScope scope(RIB_KERNEL_BWD_FINISH, stream); (p.narrow ? rib_bwd_finish_kernel<R, true> : rib_bwd_finish_kernel<R, false>)<<<grid_fin, 128, 0, stream>>>(ap, per_group); }
     return cudaGetLastError();
 }
+
+bool sm100_bwd_takes_narrow(const Problem& p) { return !sm100_window8(p) && !sm100_window16(p); }
 
 int sm100_bwd_launches(const Problem& p) { return sm100_window8(p) ? 2 : 3; }      // clear, main; else two clears, main or prepare, main, finish
 

@@ -41,6 +41,7 @@ struct Problem {
     bool masked;                      // shifted windows: the wrapped parts of a border window do not attend to each other
     int d_true, r_true;               // tcgen05 kernels on zero-padded copies (rib_repack.cu): the widths the scales 1/sqrt(d),
                                       // 1/sqrt(r) are taken from; 0 = d, r themselves
+    int narrow;                       // general tcgen05 backward on such copies: width of the rows of `out` and `dq`, which are the caller's; 0 = d
 };
 
 // Pq/Pk tables: one shared by the heads, or one per head (Sec. 3.1, after Eq. 3: head-wise projections of the shared h).
@@ -69,6 +70,7 @@ bool sm100_bwd_supported(const Problem& p);
 size_t sm100_bwd_workspace_bytes(long long pairs, int n, int tables, int r);
 cudaError_t sm100_bwd(const Problem& p, cudaStream_t stream);
 int sm100_bwd_launches(const Problem& p);     // kernels it enqueues
+bool sm100_bwd_takes_narrow(const Problem& p);    // Problem::narrow may be set
 // Windows of 8 x 8 tokens (rib_window8_sm100.cu); the backward launches 2 kernels.
 bool sm100_window8(const Problem& p);
 cudaError_t sm100_window8_fwd(const Problem& p, cudaStream_t stream);

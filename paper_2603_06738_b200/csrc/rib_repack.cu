@@ -2,7 +2,7 @@
 // r = 18 gives 36-byte rows -- the SST rows of the paper's network table).  For even d, r <= 32 the tensors are copied
 // into scratch with every row filled up with zeros to the next multiple of 8 elements, the tcgen05 kernels run on the
 // copies (zero channels change no dot product; the scales of Eq. 6 keep the true d and r), and the results are copied
-// back.  The scratch comes from a stream-ordered memory pool of the library's own, one per device, that keeps what is
+// back, all copies of a pass in one launch.  The scratch comes from a stream-ordered memory pool of the library's own, one per device, that keeps what is
 // freed (cudaMallocFromPoolAsync / cudaFreeAsync on the caller's stream): after the first call of a shape nothing here
 // talks to the driver's allocator and nothing synchronises.  The attention passes are bound by arithmetic, so the copies (a few hundred bytes per
 // token-head) cost little next to them; the any-shape kernels these shapes would otherwise take are about a hundred
@@ -113,50 +113,83 @@ __global__ void __launch_bounds__(256) rib_rank_tail_grads_kernel(const __nv_bfl
     }
 }
 
-// The image tensors (rows of bf16, widths in 4-byte words; the wide side is a multiple of 4 words): a thread moves one
-// 16-byte piece of the wide side, which is one vector access there and up to four word accesses on the narrow side.
-// kWiden: narrow src -> wide dst with zeros behind; else wide src -> narrow dst.
-template <bool kWiden>
-__global__ void __launch_bounds__(256) rib_resize_rows_kernel(const uint32_t* __restrict__ src, uint32_t* __restrict__ dst, int narrow, int wide,
-                                                             unsigned rows)
-{
-    const unsigned per_row = (unsigned)wide / 4u, total = rows * per_row;
-    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
-        const unsigned row = e / per_row, piece = e - row * per_row;
-        const int w0 = 4 * (int)piece;
-        if (kWiden) {
-            const uint32_t* in = src + (size_t)row * narrow + w0;
-            uint32_t v[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] = w0 + k < narrow ? in[k] : 0u;
-            *reinterpret_cast<uint4*>(dst + (size_t)row * wide + w0) = make_uint4(v[0], v[1], v[2], v[3]);
-        } else {
-            const uint4 v = *reinterpret_cast<const uint4*>(src + (size_t)row * wide + w0);
-            uint32_t* out = dst + (size_t)row * narrow + w0;
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (w0 + k < narrow) out[k] = w[k];
-        }
+// All copies of a pass in one launch.  A copy: rows of 4-byte words, one side `wide` words a row (a multiple of 4, 16-byte aligned),
+// the other `narrow`; widen: narrow to wide with zeros behind, else wide to narrow.  A thread moves 16-byte pieces of the wide side,
+// which is one vector access there and up to four word accesses on the narrow side; a block 1024 of them, all loads of a thread
+// before its stores.
+struct RowCopy { const uint32_t* src; uint32_t* dst; size_t rows; unsigned first_block; int narrow, wide, widen; };
+constexpr int kMostCopies = 8, kCopyPieces = 4;
+struct RowCopies {
+    RowCopy copy[kMostCopies];
+    int count;
+    unsigned blocks;
+    // src rows of ws words -> dst rows of wd words
+    void add(const void* src, int ws, void* dst, int wd, size_t rows)
+    {
+        RowCopy& c = copy[count++];
+        c.src = static_cast<const uint32_t*>(src); c.dst = static_cast<uint32_t*>(dst); c.rows = rows;
+        c.widen = wd >= ws; c.wide = c.widen ? wd : ws; c.narrow = c.widen ? ws : wd;
+        c.first_block = blocks;
+        blocks += (unsigned)((rows * (size_t)(c.wide / 4) + 256 * kCopyPieces - 1) / (256 * kCopyPieces));
     }
+};
+
+__global__ void __launch_bounds__(256) rib_copy_rows_kernel(const __grid_constant__ RowCopies all)
+{
+    int which = 0;
+    while (which + 1 < all.count && blockIdx.x >= all.copy[which + 1].first_block) ++which;
+    const RowCopy& c = all.copy[which];
+    const unsigned per_row = (unsigned)c.wide / 4u;
+    const size_t piece0 = (size_t)(blockIdx.x - c.first_block) * (256 * kCopyPieces), row0 = piece0 / per_row;
+    const unsigned rem = (unsigned)(piece0 - row0 * per_row) + threadIdx.x;
+    uint4 v[kCopyPieces];
+    auto place = [&](int k, size_t& row, int& w0) {
+        const unsigned at = rem + 256u * k, r = at / per_row;
+        row = row0 + r;
+        w0 = 4 * (int)(at - r * per_row);
+        return row < c.rows;
+    };
+#pragma unroll
+    for (int k = 0; k < kCopyPieces; ++k) {
+        size_t row;
+        int w0;
+        v[k] = make_uint4(0u, 0u, 0u, 0u);
+        if (!place(k, row, w0)) continue;
+        if (!c.widen) { v[k] = *reinterpret_cast<const uint4*>(c.src + row * c.wide + w0); continue; }
+        const uint32_t* in = c.src + row * c.narrow + w0;
+        if (w0 < c.narrow) v[k].x = in[0];
+        if (w0 + 1 < c.narrow) v[k].y = in[1];
+        if (w0 + 2 < c.narrow) v[k].z = in[2];
+        if (w0 + 3 < c.narrow) v[k].w = in[3];
+    }
+#pragma unroll
+    for (int k = 0; k < kCopyPieces; ++k) {
+        size_t row;
+        int w0;
+        if (!place(k, row, w0)) continue;
+        if (c.widen) { *reinterpret_cast<uint4*>(c.dst + row * c.wide + w0) = v[k]; continue; }
+        uint32_t* out = c.dst + row * c.narrow + w0;
+        if (w0 < c.narrow) out[0] = v[k].x;
+        if (w0 + 1 < c.narrow) out[1] = v[k].y;
+        if (w0 + 2 < c.narrow) out[2] = v[k].z;
+        if (w0 + 3 < c.narrow) out[3] = v[k].w;
+    }
+}
+
+cudaError_t run_copies(const RowCopies& all, cudaStream_t stream, int* launches)
+{
+    if (!all.blocks) return cudaSuccess;
+    rib_copy_rows_kernel<<<all.blocks, 256, 0, stream>>>(all);
+    ++*launches;
+    return cudaGetLastError();
 }
 
 // bf16 image rows of `ws` elements -> rows of `wd` elements (one of the two a multiple of 8, the other smaller or equal)
 cudaError_t resize_rows(const void* src, int ws, void* dst, int wd, size_t rows, cudaStream_t stream, int* launches)
 {
-    const int wide = (ws > wd ? ws : wd) / 2, narrow = (ws > wd ? wd : ws) / 2;      // words
-    const size_t chunk = (size_t)0x7fffffff / (size_t)wide;
-    for (size_t r0 = 0; r0 < rows; r0 += chunk) {
-        const size_t nrows = rows - r0 < chunk ? rows - r0 : chunk, total = nrows * (size_t)(wide / 4);
-        const unsigned blocks = (unsigned)((total + 255) / 256 < 148 * 32 ? (total + 255) / 256 : 148 * 32);
-        const uint32_t* s32 = static_cast<const uint32_t*>(src) + r0 * (size_t)(ws / 2);
-        uint32_t* d32 = static_cast<uint32_t*>(dst) + r0 * (size_t)(wd / 2);
-        if (wd >= ws) rib_resize_rows_kernel<true><<<blocks, 256, 0, stream>>>(s32, d32, narrow, wide, (unsigned)nrows);
-        else rib_resize_rows_kernel<false><<<blocks, 256, 0, stream>>>(s32, d32, narrow, wide, (unsigned)nrows);
-        ++*launches;
-        if (cudaError_t e = cudaGetLastError()) return e;
-    }
-    return cudaSuccess;
+    RowCopies one{};
+    one.add(src, ws / 2, dst, wd / 2, rows);
+    return run_copies(one, stream, launches);
 }
 
 template <typename T>
@@ -210,21 +243,34 @@ Problem padded_shape(const Problem& p)
     return pp;
 }
 
-// q and k into their padded copies; with a rank above 32 the tail of the tables rides in the spare channels
-cudaError_t pack_qk(const Problem& p, const __nv_bfloat16* q, __nv_bfloat16* q2, const __nv_bfloat16* k, __nv_bfloat16* k2, size_t rows,
-                    cudaStream_t stream, int* launches)
+// the tables lie behind one another, their rows no wider than the copies': they are one copy
+bool tables_in_a_row(const Problem& p) { return !rank_tail(p) && (!p.pos_head_stride || p.pos_head_stride == (long long)p.n * p.r); }
+
+// q, k and the tables into their padded copies: what is a plain copy is added to `copies`; with a rank above 32 the tail of the tables
+// rides in the spare channels
+cudaError_t pack(const Problem& p, __nv_bfloat16* q2, __nv_bfloat16* k2, __nv_bfloat16* pq2, __nv_bfloat16* pk2, int rp, size_t rows, RowCopies* copies,
+                 cudaStream_t stream, int* launches)
 {
-    const int dp = repacked_width(p.d);
+    const int dp = repacked_width(p.d), tables = pos_tables(p);
+    if (tables_in_a_row(p)) {
+        copies->add(p.pq, p.r / 2, pq2, rp / 2, (size_t)tables * p.n);
+        copies->add(p.pk, p.r / 2, pk2, rp / 2, (size_t)tables * p.n);
+    } else {
+        const long long stride = (long long)p.n * rp;
+        if (cudaError_t e = copy_tables<uint32_t>(p.pq, p.pos_head_stride, p.r, pq2, stride, rp, tables, p.n, stream, launches)) return e;
+        if (cudaError_t e = copy_tables<uint32_t>(p.pk, p.pos_head_stride, p.r, pk2, stride, rp, tables, p.n, stream, launches)) return e;
+    }
     if (!rank_tail(p)) {
-        if (cudaError_t e = resize_rows(q, p.d, q2, dp, rows, stream, launches)) return e;
-        return resize_rows(k, p.d, k2, dp, rows, stream, launches);
+        copies->add(p.q, p.d / 2, q2, dp / 2, rows);
+        copies->add(p.k, p.d / 2, k2, dp / 2, rows);
+        return cudaSuccess;
     }
     PlaceGeom g = place_geom(p);
     const size_t total = rows * (size_t)(dp / 2);
     const unsigned blocks = (unsigned)((total + 255) / 256 < 148 * 16 ? (total + 255) / 256 : 148 * 16);
-    rib_pack_with_rank_tail_kernel<<<blocks, 256, 0, stream>>>(reinterpret_cast<const uint32_t*>(q), reinterpret_cast<uint32_t*>(q2), p.pq, g, (unsigned)rows);
+    rib_pack_with_rank_tail_kernel<<<blocks, 256, 0, stream>>>(reinterpret_cast<const uint32_t*>(p.q), reinterpret_cast<uint32_t*>(q2), p.pq, g, (unsigned)rows);
     g.scale = 1.f;
-    rib_pack_with_rank_tail_kernel<<<blocks, 256, 0, stream>>>(reinterpret_cast<const uint32_t*>(k), reinterpret_cast<uint32_t*>(k2), p.pk, g, (unsigned)rows);
+    rib_pack_with_rank_tail_kernel<<<blocks, 256, 0, stream>>>(reinterpret_cast<const uint32_t*>(p.k), reinterpret_cast<uint32_t*>(k2), p.pk, g, (unsigned)rows);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -268,12 +314,11 @@ cudaError_t sm100_fwd_repacked(const Problem& p, cudaStream_t stream, int* launc
     __nv_bfloat16* g2 = reinterpret_cast<__nv_bfloat16*>(buf + 4 * img);          // the CLA gate, if any (layout of out)
     __nv_bfloat16* pq2 = reinterpret_cast<__nv_bfloat16*>(buf + 5 * img);
     __nv_bfloat16* pk2 = reinterpret_cast<__nv_bfloat16*>(buf + 5 * img + tab);
-    const long long tstride = (long long)p.n * pp.r;
-    cudaError_t e = pack_qk(p, p.q, q2, p.k, k2, rows, stream, launches);
-    if (!e) e = resize_rows(p.v, p.d, v2, pp.d, rows, stream, launches);
-    if (!e && p.gate) { e = resize_rows(p.gate, p.d, g2, pp.d, rows, stream, launches); pp.gate = g2; }
-    if (!e) e = copy_tables<uint32_t>(p.pq, p.pos_head_stride, p.r, pq2, tstride, pp.r, tables, p.n, stream, launches);
-    if (!e) e = copy_tables<uint32_t>(p.pk, p.pos_head_stride, p.r, pk2, tstride, pp.r, tables, p.n, stream, launches);
+    RowCopies in{};
+    cudaError_t e = pack(p, q2, k2, pq2, pk2, pp.r, rows, &in, stream, launches);
+    in.add(p.v, p.d / 2, v2, pp.d / 2, rows);
+    if (p.gate) { in.add(p.gate, p.d / 2, g2, pp.d / 2, rows); pp.gate = g2; }
+    if (!e) e = run_copies(in, stream, launches);
     if (!e) {
         pp.q = q2; pp.k = k2; pp.v = v2; pp.pq = pq2; pp.pk = pk2; pp.out_w = o2;
         e = sm100_frame_supported(pp) ? sm100_fwd_frame(pp, stream) : sm100_fwd(pp, stream);
@@ -300,24 +345,37 @@ cudaError_t sm100_bwd_repacked(const Problem& p, cudaStream_t stream, int* launc
     float* dpq2 = reinterpret_cast<float*>(buf + 8 * img + 2 * tab);
     float* dpk2 = reinterpret_cast<float*>(buf + 8 * img + 2 * tab + gtab);
     const long long tstride = (long long)p.n * pp.r;
-    const __nv_bfloat16* ins[5] = {p.q, p.k, p.v, p.out, p.dout};
-    cudaError_t e = cudaSuccess;
-    e = pack_qk(p, p.q, image(0), p.k, image(1), rows, stream, launches);
-    for (int i = 2; i < 5 && !e; ++i) e = resize_rows(ins[i], p.d, image(i), pp.d, rows, stream, launches);
-    if (!e) e = copy_tables<uint32_t>(p.pq, p.pos_head_stride, p.r, pq2, tstride, pp.r, tables, p.n, stream, launches);
-    if (!e) e = copy_tables<uint32_t>(p.pk, p.pos_head_stride, p.r, pk2, tstride, pp.r, tables, p.n, stream, launches);
+    // The preparation kernel reads out, and the finishing kernel writes dq, in rows of the caller's width (those of the general kernel,
+    // where no columns of the tables travel in the spare channels): two copies less.  (8 x 96 x 96 tokens, 30 channels, rank 18, windows
+    // of 32: all copies of both passes 160 -> 80 us with one launch per pass, the two kernels 87 -> 105 us; both passes 721 -> 660 us.
+    // The drain warps of the main kernel have no registers left to write dk and dv so.)
+    const bool direct = sm100_bwd_takes_narrow(pp) && !rank_tail(p);
+    pp.narrow = direct && p.d % 8 ? p.d : 0;
+    RowCopies in{};
+    cudaError_t e = pack(p, image(0), image(1), pq2, pk2, pp.r, rows, &in, stream, launches);
+    in.add(p.v, p.d / 2, image(2), pp.d / 2, rows);
+    in.add(p.dout, p.d / 2, image(4), pp.d / 2, rows);
+    if (!direct) in.add(p.out, p.d / 2, image(3), pp.d / 2, rows);
+    if (!e) e = run_copies(in, stream, launches);
     if (!e) {
-        pp.q = image(0); pp.k = image(1); pp.v = image(2); pp.out = image(3); pp.dout = image(4);
-        pp.dq = image(5); pp.dk = image(6); pp.dv = image(7);
+        pp.q = image(0); pp.k = image(1); pp.v = image(2); pp.out = direct ? p.out : image(3); pp.dout = image(4);
+        pp.dq = direct ? p.dq : image(5); pp.dk = image(6); pp.dv = image(7);
         pp.pq = pq2; pp.pk = pk2; pp.dpq = dpq2; pp.dpk = dpk2;
         e = sm100_bwd(pp, stream);
         *launches += sm100_bwd_launches(pp);
     }
-    __nv_bfloat16* outs[3] = {p.dq, p.dk, p.dv};
-    for (int i = 0; i < 3 && !e; ++i) e = resize_rows(image(5 + i), pp.d, outs[i], p.d, rows, stream, launches);
-    const long long ustride = p.pos_head_stride ? p.pos_head_stride : 0;
-    if (!e) e = copy_tables<float2>(dpq2, tstride, pp.r, p.dpq, ustride, p.r, tables, p.n, stream, launches);
-    if (!e) e = copy_tables<float2>(dpk2, tstride, pp.r, p.dpk, ustride, p.r, tables, p.n, stream, launches);
+    RowCopies back{};
+    if (!direct) back.add(image(5), pp.d / 2, p.dq, p.d / 2, rows);
+    back.add(image(6), pp.d / 2, p.dk, p.d / 2, rows);
+    back.add(image(7), pp.d / 2, p.dv, p.d / 2, rows);
+    if (tables_in_a_row(p)) {
+        back.add(dpq2, pp.r, p.dpq, p.r, (size_t)tables * p.n);
+        back.add(dpk2, pp.r, p.dpk, p.r, (size_t)tables * p.n);
+    } else {
+        if (!e) e = copy_tables<float2>(dpq2, tstride, pp.r, p.dpq, p.pos_head_stride, p.r, tables, p.n, stream, launches);
+        if (!e) e = copy_tables<float2>(dpk2, tstride, pp.r, p.dpk, p.pos_head_stride, p.r, tables, p.n, stream, launches);
+    }
+    if (!e) e = run_copies(back, stream, launches);
     if (!e && rank_tail(p)) {
         // (the copies above have cleared the columns from 32 on: the tail's gradients are summed into them)
         const PlaceGeom g = place_geom(p);
