@@ -12,6 +12,13 @@ from pathlib import Path
 
 import torch
 
+try:
+    # The checks, allocations and the C call of the hot entry points in native code (csrc/rib_marshal.cpp).  It answers None for
+    # arguments that are not plain tensors of the right kind, and the Python form below takes over.
+    from . import _rib_marshal as _marshal
+except ImportError:         # not built, or built for another torch
+    _marshal = None
+
 _LIB_PATH = Path(__file__).resolve().parent / "librib_window_attn.so"
 _lib = None
 
@@ -127,8 +134,17 @@ def library() -> ctypes.CDLL:
         lib.rib_wait_probe.argtypes = [ctypes.c_ulonglong, vp]
         lib.rib_exp_probe.restype = ctypes.c_longlong
         lib.rib_exp_probe.argtypes = [vp, ci, ci, vp]
+        lib.rib_addresses = {name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in EXPORTS}
         _lib = lib
     return _lib
+
+
+def _native(call, entry, *args):
+    """The results of a call through the native marshaller, or None: the caller then goes on in Python."""
+    got = call((_lib or library()).rib_addresses[entry], *args)
+    if type(got) is int:
+        raise RibError(got)
+    return got
 
 
 def _stream_ptr(stream) -> int:
@@ -222,6 +238,10 @@ def rib_window_attn_bwd_workspace(B, H, W, heads, d, r, window) -> int:
 
 def rib_window_attn_fwd(q, k, v, pq, pk, window, shift=0, out=None, lse=None, stream=None, want_lse=True):
     """Enqueue the forward pass; returns (out bf16 [B,H,W,heads,d], lse fp32 [B,heads,H,W] or None)."""
+    if _marshal is not None and out is None and lse is None:
+        got = _native(_marshal.fwd, "rib_window_attn_fwd_headwise", q, k, v, pq, pk, 1, window, shift, want_lse, stream)
+        if got is not None:
+            return got
     _check_image("q", q)
     B, H, W, heads, d = q.shape
     _check_image("k", k, q.shape)
@@ -243,6 +263,10 @@ def rib_window_attn_fwd(q, k, v, pq, pk, window, shift=0, out=None, lse=None, st
 
 def rib_window_attn_bwd(q, k, v, pq, pk, out, lse, dout, window, shift=0, workspace=None, stream=None):
     """Enqueue the backward pass; returns (dq, dk, dv bf16, dpq, dpk fp32 [n,r])."""
+    if _marshal is not None and workspace is not None:
+        got = _native(_marshal.bwd, "rib_window_attn_bwd_headwise", q, k, v, pq, pk, out, lse, dout, 1, window, shift, workspace, stream)
+        if got is not None:
+            return got
     _check_image("q", q)
     B, H, W, heads, d = q.shape
     for name, t in (("k", k), ("v", v), ("out", out), ("dout", dout)):
@@ -274,6 +298,10 @@ def rib_window_attn_bwd_headwise_workspace(pos_head_stride, B, H, W, heads, d, r
 
 def rib_window_attn_fwd_headwise(q, k, v, pq, pk, window, shift=0, stream=None, want_lse=True):
     """Forward pass with one Pq/Pk table per head: pq, pk bf16 [heads, n, r]; returns (out, lse)."""
+    if _marshal is not None:
+        got = _native(_marshal.fwd, "rib_window_attn_fwd_headwise", q, k, v, pq, pk, 2, window, shift, want_lse, stream)
+        if got is not None:
+            return got
     _check_image("q", q)
     B, H, W, heads, d = q.shape
     _check_image("k", k, q.shape)
@@ -294,6 +322,10 @@ def rib_window_attn_fwd_headwise(q, k, v, pq, pk, window, shift=0, stream=None, 
 def rib_window_attn_fwd_padded(q, k, v, pq, pk, window, shift=0, stream=None, want_lse=True):
     """Forward pass on a map whose sides need not be multiples of the window (positions of the extended map
     beyond H x W are not tokens); pq, pk are [n, r] or [heads, n, r].  Returns (out, lse)."""
+    if _marshal is not None:
+        got = _native(_marshal.fwd, "rib_window_attn_fwd_padded", q, k, v, pq, pk, 3, window, shift, want_lse, stream)
+        if got is not None:
+            return got
     _check_image("q", q)
     B, H, W, heads, d = q.shape
     _check_image("k", k, q.shape)
@@ -380,6 +412,10 @@ def rib_window_cycle_bwd(qs, ks, vs, pqs, pks, outs, lses, douts, windows, shift
 def rib_window_attn_bwd_padded(q, k, v, pq, pk, out, lse, dout, window, shift=0, workspace=None, stream=None):
     """Backward pass on a map whose sides need not be multiples of the window; pq, pk [n, r] or [heads, n, r].
     Returns (dq, dk, dv bf16, dpq, dpk fp32 of the shape of pq)."""
+    if _marshal is not None and workspace is not None:
+        got = _native(_marshal.bwd, "rib_window_attn_bwd_padded", q, k, v, pq, pk, out, lse, dout, 3, window, shift, workspace, stream)
+        if got is not None:
+            return got
     _check_image("q", q)
     B, H, W, heads, d = q.shape
     for name, t in (("k", k), ("v", v), ("out", out), ("dout", dout)):
@@ -413,6 +449,10 @@ def rib_window_attn_bwd_padded(q, k, v, pq, pk, out, lse, dout, window, shift=0,
 def rib_window_attn_fwd_masked(q, k, v, pq, pk, window, shift=0, stream=None, want_lse=True):
     """Forward pass with shifted windows whose wrapped parts do not attend to each other (H, W multiples of the
     window); pq, pk are [n, r] or [heads, n, r].  Returns (out, lse)."""
+    if _marshal is not None:
+        got = _native(_marshal.fwd, "rib_window_attn_fwd_masked", q, k, v, pq, pk, 3, window, shift, want_lse, stream)
+        if got is not None:
+            return got
     _check_image("q", q)
     B, H, W, heads, d = q.shape
     _check_image("k", k, q.shape)
@@ -438,6 +478,10 @@ def rib_window_attn_fwd_masked(q, k, v, pq, pk, window, shift=0, stream=None, wa
 def rib_window_attn_bwd_masked(q, k, v, pq, pk, out, lse, dout, window, shift=0, workspace=None, stream=None):
     """Backward pass of rib_window_attn_fwd_masked; pq, pk [n, r] or [heads, n, r].
     Returns (dq, dk, dv bf16, dpq, dpk fp32 of the shape of pq)."""
+    if _marshal is not None and workspace is not None:
+        got = _native(_marshal.bwd, "rib_window_attn_bwd_masked", q, k, v, pq, pk, out, lse, dout, 3, window, shift, workspace, stream)
+        if got is not None:
+            return got
     _check_image("q", q)
     B, H, W, heads, d = q.shape
     for name, t in (("k", k), ("v", v), ("out", out), ("dout", dout)):
@@ -568,6 +612,10 @@ def rib_window_attn_fwd_gated(q, k, v, pq, pk, gate, window, shift=0, stream=Non
 
 def rib_window_attn_bwd_headwise(q, k, v, pq, pk, out, lse, dout, window, shift=0, workspace=None, stream=None):
     """Backward pass with one Pq/Pk table per head; returns (dq, dk, dv bf16, dpq, dpk fp32 [heads, n, r])."""
+    if _marshal is not None and workspace is not None:
+        got = _native(_marshal.bwd, "rib_window_attn_bwd_headwise", q, k, v, pq, pk, out, lse, dout, 2, window, shift, workspace, stream)
+        if got is not None:
+            return got
     _check_image("q", q)
     B, H, W, heads, d = q.shape
     for name, t in (("k", k), ("v", v), ("out", out), ("dout", dout)):
@@ -628,6 +676,10 @@ def _check_f32(name, t, shape):
 
 def rib_generate_features(w_h, b_h, w_pq, w_pk, window, stream=None):
     """Pq, Pk (bf16 [window^2, r]) from the generator weights (Eq. 1-3); L is read off w_h's height 2 + 4 L."""
+    if _marshal is not None:
+        got = _native(_marshal.generate, "rib_generate_features", w_h, b_h, w_pq, w_pk, window, stream)
+        if got is not None:
+            return got
     rows, dh = w_h.shape
     L, r = (rows - 2) // 4, w_pq.shape[1]
     _check_f32("w_h", w_h, (2 + 4 * L, dh)); _check_f32("b_h", b_h, (dh,))
@@ -643,6 +695,10 @@ def rib_generate_features(w_h, b_h, w_pq, w_pk, window, stream=None):
 
 def rib_generate_features_bwd(w_h, b_h, w_pq, w_pk, dpq, dpk, window, stream=None):
     """Gradients (dw_h, db_h, dw_pq, dw_pk) of the generator weights given dpq, dpk fp32 [window^2, r]."""
+    if _marshal is not None:
+        got = _native(_marshal.generate_bwd, "rib_generate_features_bwd", w_h, b_h, w_pq, w_pk, dpq, dpk, window, stream)
+        if got is not None:
+            return got
     rows, dh = w_h.shape
     L, r = (rows - 2) // 4, w_pq.shape[1]
     _check_f32("w_h", w_h, (2 + 4 * L, dh)); _check_f32("b_h", b_h, (dh,))

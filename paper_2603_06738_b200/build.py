@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree: csrc/*.cu -> paper_2603_06738_b200/librib_window_attn.so.
+"""Builds the CUDA library in-tree: csrc/*.cu -> paper_2603_06738_b200/librib_window_attn.so, and the native form of the
+binding's argument marshalling, csrc/rib_marshal.cpp -> paper_2603_06738_b200/_rib_marshal.so.
 
 nvcc cross-compiles for sm_100a without a GPU.  Run as ``python -m paper_2603_06738_b200.build``.
 """
@@ -12,6 +13,7 @@ from pathlib import Path
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "librib_window_attn.so"
+MARSHAL_SOURCE, MARSHAL = CSRC / "rib_marshal.cpp", PKG / "_rib_marshal.so"
 
 NVCC_FLAGS = [
     "-std=c++17", "-O3", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -30,8 +32,30 @@ def stale() -> bool:
     return LIB.stat().st_mtime < newest
 
 
+def build_marshal(force: bool = False) -> Path:
+    """Compile the marshaller against the installed torch (host code only).  Raises on failure."""
+    if not force and MARSHAL.exists() and MARSHAL.stat().st_mtime >= MARSHAL_SOURCE.stat().st_mtime:
+        return MARSHAL
+    import sysconfig
+
+    import torch
+    root = Path(torch.__file__).resolve().parent
+    cuda = Path(os.environ.get("CUDA_HOME", "/usr/local/cuda"))
+    includes = [root / "include", root / "include" / "torch" / "csrc" / "api" / "include", sysconfig.get_path("include"), cuda / "include"]
+    tmp = MARSHAL.with_suffix(f".{os.getpid()}.tmp")
+    run = subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+                          f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *[f"-I{p}" for p in includes], str(MARSHAL_SOURCE),
+                          f"-L{root / 'lib'}", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-o", str(tmp)], capture_output=True, text=True)
+    if run.returncode:
+        sys.stderr.write(run.stdout + run.stderr)
+        raise RuntimeError("g++ failed on rib_marshal.cpp")
+    os.replace(tmp, MARSHAL)
+    return MARSHAL
+
+
 def build(force: bool = False, verbose: bool = False) -> Path:
-    """Compile every .cu for sm_100a and link the shared library.  Raises on failure."""
+    """Compile every .cu for sm_100a and link the shared library, and the marshaller.  Raises on failure."""
+    build_marshal(force)
     if not force and not stale():
         return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
