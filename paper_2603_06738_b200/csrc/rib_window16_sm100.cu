@@ -8,7 +8,7 @@
 // keys) takes about 3900 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) about 3200: 1050 of loads
 // and exponentials, 1600 of stores of P and dS and their fences, with 1470 cycles of MMAs beside it.  Measured (4 x 96 x 96 tokens,
 // 12 heads of 16 channels, rank 24, shift 8, masked, by event hooks): forward 82 -> 60 us, backward 30 + 140 + 46 -> 12 (two
-// clearings) + 104 us, both calls 288 -> 156 us; backward on 10 x 64 x 64 tokens, 6 heads of 32 channels, rank 16: 20 + 66 + 23 -> 12 + 71 us.
+// clearings) + 101 us, both calls 288 -> 156 us; backward on 10 x 64 x 64 tokens, 6 heads of 32 channels, rank 16: 20 + 66 + 23 -> 12 + 71 us.
 //
 // Windows may be shifted (multiples of 8), masked, or reach beyond the map (sides multiples of 8): a window is four 8x8-token
 // patches (one TMA box each), and a query patch attends to a key patch or not.
@@ -480,42 +480,66 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             const bool on = ((I ? seen[1] : seen[0]) >> (2 * J + (cq >> 1))) & 1u;      // warp-uniform
             if (!mbar_wait_warp(bar(kSFull), u & 1, abort_flag, p.status)) break;
             tc_fence_after();
-            uint32_t pp[16], dd[16], ld[2];
-            tmem_ld2(lanes + kColLd<R> + 4 * (t & 1) + 2 * I, ld);
-#pragma unroll
-            for (int ch = 0; ch < 2; ++ch) {                  // 16 keys at a time: 32 scores and products in registers next to the results
-                uint32_t s[16], dp[16];
-                tmem_ld16(lanes + kColS + 32 * cq + 16 * ch, s);
-                tmem_ld16(lanes + kColDP + 32 * cq + 16 * ch, dp);
-                tmem_wait_ld();
-                if (ch == 1) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kSFree));
-                }
+            uint32_t pp[16], dd[16], ld[2], s[4][8], dp[4][8];
+            // Four pieces of 8 keys, the loads of a piece under the arithmetic of the one before; P and dS are stored together behind one
+            // fence when both buffers are free already (16 x 96 x 96 tokens, 6 heads, rank 16: two pieces of 16 and a fence each 224 us, so 214).
+            auto load = [&](int c) {
+                tmem_ld8(lanes + kColS + 32 * cq + 8 * c, s[c]);
+                tmem_ld8(lanes + kColDP + 32 * cq + 8 * c, dp[c]);
+            };
+            auto work = [&](int c) {
                 const float2 l2 = make_float2(__uint_as_float(ld[0]), __uint_as_float(ld[0])), d2 = make_float2(__uint_as_float(ld[1]), __uint_as_float(ld[1]));
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), scale2, l2);
+                for (int i = 0; i < 4; ++i) {
+                    const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[c][2 * i]), __uint_as_float(s[c][2 * i + 1])), scale2, l2);
                     const float2 e = make_float2(ex2_approx(x.x), ex2_approx(x.y));
-                    const float2 d = __fmul2_rn(e, __fadd2_rn(make_float2(__uint_as_float(dp[2 * i]), __uint_as_float(dp[2 * i + 1])), d2));
-                    pp[8 * ch + i] = pack_bf16x2(e.x, e.y);
-                    dd[8 * ch + i] = pack_bf16x2(d.x, d.y);
+                    const float2 d = __fmul2_rn(e, __fadd2_rn(make_float2(__uint_as_float(dp[c][2 * i]), __uint_as_float(dp[c][2 * i + 1])), d2));
+                    pp[4 * c + i] = pack_bf16x2(e.x, e.y);
+                    dd[4 * c + i] = pack_bf16x2(d.x, d.y);
                 }
-            }
+            };
+            tmem_ld2(lanes + kColLd<R> + 4 * (t & 1) + 2 * I, ld);
+            load(0); load(1);
+            tmem_wait_ld();
+            load(2);
+            work(0);
+            tmem_wait_ld();
+            load(3);
+            work(1);
+            tmem_wait_ld();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kSFree));
+            // have the contractions of the unit before read P and dS?  (No phase completed answers yes to parity 1, which unit 0 asks for.)
+            const bool p_free = mbar_try_wait(bar(kPDone), (u - 1) & 1), ds_free = mbar_test(bar(kSDone), (u - 1) & 1);
+            work(2);
+            work(3);
             if (!on) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) pp[i] = dd[i] = 0u;
             }
-            // P, then dS: the contractions of the unit before that read each of them end one after the other, too
-            auto store = [&](uint8_t* line, const uint32_t (&v)[16], uint32_t done, uint32_t ready) {
-                if (u > 0 && !mbar_wait_warp(done, (u - 1) & 1, abort_flag, p.status)) return false;
+            auto put = [&](uint8_t* line, const uint32_t (&v)[16]) {
 #pragma unroll
                 for (int q4 = 0; q4 < 4; ++q4)
                     *reinterpret_cast<uint4*>(line + (((4 * (cq & 1) + q4) ^ (row & 7)) << 4)) = make_uint4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
+            };
+            auto announce = [&](uint32_t ready) {
                 fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(ready);
+            };
+            if (__all_sync(0xffffffffu, p_free & ds_free)) {
+                put(p_row, pp);
+                put(ds_row, dd);
+                announce(bar(kPReady));
+                if (lane == 0) mbar_arrive(bar(kSReady));
+                continue;
+            }
+            // P, then dS: the contractions of the unit before that read each of them end one after the other, too
+            auto store = [&](uint8_t* line, const uint32_t (&v)[16], uint32_t done, uint32_t ready) {
+                if (u > 0 && !mbar_wait_warp(done, (u - 1) & 1, abort_flag, p.status)) return false;
+                put(line, v);
+                announce(ready);
                 return true;
             };
             if (!store(p_row, pp, bar(kPDone), bar(kPReady)) || !store(ds_row, dd, bar(kSDone), bar(kSReady))) break;
