@@ -7,9 +7,10 @@
 // only kTokens tokens and spreads every step over all of its threads: a thread evaluates single Fourier features and then
 // 4-column pieces of the hidden rows, of the projections and, in the backward pass, of the weight gradients, which are
 // summed over the block's tokens and added to global memory with one atomic per piece.  The gradients are cleared by one
-// small kernel that the main kernel overtakes (programmatic dependent launch) up to its first atomic.  Measured at window
-// 32, L = 10, dh = 32, r = 16, a thread owning a whole token of a block of 128 before: forward 39.5 -> 14.6 us, backward 119.8 -> 19.2 us by event hooks (which
-// include about 7 us per call); forward and backward call together 140 -> 40 us, now bound by the host side.
+// small kernel that the main kernel overtakes (programmatic dependent launch) up to its first atomic.  The weights reach shared
+// memory by asynchronous copies while the features are computed.  Measured by event hooks (which include about 7 us per call) at window
+// 32, L = 10, dh = 32, r = 16: forward 10.4 us, backward 12.8 us (staged by loads and stores, 128 threads a block: 10.8 and 14.9; a
+// thread owning a whole token of a block of 128: 39.5 and 119.8); both calls at window 64, L = 12, dh = 48, r = 32: 41.4 -> 31.3 us.
 //
 // Coordinates: window points run from -1 to 1 inclusive on both axes (a single point sits at 0); token
 // i = y * window + x has the coordinate (row, column); Eq. 1 literally, frequencies 2^l without pi.
@@ -18,7 +19,7 @@
 namespace rib {
 namespace {
 
-constexpr int kThreads = 128;
+constexpr int kThreads = 256;
 constexpr int kTokens = 16;      // tokens of a block: 64 blocks at window 32; the gradients' atomics grow with the number of blocks
 
 struct GenParams {
@@ -70,12 +71,29 @@ __device__ __forceinline__ GenSmem carve(const GenParams& p, float* sm)
     return s;
 }
 
+// A matrix into shared memory, rows of ws floats to rows of wd (zeros behind, and beyond real_rows).  Rows that are whole 16-byte
+// pieces travel asynchronously: the copies of all matrices are in flight while the Fourier features are computed
+// (staged_arrived before the first use).
 __device__ __forceinline__ void stage(float* dst, int wd, const float* src, int ws, int rows, int real_rows)
 {
-    for (int i = threadIdx.x; i < rows * wd; i += kThreads) {
-        const int row = i / wd, c = i - row * wd;
-        dst[i] = row < real_rows && c < ws ? src[row * ws + c] : 0.f;
+    const int pieces = wd / 4;
+    for (int i = threadIdx.x; i < rows * pieces; i += kThreads) {
+        const int row = i / pieces, c = 4 * (i - row * pieces);
+        const float* from = src + (size_t)row * ws + c;
+        if (ws == wd && row < real_rows) {
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + 4 * i)), "l"(from) : "memory");
+        } else {
+            float v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = row < real_rows && c + k < ws ? from[k] : 0.f;
+            *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(v[0], v[1], v[2], v[3]);
+        }
     }
+}
+__device__ __forceinline__ void staged_arrived()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
 }
 
 __device__ __forceinline__ void fma4(float4& a, float x, const float4& w)
@@ -103,7 +121,7 @@ __device__ __forceinline__ void features_and_hidden(const GenParams& p, const Ge
             row[4 + 4 * l + axis] = live ? cosf(arg) : 0.f;
         }
     }
-    __syncthreads();
+    staged_arrived();
     const int pieces = s.dhp / 4;
     for (int e = threadIdx.x; e < kTokens * pieces; e += kThreads) {
         const int t = e / pieces, j = 4 * (e - t * pieces);
