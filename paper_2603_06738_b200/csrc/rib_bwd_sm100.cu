@@ -237,10 +237,10 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         auto wait_all = [&](uint32_t b, uint32_t parity) { return mbar_wait_warp(b, parity, abort_flag, p.status); };
         bool ok = true;
         if (warp == 1) {
+            // ---- S^T, dP^T of unit u as soon as the arithmetic group has read unit u - 2 (same buffers)
+            // out of tensor memory; the group is then still busy with that unit's exponentials.
             // Rank 32: of both halves of a tile at once (N = 128), whose six MMAs fetch 48 KB of operands where two sets of six fetch 72 (641 ->
             // 625 us); at rank 16 the halves kept apart are the faster (550 against 560 us).
-            // ---- S^T, dP^T of unit u as soon as the arithmetic group has read unit u - 2 (same buffers)
-            // out of tensor memory; the group is then still busy with that unit's exponentials
             uint32_t nitem = 0, I = 0;
             uint32_t slot_base = 0;
             for (uint32_t u = 0; u < total_units / kSUnits && ok; ++u) {
@@ -811,7 +811,7 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     const int windows = p.pairs / p.heads;   // pairs of one head
     const int in_line = tables == 1 ? p.pairs : windows;      // pairs whose sums go to one table
     // a block takes a run of per_group pairs (of one head, with head-wise tables)
-    // (measured on the training configuration: 4 or 8 pairs per block 62 us, 16: 74 us, 32: 74 us -- more blocks in flight
+    // (measured on the training configuration: 4 pairs per block 56 us, 2 or 8: 60, 16: 70 -- more blocks in flight
     // matter more to this kernel than fewer atomics)
     const int per_group = in_line >= 1024 ? 8 : in_line >= 16 ? 4 : 1;
     const unsigned groups = (tables == 1 ? 1u : (unsigned)p.heads) * (unsigned)((in_line + per_group - 1) / per_group);
