@@ -381,9 +381,10 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 // The warp's 32 key rows x 32 queries in four pieces of 16 x 16 (piece c: lanes 16 (c % 2) .., queries 16 (c / 2) ..), read as
                 // 16-lane fragments: a thread holds 2 key rows of 4 queries of a piece, and the per-query (-lse2, -lse2', -D, -D') cost
                 // it 16 words per unit instead of 64.  What these warps share with the operand fetches of the MMAs is the one shared-memory
-                // data pipe (a row of 32 queries per thread with 16-byte broadcasts filled it to 97 %; this form to 66 %): the reads are
-                // 4 bytes wide because a 16-byte read of four different addresses costs eight passes, four 4-byte reads one each.  With
-                // dS leaving by stmatrix and dQ~ by 16-byte adds, rank 32: 745 -> 638 us, rank 16: 565 -> 555 us (16 x 96 x 96, windows of 32).
+                // data pipe (1270 of its passes per tile of 128 x 128 were the warps' with a row of 32 queries per thread and 16-byte broadcasts,
+                // 895 with this form, beside 992 of the MMAs): the reads are 4 bytes wide because a 16-byte read of four different addresses
+                // counted eight passes.  With dS leaving by stmatrix and dQ~ by 16-byte adds, rank 32: 745 -> 638 us, rank 16: 565 -> 555 us
+                // (16 x 96 x 96, windows of 32).
                 const uint32_t ld = base + kOffRing + st * kRingBytes + kRingLD + (32 * h + 16 * cg + (lane & 3)) * 16;
                 auto ldq = [&](int gq) { return make_float4(lds_f32(ld + 64 * gq), lds_f32(ld + 64 * gq + 4), lds_f32(ld + 64 * gq + 8), lds_f32(ld + 64 * gq + 12)); };
                 const uint32_t ds_line = base + kOffDS + ((g & 1) * 2 + h) * kDSHalf + (quarter * 32 + 8 * ((lane >> 3) & 1) + (lane & 7)) * 128;
