@@ -8,6 +8,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import warnings
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
@@ -54,8 +55,20 @@ def build_marshal(force: bool = False) -> Path:
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
-    """Compile every .cu for sm_100a and link the shared library, and the marshaller.  Raises on failure."""
-    build_marshal(force)
+    """Compile every .cu for sm_100a and link the shared library; raises on failure.  Then the marshaller, which the library does
+    not need: where it cannot be compiled (no g++, no headers of Python or torch), a warning says so, none of an earlier build is
+    left behind, and the binding marshals in Python."""
+    lib = build_library(force, verbose)
+    try:
+        build_marshal(force)
+    except Exception as e:      # noqa: BLE001 - whatever is missing, the library is there
+        MARSHAL.unlink(missing_ok=True)
+        warnings.warn(f"{MARSHAL.name} was not built, calls are marshalled in Python (a few us more each): {e}", RuntimeWarning, stacklevel=2)
+    return lib
+
+
+def build_library(force: bool = False, verbose: bool = False) -> Path:
+    """Compile every .cu for sm_100a and link the shared library (nvcc alone is needed).  Raises on failure."""
     if not force and not stale():
         return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
