@@ -8,16 +8,35 @@ raises ``RibLibraryMissing``.
 from __future__ import annotations
 
 import ctypes
+import warnings
 from pathlib import Path
 
 import torch
 
-try:
-    # The checks, allocations and the C call of the hot entry points in native code (csrc/rib_marshal.cpp).  It answers None for
-    # arguments that are not plain tensors of the right kind, and the Python form below takes over.
-    from . import _rib_marshal as _marshal
-except ImportError:         # not built, or built for another torch
-    _marshal = None
+from .build import marshal_identity
+
+
+def _load_marshal():
+    """The checks, allocations and the C call of the hot entry points in native code (csrc/rib_marshal.cpp), or None.  It answers None
+    for arguments that are not plain tensors of the right kind, and the Python form below takes over."""
+    try:
+        from . import _rib_marshal as module
+    except ImportError:         # not built, or symbols that this torch does not have
+        return None
+    return module if _fits(module) else None
+
+
+def _fits(module) -> bool:
+    """Was the marshaller compiled for this torch and this Python?  It would import for many others, and read their tensors wrongly."""
+    built_for = getattr(module, "built_for", None)
+    if built_for == marshal_identity():
+        return True
+    warnings.warn(f"{module.__name__} was built for {built_for}, this is {marshal_identity()}: calls are marshalled in Python "
+                  "until `python -m paper_2603_06738_b200.build` has been run", RuntimeWarning, stacklevel=2)
+    return False
+
+
+_marshal = _load_marshal()
 
 _LIB_PATH = Path(__file__).resolve().parent / "librib_window_attn.so"
 _lib = None

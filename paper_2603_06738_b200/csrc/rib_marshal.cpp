@@ -11,6 +11,10 @@
 #include <c10/core/impl/TorchDispatchModeTLS.h>
 #include <c10/cuda/CUDAStream.h>
 
+#include <type_traits>
+
+#include "../../include/rib_window_attn.h"
+
 namespace {
 
 // The tensor behind a plain torch.Tensor of the given type: dense CUDA memory of its own, contiguous; else null.
@@ -79,11 +83,13 @@ bool get_image(PyObject* const* a, int tables, PyObject* window, PyObject* shift
     return false;
 }
 
-using Fwd = int (*)(const void*, const void*, const void*, const void*, const void*, long long, int, int, int, int, int, int, int, int, void*, float*, void*);
-using Bwd = int (*)(const void*, const void*, const void*, const void*, const void*, long long, const void*, const float*, const void*, int, int, int, int, int,
-                    int, int, int, void*, void*, void*, float*, float*, void*, size_t, void*);
-using GenFwd = int (*)(const float*, const float*, const float*, const float*, int, int, int, int, void*, void*, void*);
-using GenBwd = int (*)(const float*, const float*, const float*, const float*, const float*, const float*, int, int, int, int, float*, float*, float*, float*, void*);
+// The types of the C calls, from their header: a signature that changes there does not compile here.
+using Fwd = decltype(&rib_window_attn_fwd_headwise);
+using Bwd = decltype(&rib_window_attn_bwd_headwise);
+using GenFwd = decltype(&rib_generate_features);
+using GenBwd = decltype(&rib_generate_features_bwd);
+static_assert(std::is_same_v<Fwd, decltype(&rib_window_attn_fwd_padded)> && std::is_same_v<Fwd, decltype(&rib_window_attn_fwd_masked)>);
+static_assert(std::is_same_v<Bwd, decltype(&rib_window_attn_bwd_padded)> && std::is_same_v<Bwd, decltype(&rib_window_attn_bwd_masked)>);
 
 PyObject* status(int rc) { return PyLong_FromLong(rc); }
 PyObject* wrap(at::Tensor t) { return THPVariable_Wrap(std::move(t)); }
@@ -218,4 +224,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_rib_marshal", nullptr, -1, method
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__rib_marshal() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__rib_marshal()
+{
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", RIB_BUILT_FOR) < 0) { Py_DECREF(m); return nullptr; }      // the binding compares it
+    return m;
+}
