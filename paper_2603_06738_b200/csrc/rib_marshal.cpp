@@ -22,7 +22,7 @@ const at::Tensor* plain(PyObject* o, at::ScalarType type, int dim)
 {
     if (!THPVariable_CheckExact(o)) return nullptr;
     const at::Tensor& t = THPVariable_Unpack(o);
-    if (!t.defined() || t.layout() != at::kStrided || !t.is_cuda() || t.scalar_type() != type || t.dim() != dim || !t.has_storage() || !t.is_contiguous()) return nullptr;
+    if (!t.defined() || t.is_nested() || t.layout() != at::kStrided || !t.is_cuda() || t.scalar_type() != type || t.dim() != dim || !t.has_storage() || !t.is_contiguous()) return nullptr;
     const auto keys = t.key_set();
     if (keys.has_any(c10::DispatchKeySet({c10::DispatchKey::Python, c10::DispatchKey::FuncTorchBatched, c10::DispatchKey::FuncTorchGradWrapper,
                                           c10::DispatchKey::Functionalize, c10::DispatchKey::Conjugate, c10::DispatchKey::Negative, c10::DispatchKey::ZeroTensor}))) return nullptr;
@@ -51,9 +51,10 @@ bool get_stream(PyObject* o, void** s)
     if (o == Py_None) { *s = (void*)c10::cuda::getCurrentCUDAStream().stream(); return true; }
     PyObject* p = PyObject_GetAttrString(o, "cuda_stream");
     if (!p) { PyErr_Clear(); return false; }
-    const bool ok = PyLong_Check(p);
-    if (ok) *s = PyLong_AsVoidPtr(p);
+    if (PyLong_Check(p)) *s = PyLong_AsVoidPtr(p);
+    const bool ok = PyLong_Check(p) && !PyErr_Occurred();
     Py_DECREF(p);
+    PyErr_Clear();
     return ok;
 }
 
@@ -91,65 +92,90 @@ using GenBwd = decltype(&rib_generate_features_bwd);
 static_assert(std::is_same_v<Fwd, decltype(&rib_window_attn_fwd_padded)> && std::is_same_v<Fwd, decltype(&rib_window_attn_fwd_masked)>);
 static_assert(std::is_same_v<Bwd, decltype(&rib_window_attn_bwd_padded)> && std::is_same_v<Bwd, decltype(&rib_window_attn_bwd_masked)>);
 
+// The body of a call.  No C++ exception may leave through the C frames of the interpreter (a tensor of an unusual kind may throw
+// wherever it is asked for its sizes or its memory): the Python form meets the same condition and raises it.
+template <class Body>
+PyObject* guarded(Body&& body) noexcept
+{
+    try {
+        return body();
+    } catch (...) {
+        PyErr_Clear();
+        Py_RETURN_NONE;
+    }
+}
+
+// No lock of the interpreter while this lives, an exception or not
+struct Unlocked {
+    PyThreadState* const state = PyEval_SaveThread();
+    Unlocked() = default;
+    Unlocked(const Unlocked&) = delete;
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
 PyObject* status(int rc) { return PyLong_FromLong(rc); }
-PyObject* wrap(at::Tensor t) { return THPVariable_Wrap(std::move(t)); }
+
+// the results of a call, None in the place of an undefined one
+PyObject* results(std::initializer_list<at::Tensor*> tensors)
+{
+    PyObject* res = PyTuple_New((Py_ssize_t)tensors.size());
+    if (!res) return nullptr;
+    Py_ssize_t i = 0;
+    for (at::Tensor* t : tensors) {
+        PyObject* o = t->defined() ? THPVariable_Wrap(std::move(*t)) : Py_NewRef(Py_None);
+        if (!o) { Py_DECREF(res); return nullptr; }
+        PyTuple_SET_ITEM(res, i++, o);
+    }
+    return res;
+}
 
 // fwd(address, q, k, v, pq, pk, tables, window, shift, want_lse, stream)
 PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t count)
 {
-    Image m;
-    int tables = 0;
-    void* stream;
-    if (count != 11 || modes_active() || !get_int(a[6], &tables) || !get_image(a + 1, tables, a[7], a[8], &m) || !PyBool_Check(a[9]) || !get_stream(a[10], &stream)) Py_RETURN_NONE;
-    const Fwd fn = reinterpret_cast<Fwd>(address(a[0]));
-    try {
+    return guarded([&]() -> PyObject* {
+        Image m;
+        int tables = 0;
+        void* stream;
+        if (count != 11 || modes_active() || !get_int(a[6], &tables) || !get_image(a + 1, tables, a[7], a[8], &m) || !PyBool_Check(a[9]) || !get_stream(a[10], &stream)) Py_RETURN_NONE;
+        const Fwd fn = reinterpret_cast<Fwd>(address(a[0]));
         at::Tensor out = at::empty_like(*m.q), lse;
         if (a[9] == Py_True) lse = at::empty({m.B, m.heads, m.H, m.W}, m.q->options().dtype(at::kFloat));
         int rc;
-        Py_BEGIN_ALLOW_THREADS
-        rc = fn(m.q->const_data_ptr(), m.k->const_data_ptr(), m.v->const_data_ptr(), m.pq->const_data_ptr(), m.pk->const_data_ptr(), m.stride, m.B, m.H, m.W, m.heads,
-                m.d, m.r, m.window, m.shift, out.mutable_data_ptr(), lse.defined() ? lse.mutable_data_ptr<float>() : nullptr, stream);
-        Py_END_ALLOW_THREADS
+        {
+            const Unlocked unlocked;
+            rc = fn(m.q->const_data_ptr(), m.k->const_data_ptr(), m.v->const_data_ptr(), m.pq->const_data_ptr(), m.pk->const_data_ptr(), m.stride, m.B, m.H, m.W, m.heads,
+                    m.d, m.r, m.window, m.shift, out.mutable_data_ptr(), lse.defined() ? lse.mutable_data_ptr<float>() : nullptr, stream);
+        }
         if (rc) return status(rc);
-        PyObject* res = PyTuple_New(2);
-        PyTuple_SET_ITEM(res, 0, wrap(std::move(out)));
-        if (lse.defined()) PyTuple_SET_ITEM(res, 1, wrap(std::move(lse)));
-        else { Py_INCREF(Py_None); PyTuple_SET_ITEM(res, 1, Py_None); }
-        return res;
-    } catch (...) {
-        Py_RETURN_NONE;      // (out of memory and the like: the Python form raises it)
-    }
+        return results({&out, &lse});
+    });
 }
 
 // bwd(address, q, k, v, pq, pk, out, lse, dout, tables, window, shift, workspace, stream)
 PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t count)
 {
-    Image m;
-    int tables = 0;
-    void* stream;
-    if (count != 14 || modes_active() || !get_int(a[9], &tables) || !get_image(a + 1, tables, a[10], a[11], &m) || !get_stream(a[13], &stream)) Py_RETURN_NONE;
-    const at::Tensor *out = plain(a[6], at::kBFloat16, 5), *lse = plain(a[7], at::kFloat, 4), *dout = plain(a[8], at::kBFloat16, 5);
-    const at::Tensor* ws = plain(a[12], at::kByte, 1);
-    if (!out || !lse || !dout || !ws || out->sizes() != m.q->sizes() || dout->sizes() != m.q->sizes() ||
-        lse->size(0) != m.B || lse->size(1) != m.heads || lse->size(2) != m.H || lse->size(3) != m.W) Py_RETURN_NONE;
-    const Bwd fn = reinterpret_cast<Bwd>(address(a[0]));
-    try {
+    return guarded([&]() -> PyObject* {
+        Image m;
+        int tables = 0;
+        void* stream;
+        if (count != 14 || modes_active() || !get_int(a[9], &tables) || !get_image(a + 1, tables, a[10], a[11], &m) || !get_stream(a[13], &stream)) Py_RETURN_NONE;
+        const at::Tensor *out = plain(a[6], at::kBFloat16, 5), *lse = plain(a[7], at::kFloat, 4), *dout = plain(a[8], at::kBFloat16, 5);
+        const at::Tensor* ws = plain(a[12], at::kByte, 1);
+        if (!out || !lse || !dout || !ws || out->sizes() != m.q->sizes() || dout->sizes() != m.q->sizes() ||
+            lse->size(0) != m.B || lse->size(1) != m.heads || lse->size(2) != m.H || lse->size(3) != m.W) Py_RETURN_NONE;
+        const Bwd fn = reinterpret_cast<Bwd>(address(a[0]));
         const auto f32 = m.q->options().dtype(at::kFloat);
         at::Tensor dq = at::empty_like(*m.q), dk = at::empty_like(*m.q), dv = at::empty_like(*m.q), dpq = at::empty(m.pq->sizes(), f32), dpk = at::empty(m.pq->sizes(), f32);
         int rc;
-        Py_BEGIN_ALLOW_THREADS
-        rc = fn(m.q->const_data_ptr(), m.k->const_data_ptr(), m.v->const_data_ptr(), m.pq->const_data_ptr(), m.pk->const_data_ptr(), m.stride, out->const_data_ptr(),
-                lse->const_data_ptr<float>(), dout->const_data_ptr(), m.B, m.H, m.W, m.heads, m.d, m.r, m.window, m.shift, dq.mutable_data_ptr(), dk.mutable_data_ptr(),
-                dv.mutable_data_ptr(), dpq.mutable_data_ptr<float>(), dpk.mutable_data_ptr<float>(), ws->mutable_data_ptr(), (size_t)ws->numel(), stream);
-        Py_END_ALLOW_THREADS
+        {
+            const Unlocked unlocked;
+            rc = fn(m.q->const_data_ptr(), m.k->const_data_ptr(), m.v->const_data_ptr(), m.pq->const_data_ptr(), m.pk->const_data_ptr(), m.stride, out->const_data_ptr(),
+                    lse->const_data_ptr<float>(), dout->const_data_ptr(), m.B, m.H, m.W, m.heads, m.d, m.r, m.window, m.shift, dq.mutable_data_ptr(), dk.mutable_data_ptr(),
+                    dv.mutable_data_ptr(), dpq.mutable_data_ptr<float>(), dpk.mutable_data_ptr<float>(), ws->mutable_data_ptr(), (size_t)ws->numel(), stream);
+        }
         if (rc) return status(rc);
-        PyObject* res = PyTuple_New(5);
-        at::Tensor* all[5] = {&dq, &dk, &dv, &dpq, &dpk};
-        for (int i = 0; i < 5; ++i) PyTuple_SET_ITEM(res, i, wrap(std::move(*all[i])));
-        return res;
-    } catch (...) {
-        Py_RETURN_NONE;
-    }
+        return results({&dq, &dk, &dv, &dpq, &dpk});
+    });
 }
 
 struct Generator { const at::Tensor *w_h, *b_h, *w_pq, *w_pk; int window, L, dh, r; void* stream; };
@@ -167,51 +193,44 @@ bool get_generator(PyObject* const* w, PyObject* window, PyObject* stream, Gener
 // generate(address, w_h, b_h, w_pq, w_pk, window, stream)
 PyObject* generate(PyObject*, PyObject* const* a, Py_ssize_t count)
 {
-    Generator g;
-    if (count != 7 || modes_active() || !get_generator(a + 1, a[5], a[6], &g)) Py_RETURN_NONE;
-    const GenFwd fn = reinterpret_cast<GenFwd>(address(a[0]));
-    try {
+    return guarded([&]() -> PyObject* {
+        Generator g;
+        if (count != 7 || modes_active() || !get_generator(a + 1, a[5], a[6], &g)) Py_RETURN_NONE;
+        const GenFwd fn = reinterpret_cast<GenFwd>(address(a[0]));
         const auto options = g.w_h->options().dtype(at::kBFloat16);
         at::Tensor pq = at::empty({g.window * g.window, g.r}, options), pk = at::empty({g.window * g.window, g.r}, options);
         int rc;
-        Py_BEGIN_ALLOW_THREADS
-        rc = fn(g.w_h->const_data_ptr<float>(), g.b_h->const_data_ptr<float>(), g.w_pq->const_data_ptr<float>(), g.w_pk->const_data_ptr<float>(), g.window, g.L, g.dh, g.r,
-                pq.mutable_data_ptr(), pk.mutable_data_ptr(), g.stream);
-        Py_END_ALLOW_THREADS
+        {
+            const Unlocked unlocked;
+            rc = fn(g.w_h->const_data_ptr<float>(), g.b_h->const_data_ptr<float>(), g.w_pq->const_data_ptr<float>(), g.w_pk->const_data_ptr<float>(), g.window, g.L, g.dh, g.r,
+                    pq.mutable_data_ptr(), pk.mutable_data_ptr(), g.stream);
+        }
         if (rc) return status(rc);
-        PyObject* res = PyTuple_New(2);
-        PyTuple_SET_ITEM(res, 0, wrap(std::move(pq)));
-        PyTuple_SET_ITEM(res, 1, wrap(std::move(pk)));
-        return res;
-    } catch (...) {
-        Py_RETURN_NONE;
-    }
+        return results({&pq, &pk});
+    });
 }
 
 // generate_bwd(address, w_h, b_h, w_pq, w_pk, dpq, dpk, window, stream)
 PyObject* generate_bwd(PyObject*, PyObject* const* a, Py_ssize_t count)
 {
-    Generator g;
-    if (count != 9 || modes_active() || !get_generator(a + 1, a[7], a[8], &g)) Py_RETURN_NONE;
-    const at::Tensor *dpq = plain(a[5], at::kFloat, 2), *dpk = plain(a[6], at::kFloat, 2);
-    const int64_t n = (int64_t)g.window * g.window;
-    if (!dpq || !dpk || dpq->size(0) != n || dpk->size(0) != n || dpq->size(1) != g.r || dpk->size(1) != g.r) Py_RETURN_NONE;
-    const GenBwd fn = reinterpret_cast<GenBwd>(address(a[0]));
-    try {
+    return guarded([&]() -> PyObject* {
+        Generator g;
+        if (count != 9 || modes_active() || !get_generator(a + 1, a[7], a[8], &g)) Py_RETURN_NONE;
+        const at::Tensor *dpq = plain(a[5], at::kFloat, 2), *dpk = plain(a[6], at::kFloat, 2);
+        const int64_t n = (int64_t)g.window * g.window;
+        if (!dpq || !dpk || dpq->size(0) != n || dpk->size(0) != n || dpq->size(1) != g.r || dpk->size(1) != g.r) Py_RETURN_NONE;
+        const GenBwd fn = reinterpret_cast<GenBwd>(address(a[0]));
         at::Tensor out[4] = {at::empty_like(*g.w_h), at::empty_like(*g.b_h), at::empty_like(*g.w_pq), at::empty_like(*g.w_pk)};
         int rc;
-        Py_BEGIN_ALLOW_THREADS
-        rc = fn(g.w_h->const_data_ptr<float>(), g.b_h->const_data_ptr<float>(), g.w_pq->const_data_ptr<float>(), g.w_pk->const_data_ptr<float>(),
-                dpq->const_data_ptr<float>(), dpk->const_data_ptr<float>(), g.window, g.L, g.dh, g.r, out[0].mutable_data_ptr<float>(), out[1].mutable_data_ptr<float>(),
-                out[2].mutable_data_ptr<float>(), out[3].mutable_data_ptr<float>(), g.stream);
-        Py_END_ALLOW_THREADS
+        {
+            const Unlocked unlocked;
+            rc = fn(g.w_h->const_data_ptr<float>(), g.b_h->const_data_ptr<float>(), g.w_pq->const_data_ptr<float>(), g.w_pk->const_data_ptr<float>(),
+                    dpq->const_data_ptr<float>(), dpk->const_data_ptr<float>(), g.window, g.L, g.dh, g.r, out[0].mutable_data_ptr<float>(), out[1].mutable_data_ptr<float>(),
+                    out[2].mutable_data_ptr<float>(), out[3].mutable_data_ptr<float>(), g.stream);
+        }
         if (rc) return status(rc);
-        PyObject* res = PyTuple_New(4);
-        for (int i = 0; i < 4; ++i) PyTuple_SET_ITEM(res, i, wrap(std::move(out[i])));
-        return res;
-    } catch (...) {
-        Py_RETURN_NONE;
-    }
+        return results({&out[0], &out[1], &out[2], &out[3]});
+    });
 }
 
 PyMethodDef methods[] = {

@@ -103,3 +103,37 @@ def test_under_capture():
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, want)
+
+
+def test_tensors_that_have_no_plain_memory(monkeypatch):
+    """A nested tensor is strided, dense and five-dimensional, and throws when it is asked for its sizes; what is allocated inside a
+    gradient transform is a wrapper without storage.  Either is an exception of the Python form, not the end of the process."""
+    args, dout = inputs(False)
+    q, k, v, pq, pk = args
+    fwd, bwd = binding.rib_window_attn_fwd, binding.rib_window_attn_bwd
+    out, lse = fwd(*args, 16, 8)
+    ws = torch.empty(1 << 24, dtype=torch.uint8, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    w = [torch.randn(s, generator=gen, device="cuda") * 0.2 for s in ((42, 32), (32,), (32, 16), (32, 16))]
+    d = [torch.randn((256, 16), generator=gen, device="cuda") for _ in range(2)]
+    nest = lambda t: torch.nested.nested_tensor(list(t), dtype=t.dtype, device="cuda")
+    x = torch.ones(3, device="cuda")
+
+    def inside(transform, call):
+        def f(x):
+            call()
+            return x.sum()
+        return transform(f)
+
+    calls = (lambda: fwd(*args, 16, 8), lambda: bwd(*args, out, lse, dout, 16, 8, workspace=ws), lambda: binding.rib_generate_features(*w, 16),
+             lambda: binding.rib_generate_features_bwd(*w, *d, 16))
+    for call in (lambda: fwd(nest(q), k, v, pq, pk, 16, 8), lambda: fwd(q, k, v, nest(pq), pk, 16, 8), lambda: bwd(q, k, nest(v), pq, pk, out, lse, dout, 16, 8, workspace=ws),
+                 lambda: bwd(*args, out, nest(lse), dout, 16, 8, workspace=ws), lambda: binding.rib_generate_features(nest(w[0]), *w[1:], 16),
+                 lambda: binding.rib_generate_features_bwd(*w, nest(d[0]), d[1], 16),
+                 *(lambda c=c: inside(torch.func.grad, c)(x) for c in calls), *(lambda c=c: inside(lambda f: lambda x: torch.func.jvp(f, (x,), (x,)), c)(x) for c in calls)):
+        a, b = both(monkeypatch, call)
+        torch.cuda.synchronize()
+        assert a == b and issubclass(a[0], Exception), (a, b)
+    for call in calls:                          # (no wrapper is made under a batched map of something else)
+        a, b = both(monkeypatch, lambda: inside(torch.vmap, call)(torch.ones(2, 3, device="cuda")))
+        assert torch.equal(a, b)
