@@ -29,9 +29,13 @@ const at::Tensor* plain(PyObject* o, at::ScalarType type, int dim)
     return &t;
 }
 
+// Is something between this thread's calls and the kernels of torch: a dispatch or function mode, a transform, a trace?  (Its own
+// handlers may be in Python; what is there on every thread, and autocast, is not.)
 bool modes_active()
 {
-    return c10::impl::TorchDispatchModeTLS::any_modes_set() || at::impl::PythonTorchFunctionTLS::stack_len() > 0;
+    const c10::DispatchKeySet usual = c10::default_included_set | c10::autocast_dispatch_keyset;
+    return c10::impl::TorchDispatchModeTLS::any_modes_set() || at::impl::PythonTorchFunctionTLS::stack_len() > 0 ||
+           !(c10::impl::tls_local_dispatch_key_set().included_ - usual).empty();
 }
 
 bool get_int(PyObject* o, int* v)
@@ -105,7 +109,8 @@ PyObject* guarded(Body&& body) noexcept
     }
 }
 
-// No lock of the interpreter while this lives, an exception or not
+// No lock of the interpreter while this lives, an exception or not.  The allocations are made without it, too, as torch.empty makes
+// them: one that finds no cached memory waits for the device, and a host function on some stream may be waiting for the lock.
 struct Unlocked {
     PyThreadState* const state = PyEval_SaveThread();
     Unlocked() = default;
@@ -138,11 +143,13 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t count)
         void* stream;
         if (count != 11 || modes_active() || !get_int(a[6], &tables) || !get_image(a + 1, tables, a[7], a[8], &m) || !PyBool_Check(a[9]) || !get_stream(a[10], &stream)) Py_RETURN_NONE;
         const Fwd fn = reinterpret_cast<Fwd>(address(a[0]));
-        at::Tensor out = at::empty_like(*m.q), lse;
-        if (a[9] == Py_True) lse = at::empty({m.B, m.heads, m.H, m.W}, m.q->options().dtype(at::kFloat));
+        const bool want_lse = a[9] == Py_True;
+        at::Tensor out, lse;
         int rc;
         {
             const Unlocked unlocked;
+            out = at::empty_like(*m.q);
+            if (want_lse) lse = at::empty({m.B, m.heads, m.H, m.W}, m.q->options().dtype(at::kFloat));
             rc = fn(m.q->const_data_ptr(), m.k->const_data_ptr(), m.v->const_data_ptr(), m.pq->const_data_ptr(), m.pk->const_data_ptr(), m.stride, m.B, m.H, m.W, m.heads,
                     m.d, m.r, m.window, m.shift, out.mutable_data_ptr(), lse.defined() ? lse.mutable_data_ptr<float>() : nullptr, stream);
         }
@@ -165,10 +172,12 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t count)
             lse->size(0) != m.B || lse->size(1) != m.heads || lse->size(2) != m.H || lse->size(3) != m.W) Py_RETURN_NONE;
         const Bwd fn = reinterpret_cast<Bwd>(address(a[0]));
         const auto f32 = m.q->options().dtype(at::kFloat);
-        at::Tensor dq = at::empty_like(*m.q), dk = at::empty_like(*m.q), dv = at::empty_like(*m.q), dpq = at::empty(m.pq->sizes(), f32), dpk = at::empty(m.pq->sizes(), f32);
+        at::Tensor dq, dk, dv, dpq, dpk;
         int rc;
         {
             const Unlocked unlocked;
+            dq = at::empty_like(*m.q); dk = at::empty_like(*m.q); dv = at::empty_like(*m.q);
+            dpq = at::empty(m.pq->sizes(), f32); dpk = at::empty(m.pq->sizes(), f32);
             rc = fn(m.q->const_data_ptr(), m.k->const_data_ptr(), m.v->const_data_ptr(), m.pq->const_data_ptr(), m.pk->const_data_ptr(), m.stride, out->const_data_ptr(),
                     lse->const_data_ptr<float>(), dout->const_data_ptr(), m.B, m.H, m.W, m.heads, m.d, m.r, m.window, m.shift, dq.mutable_data_ptr(), dk.mutable_data_ptr(),
                     dv.mutable_data_ptr(), dpq.mutable_data_ptr<float>(), dpk.mutable_data_ptr<float>(), ws->mutable_data_ptr(), (size_t)ws->numel(), stream);
@@ -198,10 +207,11 @@ PyObject* generate(PyObject*, PyObject* const* a, Py_ssize_t count)
         if (count != 7 || modes_active() || !get_generator(a + 1, a[5], a[6], &g)) Py_RETURN_NONE;
         const GenFwd fn = reinterpret_cast<GenFwd>(address(a[0]));
         const auto options = g.w_h->options().dtype(at::kBFloat16);
-        at::Tensor pq = at::empty({g.window * g.window, g.r}, options), pk = at::empty({g.window * g.window, g.r}, options);
+        at::Tensor pq, pk;
         int rc;
         {
             const Unlocked unlocked;
+            pq = at::empty({g.window * g.window, g.r}, options); pk = at::empty({g.window * g.window, g.r}, options);
             rc = fn(g.w_h->const_data_ptr<float>(), g.b_h->const_data_ptr<float>(), g.w_pq->const_data_ptr<float>(), g.w_pk->const_data_ptr<float>(), g.window, g.L, g.dh, g.r,
                     pq.mutable_data_ptr(), pk.mutable_data_ptr(), g.stream);
         }
@@ -220,10 +230,11 @@ PyObject* generate_bwd(PyObject*, PyObject* const* a, Py_ssize_t count)
         const int64_t n = (int64_t)g.window * g.window;
         if (!dpq || !dpk || dpq->size(0) != n || dpk->size(0) != n || dpq->size(1) != g.r || dpk->size(1) != g.r) Py_RETURN_NONE;
         const GenBwd fn = reinterpret_cast<GenBwd>(address(a[0]));
-        at::Tensor out[4] = {at::empty_like(*g.w_h), at::empty_like(*g.b_h), at::empty_like(*g.w_pq), at::empty_like(*g.w_pk)};
+        at::Tensor out[4];
         int rc;
         {
             const Unlocked unlocked;
+            out[0] = at::empty_like(*g.w_h); out[1] = at::empty_like(*g.b_h); out[2] = at::empty_like(*g.w_pq); out[3] = at::empty_like(*g.w_pk);
             rc = fn(g.w_h->const_data_ptr<float>(), g.b_h->const_data_ptr<float>(), g.w_pq->const_data_ptr<float>(), g.w_pk->const_data_ptr<float>(),
                     dpq->const_data_ptr<float>(), dpk->const_data_ptr<float>(), g.window, g.L, g.dh, g.r, out[0].mutable_data_ptr<float>(), out[1].mutable_data_ptr<float>(),
                     out[2].mutable_data_ptr<float>(), out[3].mutable_data_ptr<float>(), g.stream);

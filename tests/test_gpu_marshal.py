@@ -1,4 +1,10 @@
 """The native form of the binding's marshalling against its Python form: the same results, the same refusals."""
+import os
+import subprocess
+import sys
+import sysconfig
+from pathlib import Path
+
 import numpy as np
 import pytest
 import torch
@@ -137,3 +143,52 @@ def test_tensors_that_have_no_plain_memory(monkeypatch):
     for call in calls:                          # (no wrapper is made under a batched map of something else)
         a, b = both(monkeypatch, lambda: inside(torch.vmap, call)(torch.ones(2, 3, device="cuda")))
         assert torch.equal(a, b)
+
+
+# an allocator that counts its calls and those in which this thread held the interpreter's lock
+COUNTING_ALLOCATOR = r"""
+#include <Python.h>
+#include <cuda_runtime_api.h>
+static int calls, locked;
+extern "C" int count_calls() { return calls; }
+extern "C" int count_locked() { return locked; }
+extern "C" void* counting_alloc(ssize_t size, int, cudaStream_t)
+{
+    void* p = nullptr;
+    ++calls;
+    locked += PyGILState_Check();
+    return cudaMalloc(&p, size) == cudaSuccess ? p : nullptr;
+}
+extern "C" void counting_free(void* p, ssize_t, int, cudaStream_t) { cudaFree(p); }
+"""
+COUNTING_PROGRAM = r"""
+import ctypes, sys
+import torch
+torch.cuda.memory.change_current_allocator(torch.cuda.memory.CUDAPluggableAllocator(sys.argv[1], "counting_alloc", "counting_free"))
+from paper_2603_06738_b200 import binding
+assert binding._marshal is not None
+count = ctypes.CDLL(sys.argv[1])
+q = torch.randn((1, 16, 16, 1, 32), device="cuda").bfloat16()
+pq = torch.randn((256, 16), device="cuda").bfloat16()
+w = [torch.randn(s, device="cuda") for s in ((6, 8), (8,), (8, 16), (8, 16))]
+d = torch.randn((256, 16), device="cuda")
+ws = torch.empty(1 << 22, dtype=torch.uint8, device="cuda")
+before, held = count.count_calls(), count.count_locked()
+out, lse = binding.rib_window_attn_fwd(q, q, q, pq, pq, 16)
+grads = binding.rib_window_attn_bwd(q, q, q, pq, pq, out, lse, q, 16, workspace=ws)
+features = binding.rib_generate_features(*w, 16)
+generator = binding.rib_generate_features_bwd(*w, d, d, 16)
+torch.cuda.synchronize()
+print(count.count_calls() - before, count.count_locked() - held)
+"""
+
+
+def test_results_are_allocated_without_the_interpreters_lock(tmp_path):
+    source, lib = tmp_path / "alloc.cpp", tmp_path / "alloc.so"
+    source.write_text(COUNTING_ALLOCATOR)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-shared", "-fPIC", f"-I{sysconfig.get_path('include')}", f"-I{cuda}/include", str(source), f"-L{cuda}/lib64", "-lcudart", "-o", str(lib)], check=True)
+    run = subprocess.run([sys.executable, "-c", COUNTING_PROGRAM, str(lib)], cwd=Path(__file__).resolve().parent.parent, capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr
+    calls, locked = map(int, run.stdout.split()[-2:])
+    assert calls >= 13 and locked == 0, run.stdout      # 2 + 5 + 2 + 4 results
