@@ -52,13 +52,14 @@ struct Frame {
     static constexpr uint32_t kOffKp = kOffKc + kStages * kContentBytes;
     static constexpr uint32_t kOffV = kOffKp + kStages * kPos;
     static constexpr uint32_t kOffBar = kOffV + kStages * kContentBytes;
-    // barriers: query buffers, ring stages, scores there (per buffer), P there (2 tile + parity of the block), P read (per buffer),
-    // completed PV per tile, merge per tile and quarter of the rows, drain per issuing warp.  A parity wait cannot tell "a phase ahead"
-    // or "a phase behind" from its own, so every barrier is one whose next phase needs what its waiters do after this one, and whose
-    // phase before they know to be complete: P of a tile's block b + 2 needs the scores that overwrite P of block b.  (By buffer it is
-    // not: the phase before belongs to the other tile, whose PV another warp issues.)
-    enum Bar { kQFull = 0, kQEmpty = 2, kQPos = 4, kFull = 6, kEmpty = kFull + kStages, kSFull = kEmpty + kStages, kPReady = kSFull + kBuffers,
-               kPFree = kPReady + 4, kPVDone = kPFree + kBuffers, kMerge = kPVDone + 2, kDrain = kMerge + 8, kNumBars = kDrain + 3 };
+    // barriers: query buffers, ring stages, scores there, P there and PV completed (each 2 tile + parity of the block, on_block), merge per
+    // tile and quarter of the rows, drain per issuing warp.  A parity wait cannot tell "a phase ahead" or "a phase behind" from its own,
+    // so every barrier is one whose next phase needs what its waiters do after this one, and whose phase before they know to have
+    // arrived: scores of a tile's block b + 2 need PV of block b, PV needs P, P the scores, and scores of block b are issued after PV
+    // of block b - 2 was seen.  (Per buffer neither holds: the phase before belongs to the other tile.  Nor does it follow that a
+    // commit has arrived when another one behind the same contractions has.  tests/test_frame_barriers.py is a model of it.)
+    enum Bar { kQFull = 0, kQEmpty = 2, kQPos = 4, kFull = 6, kEmpty = kFull + kStages, kSFull = kEmpty + kStages, kPReady = kSFull + 4,
+               kPVDone = kPReady + 4, kMerge = kPVDone + 4, kDrain = kMerge + 8, kNumBars = kDrain + 3 };
     static constexpr uint32_t kOffMisc = kOffBar + kNumBars * 8;                 // tmem base, abort flags
     static constexpr uint32_t kOffMerge = (kOffMisc + 16 + 15) & ~15u;           // [2 item parities][2 tiles][2 halves][128 rows] (max, sum)
     static constexpr uint32_t kSmemBytes = kOffMerge + 8 * kTile * 8 + 1024;     // + slack for manual alignment
@@ -171,6 +172,10 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
     auto bar = [&](int i) { return base + L::kOffBar + 8u * i; };
+    // of kSFull, kPReady, kPVDone: the barrier of a tile's block and the parity of its phase.  (Blocks -1 and -2 have the parity that a
+    // barrier without a completed phase answers yes to.)
+    auto on_block = [&](int which, int tile, uint32_t block) { return bar(which + 2 * tile + (block & 1)); };
+    auto parity = [](uint32_t block) { return (block >> 1) & 1; };
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + L::kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + L::kOffMisc + 4);
 
@@ -180,11 +185,10 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     if (threadIdx.x == 0) {
         abort_flag[0] = 0; abort_flag[1] = 0;   // [1] stays 0: used by the drain waits
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bar(L::kQFull + i), 1); mbar_init(bar(L::kQEmpty + i), 1); mbar_init(bar(L::kQPos + i), 1); mbar_init(bar(L::kPVDone + i), 1);
+            mbar_init(bar(L::kQFull + i), 1); mbar_init(bar(L::kQEmpty + i), 1); mbar_init(bar(L::kQPos + i), 1);
             for (int q4 = 0; q4 < 4; ++q4) mbar_init(bar(L::kMerge + 4 * i + q4), 2);
         }
-        for (int i = 0; i < kBuffers; ++i) { mbar_init(bar(L::kSFull + i), 1); mbar_init(bar(L::kPFree + i), 1); }
-        for (int i = 0; i < 4; ++i) mbar_init(bar(L::kPReady + i), 8);
+        for (int i = 0; i < 4; ++i) { mbar_init(bar(L::kSFull + i), 1); mbar_init(bar(L::kPReady + i), 8); mbar_init(bar(L::kPVDone + i), 1); }
         for (int s = 0; s < kStages; ++s) { mbar_init(bar(L::kFull + s), 1); mbar_init(bar(L::kEmpty + s), 2); }     // empty: both tiles' PV
         for (int i = 0; i < 3; ++i) mbar_init(bar(L::kDrain + i), 1);
         fence_barrier_init();
@@ -278,8 +282,8 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         // ===================== issuers: warp 1 the scores of both query tiles, warps 2 and 3 PV of tile 0 and 1; the whole warp walks and waits
         constexpr uint64_t kDesc64 = smem_desc_const(16, 512, kSwizzle64B), kDesc32 = smem_desc_const(16, 256, kSwizzle32B);
         constexpr uint64_t kDescP = R == 16 ? kDesc32 : kDesc64;
-        uint32_t io = 0, blk = 0, sb = warp == 3 ? 1 : 0, use = 0;      // sb, use: unit mod and div kBuffers
-        auto next_unit = [&](uint32_t by) { sb += by; if (sb >= kBuffers) { sb -= kBuffers; ++use; } };
+        uint32_t io = 0, blk = 0, sb = warp == 3 ? 1 : 0;      // sb: unit mod kBuffers
+        auto next_unit = [&](uint32_t by) { sb += by; if (sb >= kBuffers) sb -= kBuffers; };
         for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++io) {
             const int nblk = (decode_live_item(p.live, item).patches + 1) >> 1;
             const uint32_t buf = io & 1;
@@ -292,10 +296,9 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     const uint64_t kc = smem_desc_at(kDesc64, base + L::kOffKc + st * kContentBytes), kp = smem_desc_at(kDescP, base + L::kOffKp + st * kPos);
 #pragma unroll
                     for (int qt = 0; qt < 2; ++qt) {
-                        // The scores overwrite the columns that PV of three units before reads P from: it has completed.  (The barrier is the
-                        // buffer's own, so that its next phase cannot complete before this one is seen; no phase completed answers yes
-                        // to parity 1, which the first three units ask for.)
-                        if (!mbar_wait_warp(bar(L::kPFree + sb), (use - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                        // The scores overwrite the columns that PV of three units before, one of the other tile, reads P from: it has completed.
+                        const uint32_t before = blk - 2 + qt;
+                        if (!mbar_wait_warp(on_block(L::kPVDone, qt ^ 1, before), parity(before), abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
                         if (elect_one()) {
                             const uint64_t qc = smem_desc_at(kDesc64, base + L::kOffQc + (2 * buf + qt) * kContentBytes);
@@ -308,7 +311,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                             }
                             mma_ss(d_s, qc, kc, kIdescS, 1u);
                             mma_ss(d_s, qc + 2, kc + 2, kIdescS, 1u);          // + 32 bytes: second K16 step of the content rows
-                            mma_commit(bar(L::kSFull + sb));
+                            mma_commit(on_block(L::kSFull, qt, blk));
                             if (qt == 1 && j == nblk - 1) mma_commit(bar(L::kQEmpty + buf));
                         }
                         __syncwarp();
@@ -318,7 +321,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     // P of the unit is there.  (The first block of an item overwrites O: the softmax warps have read it before they
                     // arrive here for that block.)
                     if (!mbar_wait_warp(bar(L::kFull + st), (blk / kStages) & 1, abort_flag, p.status) ||
-                        !mbar_wait_warp(bar(L::kPReady + 2 * (warp - 2) + (blk & 1)), (blk >> 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                        !mbar_wait_warp(on_block(L::kPReady, warp - 2, blk), parity(blk), abort_flag, p.status)) { ok = false; break; }
                     tc_fence_after();
                     if (elect_one()) {
                         const uint64_t vd = smem_desc_at(kDesc64, base + L::kOffV + st * kContentBytes);
@@ -329,8 +332,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                             mma_ts(d, a, vd + 64 * kk, kIdescPV, (j == 0 && (kk & 3) == 0) ? 0u : 1u);
                             mma_ts(d, a + 32, vd + 64 * kk, kIdescPV, 1u);
                         }
-                        mma_commit(bar(L::kPFree + sb));
-                        mma_commit(bar(L::kPVDone + warp - 2));
+                        mma_commit(on_block(L::kPVDone, warp - 2, blk));
                         mma_commit(bar(L::kEmpty + st));
                     }
                     __syncwarp();
@@ -354,7 +356,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         float2* const merge_sets = reinterpret_cast<float2*>(base_ptr + L::kOffMerge) + qt * 2 * kTile;
         const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
         const float rescale_threshold = 8.0f / p.scale_log2; // raw-logit units: probabilities stay <= 2^8 relative to the reference
-        uint32_t blk = 0, nmerge = 0, sb = qt, use = 0;      // sb, use: (2 blk + qt) mod and div kBuffers
+        uint32_t blk = 0, nmerge = 0;
         for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++nmerge) {
             const LiveItem c = decode_live_item(p.live, item);
             const int nblk = (c.patches + 1) >> 1;
@@ -362,8 +364,9 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             const bool edge = c.wy * p.geom.M + p.geom.s + p.geom.M > p.H || c.wx * p.geom.M + p.geom.s + p.geom.M > p.W;
             float m_used = -INFINITY, l = 0.f;
             for (int j = 0; j < nblk; ++j, ++blk) {
+                const uint32_t sb = (2 * blk + qt) % kBuffers;
                 // warp-uniform outcome: the TMEM accesses below are warp-collective
-                if (!mbar_wait_warp(bar(L::kSFull + sb), use & 1, abort_flag, p.status)) { ok = false; break; }
+                if (!mbar_wait_warp(on_block(L::kSFull, qt, blk), parity(blk), abort_flag, p.status)) { ok = false; break; }
                 tc_fence_after();
                 uint32_t s[2][32];
                 tmem_ld32(t_half + sb * kTile, s[0]);
@@ -398,7 +401,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     // is exact after the final normalisation because l carries the same reference.
                     const bool need = mx > m_used + rescale_threshold;
                     if (__any_sync(0xffffffffu, need)) {
-                        if (!mbar_wait_warp(bar(L::kPVDone + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                        if (!mbar_wait_warp(on_block(L::kPVDone, qt, blk - 1), parity(blk - 1), abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
                         const float factor = need ? ex2_approx(__fmul_rn(m_used, p.scale_log2) - __fmul_rn(mx, p.scale_log2)) : 1.f;
                         if (need) { l *= factor; m_used = mx; }
@@ -433,15 +436,10 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     tmem_st8(t_half + sb * kTile + 32 + 8 * ch, lo);
                 }
                 l += (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
-                // The epilogue waits for this block's PV.  A parity wait cannot tell "two phases ahead" from "not yet", so the
-                // phase before it is seen here, while P of this block is still held back and its own phase cannot complete.
-                if (j == nblk - 1 && blk > 0 && !mbar_wait_warp(bar(L::kPVDone + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(L::kPReady + 2 * qt + (blk & 1)));
-                sb += 2;
-                if (sb >= kBuffers) { sb -= kBuffers; ++use; }
+                if (lane == 0) mbar_arrive(on_block(L::kPReady, qt, blk));
             }
             if (!ok) break;
             // ---- merge the two key halves and write this thread's 16 output columns
@@ -451,7 +449,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             if (lane == 0) mbar_arrive(bar(L::kMerge + 4 * qt + quarter));
             // The partner's (m, l) must be there and the item's last PV must have completed.
             if (!mbar_wait_warp(bar(L::kMerge + 4 * qt + quarter), nmerge & 1, abort_flag, p.status) ||
-                !mbar_wait_warp(bar(L::kPVDone + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                !mbar_wait_warp(on_block(L::kPVDone, qt, blk - 1), parity(blk - 1), abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
             uint32_t oa[16], ob[16];
             tmem_ld16(t_o + half * 16, oa);
