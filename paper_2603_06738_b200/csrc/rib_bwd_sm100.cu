@@ -811,11 +811,13 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
 
     const int windows = p.pairs / p.heads;   // pairs of one head
     const int in_line = tables == 1 ? p.pairs : windows;      // pairs whose sums go to one table
-    // a block takes a run of per_group pairs (of one head, with head-wise tables)
-    // (measured on the training configuration: 4 pairs per block 56 us, 2 or 8: 60, 16: 70 -- more blocks in flight
-    // matter more to this kernel than fewer atomics)
-    const int per_group = in_line >= 1024 ? 8 : in_line >= 16 ? 4 : 1;
-    const unsigned groups = (tables == 1 ? 1u : (unsigned)p.heads) * (unsigned)((in_line + per_group - 1) / per_group);
+    // A block takes a run of pairs (of one head, with head-wise tables): four, or one where there are fewer than sixteen.  Measured, us with
+    // the launch, for runs of 1 / 2 / 4 / 8 / 16 pairs: 864 pairs of 1024 tokens at rank 16 84 / 62 / 58 / 60 / 71, 1728 pairs 168 / 115 / 101 / 109 /
+    // 128, 3456 pairs 265 / 210 / 189 / 203 / 242, 1728 pairs at rank 32 305 / 203 / 168 / 168 / 184; 12 pairs 6.6 / 8.4 / 8.6, 24 pairs 8.6 / 8.7 / 8.7, 48 pairs
+    // 12.7 / 10.4 / 10.6: more blocks in flight matter more to this kernel than fewer atomics.  Runs of eight where the grid's y has no room.
+    auto groups_of = [&](int run) { return (tables == 1 ? 1ll : (long long)p.heads) * ((in_line + run - 1) / run); };
+    const int per_group = in_line < 16 ? 1 : groups_of(4) <= 65535 ? 4 : 8;
+    const unsigned groups = (unsigned)groups_of(per_group);
     dim3 grid_fin((unsigned)(p.n / 32), groups, (unsigned)(R / 16));
     { ProfileScope scope(RIB_KERNEL_BWD_FINISH, stream); (p.narrow ? rib_bwd_finish_kernel<R, true> : rib_bwd_finish_kernel<R, false>)<<<grid_fin, 128, 0, stream>>>(ap, per_group); }
     return cudaGetLastError();
