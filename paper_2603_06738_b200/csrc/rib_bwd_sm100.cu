@@ -4,14 +4,14 @@
 // Shapes: d = 32, r = 16 or 32 (template argument R), window side M a multiple of 16, shift a multiple of 8 (as
 // the forward).  The text below describes R = 16.  With R = 32 the RIB rows fill their 64-byte slots, dK~ and dQ~ are
 // 64 columns wide, and tensor memory has no room left for dS^T: dK~ then takes the dS tile in shared memory as a
-// K-major A operand (that tile's barrier counts two readers), and the arithmetic warps read the scores as 16-lane
-// fragments (4 key rows x 8 queries per thread), which quarters their reads of the per-query (-lse, -D) values.
+// K-major A operand (that tile's barrier counts two readers).  S^T and dP^T of both halves of a tile are then issued
+// together (N = 128), once both groups of arithmetic warps have read those of the tile before.
 //
 // Work item = one (batch, window, head) pair x one key block J of 128 tokens.  A persistent CTA keeps
 // K~_J = [k, Pk] and V_J in shared memory and dV_J, dK~_J in tensor memory, and walks the query tiles
 // I of the window.  Everything is computed transposed (keys on the TMEM lanes) so that P^T and dS^T
 // feed the dV and dK~ contractions straight from tensor memory.  The unit of the pipeline is a
-// half-tile u = (I, h): the 64 queries of patch h of tile I,
+// half-tile u = (I, h): the 64 queries of patch h of tile I (R = 32: both patches for the first two lines),
 //     S^T  = K~_J Q~_u^T                    (M128 N64 K48: content rows 2 x K16, RIB rows 1 x K16)
 //     dP^T = V_J dO_u^T                     (M128 N64 K32)
 //     P^T  = exp2(S^T * log2e/sqrt(d) - lse_i * log2e),   dS^T = P^T o (dP^T - D_i)     (ALU warps)
@@ -34,7 +34,7 @@
 // instructions from several warps at once, and one thread issuing everything was the bottleneck):
 // warp 1 issues S^T and dP^T, warp 2 (also the TMEM allocator) dV and dK~, warp 3 dQ~; warps 4-11
 // P/dS arithmetic of the even half-tiles, warps 12-19 of the odd ones (a warp per 32 key rows and 32
-// queries); warps 20-23 drain dQ~ after every tile and dK~/dV after every item.  Every wait is bounded.
+// queries, a thread 2 key rows x 4 queries of each of its four 16 x 16 pieces); warps 20-23 drain dQ~ after every tile and dK~/dV after every item.  Every wait is bounded.
 // What sets the pace is the latency of the loop  scores -> arithmetic -> gradient MMAs -> buffers free
 // divided by the two half-tiles in flight, so every buffer is handed back as early as its last reader
 // allows: the score accumulators when the arithmetic warps hold them in registers (long before their
@@ -126,7 +126,7 @@ __device__ __forceinline__ ItemCoord decode_item(const BwdParams& p, int item)
 
 // kPartial: H or W is not a multiple of the window (but of 8); windows are laid over the map extended to Hp x Wp and
 // an 8x8 patch of the extension holds no tokens.  TMA fills such patches with zeros; what is left to do: a key row that
-// is no token gets P^T = dS^T = 0 (a thread of the arithmetic warps is a key row, and the 64 rows of a patch share the
+// is no token gets P^T = dS^T = 0 (the 32 key rows of an arithmetic warp lie in one patch of 64, whose rows share the
 // answer), a query that is no token reads -inf for -lse (written by the preparation kernel), i.e. probability 0,
 // and nothing is stored for either.
 template <int R, bool kPartial>
@@ -337,7 +337,7 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         __syncwarp();
         mbar_wait(bar(kDrain + warp - 1), 0, abort_flag + 1, p.status);
     } else if (warp >= 4 && warp < 20) {
-        // ===== P^T and dS^T: group h = warps 4 + 8h .. 11 + 8h takes half-tile (I, h); one thread per key row and 32 queries
+        // ===== P^T and dS^T: group h = warps 4 + 8h .. 11 + 8h takes half-tile (I, h), a warp 32 key rows and 32 queries
         const int h = (warp - 4) >> 3;
         const int cg = ((warp - 4) >> 2) & 1;                // queries 32 cg .. 32 cg + 31 of the half-tile
         const int quarter = warp & 3;
