@@ -12,9 +12,9 @@
 //
 // What bounds it: the serial program of the softmax warps, 3300 cycles per block of both query tiles of which the exp unit is busy
 // 2048, beside 42 MMAs (2100 cycles of issue, from three warps).  Measured (180 x 320 tokens, 32 x 32 windows, 6 heads of 32
-// channels, rank 16, with the launch): 158 us = 343 TFLOP/s of the layer's own flops; one warp issuing everything 176 us (it held
-// a unit for 16 + 5 MMAs and the wait between them, 1600 cycles), the any-shape kernel 13 460 us.  Asking for the next scores
-// before P is handed over, as the general kernel does, took 178 us: P then waits for them.
+// channels, rank 16): 165 us a pass = 328 TFLOP/s of the layer's own flops (161 us on inputs that the pass before has read, too); one
+// warp issuing everything 179 us (it held a unit for 16 + 5 MMAs and the wait between them, 1600 cycles), the any-shape kernel 13 460 us.
+// Asking for the next scores before P is handed over, as the general kernel does, is 13 % slower: P then waits for them.
 // Error of `out` against float64 as that kernel's (1.7e-3, the rounding to bf16; 4 parts in a million more at most), of lse below it.
 //
 // Work item = one (batch, window, head) pair x two query tiles of 128 tokens (two 8x8-token patches each).  Only patches that

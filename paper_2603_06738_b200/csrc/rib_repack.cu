@@ -115,12 +115,13 @@ __global__ void __launch_bounds__(256) rib_rank_tail_grads_kernel(const __nv_bfl
 
 // All copies of a pass in one launch.  A copy: rows of 4-byte words, one side `wide` words a row (a multiple of 4, 16-byte aligned),
 // the other `narrow`; widen: narrow to wide with zeros behind, else wide to narrow.  A thread moves 16-byte pieces of the wide side,
-// which is one vector access there and up to four word accesses on the narrow side; a block 1024 of them, all loads of a thread
-// before its stores.
-struct RowCopy { const uint32_t* src; uint32_t* dst; size_t rows; unsigned first_block; int narrow, wide, widen; };
+// which is one vector access there and up to four word accesses on the narrow side; a block as many whole rows as make up 1024 of them
+// (the widest rows are 24 pieces), all loads of a thread before its stores.
+struct RowCopy { const uint32_t* src; uint32_t* dst; size_t rows; unsigned first_block, rows_per_block; int narrow, wide, widen; };
 constexpr int kMostCopies = 8, kCopyPieces = 4;
-struct RowCopies {
-    RowCopy copy[kMostCopies];
+template <int kMost>
+struct RowCopyList {
+    RowCopy copy[kMost];
     int count;
     unsigned blocks;
     // src rows of ws words -> dst rows of wd words
@@ -130,24 +131,30 @@ struct RowCopies {
         c.src = static_cast<const uint32_t*>(src); c.dst = static_cast<uint32_t*>(dst); c.rows = rows;
         c.widen = wd >= ws; c.wide = c.widen ? wd : ws; c.narrow = c.widen ? ws : wd;
         c.first_block = blocks;
-        blocks += (unsigned)((rows * (size_t)(c.wide / 4) + 256 * kCopyPieces - 1) / (256 * kCopyPieces));
+        c.rows_per_block = 256u * kCopyPieces / (unsigned)(c.wide / 4);
+        blocks += (unsigned)((rows + c.rows_per_block - 1) / c.rows_per_block);
     }
 };
+using RowCopies = RowCopyList<kMostCopies>;
 
-__global__ void __launch_bounds__(256) rib_copy_rows_kernel(const __grid_constant__ RowCopies all)
+// A copy on its own has an instantiation of its own, and a block begins with a row: with the parameters of eight copies, a search among
+// them and a 64-bit division for the first row the gate's backward with 96 channels on 2 x 64 x 64 pixels took 69.1 us, so 67.0 (three
+// such copies among its 14 launches; one copy kernel per tensor with scalar parameters 67.3).
+template <int kMost>
+__global__ void __launch_bounds__(256) rib_copy_rows_kernel(const __grid_constant__ RowCopyList<kMost> all)
 {
     int which = 0;
-    while (which + 1 < all.count && blockIdx.x >= all.copy[which + 1].first_block) ++which;
+    if (kMost > 1)
+        while (which + 1 < all.count && blockIdx.x >= all.copy[which + 1].first_block) ++which;
     const RowCopy& c = all.copy[which];
     const unsigned per_row = (unsigned)c.wide / 4u;
-    const size_t piece0 = (size_t)(blockIdx.x - c.first_block) * (256 * kCopyPieces), row0 = piece0 / per_row;
-    const unsigned rem = (unsigned)(piece0 - row0 * per_row) + threadIdx.x;
+    const size_t row0 = (size_t)(blockIdx.x - c.first_block) * c.rows_per_block;
     uint4 v[kCopyPieces];
     auto place = [&](int k, size_t& row, int& w0) {
-        const unsigned at = rem + 256u * k, r = at / per_row;
+        const unsigned at = threadIdx.x + 256u * k, r = at / per_row;
         row = row0 + r;
         w0 = 4 * (int)(at - r * per_row);
-        return row < c.rows;
+        return r < c.rows_per_block && row < c.rows;
     };
 #pragma unroll
     for (int k = 0; k < kCopyPieces; ++k) {
@@ -176,10 +183,12 @@ __global__ void __launch_bounds__(256) rib_copy_rows_kernel(const __grid_constan
     }
 }
 
-cudaError_t run_copies(const RowCopies& all, cudaStream_t stream, int* launches)
+template <int kMost>
+cudaError_t run_copies(const RowCopyList<kMost>& all, cudaStream_t stream, int* launches)
 {
     if (!all.blocks) return cudaSuccess;
-    rib_copy_rows_kernel<<<all.blocks, 256, 0, stream>>>(all);
+    if (kMost > 1 && all.count == 1) return run_copies(RowCopyList<1>{{all.copy[0]}, 1, all.blocks}, stream, launches);
+    rib_copy_rows_kernel<kMost><<<all.blocks, 256, 0, stream>>>(all);
     ++*launches;
     return cudaGetLastError();
 }
@@ -187,7 +196,7 @@ cudaError_t run_copies(const RowCopies& all, cudaStream_t stream, int* launches)
 // bf16 image rows of `ws` elements -> rows of `wd` elements (one of the two a multiple of 8, the other smaller or equal)
 cudaError_t resize_rows(const void* src, int ws, void* dst, int wd, size_t rows, cudaStream_t stream, int* launches)
 {
-    RowCopies one{};
+    RowCopyList<1> one{};
     one.add(src, ws / 2, dst, wd / 2, rows);
     return run_copies(one, stream, launches);
 }

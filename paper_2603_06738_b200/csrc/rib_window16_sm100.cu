@@ -5,10 +5,11 @@
 // memory) exceeds its arithmetic.  Here a CTA keeps to one head (CTA c: head c mod heads), stages the head's RIB rows once,
 // takes whole windows one after the other and lets them overlap, and no gradient but those of the tables is summed
 // outside the chip.  What bounds it: the serial program of the softmax (arithmetic) warps.  A unit of the forward (128 rows x 256
-// keys) takes about 3900 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) about 3200: 1050 of loads
-// and exponentials, 1600 of stores of P and dS and their fences, with 1470 cycles of MMAs beside it.  Measured (4 x 96 x 96 tokens,
-// 12 heads of 16 channels, rank 24, shift 8, masked, by event hooks): forward 82 -> 60 us, backward 30 + 140 + 46 -> 12 (two
-// clearings) + 101 us, both calls 288 -> 156 us; backward on 10 x 64 x 64 tokens, 6 heads of 32 channels, rank 16: 20 + 66 + 23 -> 12 + 71 us.
+// keys) takes about 3900 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) 3700 at rank 16 and 32 channels
+// (3300 at rank 24 and 16 channels): 450 until its scores are there, 1150 (1240) of loads and exponentials, 2100 (1600) of waiting for
+// the buffers of P and dS, stores into them and fences, with 1470 cycles of MMAs beside it.  Measured by event hooks against the general
+// kernels (4 x 96 x 96 tokens, 12 heads of 16 channels, rank 24, shift 8, masked): forward 82 -> 60 us, backward 30 + 140 + 46 -> 13 (two
+// clearings) + 99 us, both calls 288 -> 154 us; backward on 10 x 64 x 64 tokens, 6 heads of 32 channels, rank 16: 20 + 66 + 23 -> 13 + 70 us.
 //
 // Windows may be shifted (multiples of 8), masked, or reach beyond the map (sides multiples of 8): a window is four 8x8-token
 // patches (one TMA box each), and a query patch attends to a key patch or not.
