@@ -12,7 +12,7 @@
 //
 // What bounds it: the serial program of the softmax warps, 3300 cycles per block of both query tiles of which the exp unit is busy
 // 2048, beside 42 MMAs (2100 cycles of issue, from three warps).  Measured (180 x 320 tokens, 32 x 32 windows, 6 heads of 32
-// channels, rank 16): 165 us a pass = 328 TFLOP/s of the layer's own flops (161 us on inputs that the pass before has read, too); one
+// channels, rank 16): 163 us a pass = 332 TFLOP/s of the layer's own flops (160 us on inputs that the pass before has read, too); one
 // warp issuing everything 179 us (it held a unit for 16 + 5 MMAs and the wait between them, 1600 cycles), the any-shape kernel 13 460 us.
 // Asking for the next scores before P is handed over, as the general kernel does, is 13 % slower: P then waits for them.
 // Error of `out` against float64 as that kernel's (1.7e-3, the rounding to bf16; 4 parts in a million more at most), of lse below it.
@@ -82,6 +82,8 @@ struct FrameParams {
     WindowGeom geom;           // sides of the extended map, window, shift
     int terms;                 // terms of the scaled query RIB rows in use: 1 or kTerms
     float scale_log2;          // log2(e) / sqrt(d)
+    float rescale_threshold;   // raw-logit units: probabilities stay <= 2^8 relative to the reference.  (Here and not in a register of the softmax
+                               // warps, which have none to spare: 161.4 -> 159.5 us on the map above, inputs read before.)
     float inv_sqrt_d, inv_sqrt_r;
     float pos_scale;           // sqrt(d / r): folds 1/sqrt(r) into the content scale
     long long pos_head_stride;
@@ -355,7 +357,6 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         // [half][row]; two sets, so that a warp that is an item ahead of its partner does not overwrite what that one still reads
         float2* const merge_sets = reinterpret_cast<float2*>(base_ptr + L::kOffMerge) + qt * 2 * kTile;
         const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
-        const float rescale_threshold = 8.0f / p.scale_log2; // raw-logit units: probabilities stay <= 2^8 relative to the reference
         uint32_t blk = 0, nmerge = 0;
         for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++nmerge) {
             const LiveItem c = decode_live_item(p.live, item);
@@ -399,7 +400,7 @@ rib_fwd_frame_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 } else {
                     // Move the reference (and rescale O, l) only when the maximum grew by more than the threshold; the result
                     // is exact after the final normalisation because l carries the same reference.
-                    const bool need = mx > m_used + rescale_threshold;
+                    const bool need = mx > m_used + p.rescale_threshold;
                     if (__any_sync(0xffffffffu, need)) {
                         if (!mbar_wait_warp(on_block(L::kPVDone, qt, blk - 1), parity(blk - 1), abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
@@ -523,6 +524,7 @@ cudaError_t launch_fwd_frame(const Problem& p, cudaStream_t stream)
     fp.H = p.H; fp.W = p.W; fp.heads = p.heads; fp.d = p.d; fp.r = p.r;
     fp.geom = WindowGeom{p.Hp, p.Wp, p.M, p.s};
     fp.scale_log2 = (float)(1.4426950408889634 / sqrt((double)d));
+    fp.rescale_threshold = 8.0f / fp.scale_log2;
     fp.pos_scale = sqrtf(d / r);
     fp.terms = d == r || d == 4.f * r || 4.f * d == r ? 1 : kTerms;      // sqrt(d / r) a power of two: the product is a bf16 number
     fp.pos_head_stride = p.pos_head_stride;
