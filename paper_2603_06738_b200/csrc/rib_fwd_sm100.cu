@@ -14,9 +14,13 @@
 //                        accumulating MMAs on separately staged shared-memory slabs)
 //     P_q = exp2((S_q - m) * log2e / sqrt(d))      softmax warps, fp32 -> bf16 written back to TMEM
 //     O_q += P_q V      (A operand from TMEM, V as an MN-major shared-memory tile)
-// for the two query tiles q = 0, 1.  The two tiles run as independent pipelines; the S accumulator is
-// released as soon as the scores are in registers, so the next block's S_q is computed while the
-// exponentials of this one are being evaluated.
+// for the two query tiles q = 0, 1.
+// Tensor memory: three score buffers of 128 columns; unit u = 2 * block + query tile uses buffer u mod 3.  A softmax thread writes P
+// over its own scores (keys 0-31 of its half over the columns of keys 32-63 and so on, see the PV issuers), so a buffer is handed
+// back with P in it and S(u + 3) goes there once PV(u) has completed: scores of one tile's next block are under way while the
+// other tile's exponentials run, and between a block's scores and its P a softmax warp waits for nobody.  (Scores in one buffer per
+// tile and P in columns of its own, each with a barrier "free" that every block asked for and answered: 256 x 256 tokens in windows of 64
+// 425 -> 393 us, and with the exponentials in pieces of 16 keys 369; 360 x 640 in windows of 64 1400 -> 1220.)
 //
 // Two threads own a query row: one takes keys 0-63 of every block and the other keys 64-127, which
 // puts four softmax warps on every SM sub-partition.
@@ -35,8 +39,7 @@
 //   merge.  A row whose scores leave the representable range (a key more than ~69 nat above the
 //   reference, or a polynomial-path key more than ~83 nat below) shows up as l >= 2^100 or not finite:
 //   the item is then noted in shared memory and redone by the exact form in a second pass of the
-//   same launch.  Every third or fourth pair of exponentials (kPolyMask) is evaluated on the FMA and
-//   integer pipes instead of the MUFU.
+//   same launch.  Every fourth pair of exponentials (kPolyMask) is evaluated on the FMA and integer pipes instead of the MUFU.
 //   Exact form (second pass): classic online softmax per key half
 //   with a running maximum, lazy rescaling of O, separate accumulators and a log-sum-exp merge.
 //   On maps with partial windows (kPartial) only patches that hold tokens are walked (LiveWindows in rib_sm100_common.cuh), and
@@ -49,13 +52,13 @@
 // it is about to fetch; warp 1 issues S for both query tiles, warps 2 and 3 issue PV for tile 0 and 1 (three
 // issuers, because what bounds the bare pipeline is the serial time of an issuing warp: a group of MMAs holds
 // its issuer for several hundred cycles, and with S and PV in one warp the two dependency loops
-// scores -> S free -> next scores  and  P ready -> PV -> P free  went through the same instruction stream);
+// scores -> P ready  and  PV -> scores  went through the same instruction stream);
 // warp 2 owns the TMEM allocation; warps 4-11 softmax/epilogue of query tile 0 (4-7 first half of the keys,
 // 8-11 second half), warps 12-19 of query tile 1.  Every wait is bounded.
 #include "rib_sm100_common.cuh"
 
 #ifndef RIB_FWD_POLY_MASK
-#define RIB_FWD_POLY_MASK 0x88u         // of every 8 score pairs: which go to the FMA pipe
+#define RIB_FWD_POLY_MASK 0x88u         // of every 8 score pairs: which go to the FMA pipe (three of eight: 369 -> 374 us, other two: 375)
 #endif
 
 namespace rib {
@@ -68,9 +71,11 @@ constexpr int kThreads = 640;
 constexpr int kMaxRedo = 64;          // items a CTA can note for the exact pass (more: all of its items are redone)
 constexpr uint32_t kPolyMask = RIB_FWD_POLY_MASK;
 
-// kSFull .. kOFree: one per query tile; kDrain: one per issuing warp; kMerge: 4 * tile + quarter of the rows
-enum Bar { kQFull = 0, kQEmpty = 2, kQPos = 4, kSFull = 6, kSFree = 8, kPReady = 10, kPFree = 12, kOFree = 14, kDrain = 16, kMerge = 20,
-           kKFull = 28, kKEmpty = kKFull + kStages, kVFull = kKEmpty + kStages, kVEmpty = kVFull + kStages,
+// kSFull, kPReady, kPVDone: 2 * tile + parity of the block (on_block): a parity wait cannot tell "a phase ahead" or "a phase behind" from
+// its own, so the phase before must be known to have arrived and the next must need what the waiter does after this one
+// (tests/test_fwd_barriers.py is a model of it); kDrain: one per issuing warp; kMerge: 4 * tile + quarter of the rows
+enum Bar { kQFull = 0, kQEmpty = 2, kQPos = 4, kSFull = 6, kPReady = 10, kPVDone = 14, kDrain = 18, kMerge = 21,
+           kKFull = 29, kKEmpty = kKFull + kStages, kVFull = kKEmpty + kStages, kVEmpty = kVFull + kStages,
            kNumBars = kVEmpty + kStages };
 
 // shared-memory map (offsets from a 1024-byte aligned base) for RIB rank R = 16 (32-byte RIB rows, SWIZZLE_32B) or
@@ -88,15 +93,17 @@ struct Layout {
     static constexpr uint32_t kOffBar = kOffHalfOnes + kContentBytes;
     static constexpr uint32_t kOffMisc = kOffBar + kNumBars * 8;                 // tmem base, abort flags, redo count
     static constexpr uint32_t kOffRedo = kOffMisc + 16;                          // [kMaxRedo] item ordinals of the exact pass
-    static constexpr uint32_t kOffMerge = kOffRedo + kMaxRedo * 4;               // [2 tiles][2 halves][128 rows] (max, sum)
-    static constexpr uint32_t kSmemBytes = kOffMerge + 4 * kTile * 8 + 1024;     // + slack for manual alignment
+    static constexpr uint32_t kOffMerge = (kOffRedo + kMaxRedo * 4 + 15) & ~15u;               // [2 item parities][2 tiles][2 halves][128 rows] (max, sum)
+    static constexpr uint32_t kSmemBytes = kOffMerge + 8 * kTile * 8 + 1024;     // + slack for manual alignment
     static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
     static_assert(kOffV % 1024 == 0 && kOffOnes % 1024 == 0, "swizzle atoms need aligned tiles");
 };
 
-// tensor-memory columns (fp32 accumulators; P is bf16x2, two keys per column)
+// tensor-memory columns (fp32 accumulators; P is bf16x2, two keys per column, in the second half of its key half's score columns)
 // O, exact form: [2 tiles][2 key halves][32];  fast form: [2 tiles][48] (32 value columns, the row sum, 15 unused)
-constexpr uint32_t kColS = 0, kColO = 256, kColP = 384, kTmemCols = 512;
+constexpr int kBuffers = 3;               // score / P buffers
+constexpr uint32_t kColO = kBuffers * kTile, kTmemCols = 512;
+static_assert(kColO + 4 * kD <= kTmemCols, "tensor memory has 512 columns");
 constexpr uint32_t kFastOCols = kD + 16;
 
 constexpr uint32_t kIdescS = idesc_bf16_f32(kTile, kTile, false);
@@ -189,6 +196,10 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
     auto bar = [&](int i) { return base + kOffBar + 8u * i; };
+    // of kSFull, kPReady, kPVDone: the barrier of a tile's block and the parity of its phase.  (Blocks -1 and -2 have the parity that a
+    // barrier without a completed phase answers yes to.)
+    auto on_block = [&](int which, int tile, uint32_t block) { return bar(which + 2 * tile + (block & 1)); };
+    auto parity = [](uint32_t block) { return (block >> 1) & 1; };
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + kOffMisc + 4);
     int* redo_count = reinterpret_cast<int*>(base_ptr + kOffMisc + 12);      // notes taken (duplicates included)
@@ -203,10 +214,10 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         *redo_count = 0;
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(kQFull + i), 1); mbar_init(bar(kQEmpty + i), 1); mbar_init(bar(kQPos + i), 1);
-            mbar_init(bar(kSFull + i), 1); mbar_init(bar(kSFree + i), 8); mbar_init(bar(kOFree + i), 8);
-            mbar_init(bar(kPReady + i), 8); mbar_init(bar(kPFree + i), 1);
             for (int q4 = 0; q4 < 4; ++q4) mbar_init(bar(kMerge + 4 * i + q4), 2);
         }
+        for (int i = 0; i < 4; ++i) { mbar_init(bar(kSFull + i), 1); mbar_init(bar(kPVDone + i), 1); }
+        for (int i = 0; i < 4; ++i) mbar_init(bar(kPReady + i), 8);
         for (int i = 0; i < 3; ++i) mbar_init(bar(kDrain + i), 1);
         for (int s = 0; s < kStages; ++s) {     // keys: one commit of the S issuer; values: one commit of each PV issuer
             mbar_init(bar(kKFull + s), 1); mbar_init(bar(kKEmpty + s), 1);
@@ -240,6 +251,7 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 
     // Role state that carries over from the first pass to the exact pass: block and item counters give the barrier phases.
     uint32_t blk = 0, io = 0, nmerge = 0;
+    uint32_t sb = warp == 3 || warp >= 12 ? 1u : 0u;        // score buffer of the next unit: (2 blk + tile) mod kBuffers
     uint32_t q_armed = 0, k_armed = 0, v_armed = 0;
     bool ok = true;
 
@@ -250,16 +262,12 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         const bool all_items = pass == 0 || noted > kMaxRedo;
         const int count = all_items ? my_items : noted;
         auto item_at = [&](int i) { return (int)blockIdx.x + (all_items ? i : redo_list[i]) * (int)gridDim.x; };
-        // The loading and issuing roles below ask for every item, also where they do not need it: without this read of the notes in their
-        // loops the kernel takes 0.5 to 1 % longer (16 x 96 x 96 tokens, windows of 32, rank 16: 263.1 against 260.6 us, rank 32: 278.3
-        // against 275.6; 10 x 64 x 64, windows of 64, rank 32: 285.2 against 282.5).
         // key blocks of item i of this pass
         auto blocks_at = [&](int i) { return kPartial ? (patches_of(p, decode_item(p, item_at(i))) + 1) >> 1 : nblk; };
 
         if (warp == 0) {
             // ===================== TMA producer (lane 0) and query RIB rows bf16(Pq * sqrt(d/r)) of the same item (whole warp)
             for (int i = 0; i < count && ok; ++i, ++io) {
-                (void)item_at(i);
                 const auto c = decode_item(p, item_at(i));
                 const uint32_t buf = io & 1;
                 if (io >= 2 && !mbar_wait_warp(bar(kQEmpty + buf), ((io >> 1) - 1) & 1, abort_flag, p.status)) { ok = false; break; }
@@ -341,7 +349,6 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             // and waits; one elected lane issues (this keeps descriptors in uniform registers).
             constexpr uint64_t kDesc64 = smem_desc_const(16, 512, kSwizzle64B), kDesc32 = smem_desc_const(16, 256, kSwizzle32B);
             for (int i = 0; i < count && ok; ++i, ++io) {
-                (void)item_at(i);
                 const uint32_t buf = io & 1;
                 if (!mbar_wait_warp(bar(kQFull + buf), (io >> 1) & 1, abort_flag, p.status) ||
                     !mbar_wait_warp(bar(kQPos + buf), (io >> 1) & 1, abort_flag, p.status)) { ok = false; break; }
@@ -353,24 +360,26 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     const uint64_t kp = smem_desc_at(R == 16 ? kDesc32 : kDesc64, base + kOffKp + st * kPosBytes);
 #pragma unroll
                     for (int qt = 0; qt < 2; ++qt) {
-                        // the softmax warps have taken S(b-1) of this tile out of tensor memory
-                        if (blk > 0 && !mbar_wait_warp(bar(kSFree + qt), (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                        // The scores overwrite the columns that PV of three units before, one of the other tile, reads P from: it has completed.
+                        const uint32_t before = blk - 2 + qt;
+                        if (!mbar_wait_warp(on_block(kPVDone, qt ^ 1, before), parity(before), abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
                         if (elect_one()) {
                             const uint64_t qc = smem_desc_at(kDesc64, base + kOffQc + (2 * buf + qt) * kContentBytes);
                             const uint64_t qp = smem_desc_at(R == 16 ? kDesc32 : kDesc64, base + kOffQp + (2 * buf + qt) * kPosBytes);
-                            const uint32_t d_s = tmem + kColS + qt * kTile;
+                            const uint32_t d_s = tmem + sb * kTile;
                             mma_ss(d_s, qc, kc, kIdescS, 0u);
                             mma_ss(d_s, qc + 2, kc + 2, kIdescS, 1u);          // + 32 bytes: second K16 step of the content rows
                             mma_ss(d_s, qp, kp, kIdescS, 1u);
                             if (R == 32) mma_ss(d_s, qp + 2, kp + 2, kIdescS, 1u);
-                            mma_commit(bar(kSFull + qt));
+                            mma_commit(on_block(kSFull, qt, blk));
                             if (qt == 1) {
                                 mma_commit(bar(kKEmpty + st));
                                 if (j == nb - 1) mma_commit(bar(kQEmpty + buf));
                             }
                         }
                         __syncwarp();
+                        sb = sb == kBuffers - 1 ? 0u : sb + 1;
                     }
                 }
             }
@@ -378,41 +387,41 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             // ===================================== issuers of O_q (+)= P_q V: warp 2 for query tile 0, warp 3 for tile 1
             const int qt = warp - 2;
             constexpr uint64_t kDesc64 = smem_desc_const(16, 512, kSwizzle64B);
-            const uint32_t a_p = tmem + kColP + qt * (kTile / 2);
             const uint32_t d_o = tmem + kColO + qt * 2 * kD;              // exact form: one accumulator per key half
             const uint32_t d_o1 = tmem + kColO + qt * kFastOCols;         // fast form: one accumulator
             for (int i = 0; i < count && ok; ++i, ++io) {
-                (void)item_at(i);
                 const int patches = kPartial ? patches_of(p, decode_item(p, item_at(i))) : 0, nb = kPartial ? (patches + 1) >> 1 : nblk;
                 const bool odd = kPartial && (patches & 1);
                 for (int j = 0; j < nb; ++j, ++blk) {
                     const uint32_t st = blk % kStages;
-                    // warp-uniform outcomes, so that the warp stays converged.  The first block of an item overwrites the
-                    // accumulator: the epilogue of the item before must have read it.
+                    // warp-uniform outcomes, so that the warp stays converged.  (The first block of an item overwrites the
+                    // accumulator: the softmax warps have read it before they arrive here for that block.)
                     if (!mbar_wait_warp(bar(kVFull + st), (blk / kStages) & 1, abort_flag, p.status) ||
-                        !(j > 0 || io == 0 || mbar_wait_warp(bar(kOFree + qt), (io - 1) & 1, abort_flag, p.status)) ||
-                        !mbar_wait_warp(bar(kPReady + qt), blk & 1, abort_flag, p.status)) { ok = false; break; }
+                        !mbar_wait_warp(on_block(kPReady, qt, blk), parity(blk), abort_flag, p.status)) { ok = false; break; }
                     tc_fence_after();
                     if (elect_one()) {
                         const uint32_t v_addr = base + kOffV + st * kContentBytes;
+                        const uint32_t a_p = tmem + sb * kTile + 32;       // P of a key half: the second 32 of its 64 score columns
                         if (fast) {
                             // [V | ones] as one MN-major operand of 48 columns, the second 32-column atom `lbo` bytes behind the first
-                            // (kPartial: half a block without tokens has zero rows of V and of the second atom)
+                            // (kPartial: half a block without tokens has zero rows of V and of the second atom).  The softmax warps took
+                            // the second 32 keys of a half first.
                             const uint32_t ones = kPartial && j == nb - 1 && odd ? kOffHalfOnes : kOffOnes;
                             const uint64_t v = smem_desc(v_addr, ones - (kOffV + st * kContentBytes), 512, kSwizzle64B);
 #pragma unroll
                             for (int kk = 0; kk < 8; ++kk)
-                                mma_ts(d_o1, a_p + 8 * kk, v + 64 * kk, kIdescPV1, (j == 0 && kk == 0) ? 0u : 1u);
+                                mma_ts(d_o1, a_p + (kk >> 2) * 64 + 8 * ((kk + 2) & 3), v + 64 * kk, kIdescPV1, (j == 0 && kk == 0) ? 0u : 1u);
                         } else {
                             const uint64_t v = smem_desc_at(kDesc64, v_addr);
 #pragma unroll
                             for (int kk = 0; kk < 8; ++kk)     // keys 16 kk ..: key half kk / 4 has its own accumulator
-                                mma_ts(d_o + (kk >> 2) * kD, a_p + 8 * kk, v + 64 * kk, kIdescPV, (j == 0 && (kk & 3) == 0) ? 0u : 1u);
+                                mma_ts(d_o + (kk >> 2) * kD, a_p + (kk >> 2) * 64 + 8 * (kk & 3), v + 64 * kk, kIdescPV, (j == 0 && (kk & 3) == 0) ? 0u : 1u);
                         }
-                        mma_commit(bar(kPFree + qt));
+                        mma_commit(on_block(kPVDone, qt, blk));
                         mma_commit(bar(kVEmpty + st));
                     }
                     __syncwarp();
+                    sb = sb == 0 ? 2u : sb - 1;
                 }
             }
         } else {
@@ -422,57 +431,48 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             const int quarter = warp & 3;
             const int row = quarter * 32 + lane;                 // row of the tile == TMEM lane
             const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-            const uint32_t t_s = tmem + lane_base + kColS + qt * kTile + half * 64;
-            const uint32_t t_p = tmem + lane_base + kColP + qt * (kTile / 2) + half * 32;
-            const uint32_t b_ready = bar(kPReady + qt), b_free = bar(kPFree + qt);   // P of the tile: both key halves
+            const uint32_t t_half = tmem + lane_base + half * 64;       // + buffer: own scores, own P in the second 32 columns
             const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
 
             if (fast) {
                 // ------------------------------------------------------------------ fast form
                 const uint32_t t_o1 = tmem + lane_base + kColO + qt * kFastOCols;
-                // exp2 of 32 scores against the fixed reference, packed to bf16 pairs
-                auto exp_chunk1 = [&](const uint32_t (&s)[32], float2 sc2, float2 neg2, uint32_t (&packed)[16]) {
+                // exp2 of 16 scores against the fixed reference, packed to bf16 pairs
+                auto exp_chunk1 = [&](const uint32_t (&s)[16], float2 neg2, uint32_t (&packed)[8]) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), sc2, neg2);
-                        const float2 e = ((kPolyMask >> (i & 7)) & 1u) ? ex2_poly2_ranged(x) : make_float2(ex2_approx(x.x), ex2_approx(x.y));
+                    for (int i = 0; i < 8; ++i) {
+                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), scale2, neg2);
+                        const float2 e = ((kPolyMask >> i) & 1u) ? ex2_poly2_ranged(x) : make_float2(ex2_approx(x.x), ex2_approx(x.y));
                         packed[i] = pack_bf16x2(e.x, e.y);
                     }
                 };
-                // The epilogue of an item is run inside the first block of the NEXT item, between its exponentials and its
-                // P store: by then the last PV of the item has completed long ago (it is the very completion the P store
-                // has to wait for anyway), so nobody waits for the tensor pipe at an item boundary.
-                __nv_bfloat16* pend_out = nullptr;          // this thread's half row of the pending item
-                const __nv_bfloat16* pend_gate = nullptr;
-                float* pend_lse = nullptr;
-                float pend_ref = 0.f;
-                int pend_ordinal = -1;                      // -1: nothing pending
-                // The wait for the next block's scores is asked between the stores of P and their completion,
-                // in straight-line code (with a branch around the question the gain is gone: 3 % of the kernel).  After the
-                // last block of the pass no scores follow; there the question names the phase just used, which is complete,
-                // so that no warp sits out the time limit of a wait that nothing answers.
-                bool s_polled = false, s_ready = false;
-                const uint32_t last_blk = kPartial ? 0u : blk + (uint32_t)count * (uint32_t)nblk - 1u;
-                // O and l of the pending item are complete (the caller has waited for its last PV): normalise, store, note overflow
-                auto epilogue = [&]() {
+                // The epilogue of an item is run inside the first block of the NEXT item, behind its P store: by then the last PV of
+                // the item has completed (it was issued a block's exponentials ago), so nobody waits for the tensor pipe at an item
+                // boundary.  Where the item goes is worked out here and not kept in registers over its blocks.
+                // O and l of item i are complete (the caller has waited for its last PV): normalise, store, note overflow
+                auto epilogue = [&](int i, float ref) {
+                    const auto c = decode_item(p, item_at(i));
+                    int py, px, Y0, X0;
+                    patch_origin(p, c, 2 * (2 * c.tp + qt) + (row >> 6), py, px, Y0, X0);
+                    const int Y = Y0 + ((row >> 3) & 7), X = X0 + (row & 7);   // the patch does not straddle the border
+                    const bool no_query = kPartial && 2 * (2 * c.tp + qt) + (row >> 6) >= patches_of(p, c);   // half a tile without tokens: nothing to store
+                    const size_t tok = (((size_t)c.b * p.H + Y) * p.W + X) * p.heads + c.h;
                     uint32_t o[16], lsum[1];
                     tmem_ld16(t_o1 + half * 16, o);
                     tmem_ld1(t_o1 + kD, lsum);
                     tmem_wait_ld();
                     tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kOFree + qt));
                     const float l_all = __uint_as_float(lsum[0]);
                     // a score left the range the fixed reference covers: the exact form redoes the item
-                    const bool bad = pend_out != nullptr && !(l_all > 0.f && l_all < 1.2676506e30f);     // 2^100
+                    const bool bad = !no_query && !(l_all > 0.f && l_all < 1.2676506e30f);     // 2^100
                     if (__any_sync(0xffffffffu, bad) && lane == 0) {
                         const int slot = atomicAdd(redo_count, 1);
-                        if (slot < kMaxRedo) redo_list[slot] = pend_ordinal;
+                        if (slot < kMaxRedo) redo_list[slot] = i;
                     }
-                    if (kPartial && pend_out == nullptr) { pend_ordinal = -1; return; }
+                    if (no_query) return;
                     const float w_o = 1.f / l_all;
-                    uint4* dst = reinterpret_cast<uint4*>(pend_out);
-                    const uint4* gsrc = reinterpret_cast<const uint4*>(pend_gate);
+                    uint4* dst = reinterpret_cast<uint4*>(p.out + tok * p.d + half * 16);
+                    const uint4* gsrc = kGated ? reinterpret_cast<const uint4*>(p.gate + tok * p.d + half * 16) : nullptr;
 #pragma unroll
                     for (int g = 0; g < 2; ++g) {
                         if (half * 16 + 8 * g >= p.d) break;          // a head narrower than 32 channels: the rest of the row is padding
@@ -489,82 +489,73 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         }
                         dst[g] = make_uint4(w[0], w[1], w[2], w[3]);
                     }
-                    if (pend_lse) *pend_lse = pend_ref * p.inv_sqrt_d + logf(l_all);
-                    pend_ordinal = -1;
+                    if (p.lse && half == 0) p.lse[(((size_t)c.b * p.heads + c.h) * p.H + Y) * p.W + X] = ref * p.inv_sqrt_d + logf(l_all);
                 };
+                float m_ref = 0.f;
                 for (int i = 0; i < count && ok; ++i, ++io) {
-                    const auto c = decode_item(p, item_at(i));
-                    // where this thread's half row of the item goes
-                    int py, px, Y0, X0;
-                    patch_origin(p, c, 2 * (2 * c.tp + qt) + (row >> 6), py, px, Y0, X0);
-                    const int Y = Y0 + ((row >> 3) & 7), X = X0 + (row & 7);   // the patch does not straddle the border
-                    const bool no_query = kPartial && 2 * (2 * c.tp + qt) + (row >> 6) >= patches_of(p, c);   // half a tile without tokens: nothing to store
-                    const size_t tok = (((size_t)c.b * p.H + Y) * p.W + X) * p.heads + c.h;
-                    __nv_bfloat16* const out_row = no_query ? nullptr : p.out + tok * p.d + half * 16;
-                    const __nv_bfloat16* const gate_row = kGated ? p.gate + tok * p.d + half * 16 : nullptr;
-                    float* const lse_row = (p.lse && half == 0 && !no_query) ? p.lse + (((size_t)c.b * p.heads + c.h) * p.H + Y) * p.W + X : nullptr;
-                    float m_ref = 0.f;
+                    const float ref_before = m_ref;
                     float2 neg2 = make_float2(0.f, 0.f);
-                    const int patches = patches_of(p, c), nb = kPartial ? (patches + 1) >> 1 : nblk;
+                    const int nb = blocks_at(i);
                     for (int j = 0; j < nb; ++j, ++blk) {
                         // warp-uniform outcome: the TMEM loads below are warp-collective
-                        if (!(s_polled && __all_sync(0xffffffffu, s_ready)) && !mbar_wait_warp(bar(kSFull + qt), blk & 1, abort_flag, p.status)) { ok = false; break; }
-                        s_polled = false;
+                        if (!mbar_wait_warp(on_block(kSFull, qt, blk), parity(blk), abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
-                        uint32_t sa[32], sb[32];
+                        const uint32_t t_s = t_half + sb * kTile;
+                        sb = sb == 0 ? 2u : sb - 1;
                         if (j == 0) {
                             // the row's reference: the maximum over keys 0-31 of the window, the same for both key halves
-                            tmem_ld32(tmem + lane_base + kColS + qt * kTile, sa);
+                            uint32_t first[32];
+                            tmem_ld32(t_s - half * 64, first);
                             tmem_wait_ld();
                             float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
                             for (int e = 0; e < 32; e += 4) {
-                                mx0 = max3(mx0, __uint_as_float(sa[e]), __uint_as_float(sa[e + 1]));
-                                mx1 = max3(mx1, __uint_as_float(sa[e + 2]), __uint_as_float(sa[e + 3]));
+                                mx0 = max3(mx0, __uint_as_float(first[e]), __uint_as_float(first[e + 1]));
+                                mx1 = max3(mx1, __uint_as_float(first[e + 2]), __uint_as_float(first[e + 3]));
                             }
                             m_ref = fmaxf(mx0, mx1);
                             const float neg = -m_ref * p.scale_log2;
                             neg2 = make_float2(neg, neg);
                         }
-                        // all 64 scores of this thread at once: the accumulator goes back to the MMA warp before any exponential
-                        tmem_ld32(t_s, sa);
-                        tmem_ld32(t_s + 32, sb);
+                        // 16 keys at a time, the load of the next ones under the exponentials of these: all 64 scores and their P in
+                        // registers at once cost a tenth of the kernel (256 x 256 tokens, windows of 64: 415 against 393 us).  P goes to the second
+                        // half of the columns, whose keys are therefore taken first.
+                        uint32_t a[16], b[16], pk[8];
+                        tmem_ld16(t_s + 32, a);
+                        tmem_ld16(t_s + 48, b);
                         tmem_wait_ld();
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(bar(kSFree + qt));   // the next block's scores may overwrite the accumulator
-                        uint32_t pa[16], pb[16];
-                        // P of the tile is free once the previous block's PV has completed (long ago, as a rule).  It is asked before the
-                        // exponentials, so that the answer is there when they are done.
-                        const bool p_free = blk == 0 || mbar_try_wait(b_free, (blk - 1) & 1);
-                        exp_chunk1(sa, scale2, neg2, pa);
-                        exp_chunk1(sb, scale2, neg2, pb);
-                        if (blk > 0) {
-                            if (!__all_sync(0xffffffffu, p_free) && !mbar_wait_warp(b_free, (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
-                            tc_fence_after();
-                        }
-                        if (j == 0 && pend_ordinal >= 0) epilogue();     // that PV was the last one of the item before
-                        tmem_st16(t_p, pa);
-                        tmem_st16(t_p + 16, pb);
-                        const bool more = kPartial ? i != count - 1 || j != nb - 1 : blk != last_blk;
-                        s_ready = mbar_try_wait(bar(kSFull + qt), (blk + (more ? 1u : 0u)) & 1);
-                        s_polled = true;
+                        exp_chunk1(a, neg2, pk);
+                        tmem_st8(t_s + 32, pk);
+                        tmem_ld16(t_s, a);
+                        exp_chunk1(b, neg2, pk);
+                        tmem_wait_ld();
+                        tmem_st8(t_s + 40, pk);
+                        tmem_ld16(t_s + 16, b);
+                        exp_chunk1(a, neg2, pk);
+                        tmem_wait_ld();
+                        tmem_st8(t_s + 48, pk);
+                        exp_chunk1(b, neg2, pk);
+                        tmem_st8(t_s + 56, pk);
                         tmem_wait_st();
+                        if (j == 0 && i > 0) {       // that PV was the last one of the item before
+                            if (!mbar_wait_warp(on_block(kPVDone, qt, blk - 1), parity(blk - 1), abort_flag, p.status)) { ok = false; break; }
+                            tc_fence_after();
+                            epilogue(i - 1, ref_before);
+                        }
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(b_ready);
+                        if (lane == 0) mbar_arrive(on_block(kPReady, qt, blk));
                     }
-                    if (!ok) break;
-                    pend_out = out_row; pend_gate = gate_row; pend_lse = lse_row; pend_ref = m_ref; pend_ordinal = i;
                 }
-                if (ok && pend_ordinal >= 0) {
+                if (ok && count > 0) {
                     // the last item of the pass
-                    if (mbar_wait_warp(b_free, (blk - 1) & 1, abort_flag, p.status)) { tc_fence_after(); epilogue(); } else ok = false;
+                    if (mbar_wait_warp(on_block(kPVDone, qt, blk - 1), parity(blk - 1), abort_flag, p.status)) { tc_fence_after(); epilogue(count - 1, m_ref); } else ok = false;
                 }
             } else {
                 // ------------------------------------------------------------------ exact form
                 const uint32_t t_o = tmem + lane_base + kColO + qt * 2 * kD;        // both halves' accumulators
-                float2* merge = reinterpret_cast<float2*>(base_ptr + kOffMerge) + qt * 2 * kTile;   // [half][row]
+                // [half][row]; two sets, so that a warp that is an item ahead of its partner does not overwrite what that one still reads
+                float2* const merge_sets = reinterpret_cast<float2*>(base_ptr + kOffMerge) + qt * 2 * kTile;
                 const float rescale_threshold = 8.0f / p.scale_log2;    // raw-logit units: p stays <= 2^8
                 // exp2 of 32 scores against the reference -m * log2e/sqrt(d); returns their sum
                 auto exp_chunk = [&](const uint32_t (&s)[32], float neg_ms, uint32_t (&packed)[16]) -> float {
@@ -585,45 +576,28 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     const int patches = patches_of(p, c), nb = kPartial ? (patches + 1) >> 1 : nblk;
                     for (int j = 0; j < nb; ++j, ++blk) {
                         // warp-uniform outcome: the TMEM loads below are warp-collective
-                        if (!mbar_wait_warp(bar(kSFull + qt), blk & 1, abort_flag, p.status)) { ok = false; break; }
+                        if (!mbar_wait_warp(on_block(kSFull, qt, blk), parity(blk), abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
-                        bool p_free = blk == 0;       // P (and O) of this half are free once the previous block's PV has completed
-                        if (kPartial) {
+                        const uint32_t t_s = t_half + sb * kTile;
+                        sb = sb == 0 ? 2u : sb - 1;
+                        uint32_t pa[16], pb[16];
+                        if (kPartial && half != 0 && 2 * j + 1 >= patches) {
                             // half a block without tokens (the last one of an odd number of patches)
-                            if (half != 0 && 2 * j + 1 >= patches) {
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(bar(kSFree + qt));
-                                if (!p_free) {
-                                    if (!mbar_wait_warp(b_free, (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
-                                    tc_fence_after();
-                                }
-                                uint32_t zero[16];
 #pragma unroll
-                                for (int e = 0; e < 16; ++e) zero[e] = 0u;
-                                tmem_st16(t_p, zero);
-                                tmem_st16(t_p + 16, zero);
-                                tmem_wait_st();
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(b_ready);
-                                continue;
-                            }
-                        }
-                        const bool first_ref = j == 0;
-#pragma unroll
-                        for (int ch = 0; ch < 2; ++ch) {
-                            uint32_t s[32];
-                            tmem_ld32(t_s + 32 * ch, s);
+                            for (int e = 0; e < 16; ++e) pa[e] = pb[e] = 0u;
+                        } else {
+                            uint32_t sa[32], sc[32];
+                            tmem_ld32(t_s, sa);
+                            tmem_ld32(t_s + 32, sc);
                             tmem_wait_ld();
                             float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
-                            for (int e = 0; e < 32; e += 4) {
-                                mx0 = max3(mx0, __uint_as_float(s[e]), __uint_as_float(s[e + 1]));
-                                mx1 = max3(mx1, __uint_as_float(s[e + 2]), __uint_as_float(s[e + 3]));
+                            for (int e = 0; e < 32; e += 2) {
+                                mx0 = max3(mx0, __uint_as_float(sa[e]), __uint_as_float(sa[e + 1]));
+                                mx1 = max3(mx1, __uint_as_float(sc[e]), __uint_as_float(sc[e + 1]));
                             }
                             const float mx = fmaxf(mx0, mx1);
-                            if (first_ref && ch == 0) {
+                            if (j == 0) {
                                 m_used = mx;
                             } else {
                                 // Move the reference (and rescale O, l) only when the maximum grew by more than
@@ -631,61 +605,39 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                                 // carries the same reference.
                                 const bool need = mx > m_used + rescale_threshold;
                                 if (__any_sync(0xffffffffu, need)) {
-                                    if (!p_free) {
-                                        if (!mbar_wait_warp(b_free, (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
-                                        tc_fence_after();
-                                        p_free = true;
-                                    }
+                                    if (!mbar_wait_warp(on_block(kPVDone, qt, blk - 1), parity(blk - 1), abort_flag, p.status)) { ok = false; break; }
+                                    tc_fence_after();
                                     const float factor = need ? ex2_approx((m_used - mx) * p.scale_log2) : 1.f;
                                     if (need) { l *= factor; m_used = mx; }
-                                    if (j > 0) {
-                                        uint32_t o[32];
-                                        tmem_ld32(t_o + half * kD, o);
+                                    for (int g = 0; g < 4; ++g) {
+                                        uint32_t o[8];
+                                        tmem_ld8(t_o + half * kD + 8 * g, o);
                                         tmem_wait_ld();
 #pragma unroll
-                                        for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * factor);
-                                        tmem_st32(t_o + half * kD, o);
+                                        for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * factor);
+                                        tmem_st8(t_o + half * kD + 8 * g, o);
                                     }
-                                    if (ch == 1) {
-                                        // the first 32 keys of this block were exponentiated against the old
-                                        // reference: redo them (their sum is already in l, rescaled above)
-                                        uint32_t s0[32], packed0[16];
-                                        tmem_ld32(t_s, s0);
-                                        tmem_wait_ld();
-                                        exp_chunk(s0, -m_used * p.scale_log2, packed0);
-                                        tmem_st16(t_p, packed0);
-                                    }
-                                    tmem_wait_st();
                                 }
                             }
-                            if (ch == 1) {
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(bar(kSFree + qt));   // the next block's scores may overwrite the accumulator
-                            }
-                            uint32_t packed[16];
-                            l += exp_chunk(s, -m_used * p.scale_log2, packed);
-                            if (!p_free) {
-                                if (!mbar_wait_warp(b_free, (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
-                                tc_fence_after();
-                                p_free = true;
-                            }
-                            tmem_st16(t_p + 16 * ch, packed);
+                            l += exp_chunk(sa, -m_used * p.scale_log2, pa);
+                            l += exp_chunk(sc, -m_used * p.scale_log2, pb);
                         }
-                        if (!ok) break;
+                        tmem_st16(t_s + 32, pa);
+                        tmem_st16(t_s + 48, pb);
                         tmem_wait_st();
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(b_ready);
+                        if (lane == 0) mbar_arrive(on_block(kPReady, qt, blk));
                     }
                     if (!ok) break;
                     // ---- merge the two key halves and write this thread's 16 output columns
+                    float2* const merge = merge_sets + (nmerge & 1) * 4 * kTile;
                     merge[half * kTile + row] = make_float2(m_used, l);
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(kMerge + 4 * qt + quarter));
                     // The partner's (m, l) must be there and the item's last PV must have completed.
                     if (!mbar_wait_warp(bar(kMerge + 4 * qt + quarter), nmerge & 1, abort_flag, p.status) ||
-                        !mbar_wait_warp(b_free, (blk - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                        !mbar_wait_warp(on_block(kPVDone, qt, blk - 1), parity(blk - 1), abort_flag, p.status)) { ok = false; break; }
                     tc_fence_after();
                     uint32_t oa[16], ob[16];
                     tmem_ld16(t_o + half * 16, oa);
@@ -693,8 +645,6 @@ rib_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     tmem_wait_ld();
                     const float2 other = merge[(half ^ 1) * kTile + row];
                     tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kOFree + qt));
                     const float m_a = half ? other.x : m_used, l_a = half ? other.y : l;
                     const float m_b = half ? m_used : other.x, l_b = half ? l : other.y;
                     const float m = fmaxf(m_a, m_b);
