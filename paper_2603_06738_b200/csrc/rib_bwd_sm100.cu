@@ -4,14 +4,13 @@
 // Shapes: d = 32, r = 16 or 32 (template argument R), window side M a multiple of 16, shift a multiple of 8 (as
 // the forward).  The text below describes R = 16.  With R = 32 the RIB rows fill their 64-byte slots, dK~ and dQ~ are
 // 64 columns wide, and tensor memory has no room left for dS^T: dK~ then takes the dS tile in shared memory as a
-// K-major A operand (that tile's barrier counts two readers).  S^T and dP^T of both halves of a tile are then issued
-// together (N = 128), once both groups of arithmetic warps have read those of the tile before.
+// K-major A operand (that tile's barrier counts two readers), and dP^T has two buffers of its own.
 //
 // Work item = one (batch, window, head) pair x one key block J of 128 tokens.  A persistent CTA keeps
 // K~_J = [k, Pk] and V_J in shared memory and dV_J, dK~_J in tensor memory, and walks the query tiles
 // I of the window.  Everything is computed transposed (keys on the TMEM lanes) so that P^T and dS^T
 // feed the dV and dK~ contractions straight from tensor memory.  The unit of the pipeline is a
-// half-tile u = (I, h): the 64 queries of patch h of tile I (R = 32: both patches for the first two lines),
+// half-tile u = 2 I + h: the 64 queries of patch h of tile I,
 //     S^T  = K~_J Q~_u^T                    (M128 N64 K48: content rows 2 x K16, RIB rows 1 x K16)
 //     dP^T = V_J dO_u^T                     (M128 N64 K32)
 //     P^T  = exp2(S^T * log2e/sqrt(d) - lse_i * log2e),   dS^T = P^T o (dP^T - D_i)     (ALU warps)
@@ -19,8 +18,9 @@
 //     dK~_J += dS^T Q~_u                    (A from TMEM, B = [Q content | Q RIB] tiles, MN-major, N = 48)
 // and once per tile, when both halves of dS are in shared memory,
 //     dQ~_I  = dS K~_J                      (A = dS, MN-major, B = [K | Pk] tiles, N = 48).
-// Score accumulators, P^T and dS^T are double-buffered by h, and two groups of arithmetic warps take
-// the even and the odd half-tiles: while one group evaluates exponentials the other one's scores are
+// Three buffers of S^T and dP^T rotate among the units.  P^T and dS^T are written over the scores that they come from, piece by piece,
+// by the warp that has read them; S^T of unit u + 3 goes there once dV and dK~ have consumed unit u.  Two groups of arithmetic
+// warps take the even and the odd half-tiles: while one group evaluates exponentials the other one's scores are
 // being contracted, so neither the tensor pipe nor the exp pipe waits for a whole tile of the other.
 // The RIB rows are fetched as zero-padded 64-byte rows, so that a RIB tile has the layout of a content
 // tile and the concatenation of Eq. 5 is, for the MN-major operands, one descriptor whose second
@@ -35,10 +35,12 @@
 // warp 1 issues S^T and dP^T, warp 2 (also the TMEM allocator) dV and dK~, warp 3 dQ~; warps 4-11
 // P/dS arithmetic of the even half-tiles, warps 12-19 of the odd ones (a warp per 32 key rows and 32
 // queries, a thread 2 key rows x 4 queries of each of its four 16 x 16 pieces); warps 20-23 drain dQ~ after every tile and dK~/dV after every item.  Every wait is bounded.
-// What sets the pace is the latency of the loop  scores -> arithmetic -> gradient MMAs -> buffers free
-// divided by the two half-tiles in flight, so every buffer is handed back as early as its last reader
-// allows: the score accumulators when the arithmetic warps hold them in registers (long before their
-// exponentials are done), P^T / dS^T when dV and dK~ have consumed them.
+// What sets the pace is the loop  scores -> arithmetic -> dV and dK~ -> next scores of the buffer  (1600 cycles of issue, contraction and
+// barriers and 1350 of arithmetic), divided by the three units in flight: 2180 cycles per tile of 128 x 128 at rank 16, beside 1530 of
+// tensor pipe and, replays included, nine tenths of the shared-memory data pipe.  Measured on 16 x 96 x 96 tokens in windows of 32,
+// us at rank 16 / 32: scores, P^T and dS^T in buffers of their own, two of each 535 / 620; in place as above 515 / 640; dV and dK out by TMEM, shared
+// memory and TMA before the item's last dQ~ 488 / 618; that and dQ~ drained in pieces of 16 columns without spills 468 / 565; S^T not
+// waiting for dK~ at rank 32 468 / 550.  (At rank 16 the same costs 1 to 3 %; a third group of arithmetic warps, 64 registers each: 511.)
 #include "rib_sm100_common.cuh"
 
 namespace rib {
@@ -60,27 +62,29 @@ constexpr uint32_t kRingQc = 0, kRingQp = kContentBytes, kRingDO = kRingQp + kCo
 constexpr uint32_t kRingBytes = kRingLD + kLdBytes;              // 25600
 constexpr uint32_t kOffDS = kOffRing + kQStages * kRingBytes;    // dS: [2 tiles][2 halves of 64 queries][128 keys][128 B], SWIZZLE_128B
 constexpr uint32_t kDSHalf = kTile * 128;
-constexpr uint32_t kOffBar = kOffDS + 4 * kDSHalf;
-// kSFull, kSFree, kPFree: one per half h; kPReady: one per half and tile parity (index 2 h + parity); kDSFree: one per dS
-// tile buffer.  The rule behind the split: a barrier's next phase must not be able to complete before every waiter has seen
-// the current one, because a parity wait cannot tell "two phases ahead" from "not yet".  dQ~ of tile g waits for both halves'
-// P^T / dS^T, but nothing that the arithmetic warps need for tile g + 1 depends on dQ~ of tile g, so with one barrier per
-// half they could complete phase g + 1 before the dQ~ issuer has looked at phase g; with one per tile parity the next phase
-// belongs to tile g + 2, whose dS buffer is only released by dQ~ of tile g.
-enum Bar { kKVFull = 0, kKVEmpty = 2, kQFull = 4, kQEmpty = kQFull + kQStages, kSFull = kQEmpty + kQStages, kSFree = kSFull + 2,
-           kPReady = kSFree + 2, kPFree = kPReady + 4, kDSFree = kPFree + 2, kDQFull = kDSFree + 2, kDQFree, kAccFull, kAccFree, kDrain,
+constexpr uint32_t kOffDK = kOffDS + 4 * kDSHalf;                // dK rows of an item on their way out (dV rows leave through V's slot)
+constexpr uint32_t kOffBar = kOffDK + kContentBytes;
+// kSFull, kPReady, kPFree: unit mod 4 (on_unit); kDPFree: per half h (R = 32); kDSFree: per dS tile buffer.  The rule behind the split: a
+// barrier's next phase must not be able to complete before every waiter has seen the current one, because a parity wait
+// cannot tell "two phases ahead" from "not yet".  dQ~ of tile g waits for both halves' P^T / dS^T, but nothing that the arithmetic warps
+// need for tile g + 1 depends on dQ~ of tile g; on the barriers of units 2 g, 2 g + 1 the next phases belong to tile g + 2, whose dS
+// buffer is only released by dQ~ of tile g.  (tests/test_bwd_barriers.py is a model of these waits.)
+enum Bar { kKVFull = 0, kKVEmpty = 2, kQFull = 4, kQEmpty = kQFull + kQStages, kSFull = kQEmpty + kQStages, kPReady = kSFull + 4,
+           kPFree = kPReady + 4, kDPFree = kPFree + 4, kDSFree = kDPFree + 2, kDQFull = kDSFree + 2, kDQFree, kAccFull, kAccFree, kDrain,
            kNumBars = kDrain + 3 };
 constexpr uint32_t kOffMisc = kOffBar + kNumBars * 8;
 constexpr uint32_t kSmemBytes = kOffMisc + 16 + 1024;
+static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 static_assert(kOffRing % 1024 == 0 && kRingBytes % 1024 == 0 && kOffDS % 1024 == 0, "swizzle atoms need aligned tiles");
 
-// tensor-memory columns; S^T, dP^T (64 fp32 columns) and P^T, dS^T (32 columns of bf16 pairs) exist once per half h
-// R = 16: S 0, dP 128, P 256, dS 320, dV 384, dK~ 416 (48), dQ~ 464 (48).
+// tensor-memory columns: S^T of unit u in buffer u mod 3 (64 fp32 columns), dP^T beside it (R = 16) or in buffer h of its half (R = 32, for which
+// three do not fit); a warp writes P^T over its own scores (and, R = 16, dS^T over its dP^T): 32 queries in the first 16 of its 32 columns.
+// R = 16: 3 x (S, dP) 0, dV 384, dK~ 416 (48), dQ~ 464 (48).
 // R = 32: dK~ and dQ~ need 64 columns each, so dS^T is not kept in tensor memory (dK~ reads the dS tile in shared memory,
-//         K-major): S 0, dP 128, P 256, dV 320, dK~ 352 (64), dQ~ 416 (64).
-constexpr uint32_t kColS = 0, kColDP = 128, kColP = 256;
+//         K-major): 3 x S 0, 2 x dP 192, dV 320, dK~ 352 (64), dQ~ 416 (64).
+constexpr uint32_t kBuffers = 3;
 template <int R> struct Cols {
-    static constexpr uint32_t kColDS = 320;                              // R = 16 only
+    static constexpr uint32_t kStep = R == 16 ? 128 : 64, kColDP = R == 16 ? 64 : 192;      // between score buffers; dP^T of buffer / half 0
     static constexpr uint32_t kColDV = R == 16 ? 384 : 320, kColDK = kColDV + kD, kColDQ = kColDK + kD + R;
     static_assert(kColDQ + kD + R <= 512, "tensor memory has 512 columns");
 };
@@ -98,16 +102,14 @@ struct BwdParams {
     const float2* ld;          // [pairs][n / 2] window order, per query pair: (-lse2, -lse2', -D, -D') as two float2
     float* dq_acc;             // [pairs][48 / 4][n][4] fp32, zeroed by the preparation kernel
     float* dkp;                // [pairs][16 / 4][n][4] fp32, RIB columns of dK~ (already times 1/sqrt d)
-    __nv_bfloat16* dk;
-    __nv_bfloat16* dv;
     int* status;
     int H, W, heads, M, s, n, nWy, nWx, nblk, items;
-    int d;                     // head width (8, 16, 24, 32): tiles are 32 wide with zeros beyond d, only d channels are stored
     int Hp, Wp;                // sides of the map the windows are laid over (H, W rounded up to multiples of M)
     int pos_per_head;          // 1 when Pq/Pk are head-wise: table index = head
     int masked;                // kPartial: shifted windows with a mask (a query sees the keys of its own part of a border window)
     float scale_log2;          // log2(e) / sqrt(d)
     float inv_sqrt_d;
+    FastDiv div_nblk, div_heads, div_nwx, div_nwy, div_per_row;   // ..., M / 8
 };
 
 struct ItemCoord { int pair, b, wy, wx, h, J; };
@@ -115,12 +117,10 @@ struct ItemCoord { int pair, b, wy, wx, h, J; };
 __device__ __forceinline__ ItemCoord decode_item(const BwdParams& p, int item)
 {
     ItemCoord c;
-    c.J = item % p.nblk; item /= p.nblk;
-    c.pair = item;
-    c.h = item % p.heads; item /= p.heads;
-    c.wx = item % p.nWx; item /= p.nWx;
-    c.wy = item % p.nWy; item /= p.nWy;
-    c.b = item;
+    p.div_nblk.divmod(item, c.pair, c.J);
+    p.div_heads.divmod(c.pair, item, c.h);
+    p.div_nwx.divmod(item, item, c.wx);
+    p.div_nwy.divmod(item, c.b, c.wy);
     return c;
 }
 
@@ -134,17 +134,21 @@ __global__ void __launch_bounds__(kThreads, 1)
 rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
                      const __grid_constant__ CUtensorMap tm_pqs, const __grid_constant__ CUtensorMap tm_pk,
-                     const BwdParams p)
+                     const __grid_constant__ CUtensorMap tm_dk, const __grid_constant__ CUtensorMap tm_dv, const BwdParams p)
 {
     constexpr int kDk = kD + R;
-    constexpr uint32_t kColDS = Cols<R>::kColDS, kColDV = Cols<R>::kColDV, kColDK = Cols<R>::kColDK, kColDQ = Cols<R>::kColDQ;
-    constexpr uint32_t kSUnits = R == 32 ? 2 : 1;         // half-tiles whose S^T, dP^T are issued together
-    constexpr uint32_t kIdescSS = idesc_bf16_f32(kTile, kSUnits * kTile / 2, false);    // both operands K-major
+    constexpr uint32_t kStep = Cols<R>::kStep, kColDP = Cols<R>::kColDP, kColDV = Cols<R>::kColDV, kColDK = Cols<R>::kColDK, kColDQ = Cols<R>::kColDQ;
+    constexpr uint32_t kIdescSS = idesc_bf16_f32(kTile, kTile / 2, false);    // both operands K-major
     constexpr uint32_t kIdescT48 = Idesc<R>::kT, kIdescQ48 = Idesc<R>::kQ;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
     auto bar = [&](int i) { return base + kOffBar + 8u * i; };
+    // of kSFull, kPReady, kPFree: the barrier of a unit and the parity of its phase.  (Units -1 to -3 have the parity that a barrier without a
+    // completed phase answers yes to.)
+    auto on_unit = [&](int which, uint32_t unit) { return bar(which + (int)(unit & 3)); };
+    auto unit_parity = [](uint32_t unit) { return (unit >> 2) & 1; };
+    auto buffer_after = [](uint32_t buffer, uint32_t units) { buffer += units; return buffer >= kBuffers ? buffer - kBuffers : buffer; };
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + kOffMisc + 4);
 
@@ -153,19 +157,20 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 
     if (threadIdx.x == 0) {
         abort_flag[0] = 0; abort_flag[1] = 0;   // [1] stays 0: used by the drain waits
-        for (int s = 0; s < 2; ++s) { mbar_init(bar(kKVFull + s), 1); mbar_init(bar(kKVEmpty + s), 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(bar(kKVFull + s), 1); mbar_init(bar(kKVEmpty + s), 5); }     // empty: the item's last dQ~, and V's slot by the four warps whose dV leaves through it
         for (int s = 0; s < kQStages; ++s) { mbar_init(bar(kQFull + s), 1); mbar_init(bar(kQEmpty + s), 1); }
         for (int h = 0; h < 2; ++h) {
-            mbar_init(bar(kSFull + h), 1); mbar_init(bar(kSFree + h), 8); mbar_init(bar(kPFree + h), 1);
-            mbar_init(bar(kPReady + 2 * h), 8); mbar_init(bar(kPReady + 2 * h + 1), 8);
+            mbar_init(bar(kDPFree + h), 8);
             mbar_init(bar(kDSFree + h), R == 16 ? 1 : 2);     // R = 32: dK~ reads the dS tile as well as dQ~
         }
+        for (int i = 0; i < 4; ++i) { mbar_init(bar(kSFull + i), 1); mbar_init(bar(kPReady + i), 8); mbar_init(bar(kPFree + i), 1); }
         mbar_init(bar(kDQFull), 1); mbar_init(bar(kDQFree), 4);
         mbar_init(bar(kAccFull), 1); mbar_init(bar(kAccFree), 4);
         for (int i = 0; i < 3; ++i) mbar_init(bar(kDrain + i), 1);
         fence_barrier_init();
         prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v);
         prefetch_tensormap(&tm_do); prefetch_tensormap(&tm_pqs); prefetch_tensormap(&tm_pk);
+        prefetch_tensormap(&tm_dk); prefetch_tensormap(&tm_dv);
     }
     if (warp == 2) {
         tmem_alloc(base + kOffMisc, kTmemCols);
@@ -189,7 +194,7 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 ++kv_armed;
                 for (int sub = 0; sub < 2; ++sub) {
                     int py, px, Y0, X0;
-                    patch_origin(geom, c.wy, c.wx, 2 * c.J + sub, py, px, Y0, X0);
+                    patch_origin(geom, p.div_per_row, c.wy, c.wx, 2 * c.J + sub, py, px, Y0, X0);
                     tma_load_5d(base + kOffKc + slot * kContentBytes + sub * kPatchContent, &tm_k, bar(kKVFull + slot),
                                 0, c.h, X0, Y0, c.b);
                     tma_load_4d(base + kOffKp + slot * kContentBytes + sub * kPatchContent, &tm_pk, bar(kKVFull + slot), 0,
@@ -205,7 +210,7 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     const uint32_t ring = base + kOffRing + st * kRingBytes;
                     for (int sub = 0; sub < 2; ++sub) {
                         int py, px, Y0, X0;
-                        patch_origin(geom, c.wy, c.wx, 2 * I + sub, py, px, Y0, X0);
+                        patch_origin(geom, p.div_per_row, c.wy, c.wx, 2 * I + sub, py, px, Y0, X0);
                         tma_load_5d(ring + kRingQc + sub * kPatchContent, &tm_q, bar(kQFull + st), 0, c.h, X0, Y0, c.b);
                         tma_load_4d(ring + kRingQp + sub * kPatchContent, &tm_pqs, bar(kQFull + st), 0,
                                     px, py, c.h * p.pos_per_head);
@@ -237,62 +242,68 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         auto wait_all = [&](uint32_t b, uint32_t parity) { return mbar_wait_warp(b, parity, abort_flag, p.status); };
         bool ok = true;
         if (warp == 1) {
-            // ---- S^T, dP^T of unit u as soon as the arithmetic group has read unit u - 2 (same buffers)
-            // out of tensor memory; the group is then still busy with that unit's exponentials.
-            // Rank 32: of both halves of a tile at once (N = 128), whose six MMAs fetch 48 KB of operands where two sets of six fetch 72 (641 ->
-            // 625 us); at rank 16 the halves kept apart are the faster (550 against 560 us).
-            uint32_t nitem = 0, I = 0;
+            // ---- S^T, dP^T of unit u as soon as dV and dK~ of unit u - 3 have consumed P^T, dS^T, which lie in the same columns; the
+            // groups are then busy with units u - 1 and u - 2.  (R = 32: S^T after dV alone, dP^T when unit u - 2 has been read.)
+            uint32_t nitem = 0, I = 0, buf = 0;
             uint32_t slot_base = 0;
-            for (uint32_t u = 0; u < total_units / kSUnits && ok; ++u) {
-                const uint32_t h = kSUnits == 1 ? u & 1 : 0, g = kSUnits == 1 ? u >> 1 : u, st = g % kQStages, slot = nitem & 1;
+            for (uint32_t u = 0; u < total_units && ok; ++u) {
+                const uint32_t h = u & 1, g = u >> 1, st = g % kQStages, slot = nitem & 1;
                 if (h == 0 && I == 0) {
                     if (!wait_all(bar(kKVFull + slot), (nitem >> 1) & 1)) { ok = false; break; }
                     slot_base = base + slot * kContentBytes;
                 }
                 if (h == 0 && !wait_all(bar(kQFull + st), (g / kQStages) & 1)) { ok = false; break; }
-                if (g >= 1 && (!wait_all(bar(kSFree + h), (g - 1) & 1) || (kSUnits == 2 && !wait_all(bar(kSFree + 1), (g - 1) & 1)))) { ok = false; break; }
+                if (!wait_all(on_unit(kPFree, u - kBuffers), unit_parity(u - kBuffers))) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t ring = base + kOffRing + st * kRingBytes + h * kPatchContent;   // rows of patch h (and the next)
+                const uint32_t ring = base + kOffRing + st * kRingBytes + h * kPatchContent;   // rows of patch h
+                const uint64_t kc = smem_desc_at(kDesc64, slot_base + kOffKc), kp = smem_desc_at(kDesc64, slot_base + kOffKp);
+                const uint64_t v = smem_desc_at(kDesc64, slot_base + kOffV);
+                const uint64_t qc = smem_desc_at(kDesc64, ring + kRingQc), qp = smem_desc_at(kDesc64, ring + kRingQp);
+                const uint64_t go = smem_desc_at(kDesc64, ring + kRingDO);
+                const uint32_t d_s = tmem + kStep * buf, d_p = R == 16 ? d_s + kColDP : tmem + kColDP + 64 * h;
                 if (elect_one()) {
-                    const uint64_t kc = smem_desc_at(kDesc64, slot_base + kOffKc), kp = smem_desc_at(kDesc64, slot_base + kOffKp);
-                    const uint64_t v = smem_desc_at(kDesc64, slot_base + kOffV);
-                    const uint64_t qc = smem_desc_at(kDesc64, ring + kRingQc), qp = smem_desc_at(kDesc64, ring + kRingQp);
-                    const uint64_t go = smem_desc_at(kDesc64, ring + kRingDO);
-                    const uint32_t d_s = tmem + kColS + h * kHalfCols, d_p = tmem + kColDP + h * kHalfCols;
                     mma_ss(d_s, kc, qc, kIdescSS, 0u);
                     mma_ss(d_s, kc + 2, qc + 2, kIdescSS, 1u);     // + 32 bytes: second K16 step
                     mma_ss(d_s, kp, qp, kIdescSS, 1u);
                     if (R == 32) mma_ss(d_s, kp + 2, qp + 2, kIdescSS, 1u);
+                }
+                if (R == 32) {
+                    __syncwarp();
+                    if (!wait_all(bar(kDPFree + h), (g - 1) & 1)) { ok = false; break; }
+                    tc_fence_after();
+                }
+                if (elect_one()) {
                     mma_ss(d_p, v, go, kIdescSS, 0u);
                     mma_ss(d_p, v + 2, go + 2, kIdescSS, 1u);
-                    mma_commit(bar(kSFull + h));
-                    if (kSUnits == 2) mma_commit(bar(kSFull + 1));
+                    mma_commit(on_unit(kSFull, u));
                 }
                 __syncwarp();
-                if (h == kSUnits % 2 && ++I == (uint32_t)nblk) { I = 0; ++nitem; }
+                buf = buffer_after(buf, 1);
+                if (h == 1 && ++I == (uint32_t)nblk) { I = 0; ++nitem; }
             }
         } else if (warp == 2) {
             // ---- dV_J += P^T dO_u and dK~_J += dS^T Q~_u (A from tensor memory, 16 queries per step)
-            uint32_t nitem = 0, I = 0;
+            uint32_t nitem = 0, I = 0, buf = 0;
             for (uint32_t u = 0; u < total_units && ok; ++u) {
                 const uint32_t h = u & 1, g = u >> 1, st = g % kQStages;
                 const bool first = I == 0 && h == 0, last = I == (uint32_t)nblk - 1 && h == 1;
-                if (!wait_all(bar(kPReady + 2 * h + (g & 1)), (g >> 1) & 1) ||
+                if (!wait_all(on_unit(kPReady, u), unit_parity(u)) ||
                     (first && nitem > 0 && !wait_all(bar(kAccFree), (nitem - 1) & 1))) { ok = false; break; }
                 tc_fence_after();
                 if (elect_one()) {
                     const uint32_t ring = base + kOffRing + st * kRingBytes + h * kPatchContent;
                     const uint64_t go = smem_desc_at(kDesc64, ring + kRingDO);
                     const uint64_t q48 = smem_desc_at(kDescQ48, ring + kRingQc);
-                    const uint32_t a_p = tmem + kColP + h * (kHalfCols / 2);
+                    const uint32_t a_p = tmem + kStep * buf;          // 16 queries a step: the first 16 of every 32 columns
 #pragma unroll
                     for (int kk = 0; kk < kTile / 32; ++kk)
-                        mma_ts(tmem + kColDV, a_p + 8 * kk, go + 64 * kk, kIdescT32, (kk || !first) ? 1u : 0u);
+                        mma_ts(tmem + kColDV, a_p + 32 * (kk >> 1) + 8 * (kk & 1), go + 64 * kk, kIdescT32, (kk || !first) ? 1u : 0u);
+                    if (R == 32) mma_commit(on_unit(kPFree, u));      // S^T of unit u + 3 need not wait for dK~ as well
                     if (R == 16) {
-                        const uint32_t a_ds = tmem + kColDS + h * (kHalfCols / 2);
+                        const uint32_t a_ds = a_p + kColDP;
 #pragma unroll
                         for (int kk = 0; kk < kTile / 32; ++kk)
-                            mma_ts(tmem + kColDK, a_ds + 8 * kk, q48 + 64 * kk, kIdescT48, (kk || !first) ? 1u : 0u);
+                            mma_ts(tmem + kColDK, a_ds + 32 * (kk >> 1) + 8 * (kk & 1), q48 + 64 * kk, kIdescT48, (kk || !first) ? 1u : 0u);
                     } else {
                         // A = this half of the dS tile in shared memory, read K-major: rows are keys, the 128-byte lines the
                         // unit's 64 queries (32 bytes per K16 step)
@@ -302,19 +313,20 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                             mma_ss(tmem + kColDK, a_ds + 2 * kk, q48 + 64 * kk, kIdescT48, (kk || !first) ? 1u : 0u);
                         if (h == 1) mma_commit(bar(kDSFree + (g & 1)));
                     }
-                    mma_commit(bar(kPFree + h));
+                    if (R == 16) mma_commit(on_unit(kPFree, u));
                     // the tile's query-side rows may go: S^T, dP^T of both halves finished before P^T existed
                     if (h == 1) mma_commit(bar(kQEmpty + st));
                     if (last) mma_commit(bar(kAccFull));
                 }
                 __syncwarp();
+                buf = buffer_after(buf, 1);
                 if (h == 1 && ++I == (uint32_t)nblk) { I = 0; ++nitem; }
             }
         } else if (warp == 3) {
             // ---- dQ~_I = dS K~_J once both halves of dS are in shared memory (16 keys per step)
             uint32_t nitem = 0, I = 0;
             for (uint32_t g = 0; g < total_tiles && ok; ++g) {
-                if (!wait_all(bar(kPReady + (g & 1)), (g >> 1) & 1) || !wait_all(bar(kPReady + 2 + (g & 1)), (g >> 1) & 1) ||
+                if (!wait_all(on_unit(kPReady, 2 * g), unit_parity(2 * g)) || !wait_all(on_unit(kPReady, 2 * g + 1), unit_parity(2 * g)) ||
                     (g > 0 && !wait_all(bar(kDQFree), (g - 1) & 1))) { ok = false; break; }
                 tc_fence_after();
                 if (elect_one()) {
@@ -342,24 +354,17 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         const int cg = ((warp - 4) >> 2) & 1;                // queries 32 cg .. 32 cg + 31 of the half-tile
         const int quarter = warp & 3;
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-        const uint32_t t_s = tmem + lane_base + kColS + h * kHalfCols + 32 * cg, t_dp = tmem + lane_base + kColDP + h * kHalfCols + 32 * cg;
-        const uint32_t t_p = tmem + lane_base + kColP + h * (kHalfCols / 2) + 16 * cg, t_ds = tmem + lane_base + kColDS + h * (kHalfCols / 2) + 16 * cg;
         const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
         uint32_t g = 0;
         bool ok = true;
-        // The waits for the next unit's query tile and scores are asked between this unit's stores and their completion, in
-        // straight-line code (measured: -1 % on the kernel; behind a branch the gain is gone).  After the CTA's last unit the
-        // question names the phases just used, which are complete, so that no warp sits out the time limit of a wait that
-        // nothing answers.
-        bool polled = false, next_ready = false;
-        const uint32_t last_g = (((uint32_t)p.items - blockIdx.x + gridDim.x - 1) / gridDim.x) * (uint32_t)p.nblk - 1u;
+        uint32_t buf = h;
         for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x) {
             bool key_exists = true;       // kPartial: this warp's 32 key rows lie in one 8x8 patch of the key block
             int key_part = 0, last_window = 0;   // masked shifted windows: part of the key patch; bit 1 / 0: last window row / column
             if (kPartial) {
                 const ItemCoord c = decode_item(p, item);
                 int py, px, Y0, X0;
-                patch_origin(geom, c.wy, c.wx, 2 * c.J + (quarter >> 1), py, px, Y0, X0);
+                patch_origin(geom, p.div_per_row, c.wy, c.wx, 2 * c.J + (quarter >> 1), py, px, Y0, X0);
                 key_exists = Y0 < p.H && X0 < p.W;
                 last_window = (c.wy == p.nWy - 1 ? 2 : 0) | (c.wx == p.nWx - 1 ? 1 : 0);
                 key_part = window_part(p.M, p.s, last_window & 2, last_window & 1, py, px);
@@ -372,19 +377,17 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     key_real = key_exists && key_part == window_part(p.M, p.s, last_window & 2, last_window & 1, (qp / per_row) << 3, (qp % per_row) << 3);
                 }
                 const uint32_t st = g % kQStages;
+                const uint32_t t_s = tmem + lane_base + 32 * cg + kStep * buf, t_dp = R == 16 ? t_s + kColDP : tmem + lane_base + 32 * cg + kColDP + 64 * h;
+                buf = buffer_after(buf, 2);
                 // warp-uniform outcome: the TMEM accesses below are warp-collective
-                if (!(polled && __all_sync(0xffffffffu, next_ready)) &&
-                    !__all_sync(0xffffffffu, mbar_wait(bar(kQFull + st), (g / kQStages) & 1, abort_flag, p.status) &&
-                                                 mbar_wait(bar(kSFull + h), g & 1, abort_flag, p.status))) { ok = false; break; }
-                polled = false;
+                if (!mbar_wait_warp(on_unit(kSFull, 2 * g + h), unit_parity(2 * g), abort_flag, p.status) ||
+                    !mbar_wait_warp(bar(kQFull + st), (g / kQStages) & 1, abort_flag, p.status)) { ok = false; break; }
                 tc_fence_after();
                 // The warp's 32 key rows x 32 queries in four pieces of 16 x 16 (piece c: lanes 16 (c % 2) .., queries 16 (c / 2) ..), read as
                 // 16-lane fragments: a thread holds 2 key rows of 4 queries of a piece, and the per-query (-lse2, -lse2', -D, -D') cost
                 // it 16 words per unit instead of 64.  What these warps share with the operand fetches of the MMAs is the one shared-memory
-                // data pipe (1270 of its passes per tile of 128 x 128 were the warps' with a row of 32 queries per thread and 16-byte broadcasts,
-                // 895 with this form, beside 992 of the MMAs): the reads are 4 bytes wide because a 16-byte read of four different addresses
-                // counted eight passes.  With dS leaving by stmatrix and dQ~ by 16-byte adds, rank 32: 745 -> 638 us, rank 16: 565 -> 555 us
-                // (16 x 96 x 96, windows of 32).
+                // data pipe (840 of its passes per tile of 128 x 128 are theirs, 410 the adds' and stores', 992 the MMAs').  With four-byte columns in planes of
+                // their own these reads take as many passes and more instructions (515 against 511 us).
                 const uint32_t ld = base + kOffRing + st * kRingBytes + kRingLD + (32 * h + 16 * cg + (lane & 3)) * 16;
                 auto ldq = [&](int gq) { return make_float4(lds_f32(ld + 64 * gq), lds_f32(ld + 64 * gq + 4), lds_f32(ld + 64 * gq + 8), lds_f32(ld + 64 * gq + 12)); };
                 const uint32_t ds_line = base + kOffDS + ((g & 1) * 2 + h) * kDSHalf + (quarter * 32 + 8 * ((lane >> 3) & 1) + (lane & 7)) * 128;
@@ -411,66 +414,61 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 // m = (chunk m / 2 of the piece, rows 8 (m % 2) ..)
                 auto store = [&](int c, const uint32_t (&pp)[4], const uint32_t (&dd)[4]) {
                     const uint32_t at = ((uint32_t)(16 * (c & 1)) << 16) + 8 * (c >> 1);
-                    tmem_st_16x128b_x2(t_p + at, pp);
-                    if (R == 16) tmem_st_16x128b_x2(t_ds + at, dd);
+                    tmem_st_16x128b_x2(t_s + at, pp);
+                    if (R == 16) tmem_st_16x128b_x2(t_dp + at, dd);
                     stmatrix_x4(ds_line + 16 * (c & 1) * 128 + (((cg * 4 + 2 * (c >> 1) + (lane >> 4)) ^ (lane & 7)) << 4), dd[0], dd[1], dd[2], dd[3]);
                 };
-                // dV, dK~ of this half's previous unit still read P^T, dS^T; dQ~ of the tile before the previous one still reads this dS
-                // buffer.  (A barrier that has completed no phase answers yes to parity 1, which the first units ask for.)
-                const uint32_t b_p = bar(kPFree + h), b_ds = bar(kDSFree + (g & 1)), p_parity = (g - 1) & 1, ds_parity = ((g >> 1) - 1) & 1;
-                auto buffers_free = [&](bool polled_free) {
-                    return __all_sync(0xffffffffu, polled_free) ||
-                           __all_sync(0xffffffffu, mbar_wait(b_p, p_parity, abort_flag, p.status) && mbar_wait(b_ds, ds_parity, abort_flag, p.status));
+                // dQ~ of the tile before the previous one still reads this dS buffer.  (A barrier that has completed no phase answers yes to
+                // parity 1, which the first tiles ask for.)
+                const uint32_t b_ds = bar(kDSFree + (g & 1)), ds_parity = ((g >> 1) - 1) & 1;
+                // R = 32: dP^T of this half is in registers, the next unit's may overwrite it
+                auto dp_free = [&] {
+                    if (R == 16) return;
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kDPFree + h));
                 };
+                uint32_t pp[4], dd[4];
                 if (kPartial && !key_real) {
                     // nothing of this warp's key rows meets this half-tile's queries (no tokens, or another part of a masked
-                    // window): P^T = dS^T = 0 without reading the scores; the accumulators go back to the MMA warp at once
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kSFree + h));
-                    if (!buffers_free(false)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t zero[4] = {0u, 0u, 0u, 0u};
+                    // window): P^T = dS^T = 0 without reading the scores
+                    dp_free();
+                    if (!mbar_wait_warp(b_ds, ds_parity, abort_flag, p.status)) { ok = false; break; }
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) store(c, zero, zero);
+                    for (int e = 0; e < 4; ++e) pp[e] = dd[e] = 0u;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) store(c, pp, dd);
                 } else {
-                    uint32_t s0[8], dp0[8], s1[8], dp1[8], s2[8], dp2[8], s3[8], dp3[8], pp[4][4], dd[4][4];
+                    // a piece is stored while the next but one is on its way, over scores that this warp has read (all pieces together at the
+                    // end: 537 against 515 us; the next unit's scores asked for ahead, before the arrival: 517)
+                    uint32_t s0[8], dp0[8], s1[8], dp1[8];
                     float4 ta[2], tb[2];
-                    ta[0] = ldq(0); ta[1] = ldq(1);                         // queries 8 gq + 2 (lane % 4), + 1
+                    const bool ds_free = mbar_try_wait(b_ds, ds_parity);
                     load(0, s0, dp0);
                     load(1, s1, dp1);
+                    ta[0] = ldq(0); ta[1] = ldq(1);                         // queries 8 gq + 2 (lane % 4), + 1
                     tmem_wait_ld();
-                    load(2, s2, dp2);
+                    work(s0, dp0, ta, pp, dd);
+                    if (!__all_sync(0xffffffffu, ds_free) && !mbar_wait_warp(b_ds, ds_parity, abort_flag, p.status)) { ok = false; break; }
+                    load(2, s0, dp0);
+                    store(0, pp, dd);
                     tb[0] = ldq(2); tb[1] = ldq(3);
-                    work(s0, dp0, ta, pp[0], dd[0]);
+                    work(s1, dp1, ta, pp, dd);
                     tmem_wait_ld();
-                    load(3, s3, dp3);
-                    work(s1, dp1, ta, pp[1], dd[1]);
+                    load(3, s1, dp1);
+                    store(1, pp, dd);
+                    work(s0, dp0, tb, pp, dd);
                     tmem_wait_ld();
-                    // S^T, dP^T of this half are in registers: the next unit's scores may overwrite them
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kSFree + h));
-                    const bool free_p = mbar_try_wait(b_p, p_parity), free_ds = mbar_try_wait(b_ds, ds_parity);
-                    work(s2, dp2, tb, pp[2], dd[2]);
-                    work(s3, dp3, tb, pp[3], dd[3]);
-                    if (!buffers_free(free_p & free_ds)) { ok = false; break; }
-                    tc_fence_after();
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) store(c, pp[c], dd[c]);
-                }
-                {
-                    const uint32_t gn = g + (g != last_g ? 1u : 0u);
-                    const bool qn = mbar_try_wait(bar(kQFull + gn % kQStages), (gn / kQStages) & 1);
-                    const bool sn = mbar_try_wait(bar(kSFull + h), gn & 1);
-                    next_ready = qn & sn;
-                    polled = true;
+                    dp_free();
+                    store(2, pp, dd);
+                    work(s1, dp1, tb, pp, dd);
+                    store(3, pp, dd);
                 }
                 tmem_wait_st();
                 tc_fence_before();
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kPReady + 2 * h + (g & 1)));
+                if (lane == 0) mbar_arrive(on_unit(kPReady, 2 * g + h));
             }
         }
     } else if (warp >= 20) {
@@ -481,68 +479,87 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         uint32_t g = 0, nitem = 0;
         bool ok = true;
         for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x, ++nitem) {
-            const ItemCoord c = decode_item(p, item);
             for (int I = 0; I < p.nblk; ++I, ++g) {
-                if (!__all_sync(0xffffffffu, mbar_wait(bar(kDQFull), g & 1, abort_flag, p.status))) { ok = false; break; }
+                if (I == p.nblk - 1) {
+                    // dV and dK~ of the item, before its last dQ~: dV and dK~ of the next one wait for the accumulators.  Rows of 64 bytes, one
+                    // per thread, would touch 32 lines with every store instruction and hold up the queue that all warps' loads and stores go
+                    // through for 2000 cycles an item; so they leave by TMA, a warp's 32 rows (half a patch) at a time (510 -> 488 us
+                    // on 16 x 96 x 96 tokens in windows of 32).  Each tile goes to shared memory before the next load: held back until the
+                    // accumulators are released, its rows spill.
+                    const ItemCoord c = decode_item(p, item);
+                    int py, px, Y0, X0;
+                    patch_origin(geom, p.div_per_row, c.wy, c.wx, 2 * c.J + (quarter >> 1), py, px, Y0, X0);
+                    const bool rows_real = !kPartial || (Y0 < p.H && X0 < p.W);   // no dk / dv rows for positions beyond the image
+                    if (!mbar_wait_warp(bar(kAccFull), nitem & 1, abort_flag, p.status)) { ok = false; break; }
+                    tc_fence_after();
+                    const int sw = (row >> 1) & 3;                    // SWIZZLE_64B
+#pragma unroll
+                    for (int which = 0; which < 2; ++which) {         // dV through V's slot, dK through a tile of its own
+                        uint8_t* const stage = base_ptr + (which == 0 ? kOffV + (nitem & 1) * kContentBytes : kOffDK) + row * 64;
+                        const float f = which == 0 ? 1.f : p.inv_sqrt_d;
+                        uint32_t a[32];
+                        tmem_ld32(tmem + lane_base + (which == 0 ? kColDV : kColDK), a);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) w[e] = pack_bf16x2(__uint_as_float(a[8 * q + 2 * e]) * f, __uint_as_float(a[8 * q + 2 * e + 1]) * f);
+                            *reinterpret_cast<uint4*>(stage + ((q ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                        }
+                    }
+                    uint32_t rib[R / 16][16];
+#pragma unroll
+                    for (int part = 0; part < R / 16; ++part) tmem_ld16(tmem + lane_base + kColDK + kD + 16 * part, rib[part]);
+                    tmem_wait_ld();
+                    tc_fence_before();
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(bar(kAccFree));
+                        if (rows_real) {
+                            tma_store_5d(&tm_dv, base + kOffV + (nitem & 1) * kContentBytes + quarter * (kPatchContent / 2), 0, c.h, X0, Y0 + 4 * (quarter & 1), c.b);
+                            tma_store_5d(&tm_dk, base + kOffDK + quarter * (kPatchContent / 2), 0, c.h, X0, Y0 + 4 * (quarter & 1), c.b);
+                            bulk_commit_group();
+                        }
+                    }
+                    float* dst_p = p.dkp + (size_t)c.pair * R * p.n + 4 * ((size_t)c.J * kTile + row);
+#pragma unroll
+                    for (int col = 0; col < R; col += 4) {
+                        const uint32_t* v = rib[col >> 4] + (col & 15);
+                        *reinterpret_cast<float4*>(dst_p + (size_t)col * p.n) = make_float4(__uint_as_float(v[0]) * p.inv_sqrt_d, __uint_as_float(v[1]) * p.inv_sqrt_d,
+                                                                                            __uint_as_float(v[2]) * p.inv_sqrt_d, __uint_as_float(v[3]) * p.inv_sqrt_d);
+                    }
+                }
+                if (!mbar_wait_warp(bar(kDQFull), g & 1, abort_flag, p.status)) { ok = false; break; }
                 tc_fence_after();
-                float* dst = p.dq_acc + (size_t)c.pair * kDk * p.n + 4 * ((size_t)I * kTile + row);
-                // all columns into registers first, so that the next tile's dQ~ may start while the adds drain
-                uint32_t a[kDk / 16][16];
+                float* dst = p.dq_acc + (size_t)p.div_nblk.div(item) * kDk * p.n + 4 * ((size_t)I * kTile + row);
 #pragma unroll
-                for (int part = 0; part < kDk / 16; ++part) tmem_ld16(tmem + lane_base + kColDQ + 16 * part, a[part]);
-                tmem_wait_ld();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kDQFree));
+                for (int part = 0; part < kDk / 16; ++part) {
+                    uint32_t a[16];
+                    tmem_ld16(tmem + lane_base + kColDQ + 16 * part, a);
+                    tmem_wait_ld();
+                    if (part + 1 == kDk / 16) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar(kDQFree));
+                    }
 #pragma unroll
-                for (int col = 0; col < kDk; col += 4, dst += 4 * (size_t)p.n) {
-                    red_add_f32x4(dst, a[col >> 4] + (col & 15));
-                    // The adds of a tile in one burst hold up the loads and stores of the other warps, which go through the same queue: a short
-                    // pause after each (rank 32: after every second one) spreads them over the tile's time (550 -> 535 us at rank 16,
-                    // 641 -> 633 us at rank 32, 16 x 96 x 96 tokens in windows of 32; 50 ns pauses: 542 and 689 us).
-                    if (R == 16 || (col & 4)) __nanosleep(20);
+                    for (int col = 0; col < 16; col += 4) {
+                        red_add_f32x4(dst, a + col);
+                        dst += 4 * (size_t)p.n;
+                        if (R == 16 || (col & 4)) __nanosleep(20);
+                    }
                 }
             }
             if (!ok) break;
-            if (!__all_sync(0xffffffffu, mbar_wait(bar(kAccFull), nitem & 1, abort_flag, p.status))) { ok = false; break; }
-            tc_fence_after();
-            int i, Y, X;
-            window_order_token(geom, c.wy, c.wx, c.J * kTile + row, i, Y, X);
-            const bool row_real = !kPartial || (Y < p.H && X < p.W);      // no dk / dv row for a position beyond the image
-            const size_t tok = row_real ? (((size_t)c.b * p.H + Y) * p.W + X) * p.heads + c.h : 0;
-            uint4* dst_v = reinterpret_cast<uint4*>(p.dv + tok * p.d);
-            uint4* dst_k = reinterpret_cast<uint4*>(p.dk + tok * p.d);
-            float* dst_p = p.dkp + (size_t)c.pair * R * p.n + 4 * ((size_t)c.J * kTile + row);
-            constexpr int kParts = 4 + R / 16;
-#pragma unroll
-            for (int part = 0; part < kParts; ++part) {      // dV (2 x 16 columns), dK~ content (2 x 16), dK~ RIB (R / 16 x 16)
-                uint32_t a[16];
-                tmem_ld16(tmem + lane_base + kColDV + 16 * part, a);     // dV, dK~ are adjacent in tensor memory
-                tmem_wait_ld();
-                if (part == kParts - 1) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kAccFree));
-                }
-                if (part >= 4) {
-#pragma unroll
-                    for (int col = 0; col < 16; col += 4)
-                        *reinterpret_cast<float4*>(dst_p + (size_t)(16 * (part - 4) + col) * p.n) =
-                            make_float4(__uint_as_float(a[col]) * p.inv_sqrt_d, __uint_as_float(a[col + 1]) * p.inv_sqrt_d,
-                                        __uint_as_float(a[col + 2]) * p.inv_sqrt_d, __uint_as_float(a[col + 3]) * p.inv_sqrt_d);
-                } else if (row_real) {
-                    const float f = part < 2 ? 1.f : p.inv_sqrt_d;
-                    uint4* dst16 = (part < 2 ? dst_v : dst_k) + 2 * (part & 1);
-#pragma unroll
-                    for (int q2 = 0; q2 < 2; ++q2)
-                        if (16 * (part & 1) + 8 * q2 < p.d)       // a head narrower than 32 channels: the rest is padding
-                        dst16[q2] = make_uint4(pack_bf16x2(__uint_as_float(a[8 * q2 + 0]) * f, __uint_as_float(a[8 * q2 + 1]) * f),
-                                               pack_bf16x2(__uint_as_float(a[8 * q2 + 2]) * f, __uint_as_float(a[8 * q2 + 3]) * f),
-                                               pack_bf16x2(__uint_as_float(a[8 * q2 + 4]) * f, __uint_as_float(a[8 * q2 + 5]) * f),
-                                               pack_bf16x2(__uint_as_float(a[8 * q2 + 6]) * f, __uint_as_float(a[8 * q2 + 7]) * f));
-                }
+            if (lane == 0) {
+                bulk_wait_group_read<0>();          // (this thread's own stores)
+                mbar_arrive(bar(kKVEmpty + (nitem & 1)));
             }
+            __syncwarp();
         }
+        if (lane == 0) bulk_wait_group<0>();
     }
     // ================================================================================ common tail
     tc_fence_before();
@@ -766,10 +783,10 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     float* dkp = reinterpret_cast<float*>(ws + wl.dkp);
     __nv_bfloat16* pq_scaled = reinterpret_cast<__nv_bfloat16*>(ws + wl.pq_scaled);
 
-    CUtensorMap tm_q, tm_k, tm_v, tm_do, tm_pqs, tm_pk;
+    CUtensorMap tm_q, tm_k, tm_v, tm_do, tm_pqs, tm_pk, tm_dk, tm_dv;
     if (!encode_image_map(&tm_q, p.q, p) || !encode_image_map(&tm_k, p.k, p) || !encode_image_map(&tm_v, p.v, p) ||
         !encode_image_map(&tm_do, p.dout, p) || !encode_pos_map_padded(&tm_pqs, pq_scaled, p, tables, (long long)p.n * R, R) ||
-        !encode_pos_map_padded(&tm_pk, p.pk, p, tables, p.pos_head_stride, p.r))
+        !encode_pos_map_padded(&tm_pk, p.pk, p, tables, p.pos_head_stride, p.r) || !encode_image_map(&tm_dk, p.dk, p, 4) || !encode_image_map(&tm_dv, p.dv, p, 4))
         return cudaErrorInvalidValue;
     static KernelSetup setup;       // one per instantiation of this launcher, i.e. per kernel
     int sm_count = 0;
@@ -794,18 +811,19 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     if (e != cudaSuccess) return e;
 
     BwdParams bp{};
-    bp.ld = ld; bp.dq_acc = dq_acc; bp.dkp = dkp; bp.dk = p.dk; bp.dv = p.dv; bp.status = p.status;
+    bp.ld = ld; bp.dq_acc = dq_acc; bp.dkp = dkp; bp.status = p.status;
     bp.H = p.H; bp.W = p.W; bp.heads = p.heads; bp.M = p.M; bp.s = p.s; bp.n = p.n; bp.nWy = p.nWy; bp.nWx = p.nWx;
     bp.Hp = p.Hp; bp.Wp = p.Wp;
     bp.nblk = p.n / kTile;
     bp.items = p.pairs * bp.nblk;
     bp.pos_per_head = tables > 1 ? 1 : 0;
     bp.masked = p.masked ? 1 : 0;
-    bp.d = p.d;
     bp.scale_log2 = 1.4426950408889634f / sqrtf(scale_width_d(p));
     bp.inv_sqrt_d = ap.inv_sqrt_d;
+    bp.div_nblk = make_fast_div(bp.nblk); bp.div_heads = make_fast_div(p.heads); bp.div_nwx = make_fast_div(p.nWx); bp.div_nwy = make_fast_div(p.nWy);
+    bp.div_per_row = make_fast_div(p.M >> 3);
     const int grid = bp.items < sm_count ? bp.items : sm_count;
-    { ProfileScope scope(RIB_KERNEL_BWD_MAIN, stream); rib_bwd_sm100_kernel<R, kPartial><<<grid, kThreads, kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_do, tm_pqs, tm_pk, bp); }
+    { ProfileScope scope(RIB_KERNEL_BWD_MAIN, stream); rib_bwd_sm100_kernel<R, kPartial><<<grid, kThreads, kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_do, tm_pqs, tm_pk, tm_dk, tm_dv, bp); }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
 

@@ -258,12 +258,12 @@ inline void map_cache_counts(long long* hits, long long* misses)
 // bf16 [B][H][W][heads][d] image tensor (d = 8, 16, 24 or 32), box = one 8x8-token patch of one head, always 32 channels
 // wide: on a narrower head the channels from d on lie beyond the tensor and arrive as zeros, so a tile has one layout
 // for every head width and the zero channels change no dot product.
-inline bool encode_image_map_now(CUtensorMap* map, const void* ptr, const Problem& p)
+inline bool encode_image_map_now(CUtensorMap* map, const void* ptr, const Problem& p, int rows)
 {
     const cuuint64_t dims[5] = {(cuuint64_t)p.d, (cuuint64_t)p.heads, (cuuint64_t)p.W, (cuuint64_t)p.H, (cuuint64_t)p.B};
     const cuuint64_t row = (cuuint64_t)p.d * 2;
     const cuuint64_t strides[4] = {row, row * p.heads, row * p.heads * p.W, row * p.heads * p.W * p.H};
-    const cuuint32_t box[5] = {(cuuint32_t)kD, 1, 8, 8, 1};
+    const cuuint32_t box[5] = {(cuuint32_t)kD, 1, 8, (cuuint32_t)rows, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(ptr), dims, strides, box, estr,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -273,10 +273,11 @@ inline bool encode_image_map_now(CUtensorMap* map, const void* ptr, const Proble
 // bf16 [tables][M][M][r] positional features (one table shared by all heads, or one per head; r = p.r), box = one
 // 8x8-token patch of one table.  `tables` = 1 or heads, `table_stride` elements apart (a multiple of 8,
 // at least M * M * 16); a kernel addresses table h * (tables > 1).
-inline bool encode_image_map(CUtensorMap* map, const void* ptr, const Problem& p)
+// (`rows`: token rows of a box; 4 for the half patch that one warp holds)
+inline bool encode_image_map(CUtensorMap* map, const void* ptr, const Problem& p, int rows = 8)
 {
-    const MapKey key{ptr, 0, 0, 1, p.B, p.H, p.W, p.heads, p.d};
-    return cached_map(map, key, [&](CUtensorMap* m) { return encode_image_map_now(m, ptr, p); });
+    const MapKey key{ptr, rows, 0, 1, p.B, p.H, p.W, p.heads, p.d};
+    return cached_map(map, key, [&](CUtensorMap* m) { return encode_image_map_now(m, ptr, p, rows); });
 }
 
 inline bool encode_pos_map_now(CUtensorMap* map, const void* ptr, const Problem& p, int tables, long long table_stride,
