@@ -393,13 +393,6 @@ struct TcLayout {
     static constexpr uint32_t kTmemCols = kColW + kBlocks * D <= 256 ? 256 : 512;
 };
 
-// 32-byte store of eight 32-bit words; the address must be 32-byte aligned
-__device__ __forceinline__ void st_global_v8(float* dst, const uint32_t* v)
-{
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),
-                 "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
-}
-
 template <int D>
 __global__ void __launch_bounds__(kTcThreads, 1) rib_cla_bwd_tc_kernel(const ClaBwdParams p)
 {

@@ -333,6 +333,12 @@ __device__ __forceinline__ void red_add_f32x4(float* addr, const uint32_t* v)
     asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};"
                  ::"l"(addr), "f"(__uint_as_float(v[0])), "f"(__uint_as_float(v[1])), "f"(__uint_as_float(v[2])), "f"(__uint_as_float(v[3])) : "memory");
 }
+// 32-byte store of eight 32-bit words (one whole sector); the address must be 32-byte aligned
+__device__ __forceinline__ void st_global_v8(void* dst, const uint32_t* v)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),
+                 "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
 __device__ __forceinline__ float lds_f32(uint32_t addr)
 {
     float v;

@@ -47,3 +47,20 @@ def test_every_element(wl, form):
         assert np.abs(ref_lse).max() > 100
     compare("out", to_f64(out), ref_out, max_abs=2e-2 if far else 1e-2)
     compare("lse", to_f64(lse), ref_lse, max_abs=2e-2 * max(1.0, np.abs(ref_lse).max() / 100) if far else 1e-2)
+
+
+@pytest.mark.parametrize("d", [16, 32])
+def test_an_output_that_is_aligned_to_16_bytes_only(d):
+    """Rows of out leave as 32-byte sectors where they are such; elsewhere the same bits, and nothing beyond them."""
+    wl = Workload("b_align", 1, 64, 64, 2, d, 16, 32, 8, seed=306)
+    _, gpu = make(wl, with_dout=False)
+    args = [gpu[k] for k in ("q", "k", "v", "pq", "pk")]
+    expected, _ = binding.rib_window_attn_fwd(*args, wl.window, wl.shift)
+    n = expected.numel()
+    memory = torch.full((n + 64,), 3.0, dtype=torch.bfloat16, device="cuda")
+    out = memory[8:8 + n].view(expected.shape)
+    assert out.data_ptr() % 32 == 16
+    binding.rib_window_attn_fwd(*args, wl.window, wl.shift, out=out)
+    torch.cuda.synchronize()
+    assert torch.equal(out, expected)
+    assert (memory[:8] == 3.0).all() and (memory[8 + n:] == 3.0).all()
