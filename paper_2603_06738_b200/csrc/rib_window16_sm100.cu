@@ -5,11 +5,11 @@
 // memory) exceeds its arithmetic.  Here a CTA keeps to one head (CTA c: head c mod heads), stages the head's RIB rows once,
 // takes whole windows one after the other and lets them overlap, and no gradient but those of the tables is summed
 // outside the chip.  What bounds it: the serial program of the softmax (arithmetic) warps.  A unit of the forward (128 rows x 256
-// keys) takes about 3900 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) 3700 at rank 16 and 32 channels
-// (3300 at rank 24 and 16 channels): 450 until its scores are there, 1150 (1240) of loads and exponentials, 2100 (1600) of waiting for
-// the buffers of P and dS, stores into them and fences, with 1470 cycles of MMAs beside it.  Measured by event hooks against the general
-// kernels (4 x 96 x 96 tokens, 12 heads of 16 channels, rank 24, shift 8, masked): forward 82 -> 60 us, backward 30 + 140 + 46 -> 13 (two
-// clearings) + 99 us, both calls 288 -> 154 us; backward on 10 x 64 x 64 tokens, 6 heads of 32 channels, rank 16: 20 + 66 + 23 -> 13 + 70 us.
+// keys) takes about 3900 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) 3000 at rank 16 and 32 channels:
+// 200 until its scores are there, 1500 of loads and exponentials, 1000 of stores of P and dS and fences, with 1470 cycles of MMAs
+// beside it.  Measured by event hooks against the general kernels (4 x 96 x 96 tokens, 12 heads of 16 channels, rank 24, shift 8,
+// masked): forward 60 against 82 us, backward 13 (two clearings) + 97 against 30 + 123 + 44 us; backward on 16 x 96 x 96 tokens, 6 heads of 32
+// channels: rank 16 13 + 180 against 56 + 199 + 62, rank 32 13 + 201 against 62 + 228 + 103.
 //
 // Windows may be shifted (multiples of 8), masked, or reach beyond the map (sides multiples of 8): a window is four 8x8-token
 // patches (one TMA box each), and a query patch attends to a key patch or not.
@@ -308,20 +308,25 @@ rib_window16_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
 //     S = Q~_I K~_J^T, dP = dO_I V_J^T;   P = exp2(S log2e/sqrt(d) - lse log2e), dS = P o (dP - D);
 //     dV_J += P^T dO_I, dK~_J += dS^T Q~_I (A = the stored tiles, MN-major), dQ~_I += dS K~_J (A K-major).
 // dV_J and dK~_J leave the chip after their two units, dQ~ at the end of the window.  The content columns of dQ~ are cleared
-// when they have been read, its RIB columns (gradients of Pq) add up over the CTA's windows; those of dK~ are added to
-// global memory block by block (tensor memory has no room for both blocks at rank 32).
+// when they have been read, its RIB columns (gradients of Pq) add up over the CTA's windows; those of dK~ do so in columns of their own at
+// rank 16, and are added to global memory block by block at rank 32, for which tensor memory has no room.  (All windows' adds to one table
+// meet at the same addresses: where the tables lay on some of them the kernel took 215 us instead of 180 at rank 16.)
 //
-// Roles (768 threads): warp 0 TMA loads; warp 1 issues S and dP, warp 3 dV, dK~ and dQ~; warp 2 owns the TMEM allocation; warps
-// 4-19 P and dS (four threads per query row, 32 keys each); warps 20-23 write (-lse log2e, -D) of the next window's rows to
-// tensor memory, a row being a TMEM lane to everybody, and move the gradients out: dv from registers, dk and dq through the shared
-// memory of the window's own rows and TMA stores.
+// Roles (896 threads): warp 0 TMA loads; warp 1 issues S and dP, warp 3 dV, dK~ and dQ~; warp 2 owns the TMEM allocation; warps
+// 4-19 P and dS (four threads per query row, 32 keys each); warps 20-23 move the gradients out, dv from registers, dk and dq through the
+// shared memory of the window's own rows, from where warp 2 stores them by TMA and gives the stage back; warps 24-27 write
+// (-lse log2e, -D) of the windows to come to tensor memory, a row being a TMEM lane to everybody.  (One set of warps for both, and lanes
+// that load whole rows: 215 us on 16 x 96 x 96 tokens, 6 heads of 32 channels, rank 16, 240 at rank 32.  dv in 32-byte stores, four lanes to a
+// row of dO and O and stores by warp 2 191 / 211, warps of their own, with dO from the stage, 180 / 201: 8000 cycles of waiting for
+// loads held up dV and dK~ of the next window.)
 namespace bwd16 {
-constexpr int kThreads = 768, kStages = 2;
+constexpr int kThreads = 896, kStages = 2;
 constexpr uint32_t kQ = 0, kK = kWindowBytes, kV = 2 * kWindowBytes, kDO = 3 * kWindowBytes, kStageBytes = 4 * kWindowBytes;
 constexpr uint32_t kOffRib = kStages * kStageBytes;                           // query RIB rows, key RIB rows
 constexpr uint32_t kHalf = kTile * 128;                                       // P, dS: [2 halves of 64 keys][128 queries][128 bytes], SWIZZLE_128B
 constexpr uint32_t kOffP = kOffRib + 2 * kWindowBytes, kOffDS = kOffP + 2 * kHalf, kOffBar = kOffDS + 2 * kHalf;
-enum Bar { kFull = 0, kEmpty = kFull + kStages, kSFull = kEmpty + kStages, kSFree, kPReady, kPDone, kSReady, kSDone, kAcc, kKVFree, kQFree, kLd, kDrain = kLd + 2, kNumBars = kDrain + 2 };
+enum Bar { kFull = 0, kEmpty = kFull + kStages, kSFull = kEmpty + kStages, kSFree, kPReady, kPDone, kSReady, kSDone, kAcc, kKVFree, kQFree, kLd, kLdFree = kLd + 2, kStaged, kDrain = kStaged + 4,
+           kNumBars = kDrain + 2 };      // kStaged: 2 * parity of the window + key block
 constexpr uint32_t kOffMisc = kOffBar + kNumBars * 8;
 constexpr uint32_t kSmemBytes = kOffMisc + 16 + 1024;
 static_assert(kOffP % 1024 == 0 && kSmemBytes <= 232448, "shared memory of one CTA");
@@ -330,6 +335,7 @@ static_assert(kOffP % 1024 == 0 && kSmemBytes <= 232448, "shared memory of one C
 constexpr uint32_t kColS = 0, kColDP = 128, kColDV = 256, kColDK = 288;
 template <int R> constexpr uint32_t kColDQ = kColDK + kD + R;
 template <int R> constexpr uint32_t kColLd = kColDQ<R> + 2 * (kD + R);
+template <int R> constexpr uint32_t kColRib = kColLd<R> + 8;       // R = 16: RIB columns of dK~ of both blocks, added up over the CTA's windows
 
 constexpr uint32_t kIdescS = idesc_bf16_f32(kTile, kTile, false);
 
@@ -337,9 +343,9 @@ template <int R>
 __global__ void __launch_bounds__(kThreads, 1)
 rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                         const __grid_constant__ CUtensorMap tm_do, const __grid_constant__ CUtensorMap tm_dq, const __grid_constant__ CUtensorMap tm_dk,
-                        __nv_bfloat16* const dv, const __grid_constant__ SmallWindowParams p)
+                        __nv_bfloat16* const dv, const int dv_sectors, const __grid_constant__ SmallWindowParams p)
 {
-    static_assert(kColLd<R> + 8 <= 512, "tensor memory has 512 columns");
+    static_assert(kColRib<R> + (R == 16 ? 2 * R : 0) <= 512, "tensor memory has 512 columns");
     constexpr uint32_t kIdescDV = idesc_bf16_f32_ab(kTile, kD, true, true), kIdescDK = idesc_bf16_f32_ab(kTile, kD + R, true, true);
     constexpr uint32_t kIdescDQ = idesc_bf16_f32_ab(kTile, kD + R, false, true);
     extern __shared__ uint8_t smem_raw[];
@@ -359,6 +365,8 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         for (int s = 0; s < kStages; ++s) { mbar_init(bar(kFull + s), 1); mbar_init(bar(kEmpty + s), 1); mbar_init(bar(kLd + s), 4); }
         mbar_init(bar(kSFull), 1); mbar_init(bar(kSFree), 16); mbar_init(bar(kPReady), 16); mbar_init(bar(kPDone), 1); mbar_init(bar(kSReady), 16); mbar_init(bar(kSDone), 1);
         mbar_init(bar(kAcc), 1); mbar_init(bar(kKVFree), 4); mbar_init(bar(kQFree), 4);
+        mbar_init(bar(kLdFree), 16);
+        for (int i = 0; i < 4; ++i) mbar_init(bar(kStaged + i), 4);
         mbar_init(bar(kDrain), 1); mbar_init(bar(kDrain + 1), 1);
         fence_barrier_init();
         prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v); prefetch_tensormap(&tm_do);
@@ -426,6 +434,33 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         if (elect_one()) mma_commit(bar(kDrain));
         __syncwarp();
         mbar_wait(bar(kDrain), 0, abort_flag + 1, p.status);
+    } else if (warp == 2) {
+        // ---- gradient rows that lie staged in the window's own rows leave by TMA; then the stage may be filled again
+        if (lane == 0) {
+            for (int t = 0; t < count; ++t) {
+                const int st = t % kStages;
+                const Win16 w = decode_window(p, group0 + t * p.groups);
+                bool ok = true;
+                for (int J = 0; J < 2 && ok; ++J) {
+                    ok = mbar_wait(bar(kStaged + 2 * (t & 1) + J), (t >> 1) & 1, abort_flag, p.status);
+                    if (!ok) break;
+                    const uint32_t at = base + st * kStageBytes;
+                    for (int patch = 0; patch < 4; ++patch) {
+                        int Y0, X0;
+                        patch_at(p, w, patch, Y0, X0);
+                        if (Y0 >= p.H || X0 >= p.W) continue;
+                        if ((patch >> 1) == J) tma_store_5d(&tm_dk, at + kK + patch * kPatchContent, 0, head, X0, Y0, w.b);
+                        if (J == 1) tma_store_5d(&tm_dq, at + kQ + patch * kPatchContent, 0, head, X0, Y0, w.b);
+                    }
+                    bulk_commit_group();
+                }
+                if (!ok) break;
+                bulk_wait_group_read<0>();              // (this thread's own stores)
+                mbar_arrive(bar(kEmpty + st));
+            }
+            bulk_wait_group<0>();
+        }
+        __syncwarp();
     } else if (warp == 3) {
         // ---- dV of a unit once P is stored, dK~ and dQ~ once dS is, and the accumulators that it starts have been read
         constexpr uint64_t kDescT = smem_desc_const(kHalf, 1024, kSwizzle128B);         // MN-major: the two 64-key halves one leading step apart
@@ -510,7 +545,10 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             tmem_wait_ld();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kSFree));
+            if (lane == 0) {
+                mbar_arrive(bar(kSFree));
+                if ((u & 3) == 0) mbar_arrive(bar(kLdFree));          // nobody reads (-lse2, -D) of the window before any more
+            }
             // have the contractions of the unit before read P and dS?  (No phase completed answers yes to parity 1, which unit 0 asks for.)
             const bool p_free = mbar_try_wait(bar(kPDone), (u - 1) & 1), ds_free = mbar_test(bar(kSDone), (u - 1) & 1);
             work(2);
@@ -545,51 +583,76 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             };
             if (!store(p_row, pp, bar(kPDone), bar(kPReady)) || !store(ds_row, dd, bar(kSDone), bar(kSReady))) break;
         }
-    } else if (warp >= 20) {
-        // ---- (-lse2, -D) in, gradients out: thread = row of a tile
-        const int quarter = warp & 3, row = quarter * 32 + lane;
+    } else if (warp >= 24) {
+        // ---- (-lse2, -D) of every window: thread = row of a tile
+        const int quarter = warp & 3;
         const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
-        const size_t table = (size_t)head * p.pos_head_stride;
-        auto load_scalars = [&](int t) {
+        const uint32_t line = (uint32_t)(p.W * p.heads * p.d), in_line = (uint32_t)((lane >> 2) * p.heads * p.d + 8 * (lane & 3));
+        for (int t = 0; t < count; ++t) {
+            if (t >= 1 && !mbar_wait_warp(bar(kLdFree), (t - 1) & 1, abort_flag, p.status)) break;
+            tc_fence_after();
+            // D = dO . O: four lanes take a row (8 channels each), an instruction the 8 rows of a line of tokens; dO lies in the stage.  (With a row per
+            // lane every load touches 32 lines, which holds up the queue of everybody's loads and stores.)
             const Win16 w = decode_window(p, group0 + t * p.groups);
+            float neg_lse[2] = {-INFINITY, -INFINITY}, neg_d[2] = {0.f, 0.f};      // a query beyond the map: probability 0
+            bool exists[2];
+            uint4 y[2][4];
 #pragma unroll
             for (int I = 0; I < 2; ++I) {
                 int Y0, X0;
-                patch_at(p, w, 2 * I + (row >> 6), Y0, X0);
-                float neg_lse = -INFINITY, neg_d = 0.f;      // a query beyond the map: probability 0
-                if (Y0 < p.H && X0 < p.W) {
-                    const int Y = Y0 + ((row >> 3) & 7), X = X0 + (row & 7);
-                    const size_t tok = (((size_t)w.b * p.H + Y) * p.W + X) * p.heads + head;
-                    neg_lse = -p.lse_in[(((size_t)w.b * p.heads + head) * p.H + Y) * p.W + X] * 1.4426950408889634f;
-                    const uint4 *a = reinterpret_cast<const uint4*>(p.dout + tok * p.d), *b = reinterpret_cast<const uint4*>(p.out + tok * p.d);
+                patch_at(p, w, 2 * I + (quarter >> 1), Y0, X0);
+                exists[I] = Y0 < p.H && X0 < p.W;            // warp-uniform
+                Y0 += 4 * (quarter & 1);                     // this warp's 4 x 8 tokens; lane = 8 * row + column
+                size_t at = ((((size_t)w.b * p.H + Y0) * p.W + X0) * p.heads + head) * p.d + in_line;
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        const bool in = 8 * q4 < p.d;
-                        const uint4 zero = make_uint4(0u, 0u, 0u, 0u), x = in ? __ldg(a + q4) : zero, y = in ? __ldg(b + q4) : zero;
-                        const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+                for (int j = 0; j < 4; ++j, at += line)
+                    y[I][j] = exists[I] && 8 * (lane & 3) < p.d ? __ldg(reinterpret_cast<const uint4*>(p.out + at)) : make_uint4(0u, 0u, 0u, 0u);
+                if (exists[I]) neg_lse[I] = p.lse_in[(((size_t)w.b * p.heads + head) * p.H + Y0 + (lane >> 3)) * p.W + X0 + (lane & 7)];
+            }
+            const int st = t % kStages;
+            if (!mbar_wait_warp(bar(kFull + st), (t / kStages) & 1, abort_flag, p.status)) break;
+#pragma unroll
+            for (int I = 0; I < 2; ++I) {
+                if (exists[I]) {
+                    const uint8_t* const rows = base_ptr + st * kStageBytes + kDO + I * kContentBytes + (quarter * 32 + (lane >> 2)) * 64;
+                    neg_lse[I] *= -1.4426950408889634f;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const uint4 x = *reinterpret_cast<const uint4*>(rows + 512 * j + (((lane & 3) ^ ((lane >> 3) & 3)) << 4));      // SWIZZLE_64B
+                        const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y[I][j].x, y[I][j].y, y[I][j].z, y[I][j].w};
+                        float sum = 0.f;
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            neg_d = fmaf(-__uint_as_float(xs[e] << 16), __uint_as_float(ys[e] << 16), neg_d);
-                            neg_d = fmaf(-__uint_as_float(xs[e] & 0xffff0000u), __uint_as_float(ys[e] & 0xffff0000u), neg_d);
+                            sum = fmaf(-__uint_as_float(xs[e] << 16), __uint_as_float(ys[e] << 16), sum);
+                            sum = fmaf(-__uint_as_float(xs[e] & 0xffff0000u), __uint_as_float(ys[e] & 0xffff0000u), sum);
                         }
+                        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                        const float mine = __shfl_sync(0xffffffffu, sum, 4 * (lane & 7));
+                        if ((lane >> 3) == j) neg_d[I] = mine;
                     }
                 }
                 __syncwarp();
-                tmem_st2(lanes + kColLd<R> + 4 * (t & 1) + 2 * I, __float_as_uint(neg_lse), __float_as_uint(neg_d));
+                tmem_st2(lanes + kColLd<R> + 4 * (t & 1) + 2 * I, __float_as_uint(neg_lse[I]), __float_as_uint(neg_d[I]));
             }
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kLd + (t & 1)));
-        };
+        }
+    } else if (warp >= 20) {
+        // ---- gradients out: thread = row of a tile
+        const int quarter = warp & 3, row = quarter * 32 + lane;
+        const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
+        const size_t table = (size_t)head * p.pos_head_stride;
         auto clear32 = [&](uint32_t col) {
             uint32_t zero[32];
 #pragma unroll
             for (int e = 0; e < 32; ++e) zero[e] = 0u;
             tmem_st32(lanes + col, zero);
         };
-        load_scalars(0);
         for (int I = 0; I < 2; ++I) { clear32(kColDQ<R> + I * (kD + R)); clear32(kColDQ<R> + I * (kD + R) + R); }      // 32 + R columns each
+        if (R == 16) clear32(kColRib<R>);
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -599,10 +662,8 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         for (int t = 0; t < count && ok; ++t) {
             const int st = t % kStages;
             uint8_t* const stage = base_ptr + st * kStageBytes;
-            if (t + 1 < count) load_scalars(t + 1);
             const Win16 w = decode_window(p, group0 + t * p.groups);
             for (int J = 0; J < 2; ++J) {
-                // (the vote of the named barrier below keeps the four warps together)
                 ok = mbar_wait_warp(bar(kAcc), J, abort_flag, p.status);
                 if (ok) {
                     tc_fence_after();
@@ -613,29 +674,46 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                     patch_at(p, w, 2 * J + (row >> 6), Y0, X0);
                     if (Y0 < p.H && X0 < p.W) {              // warp-uniform
                         uint4* const dst = reinterpret_cast<uint4*>(dv + ((((size_t)w.b * p.H + Y0 + ((row >> 3) & 7)) * p.W + X0 + (row & 7)) * p.heads + head) * p.d);
+                        uint32_t v[16];
 #pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4) {
-                            if (8 * q4 >= p.d) break;
-                            uint32_t v[4];
+                        for (int e = 0; e < 16; ++e) v[e] = pack_bf16x2(__uint_as_float(a[2 * e]), __uint_as_float(a[2 * e + 1]));
+                        if (dv_sectors) {                    // rows of whole 32-byte sectors: half the instructions, each of which touches 32 lines
+                            st_global_v8(dst, v);
+                            if (p.d > 16) st_global_v8(dst + 2, v + 8);
+                        } else {
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) v[e] = pack_bf16x2(__uint_as_float(a[8 * q4 + 2 * e]), __uint_as_float(a[8 * q4 + 2 * e + 1]));
-                            dst[q4] = make_uint4(v[0], v[1], v[2], v[3]);
+                            for (int q4 = 0; q4 < 4; ++q4) {
+                                if (8 * q4 >= p.d) break;
+                                dst[q4] = make_uint4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
+                            }
                         }
                     }
                     __syncwarp();
                     tmem_ld32(lanes + kColDK, a);
                     tmem_wait_ld();
                     write_row(stage + kK + J * kContentBytes, row, a, p.inv_sqrt_d);
-                    if (R == 16) tmem_ld16(lanes + kColDK + kD, reinterpret_cast<uint32_t(&)[16]>(a));
-                    else tmem_ld32(lanes + kColDK + kD, a);
+                    uint32_t sums[16];
+                    if (R == 16) {
+                        tmem_ld16(lanes + kColDK + kD, reinterpret_cast<uint32_t(&)[16]>(a));
+                        tmem_ld16(lanes + kColRib<R> + R * J, sums);
+                    } else {
+                        tmem_ld32(lanes + kColDK + kD, a);
+                    }
                     tmem_wait_ld();
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(kKVFree));
-                    float* const gk = p.dpk + table + (size_t)table_row(J * kTile + row) * p.r;
+                    if (R == 16) {
 #pragma unroll
-                    for (int c = 0; c < R; c += 4)
-                        if (c < p.r) add_columns(gk + c, a + c, p.inv_sqrt_d);           // (the query rows carried sqrt(d / r))
+                        for (int e = 0; e < 16; ++e) sums[e] = __float_as_uint(__uint_as_float(sums[e]) + __uint_as_float(a[e]));
+                        tmem_st16(lanes + kColRib<R> + R * J, sums);
+                        tmem_wait_st();
+                    } else {
+                        float* const gk = p.dpk + table + (size_t)table_row(J * kTile + row) * p.r;
+#pragma unroll
+                        for (int c = 0; c < R; c += 4)
+                            if (c < p.r) add_columns(gk + c, a + c, p.inv_sqrt_d);       // (the query rows carried sqrt(d / r))
+                    }
                     if (J == 1) {
 #pragma unroll
                         for (int I = 0; I < 2; ++I) {
@@ -650,24 +728,10 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                         if (lane == 0) mbar_arrive(bar(kQFree));
                     }
                     fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kStaged + 2 * (t & 1) + J));
                 }
-                if (!named_barrier_and(1, 128, ok)) { ok = false; break; }
-                if (warp == 20 && lane == 0) {
-                    const uint32_t at = base + st * kStageBytes;
-                    for (int patch = 0; patch < 4; ++patch) {
-                        int Y0, X0;
-                        patch_at(p, w, patch, Y0, X0);
-                        if (Y0 >= p.H || X0 >= p.W) continue;
-                        if ((patch >> 1) == J) tma_store_5d(&tm_dk, at + kK + patch * kPatchContent, 0, head, X0, Y0, w.b);
-                        if (J == 1) tma_store_5d(&tm_dq, at + kQ + patch * kPatchContent, 0, head, X0, Y0, w.b);
-                    }
-                    bulk_commit_group();
-                    if (J == 1) {
-                        bulk_wait_group_read<0>();
-                        mbar_arrive(bar(kEmpty + st));
-                    }
-                }
-                __syncwarp();
+                if (!ok) break;
             }
         }
         if (ok) {
@@ -678,14 +742,21 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                 if (R == 16) tmem_ld16(lanes + kColDQ<R> + I * (kD + R) + kD, reinterpret_cast<uint32_t(&)[16]>(a));
                 else tmem_ld32(lanes + kColDQ<R> + I * (kD + R) + kD, a);
                 tmem_wait_ld();
+                if (R == 16) {
+                    uint32_t k[16];
+                    tmem_ld16(lanes + kColRib<R> + R * I, k);
+                    tmem_wait_ld();
+                    float* const gk = p.dpk + table + (size_t)table_row(I * kTile + row) * p.r;
+#pragma unroll
+                    for (int c = 0; c < R; c += 4)
+                        if (c < p.r) add_columns(gk + c, k + c, p.inv_sqrt_d);
+                }
                 float* const gq = p.dpq + table + (size_t)table_row(I * kTile + row) * p.r;
 #pragma unroll
                 for (int c = 0; c < R; c += 4)
                     if (c < p.r) add_columns(gq + c, a + c, p.inv_sqrt_r);
             }
         }
-        if (warp == 20 && lane == 0) bulk_wait_group<0>();
-        __syncwarp();
     }
     tc_fence_before();
     __syncthreads();
@@ -747,8 +818,9 @@ cudaError_t launch_win16_bwd(const Problem& p, cudaStream_t stream)
         ProfileScope scope(RIB_KERNEL_WINDOW16_CLEAR, stream);
         if (cudaError_t e = launch_overtaking(bwd16::rib_window16_clear_kernel, blocks, 256, 0, stream, p.dpk, tables, per_table, p.pos_head_stride)) return e;
     }
+    const int dv_sectors = p.d % 16 == 0 && (reinterpret_cast<uintptr_t>(p.dv) & 31u) == 0;
     ProfileScope scope(RIB_KERNEL_WINDOW16_BWD, stream);
-    return launch_overtaking(bwd16::rib_window16_bwd_kernel<R>, grid, bwd16::kThreads, bwd16::kSmemBytes, stream, tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, p.dv, w);
+    return launch_overtaking(bwd16::rib_window16_bwd_kernel<R>, grid, bwd16::kThreads, bwd16::kSmemBytes, stream, tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, p.dv, dv_sectors, w);
 }
 
 }  // namespace
