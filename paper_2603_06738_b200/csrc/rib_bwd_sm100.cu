@@ -585,6 +585,7 @@ struct AuxParams {
     float* dpk;
     int H, W, heads, M, s, n, nWy, nWx, pairs;
     int d, r;                    // head width and rank of the caller's tensors (the accumulators are 32 + R columns wide)
+    int dq_sectors;              // 1: 16 channels of a row of dq are one 32-byte sector
     int narrow;                  // kNarrow: width of the rows of out and dq (even, less than d)
     int Hp, Wp;                  // sides of the extended map (equal to H, W when they are multiples of the window)
     int tables;                  // Pq/Pk tables: 1 (shared by the heads) or heads
@@ -606,8 +607,9 @@ __device__ __forceinline__ bool decode_pair_token(const AuxParams& p, int pair, 
     return Y < p.H && X < p.W;
 }
 
-// One thread per (pair, token in window order): D = dO . O and lse in the layout the main kernel
-// streams; the dQ~ accumulators are cleared with 16-byte stores, (d + r) / 4 per thread, as one flat array;
+// Four lanes per (pair, token in window order), 8 channels each (a row per lane touches 32 lines with every load: 16 x 96 x 96 tokens, rank 16,
+// 56 -> 48 us = 6.2 TB/s; 10 x 64 x 64 21 -> 17): D = dO . O and lse in the layout the main kernel
+// streams; the dQ~ accumulators are cleared with 16-byte stores, (d + r) / 16 per lane, as one flat array;
 // the first threads also stage bf16(Pq sqrt(d/r)) and clear dPq, dPk.
 // kNarrow: the rows of out are p.narrow < d elements wide and aligned to 4 bytes only.
 template <int R, bool kNarrow>
@@ -615,11 +617,12 @@ __global__ void __launch_bounds__(256) rib_bwd_prepare_kernel(const AuxParams p)
 {
     constexpr int kDk = kD + R;
     const size_t total = (size_t)p.pairs * p.n;
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t thread = (size_t)blockIdx.x * blockDim.x + threadIdx.x, t = thread >> 2;
+    const int part = (int)(thread & 3);
     const size_t nthreads = (size_t)gridDim.x * blockDim.x;
     // staged rows are R wide (zeros from column r on), the caller's tables r wide
     const size_t per_table = (size_t)p.n * R;
-    for (size_t e = t; e < per_table * p.tables; e += nthreads) {
+    for (size_t e = thread; e < per_table * p.tables; e += nthreads) {
         const size_t tbl = e / per_table, rem = e % per_table;
         const int row = (int)(rem / R), col = (int)(rem % R);
         if (col < p.r) {
@@ -631,64 +634,57 @@ __global__ void __launch_bounds__(256) rib_bwd_prepare_kernel(const AuxParams p)
             p.pq_scaled[e] = __float2bfloat16_rn(0.f);
         }
     }
-    if (t >= total) return;
-    float4* z4 = reinterpret_cast<float4*>(p.dq_acc);      // pairs * (d + r) * n floats = total * kDk / 4 vectors
-#pragma unroll
-    for (int k = 0; k < kDk / 4; ++k) z4[(size_t)k * total + t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t >= total) return;                                // (whole warps: total is a multiple of 128)
     const int pair = (int)(t / p.n), w = (int)(t % p.n);
     int i; size_t tok, scalar;
-    float* ldf = reinterpret_cast<float*>(p.ld) + ((t >> 1) << 2) + (t & 1);
-    if (!decode_pair_token(p, pair, w, i, tok, scalar)) {
-        // a position beyond the image: as a query it gets probability 0 (exp2(-inf)) and D = 0
-        ldf[0] = -INFINITY;
-        ldf[2] = 0.f;
-        return;
+    const bool real = decode_pair_token(p, pair, w, i, tok, scalar);
+    uint4 x = make_uint4(0u, 0u, 0u, 0u), y = x;
+    float lse = 0.f;
+    if (real && 8 * part < p.d) {
+        x = __ldg(reinterpret_cast<const uint4*>(p.dout + tok * p.d) + part);
+        if (kNarrow) {
+            const uint32_t* v = reinterpret_cast<const uint32_t*>(p.out + tok * p.narrow) + 4 * part;
+            const int left = p.narrow - 8 * part;
+            if (left > 0) y.x = __ldg(v);
+            if (left > 2) y.y = __ldg(v + 1);
+            if (left > 4) y.z = __ldg(v + 2);
+            if (left > 6) y.w = __ldg(v + 3);
+        } else {
+            y = __ldg(reinterpret_cast<const uint4*>(p.out + tok * p.d) + part);
+        }
+        if (part == 0) lse = p.lse[scalar];
     }
-    const uint4* a = reinterpret_cast<const uint4*>(p.dout + tok * p.d);
-    const uint4* b = reinterpret_cast<const uint4*>(p.out + tok * (kNarrow ? p.narrow : p.d));
+    float4* z4 = reinterpret_cast<float4*>(p.dq_acc);      // pairs * (d + r) * n floats = total * kDk / 4 vectors
+#pragma unroll
+    for (int k = 0; k < kDk / 16; ++k) z4[(size_t)k * 4 * total + thread] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
     float acc = 0.f;
 #pragma unroll
-    for (int q4 = 0; q4 < 4; ++q4) {
-        // (predicated, not a break: the loads of all four pieces are in flight together)
-        const bool on = 8 * q4 < p.d;
-        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-        const uint4 x = on ? __ldg(a + q4) : zero;
-        uint4 y = zero;
-        if (kNarrow) {
-            const uint32_t* w = reinterpret_cast<const uint32_t*>(b) + 4 * q4;
-            const int left = p.narrow - 8 * q4;
-            if (left > 0) y.x = __ldg(w);
-            if (left > 2) y.y = __ldg(w + 1);
-            if (left > 4) y.z = __ldg(w + 2);
-            if (left > 6) y.w = __ldg(w + 3);
-        } else if (on) {
-            y = __ldg(b + q4);
-        }
-        const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            acc = fmaf(__uint_as_float(xs[k] << 16), __uint_as_float(ys[k] << 16), acc);
-            acc = fmaf(__uint_as_float(xs[k] & 0xffff0000u), __uint_as_float(ys[k] & 0xffff0000u), acc);
-        }
+    for (int k = 0; k < 4; ++k) {
+        acc = fmaf(__uint_as_float(xs[k] << 16), __uint_as_float(ys[k] << 16), acc);
+        acc = fmaf(__uint_as_float(xs[k] & 0xffff0000u), __uint_as_float(ys[k] & 0xffff0000u), acc);
     }
-    // per query pair (w even, w + 1): (-lse2, -lse2', -D, -D'), the operand order of the packed arithmetic
-    ldf[0] = -p.lse[scalar] * 1.4426950408889634f;
-    ldf[2] = -acc;
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    if (part == 0) {
+        // a position beyond the image: as a query it gets probability 0 (exp2(-inf)) and D = 0
+        float* ldf = reinterpret_cast<float*>(p.ld) + ((t >> 1) << 2) + (t & 1);
+        ldf[0] = real ? -lse * 1.4426950408889634f : -INFINITY;
+        ldf[2] = real ? -acc : 0.f;
+    }
 }
 
-// Finishing pass over the fp32 accumulators.  grid (n / 32, groups of pairs, R / 16), 32 x 4 threads: a thread
-// owns one token position w of the window and a quarter of the columns -- 8 of the 32 content columns of dQ~
-// (one 16-byte piece of the bf16 dq row) and 4 of the 16 RIB columns of this grid.z slice -- and walks
-// the pairs of its group.  Few registers per thread keep the SM full of warps, which is what this
-// kernel (a stream of 16-byte reads, 512 bytes per warp) needs to reach the memory system (4-byte column reads: 60 against 56 us on
-// 16 x 96 x 96 tokens in windows of 32).  With one
+// Finishing pass over the fp32 accumulators.  grid (n / 32, groups of pairs), 32 x (2 + R / 8) threads: a thread owns one token position w
+// of the window and either 16 of the 32 content columns of dQ~ (one 32-byte sector of the bf16 dq row) or 8 RIB columns of dQ~ and
+// of dK~, four 16-byte reads per pair in both cases, and walks the pairs of its group.  Few registers per thread keep the SM full
+// of warps, which is what this kernel (a stream of 16-byte reads, 512 bytes per warp) needs to reach the memory system.  With one
 // table for all heads a group is a run of consecutive pairs; with head-wise tables it is a run of windows of
-// one head (pair = head + heads * window), so that its sums belong to one table.  Per pair the thread turns its
-// piece of dQ~[:, :d] / sqrt(d) into bf16, and it keeps running sums of its RIB columns of dQ~ (-> dPq, times
-// 1/sqrt(r)) and of dK~ (-> dPk); the group's sums go to the zeroed results with one vector atomic each (these
+// one head (pair = head + heads * window), so that its sums belong to one table.  Per pair a content thread turns its
+// piece of dQ~[:, :d] / sqrt(d) into bf16; a RIB thread keeps running sums of its columns of dQ~ (-> dPq, times
+// 1/sqrt(r)) and of dK~ (-> dPk), and sends the group's sums to the zeroed results with vector atomics (these
 // adds all land on the same n x r addresses: a group is long enough that their number does not set the time).
 template <int R, bool kNarrow>       // kNarrow: the rows of dq are p.narrow < d elements wide
-__global__ void __launch_bounds__(128, 8) rib_bwd_finish_kernel(const AuxParams p, int pairs_per_group)
+__global__ void __launch_bounds__(32 * (2 + R / 8)) rib_bwd_finish_kernel(const AuxParams p, int pairs_per_group)
 {
     constexpr int kDk = kD + R;
     const int tx = threadIdx.x & 31, cg = threadIdx.x >> 5;
@@ -705,42 +701,60 @@ __global__ void __launch_bounds__(128, 8) rib_bwd_finish_kernel(const AuxParams 
         pair1 = min(p.pairs, pair0 + pairs_per_group * step);
         table = (size_t)head * (size_t)p.pos_head_stride;
     }
-    // blockIdx.z picks 16 of the R RIB columns (grid.z = R / 16); the slice z = 0 also writes dq
-    const int col0 = 16 * blockIdx.z + 4 * cg;
-    float sq[4] = {0.f, 0.f, 0.f, 0.f}, sk[4] = {0.f, 0.f, 0.f, 0.f};
     int i = 0;
+    size_t tok, scalar;
+    if (cg < 2) {                                            // 16 content columns
+        const int channels = min(16, (kNarrow ? p.narrow : p.d) - 16 * cg);
+        if (channels <= 0) return;
 #pragma unroll 2
-    for (int pair = pair0; pair < pair1; pair += step) {
-        size_t tok, scalar;
-        const bool real = decode_pair_token(p, pair, w, i, tok, scalar);   // its sums are zero if not
-        const float4* src = reinterpret_cast<const float4*>(p.dq_acc + (size_t)pair * kDk * p.n) + w;
-        const float4* srk = reinterpret_cast<const float4*>(p.dkp + (size_t)pair * R * p.n) + w;
-        const bool piece = blockIdx.z == 0 && real && 8 * cg < p.d;      // this thread's 8 content columns exist in the caller's dq
-        float4 f0 = make_float4(0.f, 0.f, 0.f, 0.f), f1 = f0;
-        if (piece) { f0 = src[(size_t)(2 * cg) * p.n]; f1 = src[(size_t)(2 * cg + 1) * p.n]; }
-        const float4 gq = src[(size_t)((kD + col0) / 4) * p.n], gk = srk[(size_t)(col0 / 4) * p.n];
-        if (piece) {
-            const float f = p.inv_sqrt_d;
-            const uint4 v = make_uint4(pack_bf16x2(f0.x * f, f0.y * f), pack_bf16x2(f0.z * f, f0.w * f), pack_bf16x2(f1.x * f, f1.y * f), pack_bf16x2(f1.z * f, f1.w * f));
+        for (int pair = pair0; pair < pair1; pair += step) {
+            if (!decode_pair_token(p, pair, w, i, tok, scalar)) continue;
+            const float4* src = reinterpret_cast<const float4*>(p.dq_acc + (size_t)pair * kDk * p.n) + (size_t)(4 * cg) * p.n + w;
+            float4 f[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) f[q] = 4 * q < channels ? src[(size_t)q * p.n] : make_float4(0.f, 0.f, 0.f, 0.f);
+            uint32_t v[8];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                v[2 * q] = pack_bf16x2(f[q].x * p.inv_sqrt_d, f[q].y * p.inv_sqrt_d);
+                v[2 * q + 1] = pack_bf16x2(f[q].z * p.inv_sqrt_d, f[q].w * p.inv_sqrt_d);
+            }
             if (kNarrow) {
-                uint32_t* w = reinterpret_cast<uint32_t*>(p.dq + tok * p.narrow) + 4 * cg;
-                const int left = p.narrow - 8 * cg;
-                if (left > 0) w[0] = v.x;
-                if (left > 2) w[1] = v.y;
-                if (left > 4) w[2] = v.z;
-                if (left > 6) w[3] = v.w;
+                uint32_t* dst = reinterpret_cast<uint32_t*>(p.dq + tok * p.narrow) + 8 * cg;
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    if (2 * e < channels) dst[e] = v[e];
+            } else if (p.dq_sectors) {
+                st_global_v8(p.dq + tok * p.d + 16 * cg, v);
             } else {
-                reinterpret_cast<uint4*>(p.dq + tok * p.d)[cg] = v;
+                uint4* dst = reinterpret_cast<uint4*>(p.dq + tok * p.d) + 2 * cg;
+                dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
+                if (channels > 8) dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
             }
         }
-        sq[0] += gq.x; sq[1] += gq.y; sq[2] += gq.z; sq[3] += gq.w;
-        sk[0] += gk.x; sk[1] += gk.y; sk[2] += gk.z; sk[3] += gk.w;
+        return;
+    }
+    const int col0 = 8 * (cg - 2);                           // 8 of the R RIB columns
+    if (col0 >= p.r) return;                                 // columns of the padding (ranks are multiples of 8)
+    float4 sq[2], sk[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) sq[q] = sk[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto add = [](float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; };
+#pragma unroll 2
+    for (int pair = pair0; pair < pair1; pair += step) {     // (the sums of a position beyond the image are zero)
+        const float4* src = reinterpret_cast<const float4*>(p.dq_acc + (size_t)pair * kDk * p.n) + (size_t)((kD + col0) / 4) * p.n + w;
+        const float4* srk = reinterpret_cast<const float4*>(p.dkp + (size_t)pair * R * p.n) + (size_t)(col0 / 4) * p.n + w;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) { add(sq[q], src[(size_t)q * p.n]); add(sk[q], srk[(size_t)q * p.n]); }
     }
     // (the first pair of a group always exists: the grid is sized by the groups; i is the token's row of the tables)
-    if (col0 >= p.r) return;                             // columns of the padding (ranks are multiples of 8)
-    atomicAdd(reinterpret_cast<float4*>(p.dpq + table + (size_t)i * p.r + col0),
-              make_float4(sq[0] * p.inv_sqrt_r, sq[1] * p.inv_sqrt_r, sq[2] * p.inv_sqrt_r, sq[3] * p.inv_sqrt_r));
-    atomicAdd(reinterpret_cast<float4*>(p.dpk + table + (size_t)i * p.r + col0), make_float4(sk[0], sk[1], sk[2], sk[3]));
+    decode_pair_token(p, pair0, w, i, tok, scalar);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        atomicAdd(reinterpret_cast<float4*>(p.dpq + table + (size_t)i * p.r + col0 + 4 * q),
+                  make_float4(sq[q].x * p.inv_sqrt_r, sq[q].y * p.inv_sqrt_r, sq[q].z * p.inv_sqrt_r, sq[q].w * p.inv_sqrt_r));
+        atomicAdd(reinterpret_cast<float4*>(p.dpk + table + (size_t)i * p.r + col0 + 4 * q), sk[q]);
+    }
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -799,13 +813,14 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     ap.Hp = p.Hp; ap.Wp = p.Wp;
     ap.pairs = p.pairs;
     ap.d = p.d; ap.r = p.r; ap.narrow = p.narrow;
+    ap.dq_sectors = p.d % 16 == 0 && (reinterpret_cast<uintptr_t>(p.dq) & 31u) == 0;
     ap.tables = tables;
     ap.pos_head_stride = p.pos_head_stride;
     ap.pos_scale = sqrtf(scale_width_d(p) / scale_width_r(p));
     ap.inv_sqrt_d = 1.f / sqrtf(scale_width_d(p));
     ap.inv_sqrt_r = 1.f / sqrtf(scale_width_r(p));
     const size_t tokens = (size_t)p.pairs * p.n;
-    const unsigned aux_blocks = (unsigned)((tokens + 255) / 256);
+    const unsigned aux_blocks = (unsigned)((tokens + 63) / 64);
     { ProfileScope scope(RIB_KERNEL_BWD_PREPARE, stream); (p.narrow ? rib_bwd_prepare_kernel<R, true> : rib_bwd_prepare_kernel<R, false>)<<<aux_blocks, 256, 0, stream>>>(ap); }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -830,14 +845,14 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     const int windows = p.pairs / p.heads;   // pairs of one head
     const int in_line = tables == 1 ? p.pairs : windows;      // pairs whose sums go to one table
     // A block takes a run of pairs (of one head, with head-wise tables): four, or one where there are fewer than sixteen.  Measured, us with
-    // the launch, for runs of 1 / 2 / 4 / 8 / 16 pairs: 864 pairs of 1024 tokens at rank 16 84 / 62 / 58 / 60 / 71, 1728 pairs 168 / 115 / 101 / 109 /
-    // 128, 3456 pairs 265 / 210 / 189 / 203 / 242, 1728 pairs at rank 32 305 / 203 / 168 / 168 / 184; 12 pairs 6.6 / 8.4 / 8.6, 24 pairs 8.6 / 8.7 / 8.7, 48 pairs
-    // 12.7 / 10.4 / 10.6: more blocks in flight matter more to this kernel than fewer atomics.  Runs of eight where the grid's y has no room.
+    // the launch, for runs of 2 / 4 / 8 pairs: 864 pairs of 1024 tokens at rank 16 56 / 54 / 54, at rank 32 89 / 76 / 78, 1728 pairs at rank 32 117 / 101 /
+    // 99, 60 pairs of 4096 tokens at rank 16 21 / 20 / 19; with a quarter of a token's columns per thread, 16-byte stores of dq and a pass of its
+    // own for RIB columns 16 to 31 58, 88, 138 and 21 at runs of four.  Runs of eight where the grid's y has no room.
     auto groups_of = [&](int run) { return (tables == 1 ? 1ll : (long long)p.heads) * ((in_line + run - 1) / run); };
     const int per_group = in_line < 16 ? 1 : groups_of(4) <= 65535 ? 4 : 8;
     const unsigned groups = (unsigned)groups_of(per_group);
-    dim3 grid_fin((unsigned)(p.n / 32), groups, (unsigned)(R / 16));
-    { ProfileScope scope(RIB_KERNEL_BWD_FINISH, stream); (p.narrow ? rib_bwd_finish_kernel<R, true> : rib_bwd_finish_kernel<R, false>)<<<grid_fin, 128, 0, stream>>>(ap, per_group); }
+    dim3 grid_fin((unsigned)(p.n / 32), groups);
+    { ProfileScope scope(RIB_KERNEL_BWD_FINISH, stream); (p.narrow ? rib_bwd_finish_kernel<R, true> : rib_bwd_finish_kernel<R, false>)<<<grid_fin, 32 * (2 + R / 8), 0, stream>>>(ap, per_group); }
     return cudaGetLastError();
 }
 
