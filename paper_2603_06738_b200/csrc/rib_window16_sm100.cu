@@ -5,7 +5,7 @@
 // memory) exceeds its arithmetic.  Here a CTA keeps to one head (CTA c: head c mod heads), stages the head's RIB rows once,
 // takes whole windows one after the other and lets them overlap, and no gradient but those of the tables is summed
 // outside the chip.  What bounds it: the serial program of the softmax (arithmetic) warps.  A unit of the forward (128 rows x 256
-// keys) takes about 3900 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) 3000 at rank 16 and 32 channels:
+// keys) takes about 3600 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) 3000 at rank 16 and 32 channels:
 // 200 until its scores are there, 1500 of loads and exponentials, 1000 of stores of P and dS and fences, with 1470 cycles of MMAs
 // beside it.  Measured by event hooks against the general kernels (4 x 96 x 96 tokens, 12 heads of 16 channels, rank 24, shift 8,
 // masked): forward 60 against 82 us, backward 13 (two clearings) + 97 against 30 + 123 + 44 us; backward on 16 x 96 x 96 tokens, 6 heads of 32
@@ -60,8 +60,8 @@ constexpr uint32_t kWindowBytes = 2 * kContentBytes;                          //
 // All 16 softmax warps work on one unit after the other, a thread being (row, key patch): 64 scores in registers, the row's
 // maximum exchanged among its four threads through shared memory, P written over the own columns (so that 32 .. 95 and
 // 160 .. 223 of the unit hold P), then O = P [V | ones] (N = 48: 32 channels and the row sum of the rounded probabilities) in the
-// columns 96 .. 143, whose scores have been read.  The output of a unit is stored between the maximum and the exponentials of
-// the next: its PV has completed by then, and the scores of the unit after next are computed under those exponentials.
+// columns 96 .. 143, whose scores have been read.  The output of a unit is stored before or between the exponentials of
+// the next, and the scores of the unit after next are computed under (the rest of) those.
 // Output rows are stored from registers (a tensor map of the output would be a new one on every call with a new buffer).
 // Roles (640 threads): warp 0 TMA loads, warp 1 issues S, warp 2 PV (and owns the TMEM allocation), warp 3 idles, warps 4-19
 // softmax (4-7 key patch 0, 8-11 patch 1, ...).
@@ -81,7 +81,10 @@ constexpr uint32_t kIdescS = idesc_bf16_f32(kTile, 256, false), kIdescPV = idesc
 constexpr uint32_t kColO = 96;                    // of a unit's 256 columns
 constexpr uint32_t kPolyMask = 0x88u;             // of every 8 score pairs: which go to the FMA pipe
 
-template <int R>
+// kBetween: the output of the unit before is stored between the two halves of the exponentials, where its PV has completed (16 x 96 x 96
+// tokens, 6 heads, masked, rank 16 124 -> 115 us, 360 x 632 at rank 32 189 -> 175; behind both halves, where the next scores wait for it,
+// 126 and 192).  Not for heads of up to 16 channels, whose output half of the warps have no part in: 307 against 316 us.
+template <int R, bool kBetween>
 __global__ void __launch_bounds__(kThreads, 1)
 rib_window16_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                         __nv_bfloat16* const out, const __grid_constant__ SmallWindowParams p)
@@ -256,14 +259,15 @@ rib_window16_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             mine[kq * kTile + row] = fmaxf(mx0, mx1);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kMax + quarter));
-            if (u > 0) {
-                if (!mbar_wait_warp(bar(kOFull + (g ^ 1)), ((u - 1) >> 1) & 1, abort_flag, p.status)) break;
+            auto unit_before = [&] {
+                if (!mbar_wait_warp(bar(kOFull + (g ^ 1)), ((u - 1) >> 1) & 1, abort_flag, p.status)) return false;
                 tc_fence_after();
                 epilogue(before, g ^ 1, m_last);
-            }
+                return true;
+            };
+            if (!kBetween && u > 0 && !unit_before()) break;
             if (!mbar_wait_warp(bar(kMax + quarter), u & 1, abort_flag, p.status)) break;
             const float m = fmaxf(fmaxf(mine[row], mine[kTile + row]), fmaxf(mine[2 * kTile + row], mine[3 * kTile + row]));
-            m_last = m;
             const float neg = -m * p.scale_log2;
             const float2 neg2 = make_float2(neg, neg);
 #pragma unroll
@@ -281,7 +285,10 @@ rib_window16_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                     for (int i = 0; i < 16; ++i) pk[i] = 0u;
                 }
                 tmem_st16(lanes + g * 256 + p_col + 16 * ch, pk);
+                if (kBetween && ch == 0 && u > 0 && !(ok = unit_before())) break;
             }
+            if (!ok) break;
+            m_last = m;
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
@@ -777,7 +784,7 @@ __global__ void __launch_bounds__(256) rib_window16_clear_kernel(float* grads, i
 }
 }  // namespace bwd16
 
-template <int R>
+template <int R, bool kBetween>
 cudaError_t launch_win16_fwd(const Problem& p, cudaStream_t stream)
 {
     CUtensorMap tm_q, tm_k, tm_v;
@@ -785,12 +792,12 @@ cudaError_t launch_win16_fwd(const Problem& p, cudaStream_t stream)
     if (!encode_image_map(&tm_q, p.q, p) || !encode_image_map(&tm_k, p.k, p) || !encode_image_map(&tm_v, p.v, p)) return cudaErrorInvalidValue;
     static KernelSetup setup;       // one per instantiation of this launcher, i.e. per kernel
     int sm_count = 0;
-    if (cudaError_t e = setup.prepare(fwd16::rib_window16_fwd_kernel<R>, fwd16::kSmemBytes, &sm_count)) return e;
+    if (cudaError_t e = setup.prepare(fwd16::rib_window16_fwd_kernel<R, kBetween>, fwd16::kSmemBytes, &sm_count)) return e;
     SmallWindowParams w{};
     const int grid = fill_small_window(p, sm_count, p.nWy, p.nWx, &w);
     w.lse = p.lse_w;
     ProfileScope scope(RIB_KERNEL_WINDOW16_FWD, stream);
-    fwd16::rib_window16_fwd_kernel<R><<<grid, fwd16::kThreads, fwd16::kSmemBytes, stream>>>(tm_q, tm_k, tm_v, p.out_w, w);
+    fwd16::rib_window16_fwd_kernel<R, kBetween><<<grid, fwd16::kThreads, fwd16::kSmemBytes, stream>>>(tm_q, tm_k, tm_v, p.out_w, w);
     return cudaGetLastError();
 }
 
@@ -829,9 +836,9 @@ cudaError_t launch_win16_bwd(const Problem& p, cudaStream_t stream)
 bool sm100_window16(const Problem& p) { return p.M == 16 && p.s % 8 == 0 && p.H % 8 == 0 && p.W % 8 == 0 && !p.gate; }
 // Forward, this kernel against the general one, us with the launch (6 heads of 32 channels unless stated; 12 x 16: 12 heads of 16):
 //   whole windows          rank 16: 10 x 64 x 64 tokens 40 / 35, 256 x 256 60 / 50; rank 32: 41 / 40, 62 / 59; 12 x 16, rank 24: 65 / 63, 98 / 96;
-//   with a mask            rank 16: 10 x 64 x 64 40 / 47, 16 x 96 x 96 122 / 135, 256 x 256 60 / 59; rank 32: 41 / 58, 62 / 73; 12 x 16, rank 24: 63 / 106;
-//   beyond the map         rank 16: 48 x 40 10.4 / 12.3, 120 x 200 28.8 / 28.8, 200 x 328 64 / 59, 360 x 632 189 / 175; rank 32: 120 x 200 30 / 33,
-//                          360 x 632 193 / 217; 12 x 16, rank 24: 315 / 393.
+//   with a mask            rank 16: 16 x 96 x 96 115 / 135; rank 32: 10 x 64 x 64 44 / 64; 12 x 16, rank 24: 4 x 96 x 96 60 / 90;
+//   beyond the map         rank 16: 48 x 40 10.7 / 10.8, 104 x 120 18.7 / 18.8, 120 x 200 27.0 / 27.0, 200 x 328 57 / 54, 360 x 632 171 / 162;
+//                          rank 32: 120 x 200 27 / 31, 360 x 632 174 / 203; 12 x 16, rank 24: 307 / 372.
 // So whole windows stay with the general kernel, masks come here, and windows beyond the map come here with RIB rows of 32 elements or
 // while there is little work (120 x 200 tokens are four windows per SM).
 // This kernel has the fast form of the softmax only (one exponential in four on the FMA pipe, lse from rounded probabilities):
@@ -843,7 +850,8 @@ bool sm100_window16_prefers(const Problem& p)
 }
 cudaError_t sm100_window16_fwd(const Problem& p, cudaStream_t stream)
 {
-    return padded_rank(p.r) == 32 ? launch_win16_fwd<32>(p, stream) : launch_win16_fwd<16>(p, stream);
+    if (p.d > 16) return padded_rank(p.r) == 32 ? launch_win16_fwd<32, true>(p, stream) : launch_win16_fwd<16, true>(p, stream);
+    return padded_rank(p.r) == 32 ? launch_win16_fwd<32, false>(p, stream) : launch_win16_fwd<16, false>(p, stream);
 }
 cudaError_t sm100_window16_bwd(const Problem& p, cudaStream_t stream)
 {
