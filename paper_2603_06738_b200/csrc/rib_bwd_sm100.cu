@@ -34,7 +34,8 @@
 // instructions from several warps at once, and one thread issuing everything was the bottleneck):
 // warp 1 issues S^T and dP^T, warp 2 (also the TMEM allocator) dV and dK~, warp 3 dQ~; warps 4-11
 // P/dS arithmetic of the even half-tiles, warps 12-19 of the odd ones (a warp per 32 key rows and 32
-// queries, a thread 2 key rows x 4 queries of each of its four 16 x 16 pieces); warps 20-23 drain dQ~ after every tile and dK~/dV after every item.  Every wait is bounded.
+// queries, a thread 2 key rows x 4 queries of each of its four 16 x 16 pieces); warps 20-23 drain dQ~ after every tile, they or warps
+// 24-27 dK~/dV after every item.  Every wait is bounded.
 // What sets the pace is the loop  scores -> arithmetic -> dV and dK~ -> next scores of the buffer  (1600 cycles of issue, contraction and
 // barriers and 1350 of arithmetic), divided by the three units in flight: 2180 cycles per tile of 128 x 128 at rank 16, beside 1530 of
 // tensor pipe and, replays included, nine tenths of the shared-memory data pipe.  Measured on 16 x 96 x 96 tokens in windows of 32,
@@ -49,7 +50,11 @@ namespace {
 using namespace sm100;
 
 constexpr int kQStages = 4;           // ring of query-side tiles (Q content, Q RIB rows, dO, lse/D)
-constexpr int kThreads = 768;
+// Drains of dV and dK~ in warps of their own (24-27) beside those of dQ~: 466 -> 456 us on 16 x 96 x 96 tokens in windows of 32, 488 -> 474 on
+// 10 x 64 x 64 in windows of 64.  At rank 32 and with partial windows the 72 registers that are then left per thread cost more (548
+// against 555 us, masked windows of 32 123 against 136): there warps 20-23 do both.
+template <int R, bool kPartial> constexpr bool kSplitDrains = R == 16 && !kPartial;
+template <int R, bool kPartial> constexpr int kThreads = kSplitDrains<R, kPartial> ? 896 : 768;
 // RIB rank R = 16 or 32 is a template argument of the kernels: dQ~ / dK~ have kD + R columns
 
 // shared-memory map (offsets from a 1024-byte aligned base)
@@ -130,7 +135,7 @@ __device__ __forceinline__ ItemCoord decode_item(const BwdParams& p, int item)
 // answer), a query that is no token reads -inf for -lse (written by the preparation kernel), i.e. probability 0,
 // and nothing is stored for either.
 template <int R, bool kPartial>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads<R, kPartial>, 1)
 rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
                      const __grid_constant__ CUtensorMap tm_pqs, const __grid_constant__ CUtensorMap tm_pk,
@@ -473,93 +478,108 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         }
     } else if (warp >= 20) {
         // ================================ drains: dQ~ after every tile, dV / dK~ after every item
+        constexpr bool kSplit = kSplitDrains<R, kPartial>;
         const int quarter = warp & 3;
         const int row = quarter * 32 + lane;
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-        uint32_t g = 0, nitem = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x, ++nitem) {
-            for (int I = 0; I < p.nblk; ++I, ++g) {
-                if (I == p.nblk - 1) {
-                    // dV and dK~ of the item, before its last dQ~: dV and dK~ of the next one wait for the accumulators.  Rows of 64 bytes, one
-                    // per thread, would touch 32 lines with every store instruction and hold up the queue that all warps' loads and stores go
-                    // through for 2000 cycles an item; so they leave by TMA, a warp's 32 rows (half a patch) at a time (510 -> 488 us
-                    // on 16 x 96 x 96 tokens in windows of 32).  Each tile goes to shared memory before the next load: held back until the
-                    // accumulators are released, its rows spill.
-                    const ItemCoord c = decode_item(p, item);
-                    int py, px, Y0, X0;
-                    patch_origin(geom, p.div_per_row, c.wy, c.wx, 2 * c.J + (quarter >> 1), py, px, Y0, X0);
-                    const bool rows_real = !kPartial || (Y0 < p.H && X0 < p.W);   // no dk / dv rows for positions beyond the image
-                    if (!mbar_wait_warp(bar(kAccFull), nitem & 1, abort_flag, p.status)) { ok = false; break; }
-                    tc_fence_after();
-                    const int sw = (row >> 1) & 3;                    // SWIZZLE_64B
+        auto drain_item = [&](int item, uint32_t nitem) -> bool {
+            // Rows of 64 bytes, one per thread, would touch 32 lines with every store instruction and hold up the queue that all warps' loads and stores go
+            // through for 2000 cycles an item; so they leave by TMA, a warp's 32 rows (half a patch) at a time (510 -> 488 us
+            // on 16 x 96 x 96 tokens in windows of 32).  Each tile goes to shared memory before the next load: held back until the
+            // accumulators are released, its rows spill.
+            const ItemCoord c = decode_item(p, item);
+            int py, px, Y0, X0;
+            patch_origin(geom, p.div_per_row, c.wy, c.wx, 2 * c.J + (quarter >> 1), py, px, Y0, X0);
+            const bool rows_real = !kPartial || (Y0 < p.H && X0 < p.W);   // no dk / dv rows for positions beyond the image
+            if (!mbar_wait_warp(bar(kAccFull), nitem & 1, abort_flag, p.status)) return false;
+            tc_fence_after();
+            const int sw = (row >> 1) & 3;                    // SWIZZLE_64B
 #pragma unroll
-                    for (int which = 0; which < 2; ++which) {         // dV through V's slot, dK through a tile of its own
-                        uint8_t* const stage = base_ptr + (which == 0 ? kOffV + (nitem & 1) * kContentBytes : kOffDK) + row * 64;
-                        const float f = which == 0 ? 1.f : p.inv_sqrt_d;
-                        uint32_t a[32];
-                        tmem_ld32(tmem + lane_base + (which == 0 ? kColDV : kColDK), a);
-                        tmem_wait_ld();
+            for (int which = 0; which < 2; ++which) {         // dV through V's slot, dK through a tile of its own
+                uint8_t* const stage = base_ptr + (which == 0 ? kOffV + (nitem & 1) * kContentBytes : kOffDK) + row * 64;
+                const float f = which == 0 ? 1.f : p.inv_sqrt_d;
+                uint32_t a[32];
+                tmem_ld32(tmem + lane_base + (which == 0 ? kColDV : kColDK), a);
+                tmem_wait_ld();
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            uint32_t w[4];
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t w[4];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) w[e] = pack_bf16x2(__uint_as_float(a[8 * q + 2 * e]) * f, __uint_as_float(a[8 * q + 2 * e + 1]) * f);
-                            *reinterpret_cast<uint4*>(stage + ((q ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-                        }
-                    }
-                    uint32_t rib[R / 16][16];
-#pragma unroll
-                    for (int part = 0; part < R / 16; ++part) tmem_ld16(tmem + lane_base + kColDK + kD + 16 * part, rib[part]);
-                    tmem_wait_ld();
-                    tc_fence_before();
-                    fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(bar(kAccFree));
-                        if (rows_real) {
-                            tma_store_5d(&tm_dv, base + kOffV + (nitem & 1) * kContentBytes + quarter * (kPatchContent / 2), 0, c.h, X0, Y0 + 4 * (quarter & 1), c.b);
-                            tma_store_5d(&tm_dk, base + kOffDK + quarter * (kPatchContent / 2), 0, c.h, X0, Y0 + 4 * (quarter & 1), c.b);
-                            bulk_commit_group();
-                        }
-                    }
-                    float* dst_p = p.dkp + (size_t)c.pair * R * p.n + 4 * ((size_t)c.J * kTile + row);
-#pragma unroll
-                    for (int col = 0; col < R; col += 4) {
-                        const uint32_t* v = rib[col >> 4] + (col & 15);
-                        *reinterpret_cast<float4*>(dst_p + (size_t)col * p.n) = make_float4(__uint_as_float(v[0]) * p.inv_sqrt_d, __uint_as_float(v[1]) * p.inv_sqrt_d,
-                                                                                            __uint_as_float(v[2]) * p.inv_sqrt_d, __uint_as_float(v[3]) * p.inv_sqrt_d);
-                    }
-                }
-                if (!mbar_wait_warp(bar(kDQFull), g & 1, abort_flag, p.status)) { ok = false; break; }
-                tc_fence_after();
-                float* dst = p.dq_acc + (size_t)p.div_nblk.div(item) * kDk * p.n + 4 * ((size_t)I * kTile + row);
-#pragma unroll
-                for (int part = 0; part < kDk / 16; ++part) {
-                    uint32_t a[16];
-                    tmem_ld16(tmem + lane_base + kColDQ + 16 * part, a);
-                    tmem_wait_ld();
-                    if (part + 1 == kDk / 16) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(bar(kDQFree));
-                    }
-#pragma unroll
-                    for (int col = 0; col < 16; col += 4) {
-                        red_add_f32x4(dst, a + col);
-                        dst += 4 * (size_t)p.n;
-                        if (R == 16 || (col & 4)) __nanosleep(20);
-                    }
+                    for (int e = 0; e < 4; ++e) w[e] = pack_bf16x2(__uint_as_float(a[8 * q + 2 * e]) * f, __uint_as_float(a[8 * q + 2 * e + 1]) * f);
+                    *reinterpret_cast<uint4*>(stage + ((q ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
                 }
             }
-            if (!ok) break;
+            uint32_t rib[R / 16][16];
+#pragma unroll
+            for (int part = 0; part < R / 16; ++part) tmem_ld16(tmem + lane_base + kColDK + kD + 16 * part, rib[part]);
+            tmem_wait_ld();
+            tc_fence_before();
+            fence_proxy_async();
+            __syncwarp();
             if (lane == 0) {
-                bulk_wait_group_read<0>();          // (this thread's own stores)
+                mbar_arrive(bar(kAccFree));
+                if (rows_real) {
+                    tma_store_5d(&tm_dv, base + kOffV + (nitem & 1) * kContentBytes + quarter * (kPatchContent / 2), 0, c.h, X0, Y0 + 4 * (quarter & 1), c.b);
+                    tma_store_5d(&tm_dk, base + kOffDK + quarter * (kPatchContent / 2), 0, c.h, X0, Y0 + 4 * (quarter & 1), c.b);
+                    bulk_commit_group();
+                }
+            }
+            float* dst_p = p.dkp + (size_t)c.pair * R * p.n + 4 * ((size_t)c.J * kTile + row);
+#pragma unroll
+            for (int col = 0; col < R; col += 4) {
+                const uint32_t* v = rib[col >> 4] + (col & 15);
+                *reinterpret_cast<float4*>(dst_p + (size_t)col * p.n) = make_float4(__uint_as_float(v[0]) * p.inv_sqrt_d, __uint_as_float(v[1]) * p.inv_sqrt_d,
+                                                                                    __uint_as_float(v[2]) * p.inv_sqrt_d, __uint_as_float(v[3]) * p.inv_sqrt_d);
+            }
+            return true;
+        };
+        auto release_slot = [&](uint32_t nitem) {         // V's slot, when its dV rows have been read
+            if (lane == 0) {
+                bulk_wait_group_read<0>();                // (this thread's own stores)
                 mbar_arrive(bar(kKVEmpty + (nitem & 1)));
             }
             __syncwarp();
+        };
+        auto drain_tile = [&](int item, int I, uint32_t g) -> bool {
+            if (!mbar_wait_warp(bar(kDQFull), g & 1, abort_flag, p.status)) return false;
+            tc_fence_after();
+            float* dst = p.dq_acc + (size_t)p.div_nblk.div(item) * kDk * p.n + 4 * ((size_t)I * kTile + row);
+#pragma unroll
+            for (int part = 0; part < kDk / 16; ++part) {
+                uint32_t a[16];
+                tmem_ld16(tmem + lane_base + kColDQ + 16 * part, a);
+                tmem_wait_ld();
+                if (part + 1 == kDk / 16) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kDQFree));
+                }
+#pragma unroll
+                for (int col = 0; col < 16; col += 4) {
+                    red_add_f32x4(dst, a + col);
+                    dst += 4 * (size_t)p.n;
+                    if (R == 16 || (col & 4)) __nanosleep(20);
+                }
+            }
+            return true;
+        };
+        uint32_t g = 0, nitem = 0;
+        bool ok = true;
+        for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x, ++nitem) {
+            if (kSplit && warp >= 24) {
+                ok = drain_item(item, nitem);
+                if (ok) release_slot(nitem);
+                continue;
+            }
+            for (int I = 0; I < p.nblk && ok; ++I, ++g) {
+                // (dV and dK~ before the item's last dQ~: dV and dK~ of the next item wait for the accumulators)
+                if (!kSplit && I == p.nblk - 1) ok = drain_item(item, nitem);
+                ok = ok && drain_tile(item, I, g);
+            }
+            if (!kSplit && ok) release_slot(nitem);
         }
         if (lane == 0) bulk_wait_group<0>();
+        __syncwarp();
     }
     // ================================================================================ common tail
     tc_fence_before();
@@ -838,7 +858,7 @@ cudaError_t launch_bwd(const Problem& p, cudaStream_t stream)
     bp.div_nblk = make_fast_div(bp.nblk); bp.div_heads = make_fast_div(p.heads); bp.div_nwx = make_fast_div(p.nWx); bp.div_nwy = make_fast_div(p.nWy);
     bp.div_per_row = make_fast_div(p.M >> 3);
     const int grid = bp.items < sm_count ? bp.items : sm_count;
-    { ProfileScope scope(RIB_KERNEL_BWD_MAIN, stream); rib_bwd_sm100_kernel<R, kPartial><<<grid, kThreads, kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_do, tm_pqs, tm_pk, tm_dk, tm_dv, bp); }
+    { ProfileScope scope(RIB_KERNEL_BWD_MAIN, stream); rib_bwd_sm100_kernel<R, kPartial><<<grid, kThreads<R, kPartial>, kSmemBytes, stream>>>(tm_q, tm_k, tm_v, tm_do, tm_pqs, tm_pk, tm_dk, tm_dv, bp); }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
 

@@ -1,6 +1,7 @@
 """The waits of the general backward kernel (csrc/rib_bwd_sm100.cu) in a model of its warps with random delays (tests/test_frame_barriers.py:
 a wait answers by parity, so its phase must be the one that is complete).  Rank 16: P^T and dS^T lie over the scores of one of three
-buffers.  Rank 32: dP^T has two buffers of its own, dK~ reads dS from shared memory.  No GPU needed."""
+buffers.  Rank 32: dP^T has two buffers of its own, dK~ reads dS from shared memory.  dV and dK~ are drained by the warps that drain dQ~
+or by others (`apart`).  No GPU needed."""
 import heapq
 
 import pytest
@@ -11,9 +12,9 @@ from test_frame_barriers import Model
 class Backward(Model):
     """`items` key blocks of `tiles` query tiles each; unit u = 2 * tile + half, its scores in buffer u mod 3."""
 
-    def __init__(self, items, tiles, seed, rank):
+    def __init__(self, items, tiles, seed, rank, apart):
         super().__init__([tiles] * items, seed, True)
-        self.items_, self.tiles, self.rank, self.total = items, tiles, rank, items * tiles
+        self.tiles, self.rank, self.apart, self.total = tiles, rank, apart, items * tiles
         for name in ("dq", "drain", "v"):
             self.scale[name] = self.rng.choice((0.1, 1.0, 5.0))
 
@@ -71,15 +72,22 @@ class Backward(Model):
             self.finished.add(("p", u))
             self.arrive(self.on("pready", u)[0])
 
+    def drain_item(self, item):
+        yield "wait", "accfull", item
+        u = 2 * self.tiles * (item + 1)
+        assert ("dk", u - 1) in self.finished and ("dv", u) not in self.issued
+        yield "delay", self.delay("drain")
+        self.finished.add(("acc", item))
+        self.arrive("accfree")
+
+    def drain_items(self):
+        for item in range(self.total // self.tiles):
+            yield from self.drain_item(item)
+
     def drain(self):
         for g in range(self.total):
-            if (g + 1) % self.tiles == 0:
-                item = g // self.tiles
-                yield "wait", "accfull", item
-                assert ("dk", 2 * g + 1) in self.finished and ("dv", 2 * g + 2) not in self.issued
-                yield "delay", self.delay("drain")
-                self.finished.add(("acc", item))
-                self.arrive("accfree")
+            if (g + 1) % self.tiles == 0 and not self.apart:
+                yield from self.drain_item(g // self.tiles)
             yield "wait", "dqfull", g
             assert ("dq", g) in self.finished and ("dq", g + 1) not in self.issued
             yield "delay", self.delay("drain")
@@ -91,7 +99,8 @@ class Backward(Model):
 
     def run(self):
         self.pipe = {}
-        for process in [self.scores(), self.gradients(), self.query_gradients(), self.arithmetic(0), self.arithmetic(1), self.drain()]:
+        processes = [self.scores(), self.gradients(), self.query_gradients(), self.arithmetic(0), self.arithmetic(1), self.drain()]
+        for process in processes + ([self.drain_items()] if self.apart else []):
             self.later(self.delay("soft"), lambda process=process: self.step(process))
         while self.queue:
             self.now, _, what = heapq.heappop(self.queue)
@@ -99,8 +108,8 @@ class Backward(Model):
         assert sum(f[0] == "drained" for f in self.finished) == self.total, "the warps wait for one another"
 
 
-@pytest.mark.parametrize("rank", [16, 32])
+@pytest.mark.parametrize("rank,apart", [(16, True), (16, False), (32, False)])
 @pytest.mark.parametrize("items,tiles", [(1, 8), (3, 8), (5, 1), (2, 18)])
-def test_every_wait_sees_its_own_phase(items, tiles, rank):
+def test_every_wait_sees_its_own_phase(items, tiles, rank, apart):
     for seed in range(200):
-        Backward(items, tiles, seed, rank).run()
+        Backward(items, tiles, seed, rank, apart).run()
