@@ -246,115 +246,117 @@ __global__ void __launch_bounds__(kPwThreads, 1) rib_cla_bwd_pw_kernel(const Cla
 }
 
 // ------------------------------------------------------------------------------------------------------------------
-// Depth-wise part.  A block takes a tile of 8 x 16 pixels and 32 channels: the 10 x 18 halo of dY (fp32) and of X (bf16)
-// goes to shared memory (zero outside the map), thread (channel, lane) walks 16 pixels of the tile.
+// Depth-wise part.  A block takes a tile of 16 x 16 pixels and 32 channels: the 18 x 18 halo of dY (fp32) and of X (bf16) goes to
+// shared memory by cp.async (zero outside the map), thread (channel pair, tile row) walks the 16 pixels of its row with packed
+// fp32 FMAs.  8 x 96 x 96 pixels of 192 channels 45.4 -> 38.2 us by event hooks (one channel per thread, tiles of 8 x 16 and halos through
+// registers were bound by their own instructions, 62 % of the issue slots), 4 x 96 x 96 24.9 -> 18.8.  Copies alone take 25 us, arithmetic
+// alone 25: two blocks overlap the one with the other only in part.  Three blocks per SM (80 registers, spills) 39.2; strips of 8 rows
+// with the next rows copied under the arithmetic, 12 warps per SM, 39.3.
 // ------------------------------------------------------------------------------------------------------------------
-constexpr int kDwTileH = 8, kDwTileW = 16, kDwHaloH = kDwTileH + 2, kDwHaloW = kDwTileW + 2, kDwHalo = kDwHaloH * kDwHaloW;
-constexpr int kDwCh = 32, kDwLanes = 8;
-constexpr int kDwSmemBytes = kDwHalo * kDwCh * 6 + kDwLanes * 10 * kDwCh * 4;
+constexpr int kDwTile = 16, kDwHaloW = kDwTile + 2, kDwHalo = kDwHaloW * kDwHaloW;
+constexpr int kDwCh = 32, kDwPairs = kDwCh / 2, kDwThreads = kDwPairs * kDwTile, kDwBlocks = 2;      // blocks per SM
+constexpr int kDwXPitch = kDwHaloW * kDwCh + kDwCh;       // bf16s per halo row of X: a warp's two rows lie 64 bytes apart in the banks
+constexpr int kDwXBytes = kDwHaloW * kDwXPitch * 2, kDwDyBytes = kDwHalo * kDwCh * 4;
+constexpr int kDwSmemBytes = kDwDyBytes + kDwXBytes;
+static_assert(kDwTile * 10 * kDwCh * 4 <= kDwDyBytes, "the sums are gathered over the halo of dY");
+
+// 16 bytes of global memory into shared memory, or zeros
+__device__ __forceinline__ void copy16_or_zero(uint32_t dst, const void* src, bool there)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(there ? 16 : 0) : "memory");
+}
 
 template <int D>
-__global__ void __launch_bounds__(kDwCh * kDwLanes) rib_cla_bwd_dw_kernel(const ClaBwdParams p, int tiles_y, int tiles_x)
+__global__ void __launch_bounds__(kDwThreads, kDwBlocks) rib_cla_bwd_dw_kernel(const ClaBwdParams p, int tiles_y, int tiles_x)
 {
     extern __shared__ __align__(16) uint8_t dw_smem[];
-    float* dys = reinterpret_cast<float*>(dw_smem);                                        // [180][channels]
-    __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(dw_smem + kDwHalo * kDwCh * 4);   // [180][channels]
-    float* red = reinterpret_cast<float*>(dw_smem + kDwHalo * kDwCh * 6);                  // [8 lanes][10][channels]
-    const int c = threadIdx.x, lane = threadIdx.y, tid = lane * kDwCh + c;
+    float* dys = reinterpret_cast<float*>(dw_smem);                                        // [18][18][channels]
+    __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(dw_smem + kDwDyBytes);            // [18][18 + 1][channels]
+    const uint32_t dys_at = sm100::smem_u32(dys), xs_at = sm100::smem_u32(xs);
+    const int tid = threadIdx.x, c = 2 * (tid % kDwPairs), py = tid / kDwPairs;
     constexpr int kGroups = D / kDwCh;
     // a block keeps one channel group and walks spatial tiles, so its ten sums per channel reach global memory once
     const int cg = blockIdx.x % kGroups, ch0 = cg * kDwCh;
     const int spatial = p.B * tiles_y * tiles_x, step = gridDim.x / kGroups;      // the grid is a multiple of kGroups
-    float w[9];
+    float2 w[9], gw[9], gb = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int t = 0; t < 9; ++t) w[t] = p.w_dw[(ch0 + c) * 9 + t];
-    float gw[9], gb = 0.f;
-#pragma unroll
-    for (int t = 0; t < 9; ++t) gw[t] = 0.f;
+    for (int t = 0; t < 9; ++t) {
+        w[t] = make_float2(p.w_dw[(ch0 + c) * 9 + t], p.w_dw[(ch0 + c + 1) * 9 + t]);
+        gw[t] = make_float2(0.f, 0.f);
+    }
     for (int st = blockIdx.x / kGroups; st < spatial; st += step) {
-    const int tx = st % tiles_x, ty = (st / tiles_x) % tiles_y, b = st / (tiles_x * tiles_y);
-    const int y0 = ty * kDwTileH, x0 = tx * kDwTileW;
-    // halo: a thread moves 4 channels of a pixel; all loads of a thread are issued before the
-    // first store, so the prologue costs one memory latency
-    {
-        constexpr int kPer = kDwCh / 4, kItems = kDwHalo * kPer, kIters = (kItems + kDwCh * kDwLanes - 1) / (kDwCh * kDwLanes);
-        float4 dv[kIters];
-        uint2 xv[kIters];
-#pragma unroll
-        for (int u = 0; u < kIters; ++u) {
-            const int idx = tid + u * kDwCh * kDwLanes;
-            const int hp = idx / kPer, c4 = (idx % kPer) * 4;
-            const int yy = y0 + hp / kDwHaloW - 1, xx = x0 + hp % kDwHaloW - 1;
-            dv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            xv[u] = make_uint2(0, 0);
-            if (idx < kItems && yy >= 0 && yy < p.H && xx >= 0 && xx < p.W) {
-                const size_t g = (((size_t)b * p.H + yy) * p.W + xx) * D + ch0 + c4;
-                dv[u] = __ldg(reinterpret_cast<const float4*>(p.dy + g));
-                xv[u] = __ldg(reinterpret_cast<const uint2*>(p.x + g));
-            }
+        const int tx = st % tiles_x, ty = (st / tiles_x) % tiles_y, b = st / (tiles_x * tiles_y);
+        const int y0 = ty * kDwTile, x0 = tx * kDwTile;
+        // halo: a thread keeps its 16-byte piece of a pixel (8 of dY, then 4 of X) and walks the pixels
+        const size_t image = (size_t)b * p.H * p.W;
+        for (int hp = tid / 8; hp < kDwHalo; hp += kDwThreads / 8) {
+            const int hy = hp / kDwHaloW, hx = hp - hy * kDwHaloW, yy = y0 + hy - 1, xx = x0 + hx - 1;
+            const bool there = yy >= 0 && yy < p.H && xx >= 0 && xx < p.W;
+            const size_t g = there ? (image + (size_t)yy * p.W + xx) * D + ch0 : 0;
+            copy16_or_zero(dys_at + (hp * kDwCh + 4 * (tid % 8)) * 4, p.dy + g + 4 * (tid % 8), there);
         }
-#pragma unroll
-        for (int u = 0; u < kIters; ++u) {
-            const int idx = tid + u * kDwCh * kDwLanes;
-            if (idx < kItems) {
-                const int hp = idx / kPer, c4 = (idx % kPer) * 4;
-                *reinterpret_cast<float4*>(dys + hp * kDwCh + c4) = dv[u];
-                *reinterpret_cast<uint2*>(xs + hp * kDwCh + c4) = xv[u];
-            }
+        for (int hp = tid / 4; hp < kDwHalo; hp += kDwThreads / 4) {
+            const int hy = hp / kDwHaloW, hx = hp - hy * kDwHaloW, yy = y0 + hy - 1, xx = x0 + hx - 1;
+            const bool there = yy >= 0 && yy < p.H && xx >= 0 && xx < p.W;
+            const size_t g = there ? (image + (size_t)yy * p.W + xx) * D + ch0 : 0;
+            copy16_or_zero(xs_at + (hy * kDwXPitch + hx * kDwCh + 8 * (tid % 4)) * 2, p.x + g + 8 * (tid % 4), there);
         }
-    }
-    __syncthreads();
-    // lane l takes tile row l: 16 pixels, walked left to right with the 3 x 3 windows of dY and X in registers, so each
-    // pixel costs one new halo column (6 shared-memory reads) instead of 18.  Pixels to the right of the map need no
-    // test for the sums: dY is zero there.
-    const int py = lane;
-    if (y0 + py < p.H) {
-        float dwin[3][3], xwin[3][3];                    // [halo row py + i][halo column px + j]
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        // a row of 16 pixels, left to right, with the 3 x 3 windows of dY and X in registers: a pixel costs one new halo column.
+        // Pixels to the right of the map need no test for the sums: dY is zero there.
+        if (y0 + py < p.H) {
+            float2 dwin[3][3], xwin[3][3];                    // [halo row py + i][halo column px + j]
+            const float* dcol = dys + py * kDwHaloW * kDwCh + c;
+            const __nv_bfloat16* xcol = xs + py * kDwXPitch + c;
+            auto column = [&](int j, int hx) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 1; j < 3; ++j) {
-                dwin[i][j] = dys[((py + i) * kDwHaloW + j - 1) * kDwCh + c];
-                xwin[i][j] = __bfloat162float(xs[((py + i) * kDwHaloW + j - 1) * kDwCh + c]);
-            }
-        __nv_bfloat16* dst = p.dx + (((size_t)b * p.H + y0 + py) * p.W + x0) * D + ch0 + c;
-#pragma unroll
-        for (int px = 0; px < kDwTileW; ++px) {
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                dwin[i][0] = dwin[i][1]; dwin[i][1] = dwin[i][2];
-                xwin[i][0] = xwin[i][1]; xwin[i][1] = xwin[i][2];
-                dwin[i][2] = dys[((py + i) * kDwHaloW + px + 2) * kDwCh + c];
-                xwin[i][2] = __bfloat162float(xs[((py + i) * kDwHaloW + px + 2) * kDwCh + c]);
-            }
-            const float dy_here = dwin[1][1];
-            gb += dy_here;
-            float dx = 0.f;
-#pragma unroll
-            for (int ky = 0; ky < 3; ++ky) {
-#pragma unroll
-                for (int kx = 0; kx < 3; ++kx) {
-                    // forward: Y[y, x] reads X[y + ky - 1, x + kx - 1] through tap (ky, kx); X is zero outside the map
-                    gw[ky * 3 + kx] = fmaf(dy_here, xwin[ky][kx], gw[ky * 3 + kx]);
-                    // so X[y, x] was read by the output pixel (y - ky + 1, x - kx + 1); dY is zero outside the map
-                    dx = fmaf(dwin[2 - ky][2 - kx], w[ky * 3 + kx], dx);
+                for (int i = 0; i < 3; ++i) {
+                    dwin[i][j] = *reinterpret_cast<const float2*>(dcol + (i * kDwHaloW + hx) * kDwCh);
+                    const uint32_t two = *reinterpret_cast<const uint32_t*>(xcol + i * kDwXPitch + hx * kDwCh);
+                    xwin[i][j] = make_float2(__uint_as_float(two << 16), __uint_as_float(two & 0xffff0000u));
                 }
-            }
-            if (x0 + px < p.W) dst[(size_t)px * D] = __float2bfloat16_rn(dx);
-        }
-    }
-    __syncthreads();                                     // the next tile overwrites the halos
-    }
+            };
+            column(1, 0);
+            column(2, 1);
+            uint32_t* dst = reinterpret_cast<uint32_t*>(p.dx + (image + (size_t)(y0 + py) * p.W + x0) * D + ch0 + c);
 #pragma unroll
-    for (int t = 0; t < 9; ++t) red[(lane * 10 + t) * kDwCh + c] = gw[t];
-    red[(lane * 10 + 9) * kDwCh + c] = gb;
+            for (int px = 0; px < kDwTile; ++px) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    dwin[i][0] = dwin[i][1]; dwin[i][1] = dwin[i][2];
+                    xwin[i][0] = xwin[i][1]; xwin[i][1] = xwin[i][2];
+                }
+                column(2, px + 2);
+                const float2 dy_here = dwin[1][1];
+                gb = __fadd2_rn(gb, dy_here);
+                float2 dx = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky) {
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx) {
+                        // forward: Y[y, x] reads X[y + ky - 1, x + kx - 1] through tap (ky, kx); X is zero outside the map
+                        gw[ky * 3 + kx] = __ffma2_rn(dy_here, xwin[ky][kx], gw[ky * 3 + kx]);
+                        // so X[y, x] was read by the output pixel (y - ky + 1, x - kx + 1); dY is zero outside the map
+                        dx = __ffma2_rn(dwin[2 - ky][2 - kx], w[ky * 3 + kx], dx);
+                    }
+                }
+                if (x0 + px < p.W) dst[(size_t)px * (D / 2)] = sm100::pack_bf16x2(dx.x, dx.y);
+            }
+        }
+        __syncthreads();                                     // the next tile overwrites the halos
+    }
+    float* red = dys;                                        // [16 rows][10][channels]
+#pragma unroll
+    for (int t = 0; t < 9; ++t) *reinterpret_cast<float2*>(red + (py * 10 + t) * kDwCh + c) = gw[t];
+    *reinterpret_cast<float2*>(red + (py * 10 + 9) * kDwCh + c) = gb;
     __syncthreads();
-    // 10 sums of 8 lanes per channel
-    for (int idx = tid; idx < 10 * kDwCh; idx += kDwCh * kDwLanes) {
+    // 10 sums of 16 rows per channel
+    for (int idx = tid; idx < 10 * kDwCh; idx += kDwThreads) {
         const int t = idx / kDwCh, cc = idx - t * kDwCh;
         float sum = 0.f;
 #pragma unroll
-        for (int l = 0; l < kDwLanes; ++l) sum += red[(l * 10 + t) * kDwCh + cc];
+        for (int l = 0; l < kDwTile; ++l) sum += red[(l * 10 + t) * kDwCh + cc];
         if (t < 9) atomicAdd(p.dw_dw + (ch0 + cc) * 9 + t, sum);
         else atomicAdd(p.db_dw + ch0 + cc, sum);
     }
@@ -757,12 +759,12 @@ cudaError_t launch_gate_bwd(const ClaBwdParams& p, bool tensor_cores, cudaStream
     }
     {
         ProfileScope scope(RIB_KERNEL_CLA_BWD_DW, stream);
-        const int tiles_y = (p.H + kDwTileH - 1) / kDwTileH, tiles_x = (p.W + kDwTileW - 1) / kDwTileW;
+        const int tiles_y = (p.H + kDwTile - 1) / kDwTile, tiles_x = (p.W + kDwTile - 1) / kDwTile;
         const long long spatial = (long long)p.B * tiles_y * tiles_x;
         if (spatial > 0x7fffffffLL) return cudaErrorInvalidValue;
         constexpr int kGroups = D / kDwCh;
-        const long long per_group = spatial < (long long)sms * 4 / kGroups ? spatial : (long long)sms * 4 / kGroups;   // four blocks fit on an SM
-        rib_cla_bwd_dw_kernel<D><<<(unsigned)(per_group * kGroups), dim3(kDwCh, kDwLanes), kDwSmemBytes, stream>>>(p, tiles_y, tiles_x);
+        const long long per_group = spatial < (long long)sms * kDwBlocks / kGroups ? spatial : (long long)sms * kDwBlocks / kGroups;
+        rib_cla_bwd_dw_kernel<D><<<(unsigned)(per_group * kGroups), kDwThreads, kDwSmemBytes, stream>>>(p, tiles_y, tiles_x);
     }
     return cudaGetLastError();
 }
