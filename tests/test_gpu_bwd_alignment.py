@@ -29,7 +29,7 @@ def test_gradients_that_are_aligned_to_16_bytes_only(wl):
     memory = [torch.full((size + 64,), 3.0, dtype=torch.bfloat16, device="cuda") for _ in range(3)]
     grads = [m[8:8 + size].view(q.shape) for m in memory]
     assert all(g.data_ptr() % 32 == 16 for g in grads)
-    dpq, dpk = torch.empty_like(pq), torch.empty_like(pk)
+    dpq, dpk = (torch.empty(pq.shape, dtype=torch.float32, device="cuda") for _ in range(2))
     need = binding.rib_window_attn_bwd_workspace(wl.B, wl.H, wl.W, wl.heads, wl.d, wl.r, wl.window)
     workspace = torch.empty(max(need, 256), dtype=torch.uint8, device="cuda")
     pointers = [t.data_ptr() for t in (q, k, v, pq, pk, out, lse, dout)]
