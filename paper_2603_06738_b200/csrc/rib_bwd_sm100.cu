@@ -726,6 +726,42 @@ __global__ void __launch_bounds__(32 * (2 + R / 8)) rib_bwd_finish_kernel(const 
     if (cg < 2) {                                            // 16 content columns
         const int channels = min(16, (kNarrow ? p.narrow : p.d) - 16 * cg);
         if (channels <= 0) return;
+        if (kNarrow) {
+            // A warp's 32 positions are 4 x 8 tokens, all in the map or none.  Its words change lanes through shared memory, so that a store
+            // covers 4 rows in runs of up to 32 bytes: one row per lane, every store touched 32 lines
+            // (8 x 96 x 96 tokens, 30 channels, rank 18 55.8 -> 43.5 us; one warp for both halves of the columns, two rows to a store: 88).
+            __shared__ uint32_t staged[2][32 * 9];
+            uint32_t* const mine = staged[cg];
+            const int words = p.narrow / 2, word = tx & 7;
+            auto load = [&](int pair, float4 (&to)[4]) {
+                const float4* src = reinterpret_cast<const float4*>(p.dq_acc + (size_t)pair * kDk * p.n) + (size_t)(4 * cg) * p.n + w;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) to[q] = 4 * q < channels ? src[(size_t)q * p.n] : make_float4(0.f, 0.f, 0.f, 0.f);
+            };
+            float4 f[4], ahead[4];
+            load(pair0, f);
+            for (int pair = pair0; pair < pair1; pair += step) {
+                if (pair + step < pair1) load(pair + step, ahead);
+                if (decode_pair_token(p, pair, w, i, tok, scalar)) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        mine[tx * 9 + 2 * q] = pack_bf16x2(f[q].x * p.inv_sqrt_d, f[q].y * p.inv_sqrt_d);
+                        mine[tx * 9 + 2 * q + 1] = pack_bf16x2(f[q].z * p.inv_sqrt_d, f[q].w * p.inv_sqrt_d);
+                    }
+                    __syncwarp();
+                    const size_t first = tok - (size_t)((tx >> 3) * p.W + (tx & 7)) * p.heads;
+                    uint32_t* const dst = reinterpret_cast<uint32_t*>(p.dq) + (first + (size_t)(tx >> 3) * p.heads) * words + 8 * cg + word;
+#pragma unroll
+                    for (int four = 0; four < 8; ++four)
+                        if (2 * word < channels)
+                            dst[(size_t)((four >> 1) * p.W + 4 * (four & 1)) * p.heads * words] = mine[(4 * four + (tx >> 3)) * 9 + word];
+                    __syncwarp();
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) f[q] = ahead[q];
+            }
+            return;
+        }
 #pragma unroll 2
         for (int pair = pair0; pair < pair1; pair += step) {
             if (!decode_pair_token(p, pair, w, i, tok, scalar)) continue;
@@ -739,12 +775,7 @@ __global__ void __launch_bounds__(32 * (2 + R / 8)) rib_bwd_finish_kernel(const 
                 v[2 * q] = pack_bf16x2(f[q].x * p.inv_sqrt_d, f[q].y * p.inv_sqrt_d);
                 v[2 * q + 1] = pack_bf16x2(f[q].z * p.inv_sqrt_d, f[q].w * p.inv_sqrt_d);
             }
-            if (kNarrow) {
-                uint32_t* dst = reinterpret_cast<uint32_t*>(p.dq + tok * p.narrow) + 8 * cg;
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    if (2 * e < channels) dst[e] = v[e];
-            } else if (p.dq_sectors) {
+            if (p.dq_sectors) {
                 st_global_v8(p.dq + tok * p.d + 16 * cg, v);
             } else {
                 uint4* dst = reinterpret_cast<uint4*>(p.dq + tok * p.d) + 2 * cg;
