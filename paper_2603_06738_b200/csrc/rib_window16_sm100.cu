@@ -325,7 +325,11 @@ rib_window16_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
 // (-lse log2e, -D) of the windows to come to tensor memory, a row being a TMEM lane to everybody.  (One set of warps for both, and lanes
 // that load whole rows: 215 us on 16 x 96 x 96 tokens, 6 heads of 32 channels, rank 16, 240 at rank 32.  dv in 32-byte stores, four lanes to a
 // row of dO and O and stores by warp 2 191 / 211, warps of their own, with dO from the stage, 180 / 201: 8000 cycles of waiting for
-// loads held up dV and dK~ of the next window.)
+// loads held up dV and dK~ of the next window.  That form lost up to 8 % where heads are narrow and a CTA has few windows, whose scalars then wait
+// for the first window's copies.  Those are asked for before the block's first barrier, the sums of dK~'s RIB columns are kept off the
+// hand-over of the accumulators, and 72 registers do without spills; us per call in a graph, before the warps of their own / with them / now: 64 x 64,
+// 4 heads of 24 channels 14.8 / 16.1 / 14.4; 96 x 96, 6 of 16 20.0 / 21.5 / 20.2; 16 x 96 x 96, 6 of 8 156 / 159 / 154, of 32 214 / 175 / 166.  Head-wise
+// tables, 4 x 96 x 96, 6 of 8: 43.9 / 46.9 / 46.0.)
 namespace bwd16 {
 constexpr int kThreads = 896, kStages = 2;
 constexpr uint32_t kQ = 0, kK = kWindowBytes, kV = 2 * kWindowBytes, kDO = 3 * kWindowBytes, kStageBytes = 4 * kWindowBytes;
@@ -367,6 +371,22 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
     const int count = (p.tiles - group0 + p.groups - 1) / p.groups;
     const uint32_t units = 4u * (uint32_t)count;
 
+    // (The loop is kept: unrolled, its addresses cost the arithmetic warps registers.)
+    auto load_window = [&](int t) {
+        const int st = t % kStages;
+        const Win16 w = decode_window(p, group0 + t * p.groups);
+        mbar_arrive_expect_tx(bar(kFull + st), kStageBytes);
+#pragma unroll 1
+        for (int patch = 0; patch < 4; ++patch) {
+            int Y0, X0;
+            patch_at(p, w, patch, Y0, X0);
+            const uint32_t at = base + st * kStageBytes + patch * kPatchContent;
+            tma_load_5d(at + kQ, &tm_q, bar(kFull + st), 0, head, X0, Y0, w.b);
+            tma_load_5d(at + kK, &tm_k, bar(kFull + st), 0, head, X0, Y0, w.b);
+            tma_load_5d(at + kV, &tm_v, bar(kFull + st), 0, head, X0, Y0, w.b);
+            tma_load_5d(at + kDO, &tm_do, bar(kFull + st), 0, head, X0, Y0, w.b);
+        }
+    };
     if (threadIdx.x == 0) {
         abort_flag[0] = 0; abort_flag[1] = 0;   // [1] stays 0: used by the drain waits
         for (int s = 0; s < kStages; ++s) { mbar_init(bar(kFull + s), 1); mbar_init(bar(kEmpty + s), 1); mbar_init(bar(kLd + s), 4); }
@@ -376,7 +396,8 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         for (int i = 0; i < 4; ++i) mbar_init(bar(kStaged + i), 4);
         mbar_init(bar(kDrain), 1); mbar_init(bar(kDrain + 1), 1);
         fence_barrier_init();
-        prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v); prefetch_tensormap(&tm_do);
+        fence_proxy_async();
+        load_window(0);                         // before the rows of the tables are staged and tensor memory is there
         prefetch_tensormap(&tm_dq); prefetch_tensormap(&tm_dk);
     }
     if (warp == 2) {
@@ -395,22 +416,11 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
 
     if (warp == 0) {
         if (lane == 0) {
-            int t = 0;
+            int t = 1;
             bool ok = true;
             for (; t < count; ++t) {
-                const int st = t % kStages, use = t / kStages;
-                if (use > 0 && !mbar_wait(bar(kEmpty + st), (use - 1) & 1, abort_flag, p.status)) { ok = false; break; }
-                const Win16 w = decode_window(p, group0 + t * p.groups);
-                mbar_arrive_expect_tx(bar(kFull + st), kStageBytes);
-                for (int patch = 0; patch < 4; ++patch) {
-                    int Y0, X0;
-                    patch_at(p, w, patch, Y0, X0);
-                    const uint32_t at = base + st * kStageBytes + patch * kPatchContent;
-                    tma_load_5d(at + kQ, &tm_q, bar(kFull + st), 0, head, X0, Y0, w.b);
-                    tma_load_5d(at + kK, &tm_k, bar(kFull + st), 0, head, X0, Y0, w.b);
-                    tma_load_5d(at + kV, &tm_v, bar(kFull + st), 0, head, X0, Y0, w.b);
-                    tma_load_5d(at + kDO, &tm_do, bar(kFull + st), 0, head, X0, Y0, w.b);
-                }
+                if (t >= kStages && !mbar_wait(bar(kEmpty + t % kStages), (t / kStages - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                load_window(t);
             }
             if (!ok)                            // gave up: let the copies already in flight land before the CTA may exit
                 for (int b2 = t > kStages ? t - kStages : 0; b2 < t; ++b2)
@@ -511,16 +521,15 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
         const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
         uint8_t *p_row = base_ptr + kOffP + (cq >> 1) * kHalf + row * 128, *ds_row = base_ptr + kOffDS + (cq >> 1) * kHalf + row * 128;
-        uint32_t seen[2] = {0u, 0u};
+        uint32_t seen = 0u;         // bit 4 I + 2 J + half
         for (uint32_t u = 0; u < units; ++u) {
             const uint32_t t = u >> 2, I = u & 1, J = (u >> 1) & 1;
             if ((u & 3) == 0) {
                 const Win16 w = decode_window(p, group0 + (int)t * p.groups);
-                seen[0] = attended(p, w, quarter >> 1);
-                seen[1] = attended(p, w, 2 + (quarter >> 1));
+                seen = attended(p, w, quarter >> 1) | attended(p, w, 2 + (quarter >> 1)) << 4;
                 if (!mbar_wait_warp(bar(kLd + (t & 1)), (t >> 1) & 1, abort_flag, p.status)) break;
             }
-            const bool on = ((I ? seen[1] : seen[0]) >> (2 * J + (cq >> 1))) & 1u;      // warp-uniform
+            const bool on = (seen >> (4 * I + 2 * J + (cq >> 1))) & 1u;      // warp-uniform
             if (!mbar_wait_warp(bar(kSFull), u & 1, abort_flag, p.status)) break;
             tc_fence_after();
             uint32_t pp[16], dd[16], ld[2], s[4][8], dp[4][8];
@@ -699,22 +708,27 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                     tmem_ld32(lanes + kColDK, a);
                     tmem_wait_ld();
                     write_row(stage + kK + J * kContentBytes, row, a, p.inv_sqrt_d);
-                    uint32_t sums[16];
-                    if (R == 16) {
-                        tmem_ld16(lanes + kColDK + kD, reinterpret_cast<uint32_t(&)[16]>(a));
-                        tmem_ld16(lanes + kColRib<R> + R * J, sums);
-                    } else {
-                        tmem_ld32(lanes + kColDK + kD, a);
-                    }
+                    if (R == 16) tmem_ld16(lanes + kColDK + kD, reinterpret_cast<uint32_t(&)[16]>(a));
+                    else tmem_ld32(lanes + kColDK + kD, a);
                     tmem_wait_ld();
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(kKVFree));
                     if (R == 16) {
+                        // behind the hand-over, which the next block's dV and dK~ wait for; the store is awaited with those of J = 1
+                        uint32_t sums[16];
+                        tmem_ld16(lanes + kColRib<R> + R * J, sums);
+                        tmem_wait_ld();
 #pragma unroll
                         for (int e = 0; e < 16; ++e) sums[e] = __float_as_uint(__uint_as_float(sums[e]) + __uint_as_float(a[e]));
-                        tmem_st16(lanes + kColRib<R> + R * J, sums);
-                        tmem_wait_st();
+                        if (t + 1 < count) {
+                            tmem_st16(lanes + kColRib<R> + R * J, sums);
+                        } else {
+                            float* const gk = p.dpk + table + (size_t)table_row(J * kTile + row) * p.r;
+#pragma unroll
+                            for (int c = 0; c < R; c += 4)
+                                if (c < p.r) add_columns(gk + c, sums + c, p.inv_sqrt_d);       // (the query rows carried sqrt(d / r))
+                        }
                     } else {
                         float* const gk = p.dpk + table + (size_t)table_row(J * kTile + row) * p.r;
 #pragma unroll
@@ -749,15 +763,6 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                 if (R == 16) tmem_ld16(lanes + kColDQ<R> + I * (kD + R) + kD, reinterpret_cast<uint32_t(&)[16]>(a));
                 else tmem_ld32(lanes + kColDQ<R> + I * (kD + R) + kD, a);
                 tmem_wait_ld();
-                if (R == 16) {
-                    uint32_t k[16];
-                    tmem_ld16(lanes + kColRib<R> + R * I, k);
-                    tmem_wait_ld();
-                    float* const gk = p.dpk + table + (size_t)table_row(I * kTile + row) * p.r;
-#pragma unroll
-                    for (int c = 0; c < R; c += 4)
-                        if (c < p.r) add_columns(gk + c, k + c, p.inv_sqrt_d);
-                }
                 float* const gq = p.dpq + table + (size_t)table_row(I * kTile + row) * p.r;
 #pragma unroll
                 for (int c = 0; c < R; c += 4)
