@@ -83,7 +83,8 @@ constexpr uint32_t kPolyMask = 0x88u;             // of every 8 score pairs: whi
 
 // kBetween: the output of the unit before is stored between the two halves of the exponentials, where its PV has completed (16 x 96 x 96
 // tokens, 6 heads, masked, rank 16 124 -> 115 us, 360 x 632 at rank 32 189 -> 175; behind both halves, where the next scores wait for it,
-// 126 and 192).  Not for heads of up to 16 channels, whose output half of the warps have no part in: 307 against 316 us.
+// 126 and 192).  Not for heads of up to 24 channels, whose output some of the warps have no part in: at 16 307 against 316 us; at 24, us per call in a
+// graph, masked, 4 heads, rank 8: 4 x 96 x 96 21.5 / 21.9, 256 x 256 33.7 / 34.5, 16 x 96 x 96 71.1 / 71.7, rank 24 72.2 / 72.5.
 template <int R, bool kBetween>
 __global__ void __launch_bounds__(kThreads, 1)
 rib_window16_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -855,7 +856,7 @@ bool sm100_window16_prefers(const Problem& p)
 }
 cudaError_t sm100_window16_fwd(const Problem& p, cudaStream_t stream)
 {
-    if (p.d > 16) return padded_rank(p.r) == 32 ? launch_win16_fwd<32, true>(p, stream) : launch_win16_fwd<16, true>(p, stream);
+    if (p.d > 24) return padded_rank(p.r) == 32 ? launch_win16_fwd<32, true>(p, stream) : launch_win16_fwd<16, true>(p, stream);
     return padded_rank(p.r) == 32 ? launch_win16_fwd<32, false>(p, stream) : launch_win16_fwd<16, false>(p, stream);
 }
 cudaError_t sm100_window16_bwd(const Problem& p, cudaStream_t stream)

@@ -21,6 +21,8 @@ CASES = [
     Workload("w16_partial", 2, 40, 56, 3, 24, 16, 16, 0, seed=506),
     Workload("w16_partial_s8", 1, 24, 72, 6, 32, 32, 16, 8, seed=507),
     Workload("w16_patch", 1, 8, 8, 2, 32, 16, 16, 8, seed=508),                             # one patch in the middle of the extension
+    Workload("w16_d24_r8_s8", 2, 32, 48, 4, 24, 8, 16, 8, seed=513),
+    Workload("w16_d24_r24_s8", 1, 48, 32, 3, 24, 24, 16, 8, seed=514),
     Workload("w16_d30_r18", 1, 48, 32, 6, 30, 18, 16, 8, seed=509),                         # zero-padded copies
 ]
 
