@@ -840,11 +840,13 @@ cudaError_t launch_win16_bwd(const Problem& p, cudaStream_t stream)
 
 // (sides that are no multiples of 8 have kernels of their own)
 bool sm100_window16(const Problem& p) { return p.M == 16 && p.s % 8 == 0 && p.H % 8 == 0 && p.W % 8 == 0 && !p.gate; }
-// Forward, this kernel against the general one, us with the launch (6 heads of 32 channels unless stated; 12 x 16: 12 heads of 16):
-//   whole windows          rank 16: 10 x 64 x 64 tokens 40 / 35, 256 x 256 60 / 50; rank 32: 41 / 40, 62 / 59; 12 x 16, rank 24: 65 / 63, 98 / 96;
-//   with a mask            rank 16: 16 x 96 x 96 115 / 135; rank 32: 10 x 64 x 64 44 / 64; 12 x 16, rank 24: 4 x 96 x 96 60 / 90;
-//   beyond the map         rank 16: 48 x 40 10.7 / 10.8, 104 x 120 18.7 / 18.8, 120 x 200 27.0 / 27.0, 200 x 328 57 / 54, 360 x 632 171 / 162;
-//                          rank 32: 120 x 200 27 / 31, 360 x 632 174 / 203; 12 x 16, rank 24: 307 / 372.
+// Forward, this kernel against the general one, us per call in a graph (6 heads of 32 channels unless stated; 12 x 16: 12 heads of 16):
+//   whole windows          rank 16: 10 x 64 x 64 tokens 35 / 28, 256 x 256 52 / 41, 16 x 96 x 96 108 / 83; rank 32: 36 / 33, 54 / 51; 12 x 16, rank 24:
+//                          4 x 96 x 96 53 / 51, 256 x 256 94 / 86;
+//   with a mask            rank 16: 64 x 64 9.0 / 12.1, 10 x 64 x 64 35 / 44, 256 x 256 52.8 / 53.6, 4 x 256 x 256 190 / 195, 16 x 96 x 96 110 / 128; rank 32:
+//                          10 x 64 x 64 36 / 54, 256 x 256 54 / 66; 12 x 16, rank 24: 4 x 96 x 96 53 / 79; 4 heads of 24, rank 8: 22 / 27;
+//   beyond the map         rank 16: 48 x 40 8.8 / 9.2, 104 x 120 16.0 / 16.5, 120 x 200 24.4 / 24.7, 152 x 264 36.6 / 33.3, 200 x 328 55 / 52, 360 x 632
+//                          168 / 161; 6 x 8, rank 8 157 / 152, 6 x 24 162 / 163; rank 32: 120 x 200 25 / 29, 360 x 632 171 / 202; 12 x 16, rank 24: 310 / 368.
 // So whole windows stay with the general kernel, masks come here, and windows beyond the map come here with RIB rows of 32 elements or
 // while there is little work (120 x 200 tokens are four windows per SM).
 // This kernel has the fast form of the softmax only (one exponential in four on the FMA pipe, lse from rounded probabilities):
