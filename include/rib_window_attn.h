@@ -378,8 +378,8 @@ long long rib_kernel_launches(void);
 
 /*
  * The tcgen05 kernels address their operands through TMA tensor maps, which depend on the base pointer and the
- * shape only; the library keeps the last 64 distinct ones, so a call that repeats an earlier call's buffers and
- * shape encodes none.  Writes how many maps were served from that cache (`hits`) and how many had to be encoded
+ * shape only; the library keeps 2048 of them (256 sets of 8, least recently asked for out first), more than both
+ * passes of 64 layers need, so a call that repeats an earlier call's buffers and shape encodes none.  Writes how many maps were served from that cache (`hits`) and how many had to be encoded
  * (`misses`) in this process so far; either pointer may be NULL.
  */
 void rib_tensor_map_cache_counts(long long* hits, long long* misses);

@@ -212,21 +212,32 @@ inline EncodeTiledFn encode_fn()
 }
 
 // Tensor maps depend on the base pointer and the shape only, and a training loop calls with the same few buffers
-// over and over: the last kMapCacheSlots distinct maps of the process are kept (round-robin replacement, one
-// mutex), so a repeated call encodes nothing.  The key holds every argument of the encoding.
+// over and over: the maps of the process are kept in 256 sets of 8, the one that was not asked for longest giving way (one mutex), so
+// a repeated call encodes nothing.  A layer's two passes need up to 9 maps of their own (general kernels: q, k, v and Pk of the forward, dout, Pk as
+// 64-byte rows, dk and dv in boxes of 4 rows, Pq in the workspace), so the 64 layers that the cycle entry points take need 576.  The key holds
+// every argument of the encoding.
 struct MapKey {
     const void* ptr; long long a, b; int kind, c, d, e, f, g;
     bool operator==(const MapKey& o) const
     {
         return ptr == o.ptr && a == o.a && b == o.b && kind == o.kind && c == o.c && d == o.d && e == o.e && f == o.f && g == o.g;
     }
+    unsigned hash() const
+    {
+        unsigned long long h = 0;
+        for (unsigned long long x : {(unsigned long long)(uintptr_t)ptr, (unsigned long long)a, (unsigned long long)b, (unsigned long long)(uint32_t)kind << 32 | (uint32_t)c,
+                                     (unsigned long long)(uint32_t)d << 32 | (uint32_t)e, (unsigned long long)(uint32_t)f << 32 | (uint32_t)g}) {
+            h = (h ^ x) * 0x9e3779b97f4a7c15ull;
+            h ^= h >> 32;
+        }
+        return (unsigned)h;
+    }
 };
-constexpr int kMapCacheSlots = 64;
+constexpr int kMapSets = 256, kMapWays = 8;
 struct MapCache {
+    struct Entry { CUtensorMap map; MapKey key; unsigned long long asked; };      // asked: when last (0: empty)
     std::mutex mutex;
-    MapKey keys[kMapCacheSlots];
-    CUtensorMap maps[kMapCacheSlots];
-    int used = 0, next = 0;
+    Entry entries[kMapSets][kMapWays];
     long long hits = 0, misses = 0;
 };
 inline MapCache& map_cache()
@@ -239,13 +250,15 @@ inline bool cached_map(CUtensorMap* map, const MapKey& key, Encode encode)
 {
     MapCache& c = map_cache();
     std::lock_guard<std::mutex> lock(c.mutex);
-    for (int i = 0; i < c.used; ++i)
-        if (c.keys[i] == key) { *map = c.maps[i]; ++c.hits; return true; }
+    MapCache::Entry *const set = c.entries[key.hash() % kMapSets], *slot = set;
+    const unsigned long long now = (unsigned long long)(c.hits + c.misses) + 1;
+    for (int i = 0; i < kMapWays; ++i) {
+        if (set[i].asked && set[i].key == key) { *map = set[i].map; set[i].asked = now; ++c.hits; return true; }
+        if (set[i].asked < slot->asked) slot = set + i;
+    }
     if (!encode(map)) return false;
     ++c.misses;
-    const int slot = c.used < kMapCacheSlots ? c.used++ : (c.next = (c.next + 1) % kMapCacheSlots);
-    c.keys[slot] = key;
-    c.maps[slot] = *map;
+    *slot = MapCache::Entry{*map, key, now};
     return true;
 }
 inline void map_cache_counts(long long* hits, long long* misses)

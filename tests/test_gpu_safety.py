@@ -200,3 +200,32 @@ def test_a_repeated_call_encodes_no_tensor_map():
     hits1, misses1 = binding.rib_tensor_map_cache_counts()
     assert misses1 == misses0 and hits1 == hits0 + 3 * 10      # 4 maps per forward, 6 per backward call
     assert binding.rib_query_status() == 0
+
+
+@pytest.mark.parametrize("layers", [8, 64])
+def test_the_maps_of_a_cycle_with_buffers_of_its_own_stay(layers):
+    """Both passes of layers of windows of 32 (general kernels: 4 maps and 8), no buffer shared but the workspace, up to the 64 layers
+    that the cycle entry points take: from the second round on nothing is encoded."""
+    wl = Workload("cache_w32", 1, 32, 32, 1, 32, 16, 32, 0, seed=70)
+    _, gpu = make(wl, with_dout=True)
+    names = ("q", "k", "v", "pq", "pk", "dout")
+    own = [{name: gpu[name].clone() for name in names} for _ in range(layers)]
+    outs = [run_fwd(layer, wl) for layer in own]
+    grads = [[torch.empty_like(layer["q"]) for _ in range(3)] + [torch.empty(wl.window ** 2, wl.r, device="cuda") for _ in range(2)] for layer in own]
+    ws = torch.empty(binding.rib_window_attn_bwd_workspace(wl.B, wl.H, wl.W, wl.heads, wl.d, wl.r, wl.window), dtype=torch.uint8, device="cuda")
+    sizes, lib = (wl.B, wl.H, wl.W, wl.heads, wl.d, wl.r, wl.window, wl.shift), binding.library()
+
+    def step():
+        for layer, (out, lse), res in zip(own, outs, grads):
+            inputs = [layer[name].data_ptr() for name in ("q", "k", "v", "pq", "pk")]
+            assert lib.rib_window_attn_fwd(*inputs, *sizes, out.data_ptr(), lse.data_ptr(), None) == 0
+            assert lib.rib_window_attn_bwd(*inputs, out.data_ptr(), lse.data_ptr(), layer["dout"].data_ptr(), *sizes, *(t.data_ptr() for t in res),
+                                           ws.data_ptr(), ws.numel(), None) == 0
+
+    step()
+    hits0, misses0 = binding.rib_tensor_map_cache_counts()
+    step()
+    torch.cuda.synchronize()
+    hits1, misses1 = binding.rib_tensor_map_cache_counts()
+    assert (misses1 - misses0, hits1 - hits0) == (0, layers * (4 + 8))
+    assert binding.rib_query_status() == 0
