@@ -93,7 +93,6 @@ template <int R> struct Cols {
     static constexpr uint32_t kColDV = R == 16 ? 384 : 320, kColDK = kColDV + kD, kColDQ = kColDK + kD + R;
     static_assert(kColDQ + kD + R <= 512, "tensor memory has 512 columns");
 };
-constexpr uint32_t kHalfCols = kTile / 2;
 constexpr uint32_t kTmemCols = 512;
 
 constexpr uint32_t kIdescT32 = idesc_bf16_f32(kTile, kD, true);               // A in TMEM, B MN-major, N = 32

@@ -10,7 +10,6 @@ struct SmallWindowParams {
     const __nv_bfloat16* pq;
     const __nv_bfloat16* pk;
     const __nv_bfloat16* out;  // backward at 16 x 16
-    const __nv_bfloat16* dout;
     const float* lse_in;       // backward
     float* lse;                // forward, may be null
     float* dpq;

@@ -294,7 +294,6 @@ rib_window16_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kPReady + g));
-            ok = true;
             if (u == 2 * count - 1) {
                 // the last unit
                 ok = mbar_wait_warp(bar(kOFull + g), t & 1, abort_flag, p.status);
@@ -820,7 +819,7 @@ cudaError_t launch_win16_bwd(const Problem& p, cudaStream_t stream)
     if (cudaError_t e = setup.prepare(bwd16::rib_window16_bwd_kernel<R>, bwd16::kSmemBytes, &sm_count)) return e;
     SmallWindowParams w{};
     const int grid = fill_small_window(p, sm_count, p.nWy, p.nWx, &w);
-    w.out = p.out; w.dout = p.dout; w.lse_in = p.lse_in; w.dpq = p.dpq; w.dpk = p.dpk;
+    w.out = p.out; w.lse_in = p.lse_in; w.dpq = p.dpq; w.dpk = p.dpk;
     const int tables = pos_tables(p), per_table = 256 * p.r, blocks = (tables * per_table + 255) / 256 < 64 ? (tables * per_table + 255) / 256 : 64;
     {
         ProfileScope scope(RIB_KERNEL_WINDOW16_CLEAR, stream);
