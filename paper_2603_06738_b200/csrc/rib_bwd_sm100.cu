@@ -30,7 +30,7 @@
 // bf16 and sums the RIB columns over pairs into dPq.  The RIB columns of dK~ are written per pair
 // and summed over pairs by the same finishing kernel into dPk.
 //
-// Roles (768 threads): warp 0 TMA producer; three MMA-issuing warps (the tensor pipe takes
+// Roles (896 threads at rank 16 on full windows, else 768): warp 0 TMA producer; three MMA-issuing warps (the tensor pipe takes
 // instructions from several warps at once, and one thread issuing everything was the bottleneck):
 // warp 1 issues S^T and dP^T, warp 2 (also the TMEM allocator) dV and dK~, warp 3 dQ~; warps 4-11
 // P/dS arithmetic of the even half-tiles, warps 12-19 of the odd ones (a warp per 32 key rows and 32
@@ -555,6 +555,9 @@ rib_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 }
 #pragma unroll
                 for (int col = 0; col < 16; col += 4) {
+                    // The adds of a tile in one burst fill the queue that all warps' loads, stores and fences go through: a pause after each one, at
+                    // rank 32 after every second one, spreads them over the tile's time (16 x 96 x 96 tokens in windows of 32: no pause
+                    // 502 / 589 us at rank 16 / 32, 20 ns 468 / 568, 40 ns 488 / 565).
                     red_add_f32x4(dst, a + col);
                     dst += 4 * (size_t)p.n;
                     if (R == 16 || (col & 4)) __nanosleep(20);

@@ -249,7 +249,8 @@ __global__ void __launch_bounds__(kPwThreads, 1) rib_cla_bwd_pw_kernel(const Cla
 // Depth-wise part.  A block takes a tile of 16 x 16 pixels and 32 channels: the 18 x 18 halo of dY (fp32) and of X (bf16) goes to
 // shared memory by cp.async (zero outside the map), thread (channel pair, tile row) walks the 16 pixels of its row with packed
 // fp32 FMAs.  8 x 96 x 96 pixels of 192 channels 45.4 -> 38.2 us by event hooks (one channel per thread, tiles of 8 x 16 and halos through
-// registers were bound by their own instructions, 62 % of the issue slots), 4 x 96 x 96 24.9 -> 18.8.  Copies alone take 25 us, arithmetic
+// registers were bound by their own instructions, 62 % of the issue slots), 4 x 96 x 96 27 -> 24; one map, whose blocks have a tile each, 96 x 96 of 64,
+// 128 and 192 channels 13.6 -> 12.6, 15.6 -> 13.0, 14.7 -> 13.7, two 24 -> 17, 24 -> 18.5, 18.7 -> 16.7, 64 x 64 of 192 10.5 both.  Copies alone take 25 us, arithmetic
 // alone 25: two blocks overlap the one with the other only in part.  Three blocks per SM (80 registers, spills) 39.2; strips of 8 rows
 // with the next rows copied under the arithmetic, 12 warps per SM, 39.3.
 // ------------------------------------------------------------------------------------------------------------------

@@ -20,7 +20,8 @@
 // back with P in it and S(u + 3) goes there once PV(u) has completed: scores of one tile's next block are under way while the
 // other tile's exponentials run, and between a block's scores and its P a softmax warp waits for nobody.  (Scores in one buffer per
 // tile and P in columns of its own, each with a barrier "free" that every block asked for and answered: 256 x 256 tokens in windows of 64
-// 425 -> 393 us, and with the exponentials in pieces of 16 keys 369; 360 x 640 in windows of 64 1400 -> 1220.)
+// 425 -> 393 us, and with the exponentials in pieces of 16 keys 369; 360 x 640 in windows of 64 1400 -> 1220.  These are single passes; one
+// after the other, where the card meets its power cap, they take 442 -> 399 and 1488 -> 1332.)
 //
 // Two threads own a query row: one takes keys 0-63 of every block and the other keys 64-127, which
 // puts four softmax warps on every SM sub-partition.

@@ -356,8 +356,8 @@ cudaError_t sm100_bwd_repacked(const Problem& p, cudaStream_t stream, int* launc
     const long long tstride = (long long)p.n * pp.r;
     // The preparation kernel reads out, and the finishing kernel writes dq, in rows of the caller's width (those of the general kernel,
     // where no columns of the tables travel in the spare channels): two copies less.  (8 x 96 x 96 tokens, 30 channels, rank 18, windows
-    // of 32: all copies of both passes 160 -> 80 us with one launch per pass, the two kernels 87 -> 105 us; both passes 721 -> 660 us.
-    // The drain warps of the main kernel have no registers left to write dk and dv so.)
+    // of 32: all copies of both passes 160 -> 80 us with one launch per pass, the two kernels 87 -> 105 us, both passes 721 -> 660 us; the two
+    // kernels take 74 us now.  dk and dv leave the main kernel by TMA, which has no rows of 60 bytes: its strides are multiples of 16 bytes.)
     const bool direct = sm100_bwd_takes_narrow(pp) && !rank_tail(p);
     pp.narrow = direct && p.d % 8 ? p.d : 0;
     RowCopies in{};
