@@ -321,23 +321,23 @@ rib_window16_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
 //
 // Roles (896 threads): warp 0 TMA loads; warp 1 issues S and dP, warp 3 dV, dK~ and dQ~; warp 2 owns the TMEM allocation; warps
 // 4-19 P and dS (four threads per query row, 32 keys each); warps 20-23 move the gradients out, dv from registers, dk and dq through the
-// shared memory of the window's own rows, from where warp 2 stores them by TMA and gives the stage back; warps 24-27 write
+// shared memory of the window's own rows and TMA stores; warps 24-27 write
 // (-lse log2e, -D) of the windows to come to tensor memory, a row being a TMEM lane to everybody.  (One set of warps for both, and lanes
 // that load whole rows: 215 us on 16 x 96 x 96 tokens, 6 heads of 32 channels, rank 16, 240 at rank 32.  dv in 32-byte stores, four lanes to a
-// row of dO and O and stores by warp 2 191 / 211, warps of their own, with dO from the stage, 180 / 201: 8000 cycles of waiting for
+// row of dO and O 191 / 211, warps of their own, with dO from the stage, 180 / 201: 8000 cycles of waiting for
 // loads held up dV and dK~ of the next window.  That form lost up to 8 % where heads are narrow and a CTA has few windows, whose scalars then wait
 // for the first window's copies.  Those are asked for before the block's first barrier, the sums of dK~'s RIB columns are kept off the
-// hand-over of the accumulators, and 72 registers do without spills; us per call in a graph, before the warps of their own / with them / now: 64 x 64,
-// 4 heads of 24 channels 14.8 / 16.1 / 14.4; 96 x 96, 6 of 16 20.0 / 21.5 / 20.2; 16 x 96 x 96, 6 of 8 156 / 159 / 154, of 32 214 / 175 / 166.  Head-wise
-// tables, 4 x 96 x 96, 6 of 8: 43.9 / 46.9 / 46.0.)
+// hand-over of the accumulators, 72 registers do without spills, and the TMA stores, which warp 2 issued behind barriers of their own then, are
+// warp 20's again; us per call in a graph, before the warps of their own / with them / now: 64 x 64, 4 heads of 24 channels 14.8 / 16.1 / 14.6;
+// 96 x 96, 6 of 16 20.1 / 21.5 / 20.2; 16 x 96 x 96, 6 of 8 156 / 159 / 152, of 32 214 / 175 / 162; head-wise tables, 4 x 96 x 96, 6 of 8
+// 43.7 / 46.9 / 44.3.)
 namespace bwd16 {
 constexpr int kThreads = 896, kStages = 2;
 constexpr uint32_t kQ = 0, kK = kWindowBytes, kV = 2 * kWindowBytes, kDO = 3 * kWindowBytes, kStageBytes = 4 * kWindowBytes;
 constexpr uint32_t kOffRib = kStages * kStageBytes;                           // query RIB rows, key RIB rows
 constexpr uint32_t kHalf = kTile * 128;                                       // P, dS: [2 halves of 64 keys][128 queries][128 bytes], SWIZZLE_128B
 constexpr uint32_t kOffP = kOffRib + 2 * kWindowBytes, kOffDS = kOffP + 2 * kHalf, kOffBar = kOffDS + 2 * kHalf;
-enum Bar { kFull = 0, kEmpty = kFull + kStages, kSFull = kEmpty + kStages, kSFree, kPReady, kPDone, kSReady, kSDone, kAcc, kKVFree, kQFree, kLd, kLdFree = kLd + 2, kStaged, kDrain = kStaged + 4,
-           kNumBars = kDrain + 2 };      // kStaged: 2 * parity of the window + key block
+enum Bar { kFull = 0, kEmpty = kFull + kStages, kSFull = kEmpty + kStages, kSFree, kPReady, kPDone, kSReady, kSDone, kAcc, kKVFree, kQFree, kLd, kLdFree = kLd + 2, kDrain, kNumBars = kDrain + 2 };
 constexpr uint32_t kOffMisc = kOffBar + kNumBars * 8;
 constexpr uint32_t kSmemBytes = kOffMisc + 16 + 1024;
 static_assert(kOffP % 1024 == 0 && kSmemBytes <= 232448, "shared memory of one CTA");
@@ -393,7 +393,6 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         mbar_init(bar(kSFull), 1); mbar_init(bar(kSFree), 16); mbar_init(bar(kPReady), 16); mbar_init(bar(kPDone), 1); mbar_init(bar(kSReady), 16); mbar_init(bar(kSDone), 1);
         mbar_init(bar(kAcc), 1); mbar_init(bar(kKVFree), 4); mbar_init(bar(kQFree), 4);
         mbar_init(bar(kLdFree), 16);
-        for (int i = 0; i < 4; ++i) mbar_init(bar(kStaged + i), 4);
         mbar_init(bar(kDrain), 1); mbar_init(bar(kDrain + 1), 1);
         fence_barrier_init();
         fence_proxy_async();
@@ -451,33 +450,6 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         if (elect_one()) mma_commit(bar(kDrain));
         __syncwarp();
         mbar_wait(bar(kDrain), 0, abort_flag + 1, p.status);
-    } else if (warp == 2) {
-        // ---- gradient rows that lie staged in the window's own rows leave by TMA; then the stage may be filled again
-        if (lane == 0) {
-            for (int t = 0; t < count; ++t) {
-                const int st = t % kStages;
-                const Win16 w = decode_window(p, group0 + t * p.groups);
-                bool ok = true;
-                for (int J = 0; J < 2 && ok; ++J) {
-                    ok = mbar_wait(bar(kStaged + 2 * (t & 1) + J), (t >> 1) & 1, abort_flag, p.status);
-                    if (!ok) break;
-                    const uint32_t at = base + st * kStageBytes;
-                    for (int patch = 0; patch < 4; ++patch) {
-                        int Y0, X0;
-                        patch_at(p, w, patch, Y0, X0);
-                        if (Y0 >= p.H || X0 >= p.W) continue;
-                        if ((patch >> 1) == J) tma_store_5d(&tm_dk, at + kK + patch * kPatchContent, 0, head, X0, Y0, w.b);
-                        if (J == 1) tma_store_5d(&tm_dq, at + kQ + patch * kPatchContent, 0, head, X0, Y0, w.b);
-                    }
-                    bulk_commit_group();
-                }
-                if (!ok) break;
-                bulk_wait_group_read<0>();              // (this thread's own stores)
-                mbar_arrive(bar(kEmpty + st));
-            }
-            bulk_wait_group<0>();
-        }
-        __syncwarp();
     } else if (warp == 3) {
         // ---- dV of a unit once P is stored, dK~ and dQ~ once dS is, and the accumulators that it starts have been read
         constexpr uint64_t kDescT = smem_desc_const(kHalf, 1024, kSwizzle128B);         // MN-major: the two 64-key halves one leading step apart
@@ -606,7 +578,7 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         const uint32_t line = (uint32_t)(p.W * p.heads * p.d), in_line = (uint32_t)((lane >> 2) * p.heads * p.d + 8 * (lane & 3));
         for (int t = 0; t < count; ++t) {
             // (The columns are free by then in any case: the stage is filled again after window t - 2.  But loads of `out` that run further ahead
-            // cost the kernel more than they save: without this wait 16 x 96 x 96 tokens, 6 heads of 32 channels, rank 16 180 us instead of 165.)
+            // cost the kernel more than they save: without this wait 16 x 96 x 96 tokens, 6 heads of 32 channels, rank 16 180 us instead of 162.)
             if (t >= 1 && !mbar_wait_warp(bar(kLdFree), (t - 1) & 1, abort_flag, p.status)) break;
             tc_fence_after();
             // D = dO . O: four lanes take a row (8 channels each), an instruction the 8 rows of a line of tokens; dO lies in the stage.  (With a row per
@@ -682,6 +654,7 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             uint8_t* const stage = base_ptr + st * kStageBytes;
             const Win16 w = decode_window(p, group0 + t * p.groups);
             for (int J = 0; J < 2; ++J) {
+                // (the vote of the named barrier below keeps the four warps together)
                 ok = mbar_wait_warp(bar(kAcc), J, abort_flag, p.status);
                 if (ok) {
                     tc_fence_after();
@@ -751,10 +724,24 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                         if (lane == 0) mbar_arrive(bar(kQFree));
                     }
                     fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kStaged + 2 * (t & 1) + J));
                 }
-                if (!ok) break;
+                if (!named_barrier_and(1, 128, ok)) { ok = false; break; }
+                if (warp == 20 && lane == 0) {
+                    const uint32_t at = base + st * kStageBytes;
+                    for (int patch = 0; patch < 4; ++patch) {
+                        int Y0, X0;
+                        patch_at(p, w, patch, Y0, X0);
+                        if (Y0 >= p.H || X0 >= p.W) continue;
+                        if ((patch >> 1) == J) tma_store_5d(&tm_dk, at + kK + patch * kPatchContent, 0, head, X0, Y0, w.b);
+                        if (J == 1) tma_store_5d(&tm_dq, at + kQ + patch * kPatchContent, 0, head, X0, Y0, w.b);
+                    }
+                    bulk_commit_group();
+                    if (J == 1) {
+                        bulk_wait_group_read<0>();
+                        mbar_arrive(bar(kEmpty + st));
+                    }
+                }
+                __syncwarp();
             }
         }
         if (ok) {
@@ -771,6 +758,8 @@ rib_window16_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                     if (c < p.r) add_columns(gq + c, a + c, p.inv_sqrt_r);
             }
         }
+        if (warp == 20 && lane == 0) bulk_wait_group<0>();
+        __syncwarp();
     }
     tc_fence_before();
     __syncthreads();

@@ -19,7 +19,7 @@ class Backward(Model):
         for name in ("grad", "drain", "load", "scalars"):
             self.scale[name] = self.rng.choice((0.1, 1.0, 5.0))
         self.scale["store"] = self.rng.choice((0.1, 1.0, 30.0))
-        self.counts = dict.fromkeys(("sfree", "pready", "sready", "ldfree", "ld", "kvfree", "qfree", "staged"), len(WARPS))
+        self.counts = dict.fromkeys(("sfree", "pready", "sready", "ldfree", "ld", "kvfree", "qfree", "vote"), len(WARPS))
 
     def arrive(self, bar, count=1):
         super().arrive(bar, self.counts.get(bar if isinstance(bar, str) else bar[0], 1))
@@ -34,9 +34,6 @@ class Backward(Model):
             self.finished.add(what)
             self.arrive(bar)
         self.later(self.delay(name), complete)
-
-    def staged(self, t, J):
-        return (("staged", J), t) if self.fault == "staged" else (("staged", 2 * (t & 1) + J), t >> 1)
 
     def producer(self):
         for t in range(self.windows):
@@ -134,17 +131,15 @@ class Backward(Model):
                     self.finished.add(("q", t, warp))
                     self.arrive("qfree")
                 self.finished.add(("staged", t, J, warp))
-                self.arrive(self.staged(t, J)[0])
-
-    def storer(self):
-        for t in range(self.windows):
-            for J in range(2):
-                yield ("wait", *self.staged(t, J))
-                assert self.all_done("staged", t, J) and ("window", t + 2) not in self.issued
-                yield "delay", self.delay("store")
-                self.copy("store", ("out", t, J), "group")
-            yield "group", 2 * t + 2
-            self.arrive(("empty", t & 1))
+                if self.fault != "vote":
+                    self.arrive("vote")
+                    yield "wait", "vote", 2 * t + J
+                if warp == 0:                        # its thread stores the rows of all
+                    assert self.all_done("staged", t, J) and ("window", t + 2) not in self.issued, "rows that are not there yet"
+                    self.copy("store", ("out", t, J), "group")
+                    if J == 1:
+                        yield "group", 2 * t + 2
+                        self.arrive(("empty", t & 1))
 
     def wait_group(self, process, stores):
         """Stores end in any order: asked for again until all are read."""
@@ -167,7 +162,7 @@ class Backward(Model):
 
     def run(self):
         self.pipe = {}
-        processes = [self.producer(), self.scores(), self.gradients(), self.storer()]
+        processes = [self.producer(), self.scores(), self.gradients()]
         for w in WARPS:
             processes += [self.arithmetic(w), self.scalars(w), self.drain(w)]
         for process in processes:
@@ -184,9 +179,9 @@ def test_every_wait_sees_its_own_phase(windows):
         Backward(windows, seed).run()
 
 
-@pytest.mark.parametrize("fault", ["staged", "scalars"])
+@pytest.mark.parametrize("fault", ["vote", "scalars"])
 def test_the_model_finds_a_rule_that_is_left_out(fault):
-    """staged: rows announced per key block, whatever the parity of the window.  scalars: their columns refilled without a look at the windows
+    """vote: rows stored without the barrier of the warps that stage them.  scalars: their columns refilled without a look at the windows
     under way (dO from global memory, say)."""
     found = 0
     for windows in (3, 8):
