@@ -4,6 +4,7 @@
 #include "rib_common.cuh"
 #include "sm100_primitives.cuh"
 
+#include <string.h>
 #include <mutex>
 
 namespace rib {
@@ -239,6 +240,7 @@ struct MapCache {
     std::mutex mutex;
     Entry entries[kMapSets][kMapWays];
     long long hits = 0, misses = 0;
+    MapCache() { memset(static_cast<void*>(entries), 0, sizeof entries); }      // its 512 KB of pages once, not one by one in later calls
 };
 inline MapCache& map_cache()
 {
