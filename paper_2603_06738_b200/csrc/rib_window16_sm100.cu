@@ -5,11 +5,11 @@
 // memory) exceeds its arithmetic.  Here a CTA keeps to one head (CTA c: head c mod heads), stages the head's RIB rows once,
 // takes whole windows one after the other and lets them overlap, and no gradient but those of the tables is summed
 // outside the chip.  What bounds it: the serial program of the softmax (arithmetic) warps.  A unit of the forward (128 rows x 256
-// keys) takes about 3600 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) 3000 at rank 16 and 32 channels:
+// keys) takes about 3600 cycles, of which the exp pipe is busy 1540; a unit of the backward (128 x 128) 2850 at rank 16 and 32 channels:
 // 200 until its scores are there, 1500 of loads and exponentials, 1000 of stores of P and dS and fences, with 1470 cycles of MMAs
 // beside it.  Measured by event hooks against the general kernels (4 x 96 x 96 tokens, 12 heads of 16 channels, rank 24, shift 8,
-// masked): forward 60 against 84 us, backward 13 (two clearings) + 97 against 27 + 125 + 35 us; backward on 16 x 96 x 96 tokens, 6 heads of 32
-// channels: rank 16 13 + 172 against 48 + 197 + 56, rank 32 13 + 193 against 56 + 228 + 95.
+// masked): forward 60 against 84 us, backward 13 (two clearings) + 95 against 27 + 125 + 35 us; backward on 16 x 96 x 96 tokens, 6 heads of 32
+// channels: rank 16 13 + 166 against 48 + 197 + 56, rank 32 13 + 190 against 56 + 228 + 95.
 //
 // Windows may be shifted (multiples of 8), masked, or reach beyond the map (sides multiples of 8): a window is four 8x8-token
 // patches (one TMA box each), and a query patch attends to a key patch or not.
